@@ -3,7 +3,7 @@
 // The kernels live in the .cuh files next to this one:
 //   hash_kernels.cuh, hash_tc_kernels.cuh   Eq. 2 on many rows (he_hash_keys, phase 1 of he_prefill_compress)
 //   decode_kernels.cuh, decode_sm_kernels.cuh   Algorithm 1 lines 1-5 (he_decode_step)
-//   prefill_kernels.cuh, prefill_tc_kernels.cuh   the prompt-encoding replay and the K/V gather (phases 2, 3 of
+//   prefill_kernels.cuh, prefill_block_kernels.cuh   the prompt-encoding replay and the K/V gather (phases 2, 3 of
 //                                                 he_prefill_compress)
 //
 // Eq. 2 is evaluated in one of two ways. CUDA cores (fp32 rows, odd head sizes, small calls, the per-unit decode
@@ -32,8 +32,8 @@
 #include "hash_tc_kernels.cuh"
 #include "hashevict.h"
 #include "oneshot_kernels.cuh"
+#include "prefill_block_kernels.cuh"
 #include "prefill_kernels.cuh"
-#include "prefill_tc_kernels.cuh"
 
 using namespace he;
 
@@ -452,51 +452,109 @@ int launch_replay_reg(const ReplayArgs& a, long long units, cudaStream_t stream)
   return launch_replay_smem<WORDS, GT>(a, units, stream);
 }
 
-// Tensor-core replay: one persistent CTA per SM, for budgets up to 12288 slots. Up to 4096 slots the unit's tables sit in
-// shared memory, beyond that they are the cache's own arrays.
-template <int WORDS, bool GLOBAL_TABLE, bool FP8, bool PROT = false, bool RUNS = true>
-int launch_replay_tc_one(const ReplayArgs& a0, long long units, cudaStream_t stream) {
-  ReplayArgs a = a0;
-  a.smem_slots = (a.cfg.max_budget + kRtTile - 1) / kRtTile * kRtTile;
-  const size_t smem = rt_layout(WORDS, a.smem_slots, a.cfg.group_size, !GLOBAL_TABLE, FP8).total;
-  if (int rc = set_smem(prefill_replay_tc_kernel<WORDS, GLOBAL_TABLE, FP8, PROT, RUNS>, smem)) return rc;
-  int sms = 0;
+// Block replay (prefill_block_kernels.cuh) on `ncta` CTAs per unit. At least 120 KB of shared memory are asked for, so
+// that an SM never hosts two of its CTAs: each takes all of tensor memory, and one that waited for another's while its
+// cluster peers wait for it could wait for good.
+constexpr size_t kRbMinSmem = 120 * 1024;
+constexpr size_t kMaxDynSmem = 227 * 1024 - 2048;  // dynamic shared memory of a CTA beside the kernel's static arrays
+
+// Shared memory of the block replay with as many operand stages as fit (fewer for large two-word tables); 0: does not fit.
+size_t rb_fit(int words, int slots, int G, int ncta, int* lg_stage, int* abuf) {
+  for (*abuf = 2; *abuf >= 1; --*abuf)
+    for (*lg_stage = 2; *lg_stage >= 1; --*lg_stage) {
+      const size_t smem = rb_layout(words, slots, G, ncta, 1 << *lg_stage, *abuf).total;
+      if (smem <= kMaxDynSmem) return smem < kRbMinSmem ? kRbMinSmem : smem;
+    }
+  return 0;
+}
+
+template <int WORDS, int GT, bool PROT>
+int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t stream) {
+  auto kernel = prefill_replay_block_kernel<WORDS, GT, PROT>;
+  RbArgs ra{};
+  ra.r = a;
+  ra.r.smem_slots = (a.cfg.max_budget + kRbTile - 1) / kRbTile * kRbTile;
+  int sms = 0, dev = 0;
   if (int rc = sm_count(&sms)) return rc;
-  const int nbins = sms < kMaxBins ? sms : kMaxBins;
-  // a step of this kernel costs about 400 cycles of resolver time plus 0.06 cycles per slot of tile work
-  prefill_schedule_kernel<<<1, kSchedThreads, 0, stream>>>(a.cfg, a.ca.budget, a.prompt_len, nbins, a.sched, 6700);
-  HE_CUDA_CHECK(cudaGetLastError());
-  const long long grid = units < sms ? units : sms;
-  prefill_replay_tc_kernel<WORDS, GLOBAL_TABLE, FP8, PROT, RUNS><<<(unsigned)grid, kRtThreads, smem, stream>>>(a);
-  HE_CUDA_CHECK(cudaGetLastError());
+  HE_CUDA_CHECK(cudaGetDevice(&dev));
+  // Cluster size: a block costs a CTA about 8000 cycles of settling, 380 per tile of its own and 3000 for the exchange with
+  // its peers; the number of rounds is what the clusters that fit the GPU need for the units.
+  static int max_clusters[64][4] = {};
+  const int tiles = ra.r.smem_slots / kRbTile;
+  double best = 0.;
+  int best_lg = -1;
+  for (int lg = 0; (1 << lg) <= kRbMaxCluster && (lg == 0 || (1 << lg) <= tiles); ++lg) {
+    const int n = 1 << lg;
+    if (rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, &ra.lg_stage, &ra.abuf) == 0) continue;
+    int fit = sms;
+    if (n > 1) {
+      int& cached = max_clusters[dev][lg];
+      if (cached == 0) {
+        if (int rc = set_smem(kernel, kMaxDynSmem)) return rc;
+        cudaLaunchConfig_t lc{};
+        lc.gridDim = dim3((unsigned)(sms / n * n));
+        lc.blockDim = dim3(kRbThreads);
+        lc.dynamicSmemBytes = kMaxDynSmem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)n;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        lc.attrs = attr;
+        lc.numAttrs = 1;
+        int got = 0;
+        if (cudaOccupancyMaxActiveClusters(&got, kernel, &lc) != cudaSuccess || got < 1) {
+          (void)cudaGetLastError();
+          got = -1;
+        }
+        cached = got;
+      }
+      if (cached < 1) continue;
+      fit = cached;
+    }
+    const double rounds = (double)((units + fit - 1) / fit);
+    const double cost = rounds * (8000. + (n > 1 ? 3000. : 0.) + 380. * ((tiles + n - 1) / n));
+    if (best_lg < 0 || cost < best) best = cost, best_lg = lg;
+  }
+  if (best_lg < 0) return fail(HE_ERR_UNSUPPORTED, "max_budget %d does not fit the block replay's shared memory", a.cfg.max_budget);
+  const int n = 1 << best_lg;
+  const size_t smem = rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, &ra.lg_stage, &ra.abuf);
+  if (int rc = set_smem(kernel, smem)) return rc;
+  const long long fit = n > 1 ? max_clusters[dev][best_lg] : sms;
+  const long long clusters = units < fit ? units : fit;
+  ra.L = rb_layout(WORDS, ra.r.smem_slots, a.cfg.group_size, n, 1 << ra.lg_stage, ra.abuf);
+  ra.ncta = n;
+  ra.scheduled = units > clusters ? 1 : 0;
+  if (ra.scheduled) {  // one queue, largest unit first
+    prefill_schedule_kernel<<<1, kSchedThreads, 0, stream>>>(a.cfg, a.ca.budget, a.prompt_len, 1, a.sched, 2700);
+    HE_CUDA_CHECK(cudaGetLastError());
+  }
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3((unsigned)(clusters * n));
+  lc.blockDim = dim3(kRbThreads);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)n;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  lc.attrs = attr;
+  lc.numAttrs = n > 1 ? 1 : 0;
+  HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, kernel, ra));
   return HE_OK;
 }
 
-// 8-bit operands when the group's code sum fits e5m2 exactly (group sizes up to 7); HE_TC_REPLAY_BF16=1 keeps bf16.
-template <int WORDS, bool GLOBAL_TABLE>
-int launch_replay_tc(const ReplayArgs& a, long long units, cudaStream_t stream) {
-  static const bool bf16_forced = [] {
-    const char* e = getenv("HE_TC_REPLAY_BF16");
-    return e && e[0] == '1';
-  }();
-  const bool fp8 = a.cfg.group_size <= 7 && !bf16_forced;
-  if (a.cfg.n_sink > 0 || a.cfg.n_recent > 0)  // protected windows
-    return fp8 ? launch_replay_tc_one<WORDS, GLOBAL_TABLE, true, true>(a, units, stream)
-               : launch_replay_tc_one<WORDS, GLOBAL_TABLE, false, true>(a, units, stream);
-  if (fp8) {
-    // no unit of such a launch can use the run-based resolver loop (every table keeps its tiles' second-largest keys)
-    if (!GLOBAL_TABLE && a.cfg.max_budget <= kRtSecondMaxTiles * kRtTile)
-      return launch_replay_tc_one<WORDS, false, true, false, false>(a, units, stream);
-    return launch_replay_tc_one<WORDS, GLOBAL_TABLE, true>(a, units, stream);
+template <int WORDS>
+int launch_replay_block(const ReplayArgs& a, long long units, cudaStream_t stream) {
+  const bool prot = a.cfg.n_sink > 0 || a.cfg.n_recent > 0;
+  switch (a.cfg.group_size) {
+    case 1: return prot ? launch_replay_block_one<WORDS, 1, true>(a, units, stream) : launch_replay_block_one<WORDS, 1, false>(a, units, stream);
+    case 4: return prot ? launch_replay_block_one<WORDS, 4, true>(a, units, stream) : launch_replay_block_one<WORDS, 4, false>(a, units, stream);
+    default: return prot ? launch_replay_block_one<WORDS, 0, true>(a, units, stream) : launch_replay_block_one<WORDS, 0, false>(a, units, stream);
   }
-  return launch_replay_tc_one<WORDS, GLOBAL_TABLE, false>(a, units, stream);
 }
 
-// HE_TC_REPLAY=0 keeps the replay on the CUDA-core kernels, =1 sends every eligible shape to the tensor-core kernel.
-// Unset: the tensor-core kernel runs one unit per SM at about 400 cycles per step whatever the budget, the register
-// kernel several units per SM at a cost that grows with the budget; measured on B200 (512 units, b = 64, G = 4) they
-// cross between 1024 and 1280 slots, and with no more units than SMs already around 512 slots.
-int tc_replay_mode() {
+// HE_TC_REPLAY=0 keeps the replay on the CUDA-core kernels, =1 sends every shape that fits to the block kernel.
+int block_replay_mode() {
   static const int mode = [] {
     const char* e = getenv("HE_TC_REPLAY");
     if (!tc_enabled() || (e && e[0] == '0')) return 0;
@@ -507,23 +565,27 @@ int tc_replay_mode() {
 
 template <int WORDS>
 int launch_replay(const ReplayArgs& a, long long units, cudaStream_t stream) {
-  const int mode = tc_replay_mode();
-  int sms = 0;
+  const int slots = (a.cfg.max_budget + kRbTile - 1) / kRbTile * kRbTile;
+  int lg_stage = 0, abuf = 0, sms = 0;
   if (int rc = sm_count(&sms)) return rc;
-  const int min_budget = units <= sms ? 512 : 1152;
-  bool tc_ok = mode != 0 && a.cfg.max_budget <= kRtMaxSlotsGlobal && (mode == 2 || a.cfg.max_budget >= min_budget);
-  // beyond 4096 slots the tensor-core kernel keeps its working table in the cache's own code array: word layout only
-  if (a.cfg.max_budget > kRtMaxSlots && packed_code_bytes(a.cfg) != 0) tc_ok = false;
-  if (tc_ok && (a.cfg.n_sink > 0 || a.cfg.n_recent > 0)) {
+  const int mode = block_replay_mode();
+  // The block kernel has one CTA per SM and pays a block's settling (8000 cycles) whatever the budget; the CUDA-core kernels
+  // scan every slot at every step, several units per SM. Measured on B200 (N = 2 C, ms with CUDA cores / block kernel): up
+  // to one unit per SM the block kernel is ahead from the smallest budgets where the register kernel exists (64 slots, G =
+  // 4, b = 32: 0.038 / 0.031) and from 128 slots where it does not (G = 8, b = 64: 0.066 / 0.053); with more units they
+  // cross between 256 and 512 slots (592 units, b = 32: 0.16 / 0.18 and 0.30 / 0.25), sooner with two code words and G = 4
+  // (256 slots: 0.22 / 0.18).
+  const bool has_reg = a.cfg.group_size == 1 || a.cfg.group_size == 4;
+  const int min_budget = units <= sms ? (has_reg ? 1 : 128) : (WORDS == 2 && a.cfg.group_size == 4 ? 256 : 384);
+  bool block_ok = mode != 0 && (mode == 2 || a.cfg.max_budget >= min_budget) && a.cfg.max_budget <= kRbMaxSlots &&
+                  rb_fit(WORDS, slots, a.cfg.group_size, 1, &lg_stage, &abuf) != 0;
+  if (block_ok && (a.cfg.n_sink > 0 || a.cfg.n_recent > 0)) {
     // protected windows: every budget must leave an eligible slot at every step (n_sink + n_recent < C), which the host
-    // can only check on the caller's mirror of the budgets; with the tables in global memory the kernel tracks the
-    // recent tokens in a 32-entry ring
-    tc_ok = a.cfg.n_recent <= (a.cfg.max_budget <= kRtMaxSlots ? kRtRows - 1 : 32) && a.ca.budget_host != nullptr;
-    for (int s = 0; tc_ok && s < a.cfg.batch; ++s) tc_ok = a.ca.budget_host[s] > a.cfg.n_sink + a.cfg.n_recent;
+    // can only check on the caller's mirror of the budgets
+    block_ok = a.cfg.n_sink <= kRbTile && a.cfg.n_recent < kRbRows && a.ca.budget_host != nullptr;
+    for (int s = 0; block_ok && s < a.cfg.batch; ++s) block_ok = a.ca.budget_host[s] > a.cfg.n_sink + a.cfg.n_recent;
   }
-  if (tc_ok)
-    return a.cfg.max_budget <= kRtMaxSlots ? launch_replay_tc<WORDS, false>(a, units, stream)
-                                           : launch_replay_tc<WORDS, true>(a, units, stream);
+  if (block_ok) return launch_replay_block<WORDS>(a, units, stream);
   switch (a.cfg.group_size) {
     case 1: return launch_replay_reg<WORDS, 1>(a, units, stream);
     case 4: return launch_replay_reg<WORDS, 4>(a, units, stream);

@@ -1,0 +1,955 @@
+// he_prefill_compress, phase 2: the sequential replay of Algorithm 1 over the prompt ("Prompt Encoding Stage" of Section
+// 3), a block of up to 128 evicting steps at a time.
+//
+// Distances as a contraction. With codes read as +-1 vectors s, the group distance of slot j at step t is
+//   D(j, t) = sum_g popc(h_j xor h(q_{t,g})) = (G K - <s_j, u_t>) / 2,   u_t = sum_g s(q_{t,g})  (entries in -G..G),
+// so the distances of a block of steps to every slot are one [steps x K] * [K x slots] product of small integers. The
+// operands are 8-bit (e5m2 holds 2^n u for |u| <= 8, e4m3 every whole number up to 16), accumulation is fp32 over whole
+// numbers below 2^24, so the result is exact in any order. For even G the parity of D is the same for every slot of a
+// step, so the RANK D >> 1 orders the slots (D itself for odd G). Operands A = -alpha u, B = +-2 with 2 alpha = 2^12 (even
+// G) or 2^13 (odd G) and two index columns make the accumulator 2^14 * rank + (127 - slot in tile) + a constant of the
+// step: with the tile's number added, the largest accumulator of a 128-slot tile is the arg-max key of Eq. 6 over the
+// tile (largest distance, lowest slot on ties). A third column pushes slots past the budget and protected first tokens
+// below everything else.
+//
+// What is sequential, and how it is settled side by side. Step r's victim depends on the victims s[0..r-1] of the block:
+// a base slot (the table as the block found it) may be taken already, and the keys of earlier steps are candidates
+// themselves. Written as s[r] = F_r(s[0..r-1]), any vector s with s = F(s) is the sequential result (by induction on r),
+// so the block iterates s <- F(s), all steps at once, from s[r] = best base slot, until nothing changes. After k passes
+// at least the first k entries are final; on the workloads' keys 2 to 4 passes settle a block, because few steps
+// depend on one another. A step is EASY when its best base slot is not taken by an earlier step and no earlier key can
+// reach its rank; easy steps cost nothing. The others ("hard", 5-40 %) are evaluated by a warp each: best new
+// entry still resident, best base slot (a taken one makes its tile be scanned again with popcounts). If passes
+// do not converge quickly (queries that keep preferring the same slots) the window that is evaluated at a
+// time shrinks to a dozen steps, so that no more than that is evaluated in vain.
+//
+// Few units: a cluster of up to 8 CTAs shares one unit. Tiles are dealt round-robin over its CTAs; each CTA keeps the
+// whole packed code table (at most 48 KB at 32 bits), copies its tiles' maxima to the others through distributed shared
+// memory, and all of them settle the block redundantly: one exchange per block.
+//
+// One CTA per SM, 512 threads (16 warps, so that each may have 128 registers: with 96 the accumulator loads spill and a
+// tile takes the readers 540 cycles instead of 160):
+//   warps 0-7    tile phase: read accumulators from tensor memory, one step per thread, four warps a tile
+//   warps 8-11   tile phase: expand packed codes into +-2 operand tiles (K-major, 128-byte swizzle), one slot per thread
+//   warps 12-13  issue tcgen05.mma (M = 128 steps, N = 128 slots, K = 32) for every other pair of tiles: one warp's chain of
+//                waits, instructions and commits is 800 cycles a pair, twice what the tensor pipe needs. The loop is
+//                warp-uniform and one elected lane issues, which keeps the descriptors in uniform registers
+//   warps 12-15  prepare the next block beside everything else: its codes, its operand A (14-15) and the distances between
+//                its own keys and queries, none of which depend on this block's outcome
+//   afterwards   warps 0-11 settle the block's steps
+// Every wait on an mbarrier is bounded; a CTA that gives up raises a flag that turns its later waits into no-ops, but it
+// still walks the same blocks and cluster barriers as its peers (their copies into its shared memory must find it), then
+// releases tensor memory and raises the device error counter.
+#pragma once
+#include <cuda_fp16.h>
+
+#include "hash_tc_kernels.cuh"
+#include "prefill_kernels.cuh"
+
+namespace he {
+
+constexpr int kRbThreads = 512;
+constexpr int kRbReadGroups = 2;         // groups of four warps that read accumulators
+constexpr int kRbExpWarp = 4 * kRbReadGroups, kRbMmaWarp = kRbExpWarp + 4;
+constexpr int kRbResWarps = 12;          // warps that settle a block
+constexpr int kRbResThreads = 32 * kRbResWarps;
+constexpr int kRbAuxThreads = 128;       // warps kRbMmaWarp .. kRbMmaWarp + 3
+constexpr int kRbBuildThreads = 64;      // ... of which the last two build operand A
+constexpr int kRbRows = 128;             // steps per block at most = MMA M
+constexpr int kRbTile = 128;             // slots per tile = MMA N
+constexpr int kRbKeyShift = 14;
+constexpr int kRbIdxMask = (1 << kRbKeyShift) - 1;
+constexpr int kRbMaxSlots = 12288;
+constexpr int kRbMaxCluster = 8;
+constexpr int kRbWidePasses = 6;         // passes over the whole block before the window shrinks
+constexpr int kRbAtom = 128 * 128;       // 128 operand rows x one 128-byte swizzle atom
+constexpr int kRbDnPitch = 136;          // 16-bit entries between rows of the new-entry table
+constexpr int kRbMaxStages = 4;          // pairs of operand tiles
+
+// Byte offsets of the kernel's dynamic shared memory (after rounding its base up to 1024 bytes). Tile maxima: per CTA of the
+// cluster one block of fp32 keys, a row for each step, an odd number of words apart (a warp stores a column, a lane per
+// step), then the best key of each step over each reader group's tiles.
+struct RbLayout {
+  uint32_t a, bidx, b, codes, own, mx, mx_pitch, mx_block, dn, rn, nr, sv, sn, list, par, qraw, kraw, rec, total;
+};
+__host__ __device__ inline RbLayout rb_layout(int words, int slots, int G, int ncta, int nstage, int abuf) {
+  RbLayout L;
+  const uint32_t nt = (uint32_t)slots / kRbTile, ntl = (nt + ncta - 1) / ncta;
+  uint32_t o = 0;
+  auto take = [&](uint32_t bytes) {
+    const uint32_t at = o;
+    o += (bytes + 15u) & ~15u;
+    return at;
+  };
+  // a 128-byte atom row holds two tiles' 64-bit rows or four tiles' 32-bit rows, and both buffers of a 32-bit operand A
+  L.a = take(words == 2 ? (uint32_t)abuf * kRbAtom : kRbAtom);
+  L.bidx = take(kRbAtom);  // index columns: four variants side by side
+  L.b = take(words == 2 ? (uint32_t)nstage * kRbAtom : (uint32_t)(nstage + 1) / 2 * kRbAtom);
+  L.codes = take((uint32_t)slots * words * 4u);
+  L.own = take((uint32_t)slots);
+  L.mx_pitch = ntl | 1u;  // words
+  L.mx_block = (L.mx_pitch + kRbReadGroups) * kRbRows;
+  L.mx = take(L.mx_block * ncta * 4u);
+  L.dn = take(2u * (kRbRows / 2) * kRbDnPitch * 2u);
+  L.rn = take(kRbRows * 4u);
+  L.nr = take(2u * kRbRows * 4u);
+  L.sv = take(kRbRows * 2u);
+  L.sn = take(kRbRows * 4u);
+  L.list = take(kRbRows);
+  L.par = take(2u * kRbRows * 4u);
+  L.qraw = take(2u * kRbRows * G * words * 4u);  // this block's codes and the next block's
+  L.kraw = take(2u * kRbRows * words * 4u);
+  L.rec = take(kRbRows * 4u);
+  L.total = o + 1024u;
+  return L;
+}
+
+struct RbArgs {
+  ReplayArgs r;
+  int ncta;       // CTAs per unit (cluster size, a power of two)
+  int scheduled;  // units are claimed from r.sched; 0: unit = cluster index
+  int lg_stage;   // log2 of the pairs of operand tiles in shared memory
+  int abuf;       // operand A buffers (2: the next block's is built during the tile phase)
+  RbLayout L;     // computed by the host: kernel parameters cost no registers
+};
+
+// Steps per block. A block of R steps against C slots meets about R / (2 C) taken slots per step, and the passes it needs
+// grow with them, so smaller tables use shorter blocks (1024 slots, b = 16: 42 000 cycles to settle 128 steps at once,
+// 2 x 14 000 in two blocks).
+__host__ __device__ inline int rb_block_rows(int C) { return C >= 1536 ? 128 : (C >= 128 ? 64 : 32); }
+
+__device__ __forceinline__ void rb_mma_f8(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
+      : "memory");
+}
+
+// e4m3 bit pattern of a small non-negative integer with at most four significant bits (exact), e5m2 of an integer with at
+// most three (e5m2 is the high half of f16).
+__device__ __forceinline__ uint32_t rb_e4m3(int v) {
+  if (v <= 0) return 0u;
+  const int p = 31 - __clz(v);
+  const uint32_t mant = p >= 3 ? ((uint32_t)v >> (p - 3)) & 7u : ((uint32_t)v << (3 - p)) & 7u;
+  return ((uint32_t)(p + 7) << 3) | mant;
+}
+__device__ __forceinline__ uint32_t rb_e5m2(int v) { return (uint32_t)__half_as_ushort(__int2half_rn(v)) >> 8; }
+
+// Byte offset of 16-byte chunk `chunk` (0..7) of row `row` inside one swizzle atom.
+__device__ __forceinline__ uint32_t rb_swz(int row, int chunk) {
+  return (uint32_t)((row >> 3) * 1024 + (row & 7) * 128 + ((chunk ^ (row & 7)) << 4));
+}
+
+__device__ __forceinline__ float rb_fmax3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
+// Columns of a code word in operand order: output word m (four bytes) holds bits m, m + 8, m + 16, m + 24, in both
+// operands, so that one shift and one logic operation expand four bits. Set: +2 (e4m3 0x40), clear: -2 (0xC0).
+__device__ __forceinline__ uint32_t rb_expand4(uint32_t h, int m) { return lop3<0x6A>(h << (7 - m), 0x80808080u, 0xC0C0C0C0u); }
+
+__device__ __forceinline__ bool rb_elect() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xFFFFFFFF;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
+// The ranks of a block's own keys at its steps: step r only needs those of the r steps before it, so steps 64 + k and 63 - k
+// share a row (64 + k entries from its start, 63 - k from the next multiple of four).
+__device__ __forceinline__ int rb_dn_at(int r) {
+  return r >= 64 ? (r - 64) * kRbDnPitch : (63 - r) * kRbDnPitch + ((127 - r + 3) & ~3);
+}
+
+__device__ __forceinline__ uint32_t rb_cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t rb_mapa(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void rb_st_remote(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// Copy to a peer's shared memory that counts its bytes on the peer's mbarrier. (Stores by the reading warps, fenced by a
+// releasing arrive, took about 2000 cycles a block with four CTAs; asynchronous 4-byte stores 10 000 with eight.)
+__device__ __forceinline__ void rb_copy_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src), "r"(bytes),
+               "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void rb_arrive_remote(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// Bounded wait for copies and arrivals of other CTAs of the cluster.
+__device__ __forceinline__ bool rb_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  for (uint32_t i = 0; i < kTcSpinLimit; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (*abort_flag) return false;
+  }
+  *abort_flag = 1;
+  return false;
+}
+__device__ __forceinline__ void rb_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <int ID, int THREADS>
+__device__ __forceinline__ void rb_bar() {
+  asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
+}
+
+// Rank of one slot's code at a step from the packed words. GT = 4 uses the bit-plane form, which yields (D - pc) / 2 with pc
+// the bits set in the exclusive or of the step's query codes (`parity_bits`, worked out with operand A).
+template <int WORDS, int GT>
+struct RbRank {
+  static constexpr int kQ = (GT > 0 ? GT : kMaxGroup) * WORDS;
+  uint32_t q[kQ];
+  Planes4 p[WORDS];
+  int add, G;
+  __device__ __forceinline__ void load(const uint32_t* src, int G_, int parity_bits) {
+    G = G_;
+    add = parity_bits;
+    if (GT * WORDS % 4 == 0 && GT > 0) {
+#pragma unroll
+      for (int i = 0; i < kQ; i += 4) *reinterpret_cast<uint4*>(q + i) = *reinterpret_cast<const uint4*>(src + i);
+    } else {
+#pragma unroll
+      for (int i = 0; i < kQ; ++i) q[i] = (GT > 0 || i < G * WORDS) ? src[i] : 0u;
+    }
+    if (GT == 4) {
+#pragma unroll
+      for (int w = 0; w < WORDS; ++w) {
+        uint32_t parity;
+        p[w] = make_planes4(q[w], q[WORDS + w], q[(2 * WORDS + w) % kQ], q[(3 * WORDS + w) % kQ], &parity);
+      }
+    }
+  }
+  __device__ __forceinline__ int dist(const uint32_t (&h)[WORDS]) const {
+    if (GT == 4) return 2 * half_distance4<WORDS>(h, p) + add;
+    int d = 0;
+#pragma unroll
+    for (int g = 0; g < (GT > 0 ? GT : kMaxGroup); ++g)
+      if (GT > 0 || g < G) {
+#pragma unroll
+        for (int w = 0; w < WORDS; ++w) d += __popc(h[w] ^ q[g * WORDS + w]);
+      }
+    return d;
+  }
+  __device__ __forceinline__ int rank(const uint32_t (&h)[WORDS]) const {
+    if (GT == 4) return half_distance4<WORDS>(h, p) + (add >> 1);
+    if (GT == 1) return dist(h);
+    return (G & 1) ? dist(h) : dist(h) >> 1;
+  }
+};
+
+// PROT: protected windows (Section 4 setup). The first n_sink tokens never leave slots 0 .. n_sink-1, so those slots are
+// masked like slots past the budget. A recent token that is already in the table is recognised by the list of the newest
+// slots, one of this block's own keys by its step. Needs every budget > n_sink + n_recent (so that some slot is always
+// eligible), n_sink <= 128 (one tile) and n_recent < 128.
+template <int WORDS, int GT, bool PROT>
+__global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(const __grid_constant__ RbArgs ar) {
+  constexpr int NT = kRbThreads;
+  constexpr int MS = kRbMaxStages;
+  extern __shared__ unsigned char rb_smem_raw[];
+  __shared__ __align__(8) unsigned long long bars[2 * MS + 4 + 4];
+  __shared__ uint32_t tmem_base_s;
+  __shared__ volatile int abort_flag;
+  __shared__ int s_unit[2];
+  __shared__ int s_change[2];                    // by pass parity: first step that changed
+  __shared__ __align__(4) uint8_t s_hard[2][4];  // by pass parity: lengths of warps 0-3's lists of hard steps
+
+  const ReplayArgs& a = ar.r;
+  const he_config& cfg = a.cfg;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G = GT > 0 ? GT : cfg.group_size;
+  const int GW = G * WORDS;
+  const long long Cmax = cfg.max_budget;
+  const bool write_scores = (cfg.flags & HE_FLAG_WRITE_SCORES) != 0;
+  const int ncta = ar.ncta, lg_ncta = 31 - __clz(ncta), lg_stage = ar.lg_stage, abuf = ar.abuf;
+  const int rank = ncta > 1 ? (int)rb_cluster_rank() : 0;
+  // rounded up to 1024 bytes by an offset from the array itself: the accesses stay shared-memory accesses
+  unsigned char* smem = rb_smem_raw + ((1024u - (smem_u32(rb_smem_raw) & 1023u)) & 1023u);
+  const RbLayout& L = ar.L;
+  unsigned char* As = smem + L.a;
+  unsigned char* Bx = smem + L.bidx;
+  unsigned char* Bs = smem + L.b;
+  uint32_t* codes = reinterpret_cast<uint32_t*>(smem + L.codes);
+  uint8_t* own = smem + L.own;
+  float* Mx = reinterpret_cast<float*>(smem + L.mx);
+  const int top_at = kRbRows * L.mx_pitch;  // where a CTA's block of Mx holds its groups' best keys
+  uint16_t* Dn = reinterpret_cast<uint16_t*>(smem + L.dn);
+  int32_t* RN = reinterpret_cast<int32_t*>(smem + L.rn);    // per step: best base key
+  int32_t* NR = reinterpret_cast<int32_t*>(smem + L.nr);    // per step: largest rank of any earlier key of the block, two buffers
+  uint16_t* SV = reinterpret_cast<uint16_t*>(smem + L.sv);  // per step: the slot it writes, as far as known
+  int32_t* SN = reinterpret_cast<int32_t*>(smem + L.sn);    // what the evaluation of a hard step gave
+  uint8_t* LIST = smem + L.list;                            // hard steps that warps 0-3 found in the pass: step | stale << 7
+  int32_t* PAR = reinterpret_cast<int32_t*>(smem + L.par);  // per step: bits set in the xor of its query codes, two buffers
+  uint32_t* qraw = reinterpret_cast<uint32_t*>(smem + L.qraw);
+  uint32_t* kraw = reinterpret_cast<uint32_t*>(smem + L.kraw);
+  int32_t* REC = reinterpret_cast<int32_t*>(smem + L.rec);  // PROT: slot of the m-th newest token before the block at [m - 1]
+  const int a_step = WORDS == 2 ? kRbAtom : 64;             // bytes between the two buffers of operand A
+
+  const uint32_t bar0 = smem_u32(bars);
+  auto full_bar = [&](int s) { return bar0 + 8u * s; };                  // expanders -> MMA: the pair's operand tiles are written
+  auto sfree_bar = [&](int s) { return bar0 + 8u * (MS + s); };          // MMA -> expanders: they may be rewritten
+  auto afull_bar = [&](int x) { return bar0 + 8u * (2 * MS + x); };      // MMA -> readers: the pair's accumulators are complete
+  auto afree_bar = [&](int x) { return bar0 + 8u * (2 * MS + 2 + x); };  // readers -> MMA: they have been read
+  const uint32_t peer_bar = bar0 + 8u * (2 * MS + 4);                    // peers' copies of their tiles' maxima have arrived
+  const uint32_t used_bar = bar0 + 8u * (2 * MS + 5);                    // peers: they are done with this CTA's maxima
+  const uint32_t adone_bar = bar0 + 8u * (2 * MS + 6);                   // one operand A buffer: the block's tiles are multiplied
+  const uint32_t drain_bar = bar0 + 8u * (2 * MS + 7);                   // abort path
+  if (tid == 0) {
+    abort_flag = 0;
+    mbar_init(drain_bar, 2);
+    mbar_init(adone_bar, 2);
+    for (int i = 0; i < MS; ++i) {
+      mbar_init(full_bar(i), 4);
+      mbar_init(sfree_bar(i), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(afull_bar(i), 1);
+      mbar_init(afree_bar(i), 8);
+    }
+    mbar_init(peer_bar, 1);
+    mbar_init(used_bar, ncta > 1 ? ncta - 1 : 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kRbMmaWarp) {  // four accumulators of 128 columns
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(4 * kRbTile)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  // Scaling of the operands (file comment) and the e5m2 codes of -alpha (2 c - G) for c = 0..7 set bits among the group's
+  // queries, as two words of a byte table; c = 8 (G = 8 only) is patched where it occurs.
+  const bool even = (G & 1) == 0;
+  const int alpha = even ? 2048 : 4096;
+  const float off = (float)((even ? 4096 : 8192) * G * 32 * WORDS);  // accumulator + off - 2^13 parity (even G) = 2^14 * rank + index
+  uint32_t lut_lo = 0u, lut_hi = 0u;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    lut_lo |= rb_e5m2(-alpha * (2 * c - G)) << (8 * c);
+    lut_hi |= (c + 4 <= G ? rb_e5m2(-alpha * (2 * (c + 4) - G)) : 0u) << (8 * c);
+  }
+  for (int i = tid; i < a.smem_slots / 4; i += NT) reinterpret_cast<uint32_t*>(own)[i] = 0xFFFFFFFFu;
+  tc_fence_before();
+  __syncthreads();
+  if (ncta > 1) rb_cluster_sync();  // every CTA of the cluster runs before anyone copies into it
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_base_s;
+  // instruction descriptor: fp32 accumulate, e5m2 x e4m3, both operands K-major, N = 128, M = 128
+  const uint32_t idesc = (1u << 4) | (1u << 7) | ((uint32_t)(kRbTile >> 3) << 17) | ((uint32_t)(kRbRows >> 4) << 24);
+  // Pairs of tiles so far; every role counts the same sequence. Pair n lives in operand stage n mod (1 << lg_stage) and
+  // accumulator pair n mod 2.
+  int it = 0;
+  int blk = 0;  // blocks so far
+  auto stage_of = [&](int n) { return n & ((1 << lg_stage) - 1); };
+  auto stage_phase = [&](int n) { return (uint32_t)(n >> lg_stage) & 1u; };
+
+  // (the unit number is double-buffered: a peer may still be reading the one before)
+  for (int nunit = 0;; ++nunit) {
+    if (ar.scheduled) {
+      if (rank == 0 && warp == 0) {
+        const int u = claim_unit(a.sched, lane);
+        if (lane < ncta) {
+          if (ncta > 1) rb_st_remote(rb_mapa(smem_u32(&s_unit[nunit & 1]), (uint32_t)lane), (uint32_t)u);
+          else s_unit[nunit & 1] = u;
+        }
+      }
+      __syncthreads();
+      if (ncta > 1) rb_cluster_sync();
+    } else {
+      if (nunit > 0) break;
+      if (tid == 0) s_unit[0] = (int)blockIdx.x >> lg_ncta;
+      __syncthreads();
+    }
+    const long long unit = s_unit[nunit & 1];
+    if (unit < 0) break;
+    const int s = (int)(unit / cfg.n_kv_heads);
+    const int C = clamp_budget(a.ca.budget[s], (int)Cmax);
+    const int N = clamp_len(a.prompt_len[s], a.Nmax, C);
+    const int fill0 = N < C ? N : C;
+    const uint32_t* kc_u = a.kcodes + unit * a.Nmax * WORDS;
+    const uint32_t* qc_u = a.qcodes + unit * a.Nmax * G * WORDS;
+    float* sc = a.ca.scores + unit * Cmax;
+    int32_t* pos_g = a.ca.pos + unit * Cmax;
+    const int S = PROT ? cfg.n_sink : 0, Rn = PROT ? cfg.n_recent : 0;
+    const int nbase = (C + kRbTile - 1) / kRbTile;
+    const int ntl = nbase > rank ? (nbase - rank + ncta - 1) >> lg_ncta : 0;  // this CTA's tiles: rank, rank + ncta, ...
+    const int R = rb_block_rows(C);
+    // the first C tokens fill the cache in order; everything beyond `fill` is reset
+    for (int j = tid; j < nbase * kRbTile; j += NT) {
+#pragma unroll
+      for (int w = 0; w < WORDS; ++w) codes[j * WORDS + w] = j < fill0 ? __ldg(kc_u + (long long)j * WORDS + w) : 0u;
+    }
+    for (int j = rank * NT + tid; j < (int)Cmax; j += ncta * NT) pos_g[j] = j < fill0 ? j : -1;
+    if (PROT && tid < Rn) REC[tid] = C - 1 - tid;  // (the first C tokens sit in slot = position)
+    // Index columns of operand B (columns of A: 16, 1, 2^15): digits of 127 - x, and -256 for rows that may not win. Variant
+    // bit 0: the tile holds the protected first tokens, bit 1: the budget ends inside the tile.
+    if (tid < 4 * kRbTile) {
+      const int x = tid & 127, v = tid >> 7;
+      const bool bad = ((v & 1) && x < S) || ((v & 2) && x >= C - (nbase - 1) * kRbTile);
+      *reinterpret_cast<uint4*>(Bx + rb_swz(x, 2 * v)) =
+          make_uint4(rb_e4m3((127 - x) >> 4) | (rb_e4m3((127 - x) & 15) << 8) | (bad ? 0xF8u << 16 : 0u), 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(Bx + rb_swz(x, 2 * v + 1)) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    // The block's query and key codes into buffer `buf` (rows past the prompt keep what was there: nothing reads them).
+    auto stage_codes = [&](int buf, int tb, int nrows, int first, int nthreads) {
+      uint32_t* qd = qraw + buf * kRbRows * GW;
+      uint32_t* kd = kraw + buf * kRbRows * WORDS;
+      const uint32_t* qs = qc_u + (long long)tb * GW;
+      const uint32_t* ks = kc_u + (long long)tb * WORDS;
+      for (int i = first; i < nrows * GW; i += nthreads)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(qd + i)), "l"(qs + i) : "memory");
+      for (int i = first; i < nrows * WORDS; i += nthreads)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(kd + i)), "l"(ks + i) : "memory");
+      cp_async_commit();
+    };
+    // Operand A, row r = step r of the block: -alpha u_t, then the three index columns. One thread per (row, word).
+    auto build_a = [&](int buf, int nrows, int first, int nthreads) {
+      const uint32_t* qd = qraw + buf * kRbRows * GW;
+      unsigned char* ad = As + (WORDS == 2 && abuf > 1 ? buf * kRbAtom : 0);
+      const int c0 = WORDS == 1 && abuf > 1 ? 4 * buf : 0;
+      for (int item = first; item < kRbRows * WORDS; item += nthreads) {
+        const int r = item & (kRbRows - 1), w = item >> 7;
+        const bool valid = r < nrows;
+        uint32_t cnt[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) cnt[m] = 0u;
+        if (valid)
+          for (int g = 0; g < G; ++g) {
+            const uint32_t x = qd[r * GW + g * WORDS + w];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) cnt[m] += (x >> m) & 0x01010101u;  // set bits among the queries, one counter per byte
+          }
+        uint32_t v[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+          const uint32_t t = cnt[m] | (cnt[m] >> 4);
+          v[m] = __byte_perm(lut_lo, lut_hi, __byte_perm(t, 0u, 0x4420));
+          // eight of eight: -2^14 = 0xF4 (selector 8 made the lookup give 0 there)
+          if (GT == 0) v[m] |= ((cnt[m] & 0x08080808u) * 0x1Eu) | ((cnt[m] & 0x08080808u) >> 1);
+          if (!valid) v[m] = 0u;
+        }
+        *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * w)) = make_uint4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * w + 1)) = make_uint4(v[4], v[5], v[6], v[7]);
+        if (w == 0) {
+          *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * WORDS)) = make_uint4(valid ? 0x4Cu | (0x3Cu << 8) | (0x78u << 16) : 0u, 0u, 0u, 0u);
+          *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * WORDS + 1)) = make_uint4(0u, 0u, 0u, 0u);
+          int pc = 0;
+          if (even && valid) {
+#pragma unroll
+            for (int v2 = 0; v2 < WORDS; ++v2) {
+              uint32_t x = 0u;
+              for (int g = 0; g < G; ++g) x ^= qd[r * GW + g * WORDS + v2];
+              pc += __popc(x);
+            }
+          }
+          PAR[buf * kRbRows + r] = pc;
+        }
+      }
+    };
+    // One tile's row of operand B in operand stage sx (tile g of the pair): this thread's slot or key.
+    auto expand_row = [&](const uint32_t* h, int x, int sx, int g) {
+      unsigned char* bt = Bs + (WORDS == 2 ? sx : sx >> 1) * kRbAtom + (x >> 3) * 1024 + (x & 7) * 128;
+      const int c0 = WORDS == 2 ? 4 * g : 2 * (2 * (sx & 1) + g);
+#pragma unroll
+      for (int c = 0; c < 2 * WORDS; ++c) {
+        const uint32_t hw = h[c >> 1];
+        const int m = (c & 1) * 4;
+        *reinterpret_cast<uint4*>(bt + (((c0 + c) ^ (x & 7)) << 4)) =
+            make_uint4(rb_expand4(hw, m), rb_expand4(hw, m + 1), rb_expand4(hw, m + 2), rb_expand4(hw, m + 3));
+      }
+    };
+    auto a_desc_of = [&](int buf) { return umma_desc_k128(smem_u32(As)) + (uint64_t)((abuf > 1 ? buf * a_step : 0) >> 4); };
+    auto b_desc_of = [&](int sx, int g) {
+      return umma_desc_k128(smem_u32(Bs)) +
+             (uint64_t)((WORDS == 2 ? sx * kRbAtom + g * 64 : (sx >> 1) * kRbAtom + (2 * (sx & 1) + g) * 32) >> 4);
+    };
+    // Ranks of a block's own keys (buffer `buf`) at its steps, by warps 12-15: one more tile, as pair n, without index
+    // columns. Also each step's largest rank of any key that enters before it (and is no longer recent): no new entry can
+    // beat that. (Both MMA warps have issued every earlier pair when this runs, so no wait here can meet an older phase.)
+    auto new_keys = [&](int buf, int n) {
+      const int x = tid & 127, acc = n & 1, ph = (n >> 1) & 1, sx = stage_of(n);
+      const uint32_t px = stage_phase(n);
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait(sfree_bar(sx), px ^ 1, &abort_flag))) return;
+      uint32_t h[WORDS];
+#pragma unroll
+      for (int w = 0; w < WORDS; ++w) h[w] = kraw[(buf * kRbRows + x) * WORDS + w];
+      expand_row(h, x, sx, 0);
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full_bar(sx));
+      if (warp == kRbMmaWarp) {
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait2(afree_bar(acc), ph ^ 1, full_bar(sx), px, &abort_flag))) return;
+        tc_fence_after();
+        const uint64_t ad = a_desc_of(buf), bd = b_desc_of(sx, 0);
+        if (rb_elect()) {
+#pragma unroll
+          for (int w = 0; w < WORDS; ++w)
+            rb_mma_f8(tmem_base + (uint32_t)(2 * acc * kRbTile), ad + (uint64_t)(2 * w), bd + (uint64_t)(2 * w), idesc, w > 0);
+          tc_commit(afull_bar(acc));
+          tc_commit(sfree_bar(sx));
+        }
+        __syncwarp();
+      }
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait(afull_bar(acc), ph, &abort_flag))) return;
+      tc_fence_after();
+      // Conversions by an fp32 addition (the integer conversions run at a sixteenth of its rate): 2^22 + rank has 2 * rank
+      // in its low bits, which is what is kept.
+      const int r = x, last = PROT ? r - Rn : r;  // entries below `last` are candidates
+      const float magic = (off - (float)((PAR[buf * kRbRows + r] & 1) << 13)) * (1.f / 16384.f) + 4194304.f;
+      const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(2 * acc * kRbTile);
+      uint16_t* dst = Dn + buf * (kRbRows / 2) * kRbDnPitch + rb_dn_at(r);
+      float dmax = -1e9f;
+#pragma unroll 1
+      for (int c = 0; c < 4; ++c) {
+        uint32_t v[32];
+        tc_ld32(taddr + c * 32, v);
+        tc_wait_ld();
+        if (c == 3) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane < 2) mbar_arrive(afree_bar(acc));  // (four warps, eight arrivals)
+        }
+        if (c > (warp & 3)) continue;  // no step of this warp comes after those keys
+        const int lc = last - c * 32;
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+          if (k < lc) dmax = fmaxf(dmax, __uint_as_float(v[k]));
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          uint32_t pk[2];
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const float y0 = fmaf(__uint_as_float(v[4 * k + 2 * e]), 1.f / 16384.f, magic);
+            const float y1 = fmaf(__uint_as_float(v[4 * k + 2 * e + 1]), 1.f / 16384.f, magic);
+            pk[e] = __byte_perm(__float_as_uint(y0), __float_as_uint(y1), 0x5410);
+          }
+          if (c * 32 + 4 * k < r) *reinterpret_cast<uint2*>(dst + c * 32 + 4 * k) = make_uint2(pk[0], pk[1]);
+        }
+      }
+      NR[buf * kRbRows + r] = last > 0 ? (int)(__float_as_uint(fmaf(dmax, 1.f / 16384.f, magic)) & 0xFFFFu) >> 1 : -1;
+    };
+    int cur = 0;
+    if (C < N) {
+      const int rows = min(N - C, R);
+      stage_codes(0, C, rows, tid, NT);
+      cp_async_wait_all();
+      __syncthreads();
+      build_a(0, rows, tid, NT);
+      fence_proxy_async();
+      __syncthreads();
+      if (warp >= kRbMmaWarp) new_keys(0, it);
+      ++it;
+    }
+    fence_proxy_async();
+    __syncthreads();
+
+    for (int t0 = C; t0 < N; t0 += R) {
+      const int rows = min(N - t0, R);
+      const int tn = t0 + rows;
+      const uint32_t* qb = qraw + cur * kRbRows * GW;
+      const uint32_t* kb_codes = kraw + cur * kRbRows * WORDS;
+      // ---------------------------------------------------------------- tile phase
+      // this CTA's base tiles 0 .. ntl - 1 (tile i of the CTA is tile i * ncta + rank of the unit)
+      const int npair = (ntl + 1) >> 1;
+      float topf = -1.f;  // readers: best base key of the thread's step so far
+      if (warp < kRbExpWarp) {
+        const int r = tid & 127, grp = warp >> 2;  // this thread's step = its tensor-memory lane; tile grp of each pair
+        float* mrow = Mx + rank * L.mx_block + r * L.mx_pitch;
+        // 2^14 rank + index: the step's constant, and 127 - tile above the index within the tile (lower tiles first)
+        float ct = off - (float)((PAR[cur * kRbRows + r] & 1) << 13) + (float)((127 - ((grp << lg_ncta) + rank)) * 128);
+        const float cstep = (float)(256 << lg_ncta);
+        const uint32_t taddr0 = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(grp * kRbTile);
+        if (ncta > 1 && blk > 0) rb_wait_cluster(used_bar, (blk - 1) & 1, &abort_flag);  // peers still read the block before
+        for (int p = 0; p < npair; ++p) {
+          const int n = it + p, acc = n & 1, ph = (n >> 1) & 1, i = 2 * p + grp;
+          if (!__all_sync(0xFFFFFFFFu, mbar_wait(afull_bar(acc), ph, &abort_flag))) break;
+          tc_fence_after();
+          // (the second tile of an odd last pair holds an older product; nobody looks at its key)
+          const uint32_t taddr = taddr0 + (uint32_t)(2 * acc * kRbTile);
+          uint32_t v0[32], v1[32];
+          float m[8];
+          tc_ld32(taddr, v0);
+          tc_ld32(taddr + 32, v1);
+          tc_wait_ld();
+#pragma unroll
+          for (int k = 0; k < 8; ++k) m[k] = rb_fmax3(__uint_as_float(v0[k]), __uint_as_float(v0[k + 8]), __uint_as_float(v0[k + 16]));
+#pragma unroll
+          for (int k = 0; k < 8; ++k) m[k] = rb_fmax3(m[k], __uint_as_float(v0[k + 24]), __uint_as_float(v1[k]));
+          tc_ld32(taddr + 64, v0);
+#pragma unroll
+          for (int k = 0; k < 8; ++k) m[k] = rb_fmax3(m[k], __uint_as_float(v1[k + 8]), __uint_as_float(v1[k + 16]));
+#pragma unroll
+          for (int k = 0; k < 4; ++k) m[k] = rb_fmax3(m[k], __uint_as_float(v1[k + 24]), __uint_as_float(v1[k + 28]));
+          tc_ld32(taddr + 96, v1);
+          tc_wait_ld();
+          tc_fence_before();  // the last read: the accumulators go back
+          __syncwarp();
+          if (lane == 0) mbar_arrive(afree_bar(acc));
+#pragma unroll
+          for (int k0 = 0; k0 < 32; k0 += 8)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) m[k] = rb_fmax3(m[k], __uint_as_float(v0[k0 + k]), __uint_as_float(v1[k0 + k]));
+          // the tile's best key; negative: no slot of the tile may win
+          const float key = rb_fmax3(rb_fmax3(m[0], m[1], m[2]), rb_fmax3(m[3], m[4], m[5]), fmaxf(m[6], m[7])) + ct;
+          ct -= cstep;
+          if (i < ntl) {
+            topf = fmaxf(topf, key);
+            mrow[i] = key;
+          }
+        }
+        Mx[rank * L.mx_block + top_at + grp * kRbRows + r] = topf;  // this group's best key of the step
+        if (ncta > 1) fence_proxy_async();
+        rb_bar<4, 32 * kRbExpWarp>();  // the reader groups see each other's results
+        if (tid < ncta - 1) {          // ... and every peer gets this CTA's block
+          const uint32_t peer = (uint32_t)((rank + 1 + tid) & (ncta - 1)), la = smem_u32(Mx + rank * L.mx_block);
+          rb_copy_to_peer(rb_mapa(la, peer), la, L.mx_block * 4u, rb_mapa(peer_bar, peer));
+        }
+        __syncwarp();
+      } else if (warp < kRbMmaWarp) {
+        if (ncta > 1 && tid == 32 * kRbExpWarp) mbar_arrive_expect_tx(peer_bar, L.mx_block * 4u * (uint32_t)(ncta - 1));
+        const int x = tid & 127;  // this thread's row of both tiles of a pair
+        const uint32_t* base = codes + (rank * kRbTile + x) * WORDS;
+        const int tstep = (kRbTile * WORDS) << lg_ncta;  // words between this CTA's tiles
+        for (int p = 0; p < npair; ++p) {
+          uint32_t h0[WORDS], h1[WORDS];
+          const bool two = 2 * p + 1 < ntl;
+#pragma unroll
+          for (int w = 0; w < WORDS; ++w) {
+            h0[w] = base[2 * p * tstep + w];
+            h1[w] = two ? base[(2 * p + 1) * tstep + w] : 0u;
+          }
+          const int sx = stage_of(it + p);
+          if (!__all_sync(0xFFFFFFFFu, mbar_wait(sfree_bar(sx), stage_phase(it + p) ^ 1, &abort_flag))) break;
+          expand_row(h0, x, sx, 0);
+          expand_row(h1, x, sx, 1);
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(full_bar(sx));
+        }
+      } else {
+        if (warp < kRbMmaWarp + 2) {
+          const uint64_t a_desc = a_desc_of(cur), x_desc = umma_desc_k128(smem_u32(Bx));
+          // index-column variants: the unit's first tile (protected first tokens) and its last (the budget ends in it)
+          const int first_i = S > 0 && rank == 0 ? 0 : -1, last_i = ((nbase - 1 - rank) & (ncta - 1)) == 0 ? ntl - 1 : -1;
+          for (int p = (it ^ warp) & 1; p < npair; p += 2) {  // pairs of this warp's parity
+            const int n = it + p, acc = n & 1, ph = (n >> 1) & 1, i = 2 * p, sx = stage_of(n);
+            const uint64_t bd = b_desc_of(sx, 0), bd1 = bd + (uint64_t)((WORDS == 2 ? 64 : 32) >> 4);
+            const uint64_t x0 = x_desc + (uint64_t)((i == first_i ? 2 : 0) + (i == last_i ? 4 : 0));
+            const uint64_t x1 = x_desc + (uint64_t)(i + 1 == last_i ? 4 : 0);
+            if (!__all_sync(0xFFFFFFFFu, mbar_wait2(afree_bar(acc), ph ^ 1, full_bar(sx), stage_phase(n), &abort_flag))) break;
+            tc_fence_after();
+            if (rb_elect()) {
+              const uint32_t d = tmem_base + (uint32_t)(2 * acc * kRbTile);
+#pragma unroll
+              for (int w = 0; w < WORDS; ++w) rb_mma_f8(d, a_desc + (uint64_t)(2 * w), bd + (uint64_t)(2 * w), idesc, w > 0);
+              rb_mma_f8(d, a_desc + (uint64_t)(2 * WORDS), x0, idesc, true);
+              if (i + 1 < ntl) {
+#pragma unroll
+                for (int w = 0; w < WORDS; ++w) rb_mma_f8(d + kRbTile, a_desc + (uint64_t)(2 * w), bd1 + (uint64_t)(2 * w), idesc, w > 0);
+                rb_mma_f8(d + kRbTile, a_desc + (uint64_t)(2 * WORDS), x1, idesc, true);
+              }
+              tc_commit(afull_bar(acc));
+              tc_commit(sfree_bar(sx));
+            }
+            __syncwarp();
+          }
+          if (abuf == 1 && rb_elect()) tc_commit(adone_bar);
+          __syncwarp();
+        }
+        if (tn < N) {  // the next block: its codes and operand A (warps 14-15, meanwhile), its own keys' ranks (all four)
+          const int nrows = min(N - tn, R), first = tid - 32 * (kRbMmaWarp + 2);
+          if (first >= 0) {
+            stage_codes(cur ^ 1, tn, nrows, first, kRbBuildThreads);
+            cp_async_wait_all();
+            if (abuf == 1) mbar_wait(adone_bar, blk & 1, &abort_flag);  // a single operand A is free after the block's last tile
+            rb_bar<5, kRbBuildThreads>();
+            build_a(cur ^ 1, nrows, first, kRbBuildThreads);
+            fence_proxy_async();
+          }
+          rb_bar<3, kRbAuxThreads>();
+          new_keys(cur ^ 1, it + npair);
+        }
+      }
+      it += npair + (tn < N ? 1 : 0);
+      // ---------------------------------------------------------------- settle the block's steps
+      // Owner table: own[slot] = first step that claims the slot in this pass | pass parity << 7, so that claims of the
+      // pass before need not be cleared first; (own ^ tag) < r says that a step before r claims the slot (0xFF: nobody).
+      if (warp < kRbResWarps) {
+        tc_fence_before();
+        const int r = tid;  // warps 0-3: this thread's step
+        const bool mine = tid < rows;
+        int top_slot = 0, sv = 0, prev = 0;  // warps 0-3: best base slot, slot that the step writes (now, a pass ago)
+        bool forced = false, flagged = false;  // ... the best base slot may hold a recent token; or a new entry may win
+        if (warp < 4) {
+          if (ncta > 1) rb_wait_cluster(peer_bar, blk & 1, &abort_flag);
+          for (int c = 0; c < kRbReadGroups * ncta; ++c) topf = fmaxf(topf, Mx[(c >> 1) * L.mx_block + top_at + (c & 1) * kRbRows + r]);
+          const int top = __float2int_rn(topf);
+          top_slot = max(0, min(kRbIdxMask - (top & kRbIdxMask), C - 1));
+          sv = prev = top_slot;
+          forced = PROT && r < Rn;
+          flagged = forced || NR[cur * kRbRows + r] >= (top >> kRbKeyShift);
+          RN[r] = top;
+          if (tid < 2) s_change[tid] = kRbRows;
+        }
+        int fb = 0;                    // steps below are final
+        for (int pass = 0;; ++pass) {  // every pass but the last of a window makes at least one more step final
+          const int wend = min(fb + (pass < kRbWidePasses ? kRbRows : kRbResWarps), rows);
+          const uint32_t tag = (uint32_t)(pass & 1) << 7;
+          const int par = pass & 1;
+          bool is_hard = false;
+          if (warp < 4) {
+            // Claims: earlier warps store after later ones, so that a slot goes to its first warp; among that warp's lanes any
+            // may win, the earlier ones store again.
+            SV[r] = mine ? (uint16_t)sv : (uint16_t)0xFFFFu;
+#pragma unroll
+            for (int k = 3; k >= 0; --k) {
+              if (warp == k && mine) own[sv] = (uint8_t)((uint32_t)r | tag);
+              rb_bar<1, kRbRows>();
+            }
+            for (;;) {
+              const uint32_t o = own[sv] ^ tag;
+              const bool again = mine && (int)(o >> 5) == warp && o > (uint32_t)r;
+              if (!__any_sync(0xFFFFFFFFu, again)) break;
+              if (again) own[sv] = (uint8_t)((uint32_t)r | tag);
+              __syncwarp();
+            }
+            rb_bar<1, kRbRows>();
+            const uint32_t o_top = own[top_slot];
+            if (prev != sv && (own[prev] ^ (tag ^ 0x80u)) < 128u) own[prev] = 0xFFu;  // claimed a pass ago, by nobody now
+            // hard steps of the window
+            const bool stale = (o_top ^ tag) < (uint32_t)r;
+            is_hard = r >= fb && r < wend && (flagged || stale);
+            const uint32_t hm = __ballot_sync(0xFFFFFFFFu, is_hard);
+            if (is_hard) LIST[warp * 32 + __popc(hm & ((1u << lane) - 1u))] = (uint8_t)((uint32_t)r | (stale || forced ? 0x80u : 0u));
+            if (lane == 0) s_hard[par][warp] = (uint8_t)__popc(hm);
+            if (!is_hard && r >= fb && r < wend && sv != top_slot) atomicMin(&s_change[par], r);
+          }
+          rb_bar<2, kRbResThreads>();
+          if (tid == 0) s_change[par ^ 1] = kRbRows;
+          // The hard steps are dealt round-robin over all warps (later steps are hard more often than earlier ones): entry e
+          // of the four lists one after another.
+          const uint32_t nhard = *reinterpret_cast<const uint32_t*>(s_hard[par]);
+          const int n0 = nhard & 0xFFu, n1 = n0 + ((nhard >> 8) & 0xFFu), n2 = n1 + ((nhard >> 16) & 0xFFu), n3 = n2 + (nhard >> 24);
+          for (int e0 = warp; e0 < n3; e0 += kRbResWarps) {
+            const int entry = LIST[e0 < n1 ? (e0 < n0 ? e0 : 32 + e0 - n0) : (e0 < n2 ? 64 + e0 - n1 : 96 + e0 - n2)];
+            const int r2 = entry & 127;
+            const uint2 dd = *reinterpret_cast<const uint2*>(Dn + cur * (kRbRows / 2) * kRbDnPitch + rb_dn_at(r2) + (4 * lane < r2 ? 4 * lane : 0));
+            const uint2 s4 = *reinterpret_cast<const uint2*>(SV + 4 * lane);
+            int kb = RN[r2];
+            const int sv2 = SV[r2];
+            // best new entry: written by an earlier step and no longer recent (whether a later step has overwritten it is
+            // looked at below, if it matters)
+            const int elim = (PROT ? r2 - Rn : r2) - 4 * lane;
+            auto ekey = [&](int e, uint32_t d2, uint32_t slot) {
+              return e < elim ? (int)((d2 << (kRbKeyShift - 1)) + (kRbIdxMask - slot)) : -1;
+            };
+            int k0 = ekey(0, dd.x & 0xFFFFu, s4.x & 0xFFFFu), k1 = ekey(1, dd.x >> 16, s4.x >> 16);
+            int k2 = ekey(2, dd.y & 0xFFFFu, s4.y & 0xFFFFu), k3 = ekey(3, dd.y >> 16, s4.y >> 16);
+            int kn = __reduce_max_sync(0xFFFFFFFFu, max(max(k0, k1), max(k2, k3)));
+            // Both candidates are upper bounds until looked at; the larger one is, until it holds. A base slot may be taken
+            // (or recent): its tile is scanned again for this step and its live slots replace the tile's maximum. A new
+            // entry may have been overwritten: it leaves the race. Each round takes a tile or an entry out.
+            bool exact = (entry & 0x80) == 0;  // kb is a live slot's key
+            bool loaded = false;
+            float mt[4];  // lane l: tiles l, l + 32, ...
+            RbRank<WORDS, GT> rk;
+            int live = -1;  // best live slot of the tiles scanned so far, this lane's share
+            for (int round = 0; round <= nbase + kRbRows; ++round) {
+              if (kn > kb) {
+                const uint32_t slot = (uint32_t)(kRbIdxMask - (kn & kRbIdxMask));
+                const bool e0s = (s4.x & 0xFFFFu) == slot, e1s = (s4.x >> 16) == slot, e2s = (s4.y & 0xFFFFu) == slot, e3s = (s4.y >> 16) == slot;
+                const int before = r2 - 4 * lane;  // entries of this lane below it were written before step r2
+                int l = -1, kl = -1;
+                if (e0s && 0 < before) l = 0, kl = k0;
+                if (e1s && 1 < before) l = 1, kl = k1;
+                if (e2s && 2 < before) l = 2, kl = k2;
+                if (e3s && 3 < before) l = 3, kl = k3;
+                const int newest = __reduce_max_sync(0xFFFFFFFFu, l < 0 ? -1 : 4 * lane + l);
+                if (__any_sync(0xFFFFFFFFu, l >= 0 && 4 * lane + l == newest && kl == kn)) break;
+                // the slot holds a later entry with another rank, or one that is still recent
+                if (e0s && 4 * lane != newest) k0 = -1;
+                if (e1s && 4 * lane + 1 != newest) k1 = -1;
+                if (e2s && 4 * lane + 2 != newest) k2 = -1;
+                if (e3s && 4 * lane + 3 != newest) k3 = -1;
+                kn = __reduce_max_sync(0xFFFFFFFFu, max(max(k0, k1), max(k2, k3)));
+                continue;
+              }
+              if (exact || kb < 0) break;
+              const int sb = min(kRbIdxMask - (kb & kRbIdxMask), C - 1);
+              if (loaded || PROT) {  // (the first time it is known to be taken)
+                bool bad = (own[sb] ^ tag) < (uint32_t)r2;
+                if (PROT && r2 < Rn && !bad) {  // REC[m - 1] entered m steps before the block: recent while r2 + m <= Rn
+                  bool hit = false;
+                  for (int m0 = 0; m0 < Rn - r2; m0 += 32) hit |= m0 + lane < Rn - r2 && REC[m0 + lane] == sb;
+                  bad = __any_sync(0xFFFFFFFFu, hit);
+                }
+                if (!bad) break;
+              }
+              if (!loaded) {
+                loaded = true;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const int T = lane + 32 * i;
+                  mt[i] = T < nbase ? Mx[(T & (ncta - 1)) * L.mx_block + r2 * L.mx_pitch + (T >> lg_ncta)] : -1.f;
+                }
+                rk.load(qb + r2 * GW, G, PAR[cur * kRbRows + r2]);
+              }
+              const int cb = sb >> 7, j0 = cb * kRbTile + 4 * lane;
+              const uint32_t o4 = *reinterpret_cast<const uint32_t*>(own + j0) ^ (tag * 0x01010101u);
+              uint32_t hw[4 * WORDS];
+#pragma unroll
+              for (int i = 0; i < WORDS; ++i) *reinterpret_cast<uint4*>(hw + 4 * i) = *reinterpret_cast<const uint4*>(codes + j0 * WORDS + 4 * i);
+              // bit 7 of a byte: nobody claims the slot before r2 (unclaimed bytes have bit 7 set, claims are below 128)
+              uint32_t ok4 = (((o4 | 0x80808080u) - (uint32_t)r2 * 0x01010101u) | o4);
+              if (PROT && r2 < Rn)
+                for (int m0 = 0; m0 < Rn - r2; ++m0) {
+                  const int q = REC[m0] - j0;
+                  if (q >= 0 && q < 4) ok4 &= ~(0x80u << (8 * q));
+                }
+              const int hi = C - j0, lo = PROT ? S - j0 : 0;
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                uint32_t h[WORDS];
+#pragma unroll
+                for (int w = 0; w < WORDS; ++w) h[w] = hw[e * WORDS + w];
+                const int key = (rk.rank(h) << kRbKeyShift) + (kRbIdxMask - (j0 + e));
+                const bool ok = (ok4 & (0x80u << (8 * e))) != 0u && e < hi && (!PROT || e >= lo);
+                live = max(live, ok ? key : -1);
+              }
+              float mm = -1.f;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                if (cb == lane + 32 * i) mt[i] = -1.f;
+                mm = fmaxf(mm, mt[i]);
+              }
+              // (keys are whole numbers below 2^23: the sum has them in its mantissa)
+              const int km = mm < 0.f ? -1 : (int)(__float_as_uint(mm + 8388608.f) & 0x7FFFFFu);
+              kb = __reduce_max_sync(0xFFFFFFFFu, max(live, km));
+            }
+            const int slot = min(kRbIdxMask - (max(max(kb, kn), 0) & kRbIdxMask), C - 1);
+            if (lane == 0) {
+              SN[r2] = slot;
+              if (slot != sv2) atomicMin(&s_change[par], r2);
+            }
+          }
+          rb_bar<2, kRbResThreads>();
+          const int ch = s_change[par];
+          prev = sv;
+          if (ch < kRbRows) {
+            fb = ch + 1;
+            if (warp < 4 && r < wend && r >= ch) sv = is_hard ? SN[r] : top_slot;
+          } else {
+            fb = wend;
+            if (fb >= rows) break;
+          }
+        }
+        if (ncta > 1 && warp == 4 && lane < ncta - 1) rb_arrive_remote(rb_mapa(used_bar, (uint32_t)((rank + 1 + lane) & (ncta - 1))));
+        // ------------------------------------------------------------ Algorithm 1 lines 2-5 on the table
+        const bool scoring = write_scores && tn == N;
+        auto apply = [&](int slot) {
+          if (!HE_IN_RANGE(slot, C)) return;
+#pragma unroll
+          for (int w = 0; w < WORDS; ++w) codes[slot * WORDS + w] = kb_codes[r * WORDS + w];
+          if (rank == 0) pos_g[slot] = t0 + r;
+        };
+        // last writers: the steps claim again, later ones over earlier ones (the prompt's last step waits until its scores
+        // are taken)
+        if (warp < 4) {
+          const bool in = mine && !(scoring && r == rows - 1);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (warp == k && in) own[sv] = (uint8_t)r;
+            rb_bar<1, kRbRows>();
+          }
+          for (;;) {
+            const int o = own[sv];
+            const bool again = in && (o >> 5) == warp && o < r;
+            if (!__any_sync(0xFFFFFFFFu, again)) break;
+            if (again) own[sv] = (uint8_t)r;
+            __syncwarp();
+          }
+          rb_bar<1, kRbRows>();
+          if (in && own[sv] == (uint8_t)r) apply(sv);
+          rb_bar<1, kRbRows>();
+          if (mine) own[sv] = 0xFFu;
+        }
+        int keep = 0;
+        if (PROT && tid < Rn) keep = tid < rows ? 0 : REC[tid - rows];
+        if (scoring) {  // Eq. 5 for every slot as the prompt's last step sees the table
+          rb_bar<2, kRbResThreads>();
+          RbRank<WORDS, GT> rk;
+          rk.load(qb + (rows - 1) * GW, G, PAR[cur * kRbRows + rows - 1]);
+          for (int j = rank * kRbResThreads + tid; j < C; j += ncta * kRbResThreads) {
+            uint32_t h[WORDS];
+#pragma unroll
+            for (int w = 0; w < WORDS; ++w) h[w] = codes[j * WORDS + w];
+            sc[j] = -(float)rk.dist(h);
+          }
+          rb_bar<2, kRbResThreads>();
+          if (tid == rows - 1) apply(sv);
+        }
+        if (PROT && Rn > 0) {  // the newest tokens before the next block
+          rb_bar<2, kRbResThreads>();
+          if (tid < Rn) REC[tid] = tid < rows ? (int)SV[rows - 1 - tid] : keep;
+        }
+      }
+      ++blk;
+      cur ^= 1;
+      __syncthreads();
+      tc_fence_after();
+    }
+    // final state of the unit; everything beyond `fill` is reset
+    const bool scored = write_scores && N > C;
+    for (int j = rank * NT + tid; j < (int)Cmax; j += ncta * NT) {
+      const bool valid = j < fill0;
+      uint32_t cw[WORDS];
+#pragma unroll
+      for (int w = 0; w < WORDS; ++w) cw[w] = valid ? codes[j * WORDS + w] : 0u;
+      store_slot_code<WORDS>(cfg, a.ca.codes, unit * Cmax + j, cw);
+      if (!(valid && scored)) sc[j] = 0.f;
+    }
+    if (rank == 0 && tid == 0) {
+      a.ca.fill[unit] = fill0;
+      a.ca.next_pos[unit] = N;
+    }
+    __syncthreads();  // the tables and s_unit are reused by the next unit
+  }
+
+  // A CTA that gave up must not free tensor memory under an MMA that is still writing it (the operands are written by
+  // this CTA's own threads, so no copy from outside is ever in flight): one more commit of each MMA warp tracks everything
+  // it has issued, and their completion is awaited (bounded) first.
+  if (abort_flag && (warp == kRbMmaWarp || warp == kRbMmaWarp + 1) && rb_elect()) {
+    tc_commit(drain_bar);
+    mbar_drain(drain_bar, 0);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kRbMmaWarp) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(4 * kRbTile) : "memory");
+  }
+  if (tid == 0 && abort_flag) atomicAdd(&g_tc_error, 1);
+  if (ncta > 1) rb_cluster_sync();  // no CTA leaves while a peer may still copy into its shared memory
+}
+
+}  // namespace he
