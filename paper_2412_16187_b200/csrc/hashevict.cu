@@ -179,21 +179,54 @@ int sm_count(int* out) {
   return HE_OK;
 }
 
-// Tensor map of the rows to hash, as a 4-D bf16 tensor {channel, row or token, head, sequence} with a box of
-// 64 channels x 128 rows and the 128-byte shared-memory swizzle. Returns false when the driver's encoder is not
-// available or rejects the strides (the kernel then stages rows with cp.async instead).
-bool encode_rows_tmap(const HashJob& job, long long max_rows_per_segment, int segments, CUtensorMap* out) {
-  using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static EncodeFn encode = [] {
+// The driver's tensor-map encoder, or null.
+using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn tmap_encoder() {
+  static EncodeTiledFn encode = [] {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess ||
         q != cudaDriverEntryPointSuccess)
       fn = nullptr;
-    return reinterpret_cast<EncodeFn>(fn);
+    return reinterpret_cast<EncodeTiledFn>(fn);
   }();
+  return encode;
+}
+
+// Tensor map of a K or V cache [rows, d] in bf16: boxes of 64 channels x 32 rows, 128-byte swizzle. A map depends on the address
+// and the shape alone, so the last few are kept per thread (a decode loop asks for the same ones at every token).
+bool cache_rows_tmap(const void* base, long long rows, int d, CUtensorMap* out) {
+  struct Entry {
+    const void* base;
+    long long rows;
+    int d;
+    CUtensorMap map;
+  };
+  constexpr int kEntries = 128;
+  thread_local Entry cache[kEntries] = {};
+  Entry& e = cache[(reinterpret_cast<uintptr_t>(base) >> 9) * 0x9E3779B97F4A7C15ull >> 57];
+  if (e.base != base || e.rows != rows || e.d != d) {
+    const EncodeTiledFn encode = tmap_encoder();
+    if (encode == nullptr || rows > 0x7FFFFFFF) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)d * 2};
+    const cuuint32_t box[2] = {64, (cuuint32_t)kAttendGroup}, estr[2] = {1, 1};
+    if (encode(&e.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+      e.base = nullptr;
+      return false;
+    }
+    e.base = base, e.rows = rows, e.d = d;
+  }
+  *out = e.map;
+  return true;
+}
+
+// Tensor map of the rows to hash, as a 4-D bf16 tensor {channel, row or token, head, sequence} with a box of
+// 64 channels x 128 rows and the 128-byte shared-memory swizzle. Returns false when the driver's encoder is not
+// available or rejects the strides (the kernel then stages rows with cp.async instead).
+bool encode_rows_tmap(const HashJob& job, long long max_rows_per_segment, int segments, CUtensorMap* out) {
+  const EncodeTiledFn encode = tmap_encoder();
   memset(out, 0, sizeof(*out));
   if (encode == nullptr || env_flag_set<2>("HE_DISABLE_TMA")) return false;
   cuuint64_t dims[4], strides[3];
@@ -593,6 +626,81 @@ int launch_replay(const ReplayArgs& a, long long units, cudaStream_t stream) {
   }
 }
 
+template <int D, int NW>
+int launch_attend_on(const AttendArgs& a, int S, size_t smem, cudaStream_t st) {
+  if (int rc = set_smem(attend_bf16_kernel<D, NW>, smem)) return rc;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3((unsigned)(a.cfg.n_kv_heads * S), (unsigned)a.cfg.batch);
+  lc.blockDim = dim3(32 * NW);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)S;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = S > 1 ? 2 : 1;
+  const long long rows = (long long)a.cfg.batch * a.cfg.n_kv_heads * a.cfg.max_budget;
+  alignas(64) CUtensorMap kmap, vmap;
+  if (!cache_rows_tmap(a.ca.k_cache, rows, D, &kmap) || !cache_rows_tmap(a.ca.v_cache, rows, D, &vmap))
+    return fail(HE_ERR_CUDA, "no tensor map for a cache of %lld rows x %d", rows, D);
+  HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, attend_bf16_kernel<D, NW>, a, S, kmap, vmap));
+  return HE_OK;
+}
+
+// Tensor-core attention with S CTAs per unit. A call pays 2.5 us (one CTA) to 4 us (cluster of 8) whatever it reads, an SM pulls
+// 90 GB/s, the GPU 6.3 TB/s, so a unit is spread until the grid has one CTA per SM. Measured (us per call in a graph, caches larger
+// than L2; register-fed kernel with clusters of up to 8 before): 8 units of 9830 slots 16.9 -> 10.6, 32 of 2048 8.7 -> 7.9, 128 of
+// 1024 14.6 -> 12.9.
+template <int D>
+int launch_attend(const AttendArgs& a, cudaStream_t st) {
+  const long long units = (long long)a.cfg.batch * a.cfg.n_kv_heads;
+  int sms = 0, dev = 0;
+  if (int rc = sm_count(&sms)) return rc;
+  HE_CUDA_CHECK(cudaGetDevice(&dev));
+  static_assert(8 * kMaxGroup * (D + 2) * sizeof(float) <= AttendRing<D, 8>::kBytes, "the merge reuses the rings");
+  auto smem_of = [&](int S) { return 1024 + (size_t)AttendRing<D, 8>::kBytes + (S > 1 ? (size_t)S * a.cfg.group_size * (D + 2) * sizeof(float) : 0); };
+  // As many CTAs per unit as keep the grid within one (deep) CTA per SM, and no fewer than 256 slots (a group per warp)
+  // for each. Clusters above 8 need the driver's consent and as many free SMs in one GPC, so they are asked about.
+  int S = (int)(sms / units < 16 ? sms / units : 16);
+  if (S > a.cfg.max_budget / 256) S = a.cfg.max_budget / 256;
+  if (S > 8) {
+    static int fit[64][17] = {};  // clusters of S that the device holds at once (-1: none)
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    for (S &= ~1; S > 8; S -= 2) {
+      if (fit[dev][S] == 0) {
+        int got = 0;
+        cudaLaunchConfig_t oc{};
+        oc.gridDim = dim3(S * 16);
+        oc.blockDim = dim3(256);
+        oc.dynamicSmemBytes = kMaxDynSmem;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = S;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        oc.attrs = at;
+        oc.numAttrs = 1;
+        if (int rc = set_smem(attend_bf16_kernel<D, 8>, kMaxDynSmem)) return rc;
+        if (cudaFuncSetAttribute(attend_bf16_kernel<D, 8>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&got, attend_bf16_kernel<D, 8>, &oc) != cudaSuccess || got < 1) {
+          (void)cudaGetLastError();
+          got = -1;
+        }
+        fit[dev][S] = got;
+      }
+      if (fit[dev][S] >= units && smem_of(S) <= kMaxDynSmem) break;
+    }
+  }
+  if (S < 1) S = 1;
+  // Two small CTAs per SM once there are more units than SMs, so that one streams while the other starts or merges (512 units
+  // of 1000 slots, d = 64: 24.4 against 27.7 us; level at 256 units of 2048 slots).
+  if (units > sms) return launch_attend_on<D, 4>(a, 1, 1024 + AttendRing<D, 4>::kBytes, st);
+  return launch_attend_on<D, 8>(a, S, smem_of(S), st);
+}
+
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Scratch of he_prefill_compress_noalloc: part of the device image, so no allocation is ever needed for it.
@@ -923,33 +1031,11 @@ int he_attend(const he_config* cfg, const he_cache* cache, const void* q, float*
   const dim3 grid((unsigned)cfg->n_kv_heads, (unsigned)cfg->batch);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int G = cfg->group_size, d = cfg->head_dim;
-  if (cfg->dtype == HE_DTYPE_BF16 && d == 128 && getenv("HE_DISABLE_ATTEND_MMA") == nullptr) {
-    // Cluster size: the largest power of two (<= 8) that keeps the grid within one CTA per SM.
-    const long long units = (long long)cfg->batch * cfg->n_kv_heads;
-    int sms = 0;
-    if (int rc = sm_count(&sms)) return rc;
-    int S = 1;
-    while (S < 8 && units * (S * 2) <= sms) S *= 2;
-    const size_t smem = (size_t)(kAttendWarps + 1) * G * (d + 2) * sizeof(float);
-    if (int rc = set_smem(attend_bf16_kernel, smem)) return rc;
-    cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3((unsigned)(cfg->n_kv_heads * S), (unsigned)cfg->batch);
-    lc.blockDim = dim3(kAttendThreads);
-    lc.dynamicSmemBytes = smem;
-    lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)S;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, attend_bf16_kernel, a, S));
-  } else {
-    const size_t smem = ((size_t)G * d + (size_t)kAttendWarps * G * (d + 2)) * sizeof(float);
-    if (int rc = set_smem(attend_generic_kernel, smem)) return rc;
-    attend_generic_kernel<<<grid, kAttendThreads, smem, st>>>(a);
-  }
+  if (cfg->dtype == HE_DTYPE_BF16 && (d == 64 || d == 128) && getenv("HE_DISABLE_ATTEND_MMA") == nullptr)
+    return d == 64 ? launch_attend<64>(a, st) : launch_attend<128>(a, st);
+  const size_t smem = ((size_t)G * d + (size_t)kAttendWarps * G * (d + 2)) * sizeof(float);
+  if (int rc = set_smem(attend_generic_kernel, smem)) return rc;
+  attend_generic_kernel<<<grid, kAttendThreads, smem, st>>>(a);
   HE_CUDA_CHECK(cudaGetLastError());
   return HE_OK;
 }
