@@ -310,8 +310,8 @@ int he_device_error_count(void);
  * he_prefill_phase_events - timing aid (the paper has no counterpart). events: five cudaEvent_t handles (as void*)
  * created by the caller with timing enabled, or NULL to switch the aid off. While set, every prefill call of the
  * calling thread (he_prefill_compress and its variants) records them on its stream around its phases, launching
- * exactly the kernels it always launches: [0] start, [1] after Eq. 2 on the prompt keys (with the W image), [2] after
- * Eq. 2 on the queries, [3] after the unit schedule and the replay (or ranking), [4] after the K / V gather. An event
+ * exactly the kernels it always launches: [0], [1] start (Eq. 2 on the keys and on the queries is one launch), [2] after
+ * Eq. 2 on the prompt's keys and queries (with the W image), [3] after the unit schedule and the replay (or ranking), [4] after the K / V gather. An event
  * record is one more stream operation between two kernels, so use it for measurement runs only.
  */
 int he_prefill_phase_events(void* const* events);

@@ -107,7 +107,7 @@ def device_error_count() -> int:
 
 def prefill_phase_events(events=None):
     """he_prefill_phase_events: five torch.cuda.Event(enable_timing=True) that the next prefill calls of this thread
-    record around their phases (hash K, hash Q, schedule + replay, gather), or None to switch that off."""
+    record around their phases (nothing, hash K and Q in one launch, schedule + replay, gather), or None to switch that off."""
     if events is None:
         lib().he_prefill_phase_events(None)
         return

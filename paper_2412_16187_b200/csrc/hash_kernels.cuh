@@ -28,8 +28,12 @@ struct HashJob {
   const void* w_image;  // optional: the tensor-core kernel's shared-memory image of W's three bf16 terms (build_w_image_kernel)
 };
 
+// Segments below `segs` are job1's, the others job2's (a prompt's key rows and query rows in one launch).
 template <int WORDS>
-__global__ void __launch_bounds__(kHashThreads) hash_rows_kernel(const HashJob job) {
+__global__ void __launch_bounds__(kHashThreads) hash_rows_kernel(const __grid_constant__ HashJob job1, const __grid_constant__ HashJob job2, int segs) {
+  griddep_launch_dependents();
+  const bool first_job = (int)blockIdx.y < segs;
+  const HashJob& job = first_job ? job1 : job2;
   extern __shared__ __align__(16) float hsm[];
   constexpr int BP = 32 * WORDS;
   const int d = job.d, b = job.b, es = esize_of(job.dtype);
@@ -47,7 +51,7 @@ __global__ void __launch_bounds__(kHashThreads) hash_rows_kernel(const HashJob j
     out_base = 0;
     out_stride = WORDS;
   } else {
-    const int seg = blockIdx.y;
+    const int seg = first_job ? blockIdx.y : blockIdx.y - segs;
     const int s = seg / job.heads, hh = seg % job.heads;
     const long long C = max(job.budget[s], 0);
     const long long N = clamp_len(job.prompt_len[s], job.Nmax, (int)min(C, 1LL));

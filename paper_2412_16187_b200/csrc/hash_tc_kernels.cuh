@@ -161,6 +161,7 @@ __device__ __forceinline__ void w_image_element(const float* W, int d, int b, in
 // The image in global memory, built once per call when the caller has scratch for it (kWImageBytes at most).
 constexpr size_t kWImageBytes = 3 * 2 * 64 * 128;  // three terms, d = 128, N = 64
 __global__ void build_w_image_kernel(const float* W, int d, int b, int N, unsigned char* image) {
+  griddep_launch_dependents();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx < d * N) w_image_element(W, d, b, N, idx, image);
 }
@@ -253,9 +254,13 @@ __device__ __forceinline__ bool tc_tile(const HashJob& job, long long t, long lo
 
 // Dynamic shared memory (after rounding the base up to 1024 bytes):
 //   B: 3 terms x KH halves x [N rows x 128 bytes]      A: kTcStages x KH halves x [128 rows x 128 bytes]
+//
+// A prompt's key rows and query rows go through one launch (two jobs with the same lengths; total_tiles2 > 0, dense schedule
+// only): tile numbers first count the keys' tiles, then the queries'. Launched behind build_w_image_kernel with the programmatic
+// attribute, so only the image is read after the wait: that kernel itself started when everything earlier had ended.
 template <int WORDS, bool TMA>
-__global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJob job, long long total_tiles,
-                                                                     long long tiles_per_seg,
+__global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const __grid_constant__ HashJob job, const __grid_constant__ HashJob job2,
+                                                                     long long total_tiles, long long total_tiles2, long long tiles_per_seg,
                                                                      const __grid_constant__ CUtensorMap tmap,
                                                                      const __grid_constant__ CUtensorMap tmap2) {
   constexpr int N = 32 * WORDS;
@@ -266,7 +271,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
   __shared__ uint32_t tmem_base_s;
   __shared__ volatile int abort_flag;
   __shared__ int s_len[kTcLenCache], s_bud[kTcLenCache];
-  __shared__ unsigned s_pref[kTcLenCache + 1];  // dense schedule: non-empty tiles (all heads) of the sequences before s
+  __shared__ unsigned s_pref[2][kTcLenCache + 1];  // dense schedule, per job: non-empty tiles (all heads) of the sequences before s
   __shared__ int s_nseq_dense;
 
   // Programmatic dependent launch (used by the large-batch decode step): a kernel launched behind this one may
@@ -319,6 +324,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
   // W -> three bf16 terms, transposed to [bit][channel] (K-major), 128B-swizzled; columns beyond b are zero.
   // Either copied from an image that a one-block-per-slice kernel prepared once for this call, or built here.
   if (job.w_image != nullptr) {
+    griddep_wait();
     const uint4* src = static_cast<const uint4*>(job.w_image);
     uint4* dst = reinterpret_cast<uint4*>(Bs);
     for (int i = tid; i < 3 * KH * b_tile_bytes / 16; i += kTcThreads) dst[i] = __ldg(src + i);
@@ -328,17 +334,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
   fence_proxy_async();  // the generic-proxy writes above are read by the tensor core through the async proxy
   if (job.mode != 0 && nseq <= kTcLenCache && total_tiles < 0x7FFFFFFFll) {
     __syncthreads();  // the cached lengths are complete
-    if (warp == 0) {  // exclusive prefix over the sequences' tile counts, 32 at a time
+    if (warp < 2) {  // exclusive prefix over the sequences' tile counts, 32 at a time; warp 0: the first job, warp 1: the second
+      const HashJob& jb = warp == 0 ? job : job2;
       unsigned run = 0;
       for (int i0 = 0; i0 < nseq; i0 += 32) {
         const int i = i0 + lane;
         unsigned cnt = 0;
         if (i < nseq) {
           const long long Ni = s_len[i], Ci = s_bud[i];
-          const long long r0 = (job.mode == 1 || job.q_all) ? 0 : (Ci < Ni ? Ci : Ni);
+          const long long r0 = (jb.mode == 1 || jb.q_all) ? 0 : (Ci < Ni ? Ci : Ni);
           long long nt = Ni > r0 ? (Ni - r0 + kTcRows - 1) / kTcRows : 0;
           if (nt > tiles_per_seg) nt = tiles_per_seg;
-          cnt = (unsigned)nt * (unsigned)job.heads;
+          cnt = (unsigned)nt * (unsigned)jb.heads;
         }
         unsigned inc = cnt;
 #pragma unroll
@@ -346,12 +353,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
           const unsigned v = __shfl_up_sync(0xFFFFFFFFu, inc, o);
           if (lane >= o) inc += v;
         }
-        if (i < nseq) s_pref[i] = run + inc - cnt;
+        if (i < nseq) s_pref[warp][i] = run + inc - cnt;
         run += __shfl_sync(0xFFFFFFFFu, inc, 31);
       }
       if (lane == 0) {
-        s_pref[nseq] = run;
-        s_nseq_dense = nseq;
+        s_pref[warp][nseq] = run;
+        if (warp == 0) s_nseq_dense = nseq;
       }
     }
   }
@@ -360,8 +367,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
   const int nseq_dense = s_nseq_dense;
-  const long long n_sched = nseq_dense > 0 ? (long long)s_pref[nseq_dense] : total_tiles;  // tile numbers this grid walks
-  int cursor = 0;  // this thread's sequence cursor of the dense schedule
+  const long long n_first = nseq_dense > 0 ? (long long)s_pref[0][nseq_dense] : total_tiles;  // tile numbers of the first job
+  const long long n_sched = n_first + (total_tiles2 > 0 ? (long long)s_pref[1][nseq_dense] : 0);
+  int cursor = 0, cursor2 = 0;  // this thread's sequence cursors of the dense schedule
+  auto tile_of = [&](long long t, TcTile* tl) -> bool {
+    if (t < n_first) return tc_tile<WORDS>(job, t, tiles_per_seg, tl, s_len, s_bud, s_pref[0], nseq_dense, &cursor);
+    const bool any = tc_tile<WORDS>(job2, t - n_first, tiles_per_seg, tl, s_len, s_bud, s_pref[1], nseq_dense, &cursor2);
+    tl->second = 1;
+    return any;
+  };
 
   // Flat rows and the dense schedule number real tiles only, so every role walks t = blockIdx.x, + gridDim.x, ... and all
   // of them are tiles. There the producer warp and the epilogue warps work out the tiles' coordinates 32 at a time, a
@@ -386,7 +400,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
         const long long t = tb + (long long)lane * gridDim.x;
         int row0 = 0, c2 = 0, c3 = 0, second = 0;
         TcTile tl;
-        if (t < n_sched && tc_tile<WORDS>(job, t, tiles_per_seg, &tl, s_len, s_bud, s_pref, nseq_dense, &cursor))
+        if (t < n_sched && tile_of(t, &tl))
           row0 = (int)tl.row0, c2 = tl.c2, c3 = tl.c3, second = tl.second;
         const long long left = (n_sched - tb + gridDim.x - 1) / gridDim.x;
         const int cnt = left < 32 ? (int)left : 32;
@@ -402,7 +416,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
     } else if (lane == 0) {
       for (long long t = blockIdx.x; t < n_sched; t += gridDim.x) {
         TcTile tl;
-        if (!tc_tile<WORDS>(job, t, tiles_per_seg, &tl, s_len, s_bud, s_pref, nseq_dense, &cursor)) continue;
+        if (!tile_of(t, &tl)) continue;
         if (!issue((int)tl.row0, tl.c2, tl.c3, tl.second)) break;
         ++it;
       }
@@ -423,7 +437,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
     };
     for (long long t = blockIdx.x; t < n_sched && ok; t += gridDim.x) {
       TcTile tl;
-      if (!tc_tile<WORDS>(job, t, tiles_per_seg, &tl, s_len, s_bud, s_pref, nseq_dense, &cursor)) continue;
+      if (!tile_of(t, &tl)) continue;
       const int s = it % kTcStages;
       ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty_bar(s), ((it / kTcStages) & 1) ^ 1, &abort_flag));  // warp-uniform
       if (!ok) break;
@@ -457,7 +471,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
         // roles skip them (this thread needs nothing else of the tile, so it avoids the index arithmetic)
         if (job.mode != 0 && nseq_dense == 0) {
           TcTile tl;
-          if (!tc_tile<WORDS>(job, t, tiles_per_seg, &tl, s_len, s_bud, s_pref, nseq_dense, &cursor)) continue;
+          if (!tile_of(t, &tl)) continue;
         }
         const int s = it % kTcStages, acc = it & 1;
         // the epilogue has drained this accumulator and the stage's rows have landed
@@ -491,7 +505,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
     // ------------------------------------------------------------------ epilogue (warps 0-3, one row per thread)
     int it = 0;
     // one tile: `obase` = index of its first row's first code word in job.out, `ostride` words between rows
-    auto epi_tile = [&](long long obase, int ostride, int nrows) -> bool {
+    auto epi_tile = [&](uint32_t* out, long long obase, int ostride, int nrows) -> bool {
       const int acc = it & 1;
       if (!__all_sync(0xFFFFFFFFu, mbar_wait(tfull_bar(acc), (it >> 1) & 1, &abort_flag))) return false;  // warp-uniform
       tc_fence_after();
@@ -517,7 +531,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
       if (lane == 0) mbar_arrive(tempty_bar(acc));
       const int r = warp * 32 + lane;
       if (r < nrows) {
-        uint32_t* o = job.out + obase + (long long)r * ostride;
+        uint32_t* o = out + obase + (long long)r * ostride;
 #pragma unroll
         for (int w = 0; w < WORDS; ++w) o[w] = code[w];
       }
@@ -530,22 +544,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const HashJ
         long long ob = 0;
         int os = 0, nr = 0;  // (a tile that turned out empty would still be consumed, and store nothing)
         TcTile tl;
-        if (t < n_sched && tc_tile<WORDS>(job, t, tiles_per_seg, &tl, s_len, s_bud, s_pref, nseq_dense, &cursor))
+        if (t < n_sched && tile_of(t, &tl))
           ob = tl.out_base + tl.row0 * tl.out_stride, os = (int)tl.out_stride, nr = tl.nrows;
         const long long left = (n_sched - tb + gridDim.x - 1) / gridDim.x;
         const int cnt = left < 32 ? (int)left : 32;
         for (int j = 0; j < cnt && alive; ++j) {
           const long long obj = __shfl_sync(0xFFFFFFFFu, ob, j);
           const int osj = __shfl_sync(0xFFFFFFFFu, os, j), nrj = __shfl_sync(0xFFFFFFFFu, nr, j);
-          alive = epi_tile(obj, osj, nrj);
+          alive = epi_tile(tb + (long long)j * gridDim.x < n_first ? job.out : job2.out, obj, osj, nrj);
           if (alive) ++it;
         }
       }
     } else {
       for (long long t = blockIdx.x; t < n_sched; t += gridDim.x) {
         TcTile tl;
-        if (!tc_tile<WORDS>(job, t, tiles_per_seg, &tl, s_len, s_bud, s_pref, nseq_dense, &cursor)) continue;
-        if (!epi_tile(tl.out_base + tl.row0 * tl.out_stride, (int)tl.out_stride, tl.nrows)) break;
+        if (!tile_of(t, &tl)) continue;
+        if (!epi_tile(job.out, tl.out_base + tl.row0 * tl.out_stride, (int)tl.out_stride, tl.nrows)) break;
         ++it;
       }
     }

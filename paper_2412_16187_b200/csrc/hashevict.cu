@@ -169,6 +169,24 @@ bool tc_enabled() {
   return on;
 }
 
+// Launch with the programmatic-serialization attribute: the kernel may start while the stream's previous kernel still runs and
+// calls griddepcontrol.wait before it touches anything that kernel or an earlier one may have written.
+template <typename... P, typename... A>
+int launch_pdl(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, bool pdl, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = grid;
+  lc.blockDim = dim3(threads);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = (pdl && pdl_enabled()) ? 1 : 0;
+  HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, kernel, args...));
+  return HE_OK;
+}
+
 int sm_count(int* out) {
   static int cached[64] = {};
   int dev = 0;
@@ -259,77 +277,73 @@ bool encode_rows_tmap(const HashJob& job, long long max_rows_per_segment, int se
 }
 
 // Eq. 2 on many rows. bf16 rows with d = 64 or 128 go to the tensor-core kernel once there are enough of them to
-// pay for staging the split W per CTA; everything else runs on the CUDA-core kernel.
-int launch_hash(const HashJob& job, long long max_rows_per_segment, int segments, cudaStream_t stream, bool* image_built = nullptr,
-                bool pdl = false) {
+// pay for staging the split W per CTA; everything else runs on the CUDA-core kernel. A prompt's key rows and query rows
+// (job, job2) share a launch where the kernels allow it: a launch of the persistent kernel pays 12-15 us of set-up and tail.
+int launch_hash(const HashJob& job, long long max_rows_per_segment, int segments, cudaStream_t stream, const HashJob* job2 = nullptr,
+                int segments2 = 0) {
   if (max_rows_per_segment <= 0 || segments <= 0) return HE_OK;
   const int Wd = words_of(job.b);
   const long long tiles = (max_rows_per_segment + kHashRows - 1) / kHashRows;
   // flat rows may come as two ranges (the decode step's query rows and key rows): one launch of the tensor-core kernel
   const bool two = job.mode == 0 && job.x2 != nullptr && job.rows2 > 0;
   const long long tiles2 = two ? (job.rows2 + kHashRows - 1) / kHashRows : 0;
-  const bool tc = tc_enabled() && job.dtype == HE_DTYPE_BF16 && (job.d == 64 || job.d == 128) && (tiles + tiles2) * segments >= 64;
+  const long long total = tiles * segments + tiles2, total2 = job2 != nullptr ? tiles * segments2 : 0;
+  const bool tc = tc_enabled() && job.dtype == HE_DTYPE_BF16 && (job.d == 64 || job.d == 128) && total + total2 >= 64;
   if (two && !tc) {  // the CUDA-core kernel takes one range at a time
     HashJob j1 = job, j2 = job;
     j1.x2 = nullptr, j1.rows2 = 0;
     j2.x = job.x2, j2.rows = job.rows2, j2.out = job.out + job.rows * Wd, j2.x2 = nullptr, j2.rows2 = 0;
-    if (int rc = launch_hash(j1, j1.rows, 1, stream, image_built, pdl)) return rc;
-    return launch_hash(j2, j2.rows, 1, stream, image_built, true);
+    if (int rc = launch_hash(j1, j1.rows, 1, stream)) return rc;
+    return launch_hash(j2, j2.rows, 1, stream);
   }
+  if (job2 != nullptr && (tc ? segments / job.heads > kTcLenCache || total + total2 >= 0x7FFFFFFFLL : segments + segments2 > 65535)) {
+    if (int rc = launch_hash(job, max_rows_per_segment, segments, stream)) return rc;
+    return launch_hash(*job2, max_rows_per_segment, segments2, stream);
+  }
+  const HashJob& second = job2 != nullptr ? *job2 : job;
   if (tc) {
     static_assert(kTcRows == kHashRows, "both kernels tile rows by 128");
     const int N = 32 * Wd, KH = job.d / 64;
     const size_t smem = 1024 + (size_t)3 * KH * N * 128 + (size_t)kTcStages * KH * kTcRows * 128;
     int sms = 0;
     if (int rc = sm_count(&sms)) return rc;
-    const long long total = tiles * segments + tiles2;
-    const unsigned grid = (unsigned)(total < sms ? total : sms);
+    const unsigned grid = (unsigned)(total + total2 < sms ? total + total2 : sms);
     alignas(64) CUtensorMap tmap, tmap2;
     bool tma = encode_rows_tmap(job, max_rows_per_segment, segments, &tmap);
     if (two) {
       HashJob j2 = job;
       j2.x = job.x2, j2.rows = job.rows2;
       tma = encode_rows_tmap(j2, j2.rows, 1, &tmap2) && tma;
+    } else if (job2 != nullptr) {
+      tma = encode_rows_tmap(*job2, max_rows_per_segment, segments2, &tmap2) && tma;
     } else {
       tmap2 = tmap;
     }
-    if (job.w_image != nullptr && (image_built == nullptr || !*image_built)) {  // scratch of kWImageBytes: filled once per call
+    if (job.w_image != nullptr) {  // scratch of kWImageBytes: filled once per launch
       build_w_image_kernel<<<(job.d * N + 255) / 256, 256, 0, stream>>>(job.W, job.d, job.b, N,
                                                                        static_cast<unsigned char*>(const_cast<void*>(job.w_image)));
       HE_CUDA_CHECK(cudaGetLastError());
-      if (image_built != nullptr) *image_built = true;
     }
     auto go = [&](auto kernel) -> int {
       if (int rc = set_smem(kernel, smem)) return rc;
-      cudaLaunchConfig_t lc{};
-      lc.gridDim = dim3(grid);
-      lc.blockDim = dim3(kTcThreads);
-      lc.dynamicSmemBytes = smem;
-      lc.stream = stream;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[0].val.programmaticStreamSerializationAllowed = 1;
-      lc.attrs = attr;
-      lc.numAttrs = (pdl && pdl_enabled()) ? 1 : 0;
-      HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, kernel, job, total, tiles, tmap, tmap2));
-      return HE_OK;
+      // behind its own image kernel the launch may overlap it; the decode step's scan kernel counts on this kernel starting
+      // after everything earlier, so flat rows are launched plainly
+      return launch_pdl(kernel, dim3(grid), kTcThreads, smem, job.w_image != nullptr && job.mode != 0, stream, job, second, total, total2, tiles,
+                        tmap, tmap2);
     };
-    int rc;
-    if (Wd == 1) rc = tma ? go(hash_rows_tc_kernel<1, true>) : go(hash_rows_tc_kernel<1, false>);
-    else rc = tma ? go(hash_rows_tc_kernel<2, true>) : go(hash_rows_tc_kernel<2, false>);
-    if (rc) return rc;
-    HE_CUDA_CHECK(cudaGetLastError());
-    return HE_OK;
+    if (Wd == 1) return tma ? go(hash_rows_tc_kernel<1, true>) : go(hash_rows_tc_kernel<1, false>);
+    return tma ? go(hash_rows_tc_kernel<2, true>) : go(hash_rows_tc_kernel<2, false>);
   }
   const size_t smem = ((size_t)job.d * 32 * Wd + (size_t)kHashRows * job.d) * sizeof(float);
-  if (tiles > 0x7FFFFFFFLL || segments > 65535) return fail(HE_ERR_UNSUPPORTED, "hash grid too large (%lld x %d)", tiles, segments);
-  dim3 grid((unsigned)tiles, (unsigned)segments);
+  const int segs = segments + (job2 != nullptr ? segments2 : 0);
+  if (tiles > 0x7FFFFFFFLL || segs > 65535) return fail(HE_ERR_UNSUPPORTED, "hash grid too large (%lld x %d)", tiles, segs);
+  dim3 grid((unsigned)tiles, (unsigned)segs);
   if (Wd == 1) {
     if (int rc = set_smem(hash_rows_kernel<1>, smem)) return rc;
-    hash_rows_kernel<1><<<grid, kHashThreads, smem, stream>>>(job);
+    hash_rows_kernel<1><<<grid, kHashThreads, smem, stream>>>(job, second, segments);
   } else {
     if (int rc = set_smem(hash_rows_kernel<2>, smem)) return rc;
-    hash_rows_kernel<2><<<grid, kHashThreads, smem, stream>>>(job);
+    hash_rows_kernel<2><<<grid, kHashThreads, smem, stream>>>(job, second, segments);
   }
   HE_CUDA_CHECK(cudaGetLastError());
   return HE_OK;
@@ -442,9 +456,7 @@ int launch_replay_smem(const ReplayArgs& a, long long units, cudaStream_t stream
   if (a.cfg.max_budget > 4096) nt = 512;
   if (a.cfg.max_budget > 16384) nt = 1024;
   if (int rc = set_smem(prefill_replay_smem_kernel<WORDS, GT>, smem)) return rc;
-  prefill_replay_smem_kernel<WORDS, GT><<<(unsigned)units, nt, smem, stream>>>(a);
-  HE_CUDA_CHECK(cudaGetLastError());
-  return HE_OK;
+  return launch_pdl(prefill_replay_smem_kernel<WORDS, GT>, dim3((unsigned)units), nt, smem, true, stream, a);
 }
 
 // The register kernel is persistent: as many CTAs as fit the GPU at once, each claiming units from the schedule.
@@ -462,13 +474,10 @@ int launch_replay_reg_one(const ReplayArgs& a, long long units, cudaStream_t str
     per_sm[dev] = n > 0 ? n : 1;
   }
   const int nbins = sms < kMaxBins ? sms : kMaxBins;
-  prefill_schedule_kernel<<<1, kSchedThreads, 0, stream>>>(a.cfg, a.ca.budget, a.prompt_len, nbins, a.sched, 0);
-  HE_CUDA_CHECK(cudaGetLastError());
+  if (int rc = launch_pdl(prefill_schedule_kernel, dim3(1), kSchedThreads, 0, a.Nmax > 0, stream, a.cfg, a.ca.budget, a.prompt_len, nbins, a.sched, 0)) return rc;
   long long grid = (long long)sms * per_sm[dev];
   if (grid > units) grid = units;
-  prefill_replay_reg_kernel<WORDS, GT, SPT, NT><<<(unsigned)grid, NT, smem, stream>>>(a);
-  HE_CUDA_CHECK(cudaGetLastError());
-  return HE_OK;
+  return launch_pdl(prefill_replay_reg_kernel<WORDS, GT, SPT, NT>, dim3((unsigned)grid), NT, smem, true, stream, a);
 }
 
 // Smallest (threads x slots-per-thread) tile of the register kernel that holds max_budget slots.
@@ -558,20 +567,21 @@ int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t s
   ra.ncta = n;
   ra.scheduled = units > clusters ? 1 : 0;
   if (ra.scheduled) {  // one queue, largest unit first
-    prefill_schedule_kernel<<<1, kSchedThreads, 0, stream>>>(a.cfg, a.ca.budget, a.prompt_len, 1, a.sched, 2700);
-    HE_CUDA_CHECK(cudaGetLastError());
+    if (int rc = launch_pdl(prefill_schedule_kernel, dim3(1), kSchedThreads, 0, a.Nmax > 0, stream, a.cfg, a.ca.budget, a.prompt_len, 1, a.sched, 2700)) return rc;
   }
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3((unsigned)(clusters * n));
   lc.blockDim = dim3(kRbThreads);
   lc.dynamicSmemBytes = smem;
   lc.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)n;
-  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)n;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   lc.attrs = attr;
-  lc.numAttrs = n > 1 ? 1 : 0;
+  lc.numAttrs = n > 1 ? 2 : 1;
   HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, kernel, ra));
   return HE_OK;
 }
@@ -818,8 +828,7 @@ int he_decode_step(const he_config* cfg, const he_cache* cache, const void* q, c
     job.x2 = k;
     job.rows2 = units_ll;
     job.out = cache->step_scratch;
-    bool image_built = false;
-    if (int rc = launch_hash(job, job.rows, 1, st, &image_built)) return rc;
+    if (int rc = launch_hash(job, job.rows, 1, st)) return rc;
     a.new_codes = cache->step_scratch;
   }
   if (cache->budget_host != nullptr && cfg->batch <= kMaxBudgetVals) {
@@ -883,7 +892,6 @@ int prefill_impl(int variant /* 0: Algorithm 1, 1: averaged Hamming, 2: L2 norm 
   uint32_t* qcodes = reinterpret_cast<uint32_t*>(static_cast<char*>(workspace) +
                                                  align_up((size_t)units * max_prompt_len * Wd * 4, 256));
 
-  bool image_built = false;
   record_phase(0, st);
   // phase 1: Eq. 2 on every prompt key and on the queries of the tokens that will evict
   HashJob job{};
@@ -905,20 +913,17 @@ int prefill_impl(int variant /* 0: Algorithm 1, 1: averaged Hamming, 2: L2 norm 
   job.s0 = kv_strides[0];
   job.s1 = kv_strides[1];
   job.s2 = kv_strides[2];
-  if (int rc = launch_hash(job, max_prompt_len, (int)units, st, &image_built)) return rc;
+  HashJob qjob = job;
+  qjob.x = q;
+  qjob.out = qcodes;
+  qjob.mode = 2;
+  qjob.q_all = oneshot ? 1 : 0;  // the ranking reads the queries of all later tokens, Algorithm 1 only those that evict
+  qjob.heads = cfg->n_kv_heads * G;
+  qjob.s0 = q_strides[0];
+  qjob.s1 = q_strides[1];
+  qjob.s2 = q_strides[2];
   record_phase(1, st);
-  if (variant != 2) {
-  job.x = q;
-  job.out = qcodes;
-  job.mode = 2;
-  job.q_all = oneshot ? 1 : 0;  // the ranking reads the queries of all later tokens, Algorithm 1 only those that evict
-  job.heads = cfg->n_kv_heads * G;
-  job.s0 = q_strides[0];
-  job.s1 = q_strides[1];
-  job.s2 = q_strides[2];
-  if (int rc = launch_hash(job, max_prompt_len, (int)units * G, st, &image_built)) return rc;
-  }
-
+  if (int rc = launch_hash(job, max_prompt_len, (int)units, st, variant != 2 ? &qjob : nullptr, (int)units * G)) return rc;
   record_phase(2, st);
   // phase 2: the sequential replay of Algorithm 1 over the prompt, one CTA per unit
   int32_t* sched = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(qcodes) +
@@ -957,13 +962,16 @@ int prefill_impl(int variant /* 0: Algorithm 1, 1: averaged Hamming, 2: L2 norm 
     while ((1 << lg) < cpr) ++lg;
     const int rows_per_cta = (kGatherThreads >> lg) * kGatherRows;
     const long long gx = ((long long)cfg->max_budget + rows_per_cta - 1) / rows_per_cta;
-    prefill_gather_rows_kernel<<<dim3((unsigned)gx, (unsigned)units), kGatherThreads, 0, st>>>(ga, lg);
+    // Only a small gather is launched programmatically: blocks of a large one that settle early on the SMs the replay has left
+    // make it uneven (64 ragged prompts: 1418 us a call without, 1457 with the attribute).
+    int sms = 0;
+    if (int rc = sm_count(&sms)) return rc;
+    if (int rc = launch_pdl(prefill_gather_rows_kernel, dim3((unsigned)gx, (unsigned)units), kGatherThreads, 0, gx * units <= 2 * sms, st, ga, lg)) return rc;
   } else {
     const long long per_unit = 2LL * cfg->max_budget * cpr;
     const long long gx = (per_unit + kGatherThreads * kGatherUnroll - 1) / (kGatherThreads * kGatherUnroll);
-    prefill_gather_kernel<<<dim3((unsigned)gx, (unsigned)units), kGatherThreads, 0, st>>>(ga);
+    if (int rc = launch_pdl(prefill_gather_kernel, dim3((unsigned)gx, (unsigned)units), kGatherThreads, 0, false, st, ga)) return rc;
   }
-  HE_CUDA_CHECK(cudaGetLastError());
   record_phase(4, st);
   return HE_OK;
 }

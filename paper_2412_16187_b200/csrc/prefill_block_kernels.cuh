@@ -276,6 +276,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   __shared__ int s_change[2];                    // by pass parity: first step that changed
   __shared__ __align__(4) uint8_t s_hard[2][4];  // by pass parity: lengths of warps 0-3's lists of hard steps
 
+  griddep_launch_dependents();
   const ReplayArgs& a = ar.r;
   const he_config& cfg = a.cfg;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -349,6 +350,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
     lut_hi |= (c + 4 <= G ? rb_e5m2(-alpha * (2 * (c + 4) - G)) : 0u) << (8 * c);
   }
   for (int i = tid; i < a.smem_slots / 4; i += NT) reinterpret_cast<uint32_t*>(own)[i] = 0xFFFFFFFFu;
+  griddep_wait();  // everything above overlaps the hashing kernel's tail
   tc_fence_before();
   __syncthreads();
   if (ncta > 1) rb_cluster_sync();  // every CTA of the cluster runs before anyone copies into it

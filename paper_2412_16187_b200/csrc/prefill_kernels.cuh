@@ -70,6 +70,8 @@ constexpr int kSchedThreads = 1024;
 
 __host__ __device__ inline size_t sched_words(long long units) { return 3 + 2 * (size_t)kMaxBins + (size_t)units; }
 
+// Launched programmatically behind the hashing, which it does not depend on: it runs beside it (its output is read by the
+// kernels of this call only, and the call's first kernel started when everything earlier had ended).
 // step_cost: fixed cost of one evicting step in units of one slot scanned (0 for the register kernel, whose step is a
 // scan; several thousand for the tensor-core kernel, whose step is mostly the resolver's latency).
 __global__ void __launch_bounds__(kSchedThreads) prefill_schedule_kernel(const he_config cfg, const int32_t* budget,
@@ -79,6 +81,7 @@ __global__ void __launch_bounds__(kSchedThreads) prefill_schedule_kernel(const h
   __shared__ int start_s[kMaxBins];
   __shared__ unsigned char bin_of[kSchedSortMax];  // nbins <= 256
   __shared__ unsigned short pos_of[kSchedSortMax];  // place of the unit inside its bin
+  griddep_launch_dependents();
   const int tid = threadIdx.x;
   const int units = cfg.batch * cfg.n_kv_heads;
   int32_t* bin_start = sched + 2;
@@ -102,6 +105,7 @@ __global__ void __launch_bounds__(kSchedThreads) prefill_schedule_kernel(const h
       for (int k = 0; k < b; ++k) before += (units - k + nbins - 1) / nbins;
       order[before + u / nbins] = u;
     }
+    griddep_wait();
     return;
   }
   int n = 1;
@@ -154,6 +158,7 @@ __global__ void __launch_bounds__(kSchedThreads) prefill_schedule_kernel(const h
   __syncthreads();
   // sorted order, so each bin lists its largest unit first
   for (int i = tid; i < units; i += kSchedThreads) order[start_s[bin_of[i]] + pos_of[i]] = 0xFFFFF - (int)(keys[i] & 0xFFFFF);
+  griddep_wait();  // whoever waits for this kernel waits for the ones before it
 }
 
 // Next unit for this CTA: from the bin of the SM it runs on, else from the first other bin that still has work.
@@ -206,6 +211,8 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? 4 : (NT <= 512 ? 2 : 1))) pre
   const bool prot = cfg.n_sink > 0 || cfg.n_recent > 0;
   const bool write_scores = (cfg.flags & HE_FLAG_WRITE_SCORES) != 0;
 
+  griddep_launch_dependents();
+  griddep_wait();
   for (;;) {
     if (warp == 0) {
       const int u = claim_unit(a.sched, lane);
@@ -359,6 +366,8 @@ __global__ void prefill_replay_smem_kernel(const ReplayArgs a) {
   __shared__ uint32_t wbest[2][2][32];
   __shared__ uint32_t stage[2][kStepBlock * Stager::kRec];
 
+  griddep_launch_dependents();
+  griddep_wait();
   const he_config& cfg = a.cfg;
   const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
   const long long unit = blockIdx.x;
@@ -512,6 +521,8 @@ __global__ void __launch_bounds__(kGatherThreads) prefill_gather_kernel(const Ga
 // per thread; kGatherRows slots per group, so eight loads per thread are in flight. No division anywhere.
 constexpr int kGatherRows = 4;
 __global__ void __launch_bounds__(kGatherThreads) prefill_gather_rows_kernel(const GatherArgs a, int lg_cpr) {
+  griddep_launch_dependents();
+  griddep_wait();
   const he_config& cfg = a.cfg;
   const long long unit = blockIdx.y;
   const int s = (int)(unit / cfg.n_kv_heads), h = (int)(unit % cfg.n_kv_heads);
