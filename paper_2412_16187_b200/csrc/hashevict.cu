@@ -501,18 +501,19 @@ constexpr size_t kRbMinSmem = 120 * 1024;
 constexpr size_t kMaxDynSmem = 227 * 1024 - 2048;  // dynamic shared memory of a CTA beside the kernel's static arrays
 
 // Shared memory of the block replay with as many operand stages as fit (fewer for large two-word tables); 0: does not fit.
-size_t rb_fit(int words, int slots, int G, int ncta, int* lg_stage, int* abuf) {
-  for (*abuf = 2; *abuf >= 1; --*abuf)
-    for (*lg_stage = 2; *lg_stage >= 1; --*lg_stage) {
-      const size_t smem = rb_layout(words, slots, G, ncta, 1 << *lg_stage, *abuf).total;
-      if (smem <= kMaxDynSmem) return smem < kRbMinSmem ? kRbMinSmem : smem;
+size_t rb_fit(int words, int slots, int G, int ncta, int rows_max, RbArgs* ra) {
+  ra->rows_max = rows_max;
+  for (ra->abuf = 2; ra->abuf >= 1; --ra->abuf)
+    for (ra->lg_stage = 2; ra->lg_stage >= 1; --ra->lg_stage) {
+      ra->L = rb_layout(words, slots, G, ncta, 1 << ra->lg_stage, ra->abuf, rows_max);
+      if (ra->L.total <= kMaxDynSmem) return ra->L.total < kRbMinSmem ? kRbMinSmem : ra->L.total;
     }
   return 0;
 }
 
-template <int WORDS, int GT, bool PROT>
-int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t stream) {
-  auto kernel = prefill_replay_block_kernel<WORDS, GT, PROT>;
+template <int WORDS, int GT, bool PROT, bool HALF>
+int launch_replay_block_half(const ReplayArgs& a, long long units, cudaStream_t stream) {
+  auto kernel = prefill_replay_block_kernel<WORDS, GT, PROT, HALF>;
   RbArgs ra{};
   ra.r = a;
   ra.r.smem_slots = (a.cfg.max_budget + kRbTile - 1) / kRbTile * kRbTile;
@@ -527,7 +528,7 @@ int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t s
   int best_lg = -1;
   for (int lg = 0; (1 << lg) <= kRbMaxCluster && (lg == 0 || (1 << lg) <= tiles); ++lg) {
     const int n = 1 << lg;
-    if (rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, &ra.lg_stage, &ra.abuf) == 0) continue;
+    if (rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, HALF ? kRbRows / 2 : kRbRows, &ra) == 0) continue;
     int fit = sms;
     if (n > 1) {
       int& cached = max_clusters[dev][lg];
@@ -559,11 +560,10 @@ int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t s
   }
   if (best_lg < 0) return fail(HE_ERR_UNSUPPORTED, "max_budget %d does not fit the block replay's shared memory", a.cfg.max_budget);
   const int n = 1 << best_lg;
-  const size_t smem = rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, &ra.lg_stage, &ra.abuf);
+  const size_t smem = rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, HALF ? kRbRows / 2 : kRbRows, &ra);
   if (int rc = set_smem(kernel, smem)) return rc;
   const long long fit = n > 1 ? max_clusters[dev][best_lg] : sms;
   const long long clusters = units < fit ? units : fit;
-  ra.L = rb_layout(WORDS, ra.r.smem_slots, a.cfg.group_size, n, 1 << ra.lg_stage, ra.abuf);
   ra.ncta = n;
   ra.scheduled = units > clusters ? 1 : 0;
   if (ra.scheduled) {  // one queue, largest unit first
@@ -584,6 +584,17 @@ int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t s
   lc.numAttrs = n > 1 ? 2 : 1;
   HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, kernel, ra));
   return HE_OK;
+}
+
+// Two-word tables above about 8200 slots only fit with blocks of 64 steps.
+template <int WORDS, int GT, bool PROT>
+int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t stream) {
+  if constexpr (WORDS == 2) {
+    RbArgs fit{};
+    if (rb_fit(WORDS, (a.cfg.max_budget + kRbTile - 1) / kRbTile * kRbTile, a.cfg.group_size, 1, kRbRows, &fit) == 0)
+      return launch_replay_block_half<WORDS, GT, PROT, true>(a, units, stream);
+  }
+  return launch_replay_block_half<WORDS, GT, PROT, false>(a, units, stream);
 }
 
 template <int WORDS>
@@ -609,7 +620,8 @@ int block_replay_mode() {
 template <int WORDS>
 int launch_replay(const ReplayArgs& a, long long units, cudaStream_t stream) {
   const int slots = (a.cfg.max_budget + kRbTile - 1) / kRbTile * kRbTile;
-  int lg_stage = 0, abuf = 0, sms = 0;
+  RbArgs fit{};
+  int sms = 0;
   if (int rc = sm_count(&sms)) return rc;
   const int mode = block_replay_mode();
   // The block kernel has one CTA per SM and pays a block's settling (8000 cycles) whatever the budget; the CUDA-core kernels
@@ -621,7 +633,7 @@ int launch_replay(const ReplayArgs& a, long long units, cudaStream_t stream) {
   const bool has_reg = a.cfg.group_size == 1 || a.cfg.group_size == 4;
   const int min_budget = units <= sms ? (has_reg ? 1 : 128) : (WORDS == 2 && a.cfg.group_size == 4 ? 256 : 384);
   bool block_ok = mode != 0 && (mode == 2 || a.cfg.max_budget >= min_budget) && a.cfg.max_budget <= kRbMaxSlots &&
-                  rb_fit(WORDS, slots, a.cfg.group_size, 1, &lg_stage, &abuf) != 0;
+                  rb_fit(WORDS, slots, a.cfg.group_size, 1, WORDS == 2 ? kRbRows / 2 : kRbRows, &fit) != 0;
   if (block_ok && (a.cfg.n_sink > 0 || a.cfg.n_recent > 0)) {
     // protected windows: every budget must leave an eligible slot at every step (n_sink + n_recent < C), which the host
     // can only check on the caller's mirror of the budgets

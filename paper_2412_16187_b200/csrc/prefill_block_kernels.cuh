@@ -64,15 +64,16 @@ constexpr int kRbMaxCluster = 8;
 constexpr int kRbWidePasses = 6;         // passes over the whole block before the window shrinks
 constexpr int kRbAtom = 128 * 128;       // 128 operand rows x one 128-byte swizzle atom
 constexpr int kRbDnPitch = 136;          // 16-bit entries between rows of the new-entry table
+constexpr int kRbDnPitchHalf = 68;       // ... when blocks have at most 64 steps
 constexpr int kRbMaxStages = 4;          // pairs of operand tiles
 
 // Byte offsets of the kernel's dynamic shared memory (after rounding its base up to 1024 bytes). Tile maxima: per CTA of the
 // cluster one block of fp32 keys, a row for each step, an odd number of words apart (a warp stores a column, a lane per
 // step), then the best key of each step over each reader group's tiles.
 struct RbLayout {
-  uint32_t a, bidx, b, codes, own, mx, mx_pitch, mx_block, dn, rn, nr, sv, sn, list, par, qraw, kraw, rec, total;
+  uint32_t a, bidx, b, codes, own, mx, mx_pitch, mx_block, top_at, dn, dn_buf, rn, nr, sv, sn, list, par, qraw, kraw, rec, total;
 };
-__host__ __device__ inline RbLayout rb_layout(int words, int slots, int G, int ncta, int nstage, int abuf) {
+__host__ __device__ inline RbLayout rb_layout(int words, int slots, int G, int ncta, int nstage, int abuf, int rows_max) {
   RbLayout L;
   const uint32_t nt = (uint32_t)slots / kRbTile, ntl = (nt + ncta - 1) / ncta;
   uint32_t o = 0;
@@ -88,9 +89,12 @@ __host__ __device__ inline RbLayout rb_layout(int words, int slots, int G, int n
   L.codes = take((uint32_t)slots * words * 4u);
   L.own = take((uint32_t)slots);
   L.mx_pitch = ntl | 1u;  // words
-  L.mx_block = (L.mx_pitch + kRbReadGroups) * kRbRows;
+  // (one more row takes the threads without a step; whole 16-byte units, as the copies between CTAs want)
+  L.top_at = (L.mx_pitch * (rows_max < kRbRows ? rows_max + 1 : rows_max) + 3u) & ~3u;
+  L.mx_block = L.top_at + kRbReadGroups * rows_max;
   L.mx = take(L.mx_block * ncta * 4u);
-  L.dn = take(2u * (kRbRows / 2) * kRbDnPitch * 2u);
+  L.dn_buf = rows_max == kRbRows ? kRbRows / 2 * kRbDnPitch : rows_max * kRbDnPitchHalf;  // entries
+  L.dn = take(2u * L.dn_buf * 2u);
   L.rn = take(kRbRows * 4u);
   L.nr = take(2u * kRbRows * 4u);
   L.sv = take(kRbRows * 2u);
@@ -110,6 +114,7 @@ struct RbArgs {
   int scheduled;  // units are claimed from r.sched; 0: unit = cluster index
   int lg_stage;   // log2 of the pairs of operand tiles in shared memory
   int abuf;       // operand A buffers (2: the next block's is built during the tile phase)
+  int rows_max;   // steps per block at most: 128, or 64 (the HALF kernel)
   RbLayout L;     // computed by the host: kernel parameters cost no registers
 };
 
@@ -163,8 +168,9 @@ __device__ __forceinline__ bool rb_elect() {
 }
 
 // The ranks of a block's own keys at its steps: step r only needs those of the r steps before it, so steps 64 + k and 63 - k
-// share a row (64 + k entries from its start, 63 - k from the next multiple of four).
-__device__ __forceinline__ int rb_dn_at(int r) {
+// share a row (64 + k entries from its start, 63 - k from the next multiple of four). Blocks of 64 have a row each.
+__device__ __forceinline__ int rb_dn_at(int r, int rows_max) {
+  if (rows_max < kRbRows) return r * kRbDnPitchHalf;
   return r >= 64 ? (r - 64) * kRbDnPitch : (63 - r) * kRbDnPitch + ((127 - r + 3) & ~3);
 }
 
@@ -264,12 +270,14 @@ struct RbRank {
 // masked like slots past the budget. A recent token that is already in the table is recognised by the list of the newest
 // slots, one of this block's own keys by its step. Needs every budget > n_sink + n_recent (so that some slot is always
 // eligible), n_sink <= 128 (one tile) and n_recent < 128.
-template <int WORDS, int GT, bool PROT>
+// HALF: blocks of at most 64 steps, where the largest two-word tables leave no room for the tables of more.
+template <int WORDS, int GT, bool PROT, bool HALF>
 __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(const __grid_constant__ RbArgs ar) {
   constexpr int NT = kRbThreads;
   constexpr int MS = kRbMaxStages;
+  constexpr int RM = HALF ? kRbRows / 2 : kRbRows;
   extern __shared__ unsigned char rb_smem_raw[];
-  __shared__ __align__(8) unsigned long long bars[2 * MS + 4 + 4];
+  __shared__ __align__(8) unsigned long long bars[2 * MS + 4 + 5];
   __shared__ uint32_t tmem_base_s;
   __shared__ volatile int abort_flag;
   __shared__ int s_unit[2];
@@ -295,7 +303,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   uint32_t* codes = reinterpret_cast<uint32_t*>(smem + L.codes);
   uint8_t* own = smem + L.own;
   float* Mx = reinterpret_cast<float*>(smem + L.mx);
-  const int top_at = kRbRows * L.mx_pitch;  // where a CTA's block of Mx holds its groups' best keys
+  const int top_at = HALF ? L.top_at : RM * L.mx_pitch;  // where a CTA's block of Mx holds its groups' best keys
   uint16_t* Dn = reinterpret_cast<uint16_t*>(smem + L.dn);
   int32_t* RN = reinterpret_cast<int32_t*>(smem + L.rn);    // per step: best base key
   int32_t* NR = reinterpret_cast<int32_t*>(smem + L.nr);    // per step: largest rank of any earlier key of the block, two buffers
@@ -317,6 +325,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   const uint32_t used_bar = bar0 + 8u * (2 * MS + 5);                    // peers: they are done with this CTA's maxima
   const uint32_t adone_bar = bar0 + 8u * (2 * MS + 6);                   // one operand A buffer: the block's tiles are multiplied
   const uint32_t drain_bar = bar0 + 8u * (2 * MS + 7);                   // abort path
+  const uint32_t tops_bar = bar0 + 8u * (2 * MS + 8);                    // peers' copies of their best keys have arrived
   if (tid == 0) {
     abort_flag = 0;
     mbar_init(drain_bar, 2);
@@ -330,6 +339,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
       mbar_init(afree_bar(i), 8);
     }
     mbar_init(peer_bar, 1);
+    mbar_init(tops_bar, 1);
     mbar_init(used_bar, ncta > 1 ? ncta - 1 : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -395,7 +405,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
     const int S = PROT ? cfg.n_sink : 0, Rn = PROT ? cfg.n_recent : 0;
     const int nbase = (C + kRbTile - 1) / kRbTile;
     const int ntl = nbase > rank ? (nbase - rank + ncta - 1) >> lg_ncta : 0;  // this CTA's tiles: rank, rank + ncta, ...
-    const int R = rb_block_rows(C);
+    const int R = min(rb_block_rows(C), RM);
     // the first C tokens fill the cache in order; everything beyond `fill` is reset
     for (int j = tid; j < nbase * kRbTile; j += NT) {
 #pragma unroll
@@ -519,7 +529,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
       const int r = x, last = PROT ? r - Rn : r;  // entries below `last` are candidates
       const float magic = (off - (float)((PAR[buf * kRbRows + r] & 1) << 13)) * (1.f / 16384.f) + 4194304.f;
       const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(2 * acc * kRbTile);
-      uint16_t* dst = Dn + buf * (kRbRows / 2) * kRbDnPitch + rb_dn_at(r);
+      uint16_t* dst = Dn + buf * L.dn_buf + rb_dn_at(r, RM);
       float dmax = -1e9f;
 #pragma unroll 1
       for (int c = 0; c < 4; ++c) {
@@ -545,7 +555,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             const float y1 = fmaf(__uint_as_float(v[4 * k + 2 * e + 1]), 1.f / 16384.f, magic);
             pk[e] = __byte_perm(__float_as_uint(y0), __float_as_uint(y1), 0x5410);
           }
-          if (c * 32 + 4 * k < r) *reinterpret_cast<uint2*>(dst + c * 32 + 4 * k) = make_uint2(pk[0], pk[1]);
+          if (c * 32 + 4 * k < r && r < RM) *reinterpret_cast<uint2*>(dst + c * 32 + 4 * k) = make_uint2(pk[0], pk[1]);
         }
       }
       NR[buf * kRbRows + r] = last > 0 ? (int)(__float_as_uint(fmaf(dmax, 1.f / 16384.f, magic)) & 0xFFFFu) >> 1 : -1;
@@ -576,7 +586,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
       float topf = -1.f;  // readers: best base key of the thread's step so far
       if (warp < kRbExpWarp) {
         const int r = tid & 127, grp = warp >> 2;  // this thread's step = its tensor-memory lane; tile grp of each pair
-        float* mrow = Mx + rank * L.mx_block + r * L.mx_pitch;
+        float* mrow = Mx + rank * L.mx_block + min(r, RM) * L.mx_pitch;
         // 2^14 rank + index: the step's constant, and 127 - tile above the index within the tile (lower tiles first)
         float ct = off - (float)((PAR[cur * kRbRows + r] & 1) << 13) + (float)((127 - ((grp << lg_ncta) + rank)) * 128);
         const float cstep = (float)(256 << lg_ncta);
@@ -619,16 +629,22 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             mrow[i] = key;
           }
         }
-        Mx[rank * L.mx_block + top_at + grp * kRbRows + r] = topf;  // this group's best key of the step
+        if (r < RM) Mx[rank * L.mx_block + top_at + grp * RM + r] = topf;  // this group's best key of the step
         if (ncta > 1) fence_proxy_async();
         rb_bar<4, 32 * kRbExpWarp>();  // the reader groups see each other's results
         if (tid < ncta - 1) {          // ... and every peer gets this CTA's block
           const uint32_t peer = (uint32_t)((rank + 1 + tid) & (ncta - 1)), la = smem_u32(Mx + rank * L.mx_block);
-          rb_copy_to_peer(rb_mapa(la, peer), la, L.mx_block * 4u, rb_mapa(peer_bar, peer));
+          // the best keys, which the settling starts from, then the tiles' (1 KB each against 6 KB at 9830 slots and 8 CTAs)
+          const uint32_t tops = la + 4u * (uint32_t)top_at;
+          rb_copy_to_peer(rb_mapa(tops, peer), tops, (uint32_t)(kRbReadGroups * RM) * 4u, rb_mapa(tops_bar, peer));
+          rb_copy_to_peer(rb_mapa(la, peer), la, 4u * (uint32_t)top_at, rb_mapa(peer_bar, peer));
         }
         __syncwarp();
       } else if (warp < kRbMmaWarp) {
-        if (ncta > 1 && tid == 32 * kRbExpWarp) mbar_arrive_expect_tx(peer_bar, L.mx_block * 4u * (uint32_t)(ncta - 1));
+        if (ncta > 1 && tid == 32 * kRbExpWarp) {
+          mbar_arrive_expect_tx(tops_bar, (uint32_t)(kRbReadGroups * RM * (ncta - 1)) * 4u);
+          mbar_arrive_expect_tx(peer_bar, 4u * (uint32_t)(top_at * (ncta - 1)));
+        }
         const int x = tid & 127;  // this thread's row of both tiles of a pair
         const uint32_t* base = codes + (rank * kRbTile + x) * WORDS;
         const int tstep = (kRbTile * WORDS) << lg_ncta;  // words between this CTA's tiles
@@ -703,8 +719,8 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         int top_slot = 0, sv = 0, prev = 0;  // warps 0-3: best base slot, slot that the step writes (now, a pass ago)
         bool forced = false, flagged = false;  // ... the best base slot may hold a recent token; or a new entry may win
         if (warp < 4) {
-          if (ncta > 1) rb_wait_cluster(peer_bar, blk & 1, &abort_flag);
-          for (int c = 0; c < kRbReadGroups * ncta; ++c) topf = fmaxf(topf, Mx[(c >> 1) * L.mx_block + top_at + (c & 1) * kRbRows + r]);
+          if (ncta > 1) rb_wait_cluster(tops_bar, blk & 1, &abort_flag);
+          for (int c = 0; c < kRbReadGroups * ncta; ++c) topf = fmaxf(topf, Mx[(c >> 1) * L.mx_block + top_at + (c & 1) * RM + (r < RM ? r : 0)]);
           const int top = __float2int_rn(topf);
           top_slot = max(0, min(kRbIdxMask - (top & kRbIdxMask), C - 1));
           sv = prev = top_slot;
@@ -745,6 +761,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             if (is_hard) LIST[warp * 32 + __popc(hm & ((1u << lane) - 1u))] = (uint8_t)((uint32_t)r | (stale || forced ? 0x80u : 0u));
             if (lane == 0) s_hard[par][warp] = (uint8_t)__popc(hm);
             if (!is_hard && r >= fb && r < wend && sv != top_slot) atomicMin(&s_change[par], r);
+            if (ncta > 1 && pass == 0) rb_wait_cluster(peer_bar, blk & 1, &abort_flag);  // the peers' tile maxima
           }
           rb_bar<2, kRbResThreads>();
           if (tid == 0) s_change[par ^ 1] = kRbRows;
@@ -755,7 +772,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           for (int e0 = warp; e0 < n3; e0 += kRbResWarps) {
             const int entry = LIST[e0 < n1 ? (e0 < n0 ? e0 : 32 + e0 - n0) : (e0 < n2 ? 64 + e0 - n1 : 96 + e0 - n2)];
             const int r2 = entry & 127;
-            const uint2 dd = *reinterpret_cast<const uint2*>(Dn + cur * (kRbRows / 2) * kRbDnPitch + rb_dn_at(r2) + (4 * lane < r2 ? 4 * lane : 0));
+            const uint2 dd = *reinterpret_cast<const uint2*>(Dn + cur * L.dn_buf + rb_dn_at(r2, RM) + (4 * lane < r2 ? 4 * lane : 0));
             const uint2 s4 = *reinterpret_cast<const uint2*>(SV + 4 * lane);
             int kb = RN[r2];
             const int sv2 = SV[r2];

@@ -16,6 +16,7 @@ SHAPES = {
     "one_unit_cluster": base.scaled(n_kv_heads=1, hash_bits=32, budget=9830, prompt_len=10300),
     "one_unit_cluster_protected": base.scaled(n_kv_heads=1, hash_bits=32, budget=5000, prompt_len=5400, n_sink=4, n_recent=100),
     "two_words_large": base.scaled(n_kv_heads=1, budget=8190, prompt_len=8600),
+    "two_words_largest": base.scaled(n_kv_heads=1, budget=9830, prompt_len=10200),
     "units_over_clusters": base.scaled(batch=4, n_kv_heads=25, hash_bits=32, ragged=True, budget_lo=300, budget_hi=2600, head_dim=64),
     "units_over_sms": base.scaled(batch=10, n_kv_heads=16, ragged=True, budget_lo=200, budget_hi=500, head_dim=64),
 }
