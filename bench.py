@@ -67,7 +67,7 @@ def prefill_bytes_per_call(w, budgets, plens):
 
 
 NOMINAL_HBM_GBS = 8000.0  # the vendor's figure, for context beside the measured copy bandwidth
-RESOLVER_CYCLES_PER_STEP = 144.0  # one warp walking Algorithm 1's evicting steps in order (measured in isolation)
+CHAIN_CYCLES_PER_STEP = 144.0  # one warp walking Algorithm 1's evicting steps in order (measured in isolation)
 
 
 def profiled_traffic(kernel, workload):
@@ -83,13 +83,13 @@ def profiled_traffic(kernel, workload):
 
 
 def replay_bounds(w, budgets, plens, sms, sm_mhz):
-    """What bounds Section 3's sequential prompt replay in this design: every evicting step of a unit passes through
-    one resolver warp (a dependent chain of RESOLVER_CYCLES_PER_STEP cycles), one unit per SM at a time."""
+    """A yardstick for Section 3's sequential prompt replay: one warp per SM that walks a unit's evicting steps in order (a
+    dependent chain of CHAIN_CYCLES_PER_STEP cycles). The block replay settles steps side by side and may exceed it."""
     N = plens.astype(np.int64)
     C = np.minimum(budgets.astype(np.int64), N)
     steps = float((N - C).sum()) * w.n_kv_heads  # evicting steps of one call, all units
     clock = (sm_mhz or 1965.0) * 1e6
-    return steps, sms * clock / RESOLVER_CYCLES_PER_STEP  # steps per call, steps per second at the chain's pace
+    return steps, sms * clock / CHAIN_CYCLES_PER_STEP  # steps per call, steps per second at the chain's pace
 
 
 # ------------------------------------------------------------------------------------------------- clocks
@@ -384,8 +384,8 @@ def run_ours(args, w):
     def replay_bound_obj(wk, budgets_, plens_, replay_ms):
         steps, peak_steps = replay_bounds(wk, budgets_, plens_, sms, sm_mhz)
         ach = steps / (replay_ms * 1e-3)
-        return {"bound": "latency: one resolver warp per SM walks a unit's evicting steps in order, a dependent chain of "
-                         f"{RESOLVER_CYCLES_PER_STEP:.0f} cycles per step", "unit": "evicting steps/s", "achieved": ach,
+        return {"bound": "yardstick: one warp per SM that walks a unit's evicting steps in order, a dependent chain of "
+                         f"{CHAIN_CYCLES_PER_STEP:.0f} cycles per step", "unit": "evicting steps/s", "achieved": ach,
                 "peak": peak_steps, "frac": ach / peak_steps, "evicting_steps_per_call": steps,
                 "hbm_floor_ms_of_the_whole_call": None}
 
