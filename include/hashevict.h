@@ -86,7 +86,7 @@ typedef struct he_cache {
   int32_t* fill;
   int32_t* next_pos;
   const float* W;
-  const int32_t* budget_host; /* optional HOST copy of budget ([B]), or NULL. When given (and B <= 1024)
+  const int32_t* budget_host; /* optional HOST copy of budget ([B]), or NULL. When given (and B <= 256)
                                  he_decode_step passes the budgets in the kernel parameters, which saves the
                                  kernel one dependent device read before it can start streaming the code table.
                                  With protected windows (n_sink or n_recent > 0) he_prefill_compress also needs it to

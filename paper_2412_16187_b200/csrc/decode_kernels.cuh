@@ -15,7 +15,7 @@
 
 namespace he {
 
-constexpr int kMaxBudgetVals = 1024;  // budgets carried in the kernel parameters (4 KB)
+constexpr int kMaxBudgetVals = 256;  // budgets carried in the kernel parameters (1 KB: every launch pays for its parameters' size)
 
 struct DecodeArgs {
   he_config cfg;
@@ -29,8 +29,10 @@ struct DecodeArgs {
   const uint32_t* new_codes;               // PRE kernels: [B*Hkv*G + B*Hkv, Wd] codes of this step's q rows, then k rows
   int n_budget_vals;                       // > 0: budgets are in budget_vals (copied from he_cache.budget_host)
   int n_sched;                             // > 0: sched lists the sequences by budget, largest first (sequence << 21 | budget)
-  int32_t budget_vals[kMaxBudgetVals];
-  uint32_t sched[kMaxBudgetVals];
+  union {
+    int32_t budget_vals[kMaxBudgetVals];
+    uint32_t sched[kMaxBudgetVals];
+  };
 };
 
 constexpr int kVecsPerThread = 8;  // 16-byte code vectors per thread (the host picks the block size accordingly)
