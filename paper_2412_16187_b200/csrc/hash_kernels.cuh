@@ -1,14 +1,18 @@
 // he_hash_keys and phase 1 of he_prefill_compress: Eq. 2 on many rows with CUDA-core fp32 FMAs.
-// A CTA stages W (zero-padded to 32 or 64 columns) and a tile of 128 rows in shared memory as fp32; each warp owns
-// 16 rows and each lane one (or two) hash bits, so a row's sign bits are packed by one warp ballot per code word.
+// A CTA stages W (zero-padded to 32 or 64 columns) and a tile of 128 rows in shared memory as fp32; a warp owns 32 rows, a lane
+// a block of 8 rows x 4 bits of every code word (16 shared-memory reads for 256 FMAs with two words). fp32 rows and a dense W are
+// staged with cp.async, all of it in flight at once: staged through registers, a few loads at a time, the tile's latency
+// bound the kernel (39 000 cycles per tile where its FMAs need 8200).
 #pragma once
 #include "common.cuh"
 
 namespace he {
 
-constexpr int kHashThreads = 256;
+constexpr int kHashThreads = 128;
 constexpr int kHashRows = 128;  // rows per CTA
-constexpr int kHashRpw = 16;    // rows per warp
+constexpr int kHashRpw = 32;    // rows per warp
+constexpr int kHashRpl = 8;     // rows per lane
+constexpr int kHashPad = 4;     // floats between staged rows: neighbouring rows start on other banks
 
 struct HashJob {
   const void* x;
@@ -38,7 +42,8 @@ __global__ void __launch_bounds__(kHashThreads) hash_rows_kernel(const __grid_co
   constexpr int BP = 32 * WORDS;
   const int d = job.d, b = job.b, es = esize_of(job.dtype);
   float* Ws = hsm;            // [d][BP]
-  float* xs = hsm + d * BP;   // [kHashRows][d]
+  float* xs = hsm + d * BP;   // [kHashRows][d + kHashPad]
+  const int xp = d + kHashPad;
 
   // which rows does this CTA hash, and where do the codes go
   const char* base;
@@ -73,76 +78,88 @@ __global__ void __launch_bounds__(kHashThreads) hash_rows_kernel(const __grid_co
   if (row0 >= r_end) return;
   const int nrows = (int)((r_end - row0) < kHashRows ? (r_end - row0) : kHashRows);
 
-  for (int idx = threadIdx.x; idx < d * BP; idx += kHashThreads) {
-    const int c = idx / BP, i = idx % BP;
-    Ws[idx] = i < b ? __ldg(job.W + (long long)c * b + i) : 0.f;
-  }
-  const int cpr = d * es / 16;  // 16-byte chunks per row
-  for (int idx = threadIdx.x; idx < kHashRows * cpr; idx += kHashThreads) {
-    const int r = idx / cpr, ch = idx % cpr;
-    if (r < nrows) {
-      stage_chunk(xs + r * d, base + (row0 + r) * stride * es, ch, job.dtype);
-    } else {
-      float* o = xs + r * d + ch * (16 / es);
-      for (int i = 0; i < 16 / es; ++i) o[i] = 0.f;
+  if (b == BP && (reinterpret_cast<uintptr_t>(job.W) & 15u) == 0) {
+    for (int idx = threadIdx.x; idx < d * BP / 4; idx += kHashThreads) cp_async16(Ws + 4 * idx, job.W + 4 * idx);
+  } else {
+#pragma unroll 8
+    for (int idx = threadIdx.x; idx < d * BP; idx += kHashThreads) {
+      const int c = idx / BP, i = idx % BP;
+      Ws[idx] = i < b ? __ldg(job.W + (long long)c * b + i) : 0.f;
     }
   }
+  const int cpr = d * es / 16;  // 16-byte chunks per row
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < kHashRows * cpr; idx += kHashThreads) {
+    const int r = idx / cpr, ch = idx - r * cpr;
+    // rows past the end repeat the last one; their codes are not stored
+    const char* src = base + (row0 + min(r, nrows - 1)) * stride * es;
+    if (job.dtype == HE_DTYPE_F32) cp_async16(xs + r * xp + ch * 4, src + ch * 16);
+    else stage_chunk(xs + r * xp, src, ch, HE_DTYPE_BF16);
+  }
+  cp_async_commit();
+  cp_async_wait_all();
   __syncthreads();
 
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float* xw = xs + warp * kHashRpw * d;
-  float tot[kHashRpw][WORDS];
+  // lane (rg, bg): rows rg, rg + 4, ... of the warp's 32, bits 4 bg .. 4 bg + 3 of every code word
+  constexpr int BPL = 4 * WORDS;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, bg = lane & 7, rg = lane >> 3;
+  const float* xw = xs + (warp * kHashRpw + rg) * xp;
+  const float* ww = Ws + bg * 4;
+  float tot[kHashRpl][BPL];
 #pragma unroll
-  for (int r = 0; r < kHashRpw; ++r)
+  for (int r = 0; r < kHashRpl; ++r)
 #pragma unroll
-    for (int w = 0; w < WORDS; ++w) tot[r][w] = 0.f;
+    for (int k = 0; k < BPL; ++k) tot[r][k] = 0.f;
 
   for (int c0 = 0; c0 < d; c0 += kChunk) {
-    float acc[kHashRpw][WORDS];
+    float acc[kHashRpl][BPL];
 #pragma unroll
-    for (int r = 0; r < kHashRpw; ++r)
+    for (int r = 0; r < kHashRpl; ++r)
 #pragma unroll
-      for (int w = 0; w < WORDS; ++w) acc[r][w] = 0.f;
+      for (int k = 0; k < BPL; ++k) acc[r][k] = 0.f;
     const int cend = (d - c0) < kChunk ? (d - c0) : kChunk;
+#pragma unroll 1
     for (int cc = 0; cc < cend; cc += 4) {
-      float wv[4][WORDS];
+      float4 xv[kHashRpl];
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
+      for (int r = 0; r < kHashRpl; ++r) xv[r] = *reinterpret_cast<const float4*>(xw + r * 4 * xp + c0 + cc);
 #pragma unroll
-        for (int w = 0; w < WORDS; ++w) wv[k][w] = Ws[(c0 + cc + k) * BP + lane + 32 * w];
-#pragma unroll
-      for (int r = 0; r < kHashRpw; ++r) {
-        const float4 xv = *reinterpret_cast<const float4*>(xw + r * d + c0 + cc);
+      for (int c = 0; c < 4; ++c) {
+        float wv[BPL];
 #pragma unroll
         for (int w = 0; w < WORDS; ++w) {
-          acc[r][w] = fmaf(xv.x, wv[0][w], acc[r][w]);
-          acc[r][w] = fmaf(xv.y, wv[1][w], acc[r][w]);
-          acc[r][w] = fmaf(xv.z, wv[2][w], acc[r][w]);
-          acc[r][w] = fmaf(xv.w, wv[3][w], acc[r][w]);
+          const float4 w4 = *reinterpret_cast<const float4*>(ww + (c0 + cc + c) * BP + 32 * w);
+          wv[4 * w] = w4.x, wv[4 * w + 1] = w4.y, wv[4 * w + 2] = w4.z, wv[4 * w + 3] = w4.w;
+        }
+#pragma unroll
+        for (int r = 0; r < kHashRpl; ++r) {
+          const float x = c == 0 ? xv[r].x : (c == 1 ? xv[r].y : (c == 2 ? xv[r].z : xv[r].w));
+#pragma unroll
+          for (int k = 0; k < BPL; ++k) acc[r][k] = fmaf(x, wv[k], acc[r][k]);
         }
       }
     }
 #pragma unroll
-    for (int r = 0; r < kHashRpw; ++r)
+    for (int r = 0; r < kHashRpl; ++r)
 #pragma unroll
-      for (int w = 0; w < WORDS; ++w) tot[r][w] += acc[r][w];
+      for (int k = 0; k < BPL; ++k) tot[r][k] += acc[r][k];
   }
 
-  uint32_t mine[WORDS];
+  // a lane's four bits of a word, then the eight lanes of the row together
 #pragma unroll
-  for (int w = 0; w < WORDS; ++w) mine[w] = 0u;
-#pragma unroll
-  for (int r = 0; r < kHashRpw; ++r)
+  for (int r = 0; r < kHashRpl; ++r) {
+    const int row = warp * kHashRpw + r * 4 + rg;
 #pragma unroll
     for (int w = 0; w < WORDS; ++w) {
-      const uint32_t word = __ballot_sync(0xFFFFFFFFu, tot[r][w] >= 0.f) & word_mask(b, w);
-      if (lane == r) mine[w] = word;
-    }
-  const int r = warp * kHashRpw + lane;
-  if (lane < kHashRpw && r < nrows) {
-    uint32_t* o = job.out + out_base + (row0 + r) * out_stride;
+      uint32_t word = 0u;
 #pragma unroll
-    for (int w = 0; w < WORDS; ++w) o[w] = mine[w];
+      for (int k = 0; k < 4; ++k) word |= (tot[r][4 * w + k] >= 0.f ? 1u : 0u) << k;
+      word <<= 4 * bg;
+      word |= __shfl_xor_sync(0xFFFFFFFFu, word, 1);
+      word |= __shfl_xor_sync(0xFFFFFFFFu, word, 2);
+      word |= __shfl_xor_sync(0xFFFFFFFFu, word, 4);
+      if (bg == 0 && row < nrows) job.out[out_base + (row0 + row) * out_stride + w] = word & word_mask(b, w);
+    }
   }
 }
 

@@ -334,7 +334,7 @@ int launch_hash(const HashJob& job, long long max_rows_per_segment, int segments
     if (Wd == 1) return tma ? go(hash_rows_tc_kernel<1, true>) : go(hash_rows_tc_kernel<1, false>);
     return tma ? go(hash_rows_tc_kernel<2, true>) : go(hash_rows_tc_kernel<2, false>);
   }
-  const size_t smem = ((size_t)job.d * 32 * Wd + (size_t)kHashRows * job.d) * sizeof(float);
+  const size_t smem = ((size_t)job.d * 32 * Wd + (size_t)kHashRows * (job.d + kHashPad)) * sizeof(float);
   const int segs = segments + (job2 != nullptr ? segments2 : 0);
   if (tiles > 0x7FFFFFFFLL || segs > 65535) return fail(HE_ERR_UNSUPPORTED, "hash grid too large (%lld x %d)", tiles, segs);
   dim3 grid((unsigned)tiles, (unsigned)segs);
