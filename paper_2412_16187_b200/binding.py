@@ -126,8 +126,10 @@ def _check(rc: int):
 def _stream(stream=None) -> int:
     if stream is not None:
         return stream.cuda_stream
-    # the handle alone: building torch.cuda.current_stream()'s Python object costs 3 us per call
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    try:  # the handle alone: building torch.cuda.current_stream()'s Python object costs 3 us per call
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:  # neither function is part of torch's public interface
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t):
