@@ -9,7 +9,8 @@ _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 LIB_PATH = os.path.join(_PKG, "libhashevict.so")
 _SOURCES = sorted(glob.glob(os.path.join(_PKG, "csrc", "*.cu")))
-_HEADERS = sorted(glob.glob(os.path.join(_ROOT, "include", "*.h")) + glob.glob(os.path.join(_PKG, "csrc", "*.cuh")))
+_HEADERS = sorted(glob.glob(os.path.join(_ROOT, "include", "*.h")) + glob.glob(os.path.join(_PKG, "csrc", "*.cuh")) +
+                  glob.glob(os.path.join(_PKG, "csrc", "*.h")))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

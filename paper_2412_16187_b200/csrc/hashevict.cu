@@ -28,6 +28,7 @@
 #include "common.cuh"
 #include "decode_kernels.cuh"
 #include "decode_sm_kernels.cuh"
+#include "device_table.h"
 #include "hash_kernels.cuh"
 #include "hash_tc_kernels.cuh"
 #include "hashevict.h"
@@ -188,13 +189,14 @@ int launch_pdl(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, b
 }
 
 int sm_count(int* out) {
-  static int cached[64] = {};
+  static DeviceTable<1> table;
   int dev = 0;
   HE_CUDA_CHECK(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) return fail(HE_ERR_UNSUPPORTED, "device index %d", dev);
-  if (cached[dev] == 0) HE_CUDA_CHECK(cudaDeviceGetAttribute(&cached[dev], cudaDevAttrMultiProcessorCount, dev));
-  *out = cached[dev];
-  return HE_OK;
+  if (dev < 0 || dev >= kMaxDevices) return fail(HE_ERR_UNSUPPORTED, "device index %d", dev);
+  return table.get(dev, 0, out, [dev](int* n) -> int {
+    HE_CUDA_CHECK(cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev));
+    return HE_OK;
+  });
 }
 
 // The driver's tensor-map encoder, or null.
@@ -464,18 +466,19 @@ template <int WORDS, int GT, int SPT, int NT>
 int launch_replay_reg_one(const ReplayArgs& a, long long units, cudaStream_t stream) {
   const size_t smem = (size_t)a.cfg.max_budget * 4;
   if (int rc = set_smem(prefill_replay_reg_kernel<WORDS, GT, SPT, NT>, smem)) return rc;
-  static int per_sm[64] = {};
-  int dev = 0, sms = 0;
+  static DeviceTable<1> table;
+  int dev = 0, sms = 0, per_sm = 0;
   HE_CUDA_CHECK(cudaGetDevice(&dev));
   if (int rc = sm_count(&sms)) return rc;
-  if (per_sm[dev] == 0) {
-    int n = 0;
-    HE_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, prefill_replay_reg_kernel<WORDS, GT, SPT, NT>, NT, smem));
-    per_sm[dev] = n > 0 ? n : 1;
-  }
+  auto resident = [smem](int* n) -> int {
+    HE_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, prefill_replay_reg_kernel<WORDS, GT, SPT, NT>, NT, smem));
+    if (*n < 1) *n = 1;
+    return HE_OK;
+  };
+  if (int rc = table.get(dev, 0, &per_sm, resident)) return rc;
   const int nbins = sms < kMaxBins ? sms : kMaxBins;
   if (int rc = launch_pdl(prefill_schedule_kernel, dim3(1), kSchedThreads, 0, a.Nmax > 0, stream, a.cfg, a.ca.budget, a.prompt_len, nbins, a.sched, 0)) return rc;
-  long long grid = (long long)sms * per_sm[dev];
+  long long grid = (long long)sms * per_sm;
   if (grid > units) grid = units;
   return launch_pdl(prefill_replay_reg_kernel<WORDS, GT, SPT, NT>, dim3((unsigned)grid), NT, smem, true, stream, a);
 }
@@ -522,17 +525,16 @@ int launch_replay_block_half(const ReplayArgs& a, long long units, cudaStream_t 
   HE_CUDA_CHECK(cudaGetDevice(&dev));
   // Cluster size: a block costs a CTA about 8000 cycles of settling, 380 per tile of its own and 3000 for the exchange with
   // its peers; the number of rounds is what the clusters that fit the GPU need for the units.
-  static int max_clusters[64][4] = {};
+  static DeviceTable<4> table;  // clusters of 2^lg CTAs that the device holds at once (-1: none)
   const int tiles = ra.r.smem_slots / kRbTile;
   double best = 0.;
-  int best_lg = -1;
+  int best_lg = -1, best_fit = 0;
   for (int lg = 0; (1 << lg) <= kRbMaxCluster && (lg == 0 || (1 << lg) <= tiles); ++lg) {
     const int n = 1 << lg;
     if (rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, HALF ? kRbRows / 2 : kRbRows, &ra) == 0) continue;
     int fit = sms;
     if (n > 1) {
-      int& cached = max_clusters[dev][lg];
-      if (cached == 0) {
+      auto clusters_of = [&](int* got) -> int {
         if (int rc = set_smem(kernel, kMaxDynSmem)) return rc;
         cudaLaunchConfig_t lc{};
         lc.gridDim = dim3((unsigned)(sms / n * n));
@@ -544,26 +546,24 @@ int launch_replay_block_half(const ReplayArgs& a, long long units, cudaStream_t 
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
         lc.attrs = attr;
         lc.numAttrs = 1;
-        int got = 0;
-        if (cudaOccupancyMaxActiveClusters(&got, kernel, &lc) != cudaSuccess || got < 1) {
+        if (cudaOccupancyMaxActiveClusters(got, kernel, &lc) != cudaSuccess || *got < 1) {
           (void)cudaGetLastError();
-          got = -1;
+          *got = -1;
         }
-        cached = got;
-      }
-      if (cached < 1) continue;
-      fit = cached;
+        return HE_OK;
+      };
+      if (int rc = table.get(dev, lg, &fit, clusters_of)) return rc;
+      if (fit < 1) continue;
     }
     const double rounds = (double)((units + fit - 1) / fit);
     const double cost = rounds * (8000. + (n > 1 ? 3000. : 0.) + 380. * ((tiles + n - 1) / n));
-    if (best_lg < 0 || cost < best) best = cost, best_lg = lg;
+    if (best_lg < 0 || cost < best) best = cost, best_lg = lg, best_fit = fit;
   }
   if (best_lg < 0) return fail(HE_ERR_UNSUPPORTED, "max_budget %d does not fit the block replay's shared memory", a.cfg.max_budget);
   const int n = 1 << best_lg;
   const size_t smem = rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, HALF ? kRbRows / 2 : kRbRows, &ra);
   if (int rc = set_smem(kernel, smem)) return rc;
-  const long long fit = n > 1 ? max_clusters[dev][best_lg] : sms;
-  const long long clusters = units < fit ? units : fit;
+  const long long clusters = units < best_fit ? units : best_fit;
   ra.ncta = n;
   ra.scheduled = units > clusters ? 1 : 0;
   if (ra.scheduled) {  // one queue, largest unit first
@@ -689,12 +689,9 @@ int launch_attend(const AttendArgs& a, cudaStream_t st) {
   int S = (int)(sms / units < 16 ? sms / units : 16);
   if (S > a.cfg.max_budget / 256) S = a.cfg.max_budget / 256;
   if (S > 8) {
-    static int fit[64][17] = {};  // clusters of S that the device holds at once (-1: none)
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lock(mu);
+    static DeviceTable<17> table;  // clusters of S that the device holds at once (-1: none)
     for (S &= ~1; S > 8; S -= 2) {
-      if (fit[dev][S] == 0) {
-        int got = 0;
+      auto clusters_of = [S](int* got) -> int {
         cudaLaunchConfig_t oc{};
         oc.gridDim = dim3(S * 16);
         oc.blockDim = dim3(256);
@@ -707,13 +704,15 @@ int launch_attend(const AttendArgs& a, cudaStream_t st) {
         oc.numAttrs = 1;
         if (int rc = set_smem(attend_bf16_kernel<D, 8>, kMaxDynSmem)) return rc;
         if (cudaFuncSetAttribute(attend_bf16_kernel<D, 8>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&got, attend_bf16_kernel<D, 8>, &oc) != cudaSuccess || got < 1) {
+            cudaOccupancyMaxActiveClusters(got, attend_bf16_kernel<D, 8>, &oc) != cudaSuccess || *got < 1) {
           (void)cudaGetLastError();
-          got = -1;
+          *got = -1;
         }
-        fit[dev][S] = got;
-      }
-      if (fit[dev][S] >= units && smem_of(S) <= kMaxDynSmem) break;
+        return HE_OK;
+      };
+      int fit = 0;
+      if (int rc = table.get(dev, S, &fit, clusters_of)) return rc;
+      if (fit >= units && smem_of(S) <= kMaxDynSmem) break;
     }
   }
   if (S < 1) S = 1;
@@ -1024,10 +1023,10 @@ int he_prefill_compress_noalloc(const he_config* cfg, const he_cache* cache, con
                 need, (unsigned)HE_NOALLOC_SCRATCH_BYTES);
   // device address of the built-in array, looked up once per device with that device current
   static std::mutex mu;
-  static void* scratch_of_device[64] = {};
+  static void* scratch_of_device[kMaxDevices] = {};
   int dev = 0;
   HE_CUDA_CHECK(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) return fail(HE_ERR_UNSUPPORTED, "device index %d", dev);
+  if (dev < 0 || dev >= kMaxDevices) return fail(HE_ERR_UNSUPPORTED, "device index %d", dev);
   void* scratch = nullptr;
   {
     std::lock_guard<std::mutex> lock(mu);
