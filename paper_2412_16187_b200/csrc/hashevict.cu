@@ -672,6 +672,15 @@ int launch_attend_on(const AttendArgs& a, int S, size_t smem, cudaStream_t st) {
   return HE_OK;
 }
 
+// Dynamic shared memory of the attention kernel at most: a CTA's 227 KB less the mbarriers in static memory. One limit for every
+// cluster size.
+constexpr size_t kAttendMaxSmem = 227 * 1024 - 512;
+
+template <int D>
+constexpr size_t attend_smem(int S, int G) {
+  return 1024 + (size_t)AttendRing<D, 8>::kBytes + (S > 1 ? (size_t)S * G * (D + 2) * sizeof(float) : 0);
+}
+
 // Tensor-core attention with S CTAs per unit. A call pays 2.5 us (one CTA) to 4 us (cluster of 8) whatever it reads, an SM pulls
 // 90 GB/s, the GPU 6.3 TB/s, so a unit is spread until the grid has one CTA per SM. Measured (us per call in a graph, caches larger
 // than L2; register-fed kernel with clusters of up to 8 before): 8 units of 9830 slots 16.9 -> 10.6, 32 of 2048 8.7 -> 7.9, 128 of
@@ -683,7 +692,7 @@ int launch_attend(const AttendArgs& a, cudaStream_t st) {
   if (int rc = sm_count(&sms)) return rc;
   HE_CUDA_CHECK(cudaGetDevice(&dev));
   static_assert(8 * kMaxGroup * (D + 2) * sizeof(float) <= AttendRing<D, 8>::kBytes, "the merge reuses the rings");
-  auto smem_of = [&](int S) { return 1024 + (size_t)AttendRing<D, 8>::kBytes + (S > 1 ? (size_t)S * a.cfg.group_size * (D + 2) * sizeof(float) : 0); };
+  static_assert(attend_smem<D>(8, kMaxGroup) <= kAttendMaxSmem, "up to eight CTAs any group's partial results fit");
   // As many CTAs per unit as keep the grid within one (deep) CTA per SM, and no fewer than 256 slots (a group per warp)
   // for each. Clusters above 8 need the driver's consent and as many free SMs in one GPC, so they are asked about.
   int S = (int)(sms / units < 16 ? sms / units : 16);
@@ -695,14 +704,14 @@ int launch_attend(const AttendArgs& a, cudaStream_t st) {
         cudaLaunchConfig_t oc{};
         oc.gridDim = dim3(S * 16);
         oc.blockDim = dim3(256);
-        oc.dynamicSmemBytes = kMaxDynSmem;
+        oc.dynamicSmemBytes = kAttendMaxSmem;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = S;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         oc.attrs = at;
         oc.numAttrs = 1;
-        if (int rc = set_smem(attend_bf16_kernel<D, 8>, kMaxDynSmem)) return rc;
+        if (int rc = set_smem(attend_bf16_kernel<D, 8>, kAttendMaxSmem)) return rc;
         if (cudaFuncSetAttribute(attend_bf16_kernel<D, 8>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
             cudaOccupancyMaxActiveClusters(got, attend_bf16_kernel<D, 8>, &oc) != cudaSuccess || *got < 1) {
           (void)cudaGetLastError();
@@ -712,14 +721,14 @@ int launch_attend(const AttendArgs& a, cudaStream_t st) {
       };
       int fit = 0;
       if (int rc = table.get(dev, S, &fit, clusters_of)) return rc;
-      if (fit >= units && smem_of(S) <= kMaxDynSmem) break;
+      if (fit >= units && attend_smem<D>(S, a.cfg.group_size) <= kAttendMaxSmem) break;
     }
   }
   if (S < 1) S = 1;
   // Two small CTAs per SM once there are more units than SMs, so that one streams while the other starts or merges (512 units
   // of 1000 slots, d = 64: 24.4 against 27.7 us; level at 256 units of 2048 slots).
   if (units > sms) return launch_attend_on<D, 4>(a, 1, 1024 + AttendRing<D, 4>::kBytes, st);
-  return launch_attend_on<D, 8>(a, S, smem_of(S), st);
+  return launch_attend_on<D, 8>(a, S, attend_smem<D>(S, a.cfg.group_size), st);
 }
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
