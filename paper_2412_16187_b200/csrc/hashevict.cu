@@ -228,7 +228,7 @@ bool cache_rows_tmap(const void* base, long long rows, int d, CUtensorMap* out) 
   Entry& e = cache[(reinterpret_cast<uintptr_t>(base) >> 9) * 0x9E3779B97F4A7C15ull >> 57];
   if (e.base != base || e.rows != rows || e.d != d) {
     const EncodeTiledFn encode = tmap_encoder();
-    if (encode == nullptr || rows > 0x7FFFFFFF) return false;
+    if (encode == nullptr || rows > 0x7FFFFFFF || env_flag_set<3>("HE_DISABLE_TMA")) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)d * 2};
     const cuuint32_t box[2] = {64, (cuuint32_t)kAttendGroup}, estr[2] = {1, 1};
     if (encode(&e.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -648,8 +648,12 @@ int launch_replay(const ReplayArgs& a, long long units, cudaStream_t stream) {
   }
 }
 
+struct AttendMaps {
+  alignas(64) CUtensorMap k, v;
+};
+
 template <int D, int NW>
-int launch_attend_on(const AttendArgs& a, int S, size_t smem, cudaStream_t st) {
+int launch_attend_on(const AttendArgs& a, const AttendMaps& maps, int S, size_t smem, cudaStream_t st) {
   if (int rc = set_smem(attend_bf16_kernel<D, NW>, smem)) return rc;
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3((unsigned)(a.cfg.n_kv_heads * S), (unsigned)a.cfg.batch);
@@ -664,11 +668,7 @@ int launch_attend_on(const AttendArgs& a, int S, size_t smem, cudaStream_t st) {
   at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   lc.attrs = at;
   lc.numAttrs = S > 1 ? 2 : 1;
-  const long long rows = (long long)a.cfg.batch * a.cfg.n_kv_heads * a.cfg.max_budget;
-  alignas(64) CUtensorMap kmap, vmap;
-  if (!cache_rows_tmap(a.ca.k_cache, rows, D, &kmap) || !cache_rows_tmap(a.ca.v_cache, rows, D, &vmap))
-    return fail(HE_ERR_CUDA, "no tensor map for a cache of %lld rows x %d", rows, D);
-  HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, attend_bf16_kernel<D, NW>, a, S, kmap, vmap));
+  HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, attend_bf16_kernel<D, NW>, a, S, maps.k, maps.v));
   return HE_OK;
 }
 
@@ -686,7 +686,7 @@ constexpr size_t attend_smem(int S, int G) {
 // than L2; register-fed kernel with clusters of up to 8 before): 8 units of 9830 slots 16.9 -> 10.6, 32 of 2048 8.7 -> 7.9, 128 of
 // 1024 14.6 -> 12.9.
 template <int D>
-int launch_attend(const AttendArgs& a, cudaStream_t st) {
+int launch_attend(const AttendArgs& a, const AttendMaps& maps, cudaStream_t st) {
   const long long units = (long long)a.cfg.batch * a.cfg.n_kv_heads;
   int sms = 0, dev = 0;
   if (int rc = sm_count(&sms)) return rc;
@@ -727,8 +727,8 @@ int launch_attend(const AttendArgs& a, cudaStream_t st) {
   if (S < 1) S = 1;
   // Two small CTAs per SM once there are more units than SMs, so that one streams while the other starts or merges (512 units
   // of 1000 slots, d = 64: 24.4 against 27.7 us; level at 256 units of 2048 slots).
-  if (units > sms) return launch_attend_on<D, 4>(a, 1, 1024 + AttendRing<D, 4>::kBytes, st);
-  return launch_attend_on<D, 8>(a, S, attend_smem<D>(S, a.cfg.group_size), st);
+  if (units > sms) return launch_attend_on<D, 4>(a, maps, 1, 1024 + AttendRing<D, 4>::kBytes, st);
+  return launch_attend_on<D, 8>(a, maps, S, attend_smem<D>(S, a.cfg.group_size), st);
 }
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -1059,8 +1059,13 @@ int he_attend(const he_config* cfg, const he_cache* cache, const void* q, float*
   const dim3 grid((unsigned)cfg->n_kv_heads, (unsigned)cfg->batch);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int G = cfg->group_size, d = cfg->head_dim;
-  if (cfg->dtype == HE_DTYPE_BF16 && (d == 64 || d == 128) && getenv("HE_DISABLE_ATTEND_MMA") == nullptr)
-    return d == 64 ? launch_attend<64>(a, st) : launch_attend<128>(a, st);
+  if (cfg->dtype == HE_DTYPE_BF16 && (d == 64 || d == 128) && getenv("HE_DISABLE_ATTEND_MMA") == nullptr) {
+    // without tensor maps (a driver that lacks the encoder, more than 2^31 rows) the generic kernel serves, which needs none
+    const long long rows = (long long)cfg->batch * cfg->n_kv_heads * cfg->max_budget;
+    AttendMaps maps;
+    if (cache_rows_tmap(cache->k_cache, rows, d, &maps.k) && cache_rows_tmap(cache->v_cache, rows, d, &maps.v))
+      return d == 64 ? launch_attend<64>(a, maps, st) : launch_attend<128>(a, maps, st);
+  }
   const size_t smem = ((size_t)G * d + (size_t)kAttendWarps * G * (d + 2)) * sizeof(float);
   if (int rc = set_smem(attend_generic_kernel, smem)) return rc;
   attend_generic_kernel<<<grid, kAttendThreads, smem, st>>>(a);
