@@ -86,9 +86,10 @@ typedef struct he_cache {
   int32_t* fill;
   int32_t* next_pos;
   const float* W;
-  const int32_t* budget_host; /* optional HOST copy of budget ([B]), or NULL. When given (and B <= 256)
+  const int32_t* budget_host; /* optional HOST copy of budget ([B]), or NULL. When given (and B <= 1024)
                                  he_decode_step passes the budgets in the kernel parameters, which saves the
-                                 kernel one dependent device read before it can start streaming the code table.
+                                 kernel one dependent device read before it can start streaming the code table,
+                                 and with HE_FLAG_EARLY_INPUTS deals the units by budget.
                                  With protected windows (n_sink or n_recent > 0) he_prefill_compress also needs it to
                                  check that every budget exceeds n_sink + n_recent before it picks its faster replay
                                  kernel; without it the call is correct but slower. Must hold the same values as `budget`. */

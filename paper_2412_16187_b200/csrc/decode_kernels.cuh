@@ -15,7 +15,14 @@
 
 namespace he {
 
-constexpr int kMaxBudgetVals = 256;  // budgets carried in the kernel parameters (1 KB: every launch pays for its parameters' size)
+// Sequences whose budgets (16 bits, or 32 where a cache has more than 65 535 slots) travel in the kernel parameters. Every launch
+// pays for its parameters' size (a launch waited for 9.16 us with 1.2 KB of them, 9.23 with 2.2, 9.88 with 8.4), and a call of
+// more sequences reads its budgets on the device, a dependent read ahead of the code tables, and deals its units unsorted with
+// HE_FLAG_EARLY_INPUTS. With room for 256, us per call in a graph: 600 / 1024 sequences of one unit (b = 64) 9.5 / 14.7 against 9.1
+// / 14.1 now, 1024 of eight (b = 32) 41.9 against 40.4, early 400 of one (b = 64) 5.76 against 5.45. An 8-bit bound of the
+// budget beside the copy, with the budget itself read meanwhile, did not do: 14.8 at 1024.
+constexpr int kBudgetVals = 1024;
+constexpr int kBudgetWords = kBudgetVals / 2;
 
 struct DecodeArgs {
   he_config cfg;
@@ -27,11 +34,15 @@ struct DecodeArgs {
   int32_t* evicted_pos_out;
   uint32_t* qcodes_out;
   const uint32_t* new_codes;               // PRE kernels: [B*Hkv*G + B*Hkv, Wd] codes of this step's q rows, then k rows
-  int n_budget_vals;                       // > 0: budgets are in budget_vals (copied from he_cache.budget_host)
-  int n_sched;                             // > 0: sched lists the sequences by budget, largest first (sequence << 21 | budget)
+  // What is in the union, copied from he_cache.budget_host (one of them > 0, or none):
+  int n_budget16, n_budget32;  // the sequences' budgets
+  int n_sched;                 // the sequences by budget, largest first (sequence << 21 | budget)
+  int n_order;                 // ... the sequences alone
   union {
-    int32_t budget_vals[kMaxBudgetVals];
-    uint32_t sched[kMaxBudgetVals];
+    uint16_t budget16[kBudgetVals];
+    int32_t budget32[kBudgetWords];
+    uint32_t sched[kBudgetWords];
+    uint16_t order[kBudgetVals];
   };
 };
 
@@ -112,7 +123,8 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
     const char* src = static_cast<const char*>(is_k ? a.k : a.v) + (size_t)unit * d * es;
     rowreg = __ldg(reinterpret_cast<const uint4*>(src) + (is_k ? tid : tid - cpr));
   }
-  const int C = clamp_budget(a.n_budget_vals > 0 ? a.budget_vals[s] : a.ca.budget[s], Cmax);
+  // (the bulk-hashed kernels have no register left for a third source: 59.5 us with it where 56.6)
+  const int C = clamp_budget(a.n_budget16 > 0 ? (int)a.budget16[s] : (!PRE && a.n_budget32 > 0 ? a.budget32[s] : a.ca.budget[s]), Cmax);
   const int fill = a.ca.fill[unit];
   const int t = a.ca.next_pos[unit];
 

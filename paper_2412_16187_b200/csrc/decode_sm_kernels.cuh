@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(kSmThreads, 2) decode_step_sm_kernel(const Dec
           s = (int)(sw >> kSmSchedShift);
           C = (int)(sw & ((1u << kSmSchedShift) - 1u));
         } else {
+          if (a.n_order > 0) s = a.order[so];
           C = __ldg(a.ca.budget + s);  // read-only while the cache is in use, so it may be read before the wait
         }
         u.unit = s * H + h;

@@ -422,32 +422,32 @@ int launch_decode_sm(const DecodeArgs& a, bool mma, unsigned grid, cudaStream_t 
   }
 }
 
-// Sequences ordered by budget, largest first (ties by index), each with its budget, for the unit schedule of the
-// one-CTA-per-SM decode kernel: word = sequence << 21 | budget. The caller's budget mirror is hashed on every call
-// and sorted again only when its contents changed.
+// Sequences ordered by budget, largest first (ties by index), for the unit schedule of the one-CTA-per-SM decode kernel: up
+// to kBudgetWords of them each with its budget (word = sequence << 21 | budget), more as indices alone. The caller's budget mirror
+// is hashed on every call and sorted again only when its contents changed.
 struct SchedCache {
   uint64_t hash = 0;
   int n = -1;
   int cmax = 0;
-  uint32_t sched[kMaxBudgetVals];
+  uint32_t sched[kBudgetWords];
+  uint16_t order[kBudgetVals];
 };
-const uint32_t* sched_of(const int32_t* budget_host, int n, int cmax) {
+const SchedCache& sched_of(const int32_t* budget_host, int n, int cmax) {
   thread_local SchedCache c;
   uint64_t h = 1469598103934665603ull;
   for (int i = 0; i < n; ++i) h = (h ^ (uint32_t)budget_host[i]) * 1099511628211ull;
   if (c.n != n || c.hash != h || c.cmax != cmax) {
-    uint16_t order[kMaxBudgetVals];
-    for (int i = 0; i < n; ++i) order[i] = (uint16_t)i;
-    std::stable_sort(order, order + n, [&](uint16_t x, uint16_t y) { return budget_host[x] > budget_host[y]; });
-    for (int i = 0; i < n; ++i) {
-      const int cb = budget_host[order[i]];
-      c.sched[i] = ((uint32_t)order[i] << kSmSchedShift) | (uint32_t)(cb < 0 ? 0 : (cb > cmax ? cmax : cb));
+    for (int i = 0; i < n; ++i) c.order[i] = (uint16_t)i;
+    std::stable_sort(c.order, c.order + n, [&](uint16_t x, uint16_t y) { return budget_host[x] > budget_host[y]; });
+    for (int i = 0; i < n && n <= kBudgetWords; ++i) {
+      const int cb = budget_host[c.order[i]];
+      c.sched[i] = ((uint32_t)c.order[i] << kSmSchedShift) | (uint32_t)(cb < 0 ? 0 : (cb > cmax ? cmax : cb));
     }
     c.n = n;
     c.hash = h;
     c.cmax = cmax;
   }
-  return c.sched;
+  return c;
 }
 
 template <int WORDS, int GT>
@@ -808,8 +808,8 @@ int he_decode_step(const he_config* cfg, const he_cache* cache, const void* q, c
   a.victim_out = victim_out;
   a.evicted_pos_out = evicted_pos_out;
   a.qcodes_out = qcodes_out;
-  a.n_budget_vals = 0;
-  a.n_sched = 0;
+  a.n_budget16 = a.n_budget32 = a.n_sched = a.n_order = 0;
+  const bool mirror = cache->budget_host != nullptr && cfg->batch <= kBudgetVals;
   a.new_codes = nullptr;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // Large batches: hash the step's new rows with the bulk projection kernels (tensor cores for bf16) into the
@@ -823,9 +823,15 @@ int he_decode_step(const he_config* cfg, const he_cache* cache, const void* q, c
   const bool early = cb == 0 && cfg->head_dim % kChunk == 0 && (cfg->flags & HE_FLAG_EARLY_INPUTS) != 0 &&
                      units_ll <= (long long)kSmUnits * sms && !env_flag_set<0>("HE_DISABLE_EARLY_DECODE");
   if (early) {
-    if (cache->budget_host != nullptr && cfg->batch <= kMaxBudgetVals) {
-      a.n_sched = cfg->batch;
-      memcpy(a.sched, sched_of(cache->budget_host, cfg->batch, cfg->max_budget), sizeof(uint32_t) * (size_t)cfg->batch);
+    if (mirror) {
+      const SchedCache& sc = sched_of(cache->budget_host, cfg->batch, cfg->max_budget);
+      if (cfg->batch <= kBudgetWords) {
+        a.n_sched = cfg->batch;
+        memcpy(a.sched, sc.sched, sizeof(uint32_t) * (size_t)cfg->batch);
+      } else {
+        a.n_order = cfg->batch;
+        memcpy(a.order, sc.order, sizeof(uint16_t) * (size_t)cfg->batch);
+      }
     }
     const unsigned g = (unsigned)(units_ll < sms ? units_ll : sms);
     const bool mma = tc_enabled() && cfg->dtype == HE_DTYPE_BF16 && cfg->head_dim <= 128;
@@ -851,10 +857,13 @@ int he_decode_step(const he_config* cfg, const he_cache* cache, const void* q, c
     if (int rc = launch_hash(job, job.rows, 1, st)) return rc;
     a.new_codes = cache->step_scratch;
   }
-  if (cache->budget_host != nullptr && cfg->batch <= kMaxBudgetVals) {
-    // budgets travel in the kernel parameters, so the code-table copy can start without a dependent device read
-    a.n_budget_vals = cfg->batch;
-    memcpy(a.budget_vals, cache->budget_host, sizeof(int32_t) * (size_t)cfg->batch);
+  // budgets travel in the kernel parameters, so the code-table copy can start without a dependent device read
+  if (mirror && cfg->max_budget <= 0xFFFF) {
+    a.n_budget16 = cfg->batch;
+    for (int i = 0; i < cfg->batch; ++i) a.budget16[i] = (uint16_t)cache->budget_host[i];
+  } else if (mirror && cfg->batch <= kBudgetWords) {
+    a.n_budget32 = cfg->batch;
+    memcpy(a.budget32, cache->budget_host, sizeof(int32_t) * (size_t)cfg->batch);
   }
   const dim3 grid((unsigned)cfg->n_kv_heads, (unsigned)cfg->batch);
   if (cb) return launch_decode_g<1, true>(a, nt, smem, grid, st);
