@@ -19,9 +19,16 @@
 // at least the first k entries are final; on the workloads' keys 2 to 4 passes settle a block, because few steps
 // depend on one another. A step is EASY when its best base slot is not taken by an earlier step and no earlier key can
 // reach its rank; easy steps cost nothing. The others ("hard", 5-40 %) are evaluated by a warp each: best new
-// entry still resident, best base slot (a taken one makes its tile be scanned again with popcounts). If passes
-// do not converge quickly (queries that keep preferring the same slots) the window that is evaluated at a
-// time shrinks to a dozen steps, so that no more than that is evaluated in vain.
+// entry still resident, best base slot (a taken one makes its tile be scanned again with popcounts).
+//
+// Where passes do not converge quickly, the window that is evaluated at a time shrinks to a dozen steps. Where they do not converge
+// at all (queries that keep preferring the same slots, near-constant ones, say, let a pass settle one step and make every evaluation
+// scan tile after tile), the block is finished by a walk: one step after the other, all settling warps scanning the table for each
+// (rb_walk). us per call with passes alone / with the walk, and what one warp resolving step by step took before the passes: constant
+// queries, 32 units of 2048 slots, 2048 steps, 8110 / 890 (1980); 512 units of 2304, two words, 43 700 / 6830 (13 600); 8 of 9830,
+// 4070 steps, 20 000 / 4330 (10 500); 128 of 192, 960 steps, 1860 / 460 (380 on CUDA cores); queries with a tenth of their
+// variation, the first two 7310 / 1150 (1920) and 11 900 / 7250 (6780). Independent queries, where the test for it costs 0 to 1.4 %,
+// take 150 (420), 1210 (2310), 260 (1320) and 214 (380).
 //
 // Few units: a cluster of up to 8 CTAs shares one unit. Tiles are dealt round-robin over its CTAs; each CTA keeps the
 // whole packed code table (at most 48 KB at 32 bits), copies its tiles' maxima to the others through distributed shared
@@ -62,6 +69,17 @@ constexpr int kRbIdxMask = (1 << kRbKeyShift) - 1;
 constexpr int kRbMaxSlots = 12288;
 constexpr int kRbMaxCluster = 8;
 constexpr int kRbWidePasses = 6;         // passes over the whole block before the window shrinks
+// The walk through a block takes over from the passes where hardly a step of the window is easy and as many passes at this one's cost
+// would have cost twice the walk through the steps that are final: at the second pass where more than half of the block is left,
+// later where less is (a few steps are soon settled by passes, and one slow pass is often chance). On independent queries 5 to 90 %
+// of the steps are hard, most with few distinct distances, and passes win: with three quarters as the line, 4792 slots at b = 8 took
+// 6190 us for 4960. On repeating queries 97 % are. Cycles, fitted to 8 units of 192 to 6144 slots: a pass (an evaluation scans a tile
+// or two), and a step of the walk with `slots` slots for each thread (group sizes without a form of their own scan all eight places
+// of a group).
+__device__ __forceinline__ int rb_pass_cost(int hard) { return 1000 + (hard + kRbResWarps - 1) / kRbResWarps * 1400; }
+__host__ __device__ constexpr int rb_walk_cost(int words, int gt, bool prot, int slots) {
+  return (prot ? 550 : 400) + slots * ((gt == 4 ? 55 : (gt == 1 ? 35 : 215)) * words + (prot ? 20 : 0));
+}
 constexpr int kRbAtom = 128 * 128;       // 128 operand rows x one 128-byte swizzle atom
 constexpr int kRbDnPitch = 136;          // 16-bit entries between rows of the new-entry table
 constexpr int kRbDnPitchHalf = 68;       // ... when blocks have at most 64 steps
@@ -231,7 +249,7 @@ struct RbRank {
   uint32_t q[kQ];
   Planes4 p[WORDS];
   int add, G;
-  __device__ __forceinline__ void load(const uint32_t* src, int G_, int parity_bits) {
+  __device__ __forceinline__ void fetch(const uint32_t* src, int G_, int parity_bits) {
     G = G_;
     add = parity_bits;
     if (GT * WORDS % 4 == 0 && GT > 0) {
@@ -241,6 +259,8 @@ struct RbRank {
 #pragma unroll
       for (int i = 0; i < kQ; ++i) q[i] = (GT > 0 || i < G * WORDS) ? src[i] : 0u;
     }
+  }
+  __device__ __forceinline__ void prepare() {
     if (GT == 4) {
 #pragma unroll
       for (int w = 0; w < WORDS; ++w) {
@@ -248,6 +268,10 @@ struct RbRank {
         p[w] = make_planes4(q[w], q[WORDS + w], q[(2 * WORDS + w) % kQ], q[(3 * WORDS + w) % kQ], &parity);
       }
     }
+  }
+  __device__ __forceinline__ void load(const uint32_t* src, int G_, int parity_bits) {
+    fetch(src, G_, parity_bits);
+    prepare();
   }
   __device__ __forceinline__ int dist(const uint32_t (&h)[WORDS]) const {
     if (GT == 4) return 2 * half_distance4<WORDS>(h, p) + add;
@@ -267,6 +291,88 @@ struct RbRank {
   }
 };
 
+// The walk through the steps fin .. rows - 1 of a block by the settling warps (file comment), every step on the table that the one
+// before it left. Every thread scans its slots (tid, tid + 384, ...), and a slot is rewritten by the thread that scans it, so that a
+// step needs one barrier: 400 cycles, and 35 (G = 1) or 55 (G = 4) more for each slot of a thread and word. `own` (all 0xFF before
+// and after) marks the slots of recent tokens meanwhile. Steps from writes_end on leave the table as it is; pos is null where
+// another CTA of the cluster writes the positions. Not inlined: inside the block loop it cost independent queries 2 % (64 ragged
+// prompts), and itself gains 6 %.
+extern __shared__ unsigned char rb_smem_raw[];
+template <int WORDS, int GT, bool PROT>
+__device__ __noinline__ void rb_walk(const RbLayout& L, int base, int cur, int32_t* pos, int t0, int fin, int rows, int writes_end, int C, int G,
+                                     int S, int Rn) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, GW = G * WORDS;
+  unsigned char* smem = rb_smem_raw + base;  // (not passed as pointers, so that the accesses stay shared-memory accesses)
+  uint32_t* codes = reinterpret_cast<uint32_t*>(smem + L.codes);
+  uint8_t* own = smem + L.own;
+  uint16_t* SV = reinterpret_cast<uint16_t*>(smem + L.sv);
+  int32_t* SN = reinterpret_cast<int32_t*>(smem + L.sn);
+  const int32_t* REC = reinterpret_cast<const int32_t*>(smem + L.rec);
+  const int32_t* par = reinterpret_cast<const int32_t*>(smem + L.par) + cur * kRbRows;
+  const uint32_t* qb = reinterpret_cast<const uint32_t*>(smem + L.qraw) + cur * kRbRows * GW;
+  const uint32_t* kb = reinterpret_cast<const uint32_t*>(smem + L.kraw) + cur * kRbRows * WORDS;
+  auto newest = [&](int r, int m) { return r >= m ? (int)SV[r - m] : REC[m - r - 1]; };  // slot of the m-th newest token at step r
+  rb_bar<2, kRbResThreads>();
+  if (PROT && Rn > 0) {
+    if (tid < Rn) own[newest(fin, tid + 1)] = 0;
+    rb_bar<2, kRbResThreads>();
+  }
+  const int mine = tid < C ? (C - tid + kRbResThreads - 1) / kRbResThreads : 0;  // slots of this thread
+  RbRank<WORDS, GT> rk;
+  rk.load(qb + fin * GW, G, par[fin]);
+  int last = PROT && Rn == 1 ? newest(fin, 1) : 0;  // slot of the step before
+  for (int r = fin; r < rows; ++r) {
+    // what the rewrite and the next step want and this step's outcome does not decide
+    RbRank<WORDS, GT> next;
+    const int rn = min(r + 1, rows - 1);
+    next.fetch(qb + rn * GW, G, par[rn]);
+    uint32_t kc[WORDS];
+#pragma unroll
+    for (int w = 0; w < WORDS; ++w) kc[w] = kb[r * WORDS + w];
+    const int out = PROT && Rn > 1 ? newest(r, Rn) : last;  // its token is recent no longer
+    int best = -1, kx = kRbIdxMask - tid;
+    const uint32_t* cp = codes + tid * WORDS;
+    const uint8_t* op = own + tid;
+#pragma unroll 4
+    for (int i = 0; i < mine; ++i) {
+      uint32_t h[WORDS];
+      if (WORDS == 2) {
+        const uint2 h2 = *reinterpret_cast<const uint2*>(cp);
+        h[0] = h2.x, h[WORDS - 1] = h2.y;
+      } else {
+        h[0] = *cp;
+      }
+      int key = (rk.rank(h) << kRbKeyShift) + kx;
+      if (PROT) key = kx <= kRbIdxMask - S && *op != 0 ? key : -1;
+      best = max(best, key);
+      cp += kRbResThreads * WORDS;
+      op += kRbResThreads;
+      kx -= kRbResThreads;
+    }
+    int32_t* wbest = SN + (r & 1) * 16;
+    const int wb = __reduce_max_sync(0xFFFFFFFFu, best);
+    if (lane == 0) wbest[warp] = wb;
+    rb_bar<2, kRbResThreads>();
+    const int wtop = lane < kRbResWarps ? wbest[lane] : -1;
+    rk = next;
+    rk.prepare();
+    const int top = __reduce_max_sync(0xFFFFFFFFu, wtop);
+    last = min(kRbIdxMask - (top & kRbIdxMask), C - 1);
+    if (tid == 0) SV[r] = (uint16_t)last;
+    if (best == top && HE_IN_RANGE(last, C)) {  // (keys differ between slots)
+      if (r < writes_end) {
+#pragma unroll
+        for (int w = 0; w < WORDS; ++w) codes[last * WORDS + w] = kc[w];
+        if (pos != nullptr) pos[last] = t0 + r;
+      }
+      if (PROT && Rn > 0) own[last] = 0;
+    }
+    if (PROT && Rn > 0 && out % kRbResThreads == tid) own[out] = 0xFFu;
+  }
+  rb_bar<2, kRbResThreads>();
+  if (PROT && tid < Rn) own[newest(rows, tid + 1)] = 0xFFu;
+}
+
 // PROT: protected windows (Section 4 setup). The first n_sink tokens never leave slots 0 .. n_sink-1, so those slots are
 // masked like slots past the budget. A recent token that is already in the table is recognised by the list of the newest
 // slots, one of this block's own keys by its step. Needs every budget > n_sink + n_recent (so that some slot is always
@@ -277,7 +383,6 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   constexpr int NT = kRbThreads;
   constexpr int MS = kRbMaxStages;
   constexpr int RM = HALF ? kRbRows / 2 : kRbRows;
-  extern __shared__ unsigned char rb_smem_raw[];
   __shared__ __align__(8) unsigned long long bars[2 * MS + 4 + 5];
   __shared__ uint32_t tmem_base_s;
   __shared__ volatile int abort_flag;
@@ -770,6 +875,10 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           // of the four lists one after another.
           const uint32_t nhard = *reinterpret_cast<const uint32_t*>(s_hard[par]);
           const int n0 = nhard & 0xFFu, n1 = n0 + ((nhard >> 8) & 0xFFu), n2 = n1 + ((nhard >> 16) & 0xFFu), n3 = n2 + (nhard >> 24);
+          if (__builtin_expect(32 * n3 > 31 * (wend - fb), 0)) {
+            const int walk = rb_walk_cost(WORDS, GT, PROT, (C + kRbResThreads - 1) / kRbResThreads);
+            if (pass * rb_pass_cost(n3) > 2 * fb * walk && 2 * pass * (rows - fb) > rows) break;  // the rest is walked
+          }
           for (int e0 = warp; e0 < n3; e0 += kRbResWarps) {
             const int entry = LIST[e0 < n1 ? (e0 < n0 ? e0 : 32 + e0 - n0) : (e0 < n2 ? 64 + e0 - n1 : 96 + e0 - n2)];
             const int r2 = entry & 127;
@@ -883,6 +992,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             if (fb >= rows) break;
           }
         }
+        const int fin = fb;  // the passes have settled the steps below: as a rule all of the block's
         if (ncta > 1 && warp == 4 && lane < ncta - 1) rb_arrive_remote(rb_mapa(used_bar, (uint32_t)((rank + 1 + lane) & (ncta - 1))));
         // ------------------------------------------------------------ Algorithm 1 lines 2-5 on the table
         const bool scoring = write_scores && tn == N;
@@ -895,7 +1005,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         // last writers: the steps claim again, later ones over earlier ones (the prompt's last step waits until its scores
         // are taken)
         if (warp < 4) {
-          const bool in = mine && !(scoring && r == rows - 1);
+          const bool in = tid < fin && !(scoring && r == rows - 1);
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             if (warp == k && in) own[sv] = (uint8_t)r;
@@ -912,6 +1022,10 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           if (in && own[sv] == (uint8_t)r) apply(sv);
           rb_bar<1, kRbRows>();
           if (mine) own[sv] = 0xFFu;
+        }
+        if (__builtin_expect(fin < rows, 0)) {
+          rb_walk<WORDS, GT, PROT>(L, (int)(smem - rb_smem_raw), cur, rank == 0 ? pos_g : nullptr, t0, fin, rows, scoring ? rows - 1 : rows, C, G, S, Rn);
+          if (mine) sv = SV[r];
         }
         int keep = 0;
         if (PROT && tid < Rn) keep = tid < rows ? 0 : REC[tid - rows];
