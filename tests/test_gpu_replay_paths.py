@@ -1,8 +1,8 @@
-"""The implementations of the prompt replay (tensor-core kernel with 8-bit or bf16 operands, CUDA-core kernels)
+"""The implementations of the prompt replay (the block kernel on tensor cores, the CUDA-core kernels)
 against the oracle, each forced through the environment switches in a fresh process, on shapes that cover one-word and two-word codes, group
 sizes 1, 3 and 4, budgets that are not multiples of the 128-slot tile, ragged budgets, prompts that end inside a
 128-step block, prompts shorter than the budget, protected windows, and keys with little variety (many equal distances, so the
-lowest-slot rule and the repair of stale tile maxima are exercised)."""
+lowest-slot rule and the evaluation of steps whose best slot is taken are exercised)."""
 import os
 import subprocess
 import sys
@@ -35,11 +35,11 @@ shapes = [
     C["llama3_8b_gqa"].scaled(batch=1, prompt_len=900, budget=260, hash_bits=4, decode_steps=2, n_sink=4, n_recent=10),
     C["throughput_batch"].scaled(batch=2, budget_lo=200, budget_hi=400, decode_steps=2, n_sink=2, n_recent=45),
     C["llama2_7b_layer"].scaled(prompt_len=700, budget=300, decode_steps=2, n_sink=7, n_recent=0),
-    # budgets above 4096 slots (tables in global memory), plain and with protected windows up to the 32-token ring
+    # budgets above 4096 slots (a cluster of CTAs per unit), plain and with protected windows
     C["long_prefill"].scaled(layers=1, n_kv_heads=2, prompt_len=7000, budget=4500, decode_steps=2),
     C["long_prefill"].scaled(layers=1, n_kv_heads=2, prompt_len=7000, budget=4500, decode_steps=2, n_sink=4, n_recent=10),
     C["long_prefill"].scaled(layers=1, n_kv_heads=1, prompt_len=6000, budget=4200, hash_bits=8, decode_steps=2, n_sink=3, n_recent=32),
-    # four-bit codes over several tiles: most steps hit a stale tile maximum, so blocks are cut short after 64 repairs
+    # four-bit codes over several tiles: most steps find their best slot taken
     C["llama3_8b_gqa"].scaled(batch=1, prompt_len=1800, budget=700, hash_bits=4, decode_steps=2),
 ]
 for w in shapes:
@@ -60,8 +60,7 @@ print("ok")
 """ % (ROOT, os.path.join(ROOT, "tests"))
 
 
-@pytest.mark.parametrize("env", [{"HE_TC_REPLAY": "1"}, {"HE_TC_REPLAY": "1", "HE_TC_REPLAY_BF16": "1"}, {"HE_TC_REPLAY": "0"}],
-                         ids=["tensor_cores_fp8", "tensor_cores_bf16", "cuda_cores"])
+@pytest.mark.parametrize("env", [{"HE_TC_REPLAY": "1"}, {"HE_TC_REPLAY": "0"}], ids=["tensor_cores", "cuda_cores"])
 def test_replay_path(env):
     e = dict(os.environ, **env)
     r = subprocess.run([sys.executable, "-c", SCRIPT], env=e, capture_output=True, text=True, timeout=600)
