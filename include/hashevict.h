@@ -86,7 +86,7 @@ typedef struct he_cache {
   int32_t* fill;
   int32_t* next_pos;
   const float* W;
-  const int32_t* budget_host; /* optional HOST copy of budget ([B]), or NULL. When given (and B <= 1024)
+  const int32_t* budget_host; /* optional HOST copy of budget ([B]), or NULL. When given (and B <= 792)
                                  he_decode_step passes the budgets in the kernel parameters, which saves the
                                  kernel one dependent device read before it can start streaming the code table,
                                  and with HE_FLAG_EARLY_INPUTS deals the units by budget.
@@ -300,8 +300,8 @@ int he_prefill_compress_noalloc(const he_config* cfg, const he_cache* cache, con
  * wait since the library was loaded (0 in a healthy process; the kernels never wait without a limit, and a
  * block that hits one releases what it holds and returns), plus, in the bounds-checking debug build, how many
  * indices were found out of range. A call during which the counter rose has returned HE_OK all the same (calls
- * only enqueue work), but its outputs are undefined: he_hash_keys, he_prefill_compress and its variants, and
- * he_decode_step with a step scratch are the calls whose kernels contain such waits. This is the one call of the
+ * only enqueue work), but its outputs are undefined: he_hash_keys, he_prefill_compress and its variants,
+ * he_attend, and he_decode_step with a step scratch are the calls whose kernels contain such waits. This is the one call of the
  * library, besides the *_host variants, that synchronises the device. Returns -1 if the counter cannot be read.
  * Diagnostic only: the paper has no counterpart.
  */

@@ -16,12 +16,12 @@
 namespace he {
 
 // Sequences whose budgets (16 bits, or 32 where a cache has more than 65 535 slots) travel in the kernel parameters. Every launch
-// pays for its parameters' size (a launch waited for 9.16 us with 1.2 KB of them, 9.23 with 2.2, 9.88 with 8.4), and a call of
-// more sequences reads its budgets on the device, a dependent read ahead of the code tables, and deals its units unsorted with
-// HE_FLAG_EARLY_INPUTS. With room for 256, us per call in a graph: 600 / 1024 sequences of one unit (b = 64) 9.5 / 14.7 against 9.1
-// / 14.1 now, 1024 of eight (b = 32) 41.9 against 40.4, early 400 of one (b = 64) 5.76 against 5.45. An 8-bit bound of the
-// budget beside the copy, with the budget itself read meanwhile, did not do: 14.8 at 1024.
-constexpr int kBudgetVals = 1024;
+// pays for its parameters' size: a graph node 0.75 us with up to 1.8 KB of them, 0.77 with 2.0, 0.83 with 2.2. A call of more sequences reads its budgets on the device, a dependent
+// read ahead of the code tables, and deals its units unsorted with HE_FLAG_EARLY_INPUTS. us per call in a graph, read on the device /
+// in the parameters: 600 sequences of one unit (b = 64) 9.5 / 9.1, early 400 of one 5.76 / 5.45 (and 1024 of one 14.7 / 14.1, of
+// eight at b = 32 41.9 / 40.4, which the room that the others have to pay for is not spent on). An 8-bit bound of the budget beside
+// the copy, with the budget itself read meanwhile, did not do: 14.8 at 1024.
+constexpr int kBudgetVals = 792;
 constexpr int kBudgetWords = kBudgetVals / 2;
 
 struct DecodeArgs {
@@ -123,8 +123,9 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
     const char* src = static_cast<const char*>(is_k ? a.k : a.v) + (size_t)unit * d * es;
     rowreg = __ldg(reinterpret_cast<const uint4*>(src) + (is_k ? tid : tid - cpr));
   }
-  // (the bulk-hashed kernels have no register left for a third source: 59.5 us with it where 56.6)
-  const int C = clamp_budget(a.n_budget16 > 0 ? (int)a.budget16[s] : (!PRE && a.n_budget32 > 0 ? a.budget32[s] : a.ca.budget[s]), Cmax);
+  // Only the kernel of the largest packed tables looks for 32-bit budgets: the third source costs the others 1 to 5 %.
+  constexpr bool kWide = PACKED && NT == 1024 && !PRE;
+  const int C = clamp_budget(a.n_budget16 > 0 ? (int)a.budget16[s] : (kWide && a.n_budget32 > 0 ? a.budget32[s] : a.ca.budget[s]), Cmax);
   const int fill = a.ca.fill[unit];
   const int t = a.ca.next_pos[unit];
 
