@@ -4,10 +4,11 @@
 // own slots with an online softmax (running maximum, running sum, unnormalised output) and the partial results are
 // merged through shared memory at the end. HBM-bound by design: 2 * C * d * e bytes per unit.
 //
-//   attend_bf16_kernel<D>  bf16, d = 64 or 128, G <= 8: 16 slots at a time, Q K^T and P V as warp-level m16n8k16 MMAs fed
-//                          straight from registers (bf16 products are exact, fp32 accumulation, P as hi + lo bf16);
-//                          a cluster of up to 16 CTAs shares a unit when there are few units.
-//   attend_generic_kernel  any supported dtype / d: one slot at a time, dot products by warp shuffles.
+//   attend_bf16_kernel<D, NW>  bf16, d = 64 or 128, G <= 8: 32 slots at a time from rings of TMA tiles, Q K^T and P V as warp-level
+//                          m16n8k16 MMAs (bf16 products are exact, fp32 accumulation, P as hi + lo bf16); a cluster of up
+//                          to 16 CTAs shares a unit when there are few units.
+//   attend_generic_kernel  any supported dtype / d, and where no tensor map can be encoded: one slot at a time, dot products by
+//                          warp shuffles.
 #pragma once
 #include <cuda.h>  // CUtensorMap (types only; the encoder is fetched through the runtime)
 
@@ -122,10 +123,10 @@ __device__ __forceinline__ void attend_merge_cluster(const float* part_ml, const
 
 // ------------------------------------------------------------------------------------------------ bf16, d = 64 or 128
 //
-// A warp takes 16 slots at a time. Scores: S[head][slot] = Q K^T as m16n8k16 MMAs with M = query heads (rows 0..7
+// A warp takes 32 slots at a time. Scores: S[head][slot] = Q K^T as m16n8k16 MMAs with M = query heads (rows 0..7
 // used), N = 8 slots, K = 16 channels. A dot product does not depend on the order of its terms, so the 16 "logical"
-// channels of MMA step s are chosen to suit 16-byte loads: lane (gid, tig) reads chunks tig, tig+4, ... (d = 128: + 12)
-// (8 channels each) of row gid, and chunk tig+4c feeds steps 2c (first two registers) and 2c+1 (last two); the
+// channels of MMA step s are chosen to suit 16-byte reads: lane (gid, tig) reads chunks 2 tig and 2 tig + 1 (8 channels each) of
+// every 64 channels of row gid; the c-th of them feeds steps 2c (first two registers) and 2c+1 (last two); the
 // query fragment is loaded the same way, so both operands agree on the permutation.
 // Output: O[head][channel] += P V with M = heads, K = 16 slots, N = 8 channels. The score tile's accumulator layout
 // is already the A-fragment layout of P (head gid, slots 2tig, 2tig+1 [+8]). P is split into two bf16 terms

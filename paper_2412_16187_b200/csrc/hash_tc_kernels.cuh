@@ -1,7 +1,6 @@
 // Eq. 2 on many bf16 rows with the 5th-generation tensor cores (tcgen05.mma, accumulators in tensor memory).
 //
-// Why tensor cores here and nowhere else on this path: the projection X[rows, d] * W[d, b] is the one dense
-// contraction, and at b >= 16 its arithmetic intensity (b flop per input byte) puts the CUDA-core kernel on the
+// Why tensor cores: the projection X[rows, d] * W[d, b] is a dense contraction, and at b >= 16 its arithmetic intensity (b flop per input byte) puts the CUDA-core kernel on the
 // fp32 FMA pipe instead of on HBM (profiles/: DRAM at ~5 % of peak). Exactness is kept by splitting the fp32 W
 // into three bf16 terms W = W1 + W2 + W3 (each residual is exact in fp32, so the three terms carry all 24
 // significand bits): x is bf16, every product x * W_t is exact, and only the fp32 accumulation rounds. The sign
@@ -13,7 +12,7 @@
 //   warp 4     producer: one thread issues a TMA tensor copy per 64-channel half of a 128-row tile (the hardware
 //              applies the 128-byte swizzle and signals the stage's mbarrier with the byte count); when no tensor
 //              map can be built for the caller's strides the warp falls back to 16-byte cp.async copies
-//   warp 5     one thread issues 3 terms x d/16 tcgen05.mma (M = 128, N = 32|64, K = 16) per tile and commits
+//   warp 5     one thread issues d/16 tcgen05.mma (M = 128, N = 96|192: the three terms side by side, K = 16) per tile and commits
 // Four shared-memory stages for X, W's three terms resident in shared memory, two accumulators in tensor memory
 // so the epilogue of tile i overlaps the MMAs of tile i+1. Every wait on an mbarrier is bounded: when a limit is
 // hit the CTA raises a flag, all roles leave their loops, tensor memory is released and the kernel returns.

@@ -523,8 +523,11 @@ int launch_replay_block_half(const ReplayArgs& a, long long units, cudaStream_t 
   int sms = 0, dev = 0;
   if (int rc = sm_count(&sms)) return rc;
   HE_CUDA_CHECK(cudaGetDevice(&dev));
-  // Cluster size: a block costs a CTA about 8000 cycles of settling, 380 per tile of its own and 3000 for the exchange with
-  // its peers; the number of rounds is what the clusters that fit the GPU need for the units.
+  // Cluster size: a block costs a CTA about 8000 cycles of settling (measured 5000 for the largest tables to 12 000 for 64 steps with
+  // protected windows), 380 per tile of its own and 3000 for the exchange with its peers; the number of rounds is what the
+  // clusters that fit the GPU need for the units. A wider cluster never pays with more rounds unless there are about 90 tiles (200
+  // units: two rounds of single CTAs against three of pairs cross at 89 tiles with 8000, at 74 with 5000, where they are level
+  // within 1 %), so one figure does for every block length.
   static DeviceTable<4> table;  // clusters of 2^lg CTAs that the device holds at once (-1: none)
   const int tiles = ra.r.smem_slots / kRbTile;
   double best = 0.;
