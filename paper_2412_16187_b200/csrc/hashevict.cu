@@ -501,22 +501,22 @@ int launch_replay_reg(const ReplayArgs& a, long long units, cudaStream_t stream)
 // that an SM never hosts two of its CTAs: each takes all of tensor memory, and one that waited for another's while its
 // cluster peers wait for it could wait for good.
 constexpr size_t kRbMinSmem = 120 * 1024;
-constexpr size_t kMaxDynSmem = 227 * 1024 - 2048;  // dynamic shared memory of a CTA beside the kernel's static arrays
+constexpr size_t kMaxDynSmem = 227 * 1024 - 512;  // dynamic shared memory of a CTA beside the kernel's static arrays
 
 // Shared memory of the block replay with as many operand stages as fit (fewer for large two-word tables); 0: does not fit.
-size_t rb_fit(int words, int slots, int G, int ncta, int rows_max, RbArgs* ra) {
-  ra->rows_max = rows_max;
+size_t rb_fit(int words, int slots, int G, int ncta, int form, RbArgs* ra) {
+  ra->rows_max = form == kRbHalf ? kRbRows / 2 : kRbRows;
   for (ra->abuf = 2; ra->abuf >= 1; --ra->abuf)
     for (ra->lg_stage = 2; ra->lg_stage >= 1; --ra->lg_stage) {
-      ra->L = rb_layout(words, slots, G, ncta, 1 << ra->lg_stage, ra->abuf, rows_max);
+      ra->L = rb_layout(words, slots, G, ncta, 1 << ra->lg_stage, ra->abuf, ra->rows_max, form == kRbWide);
       if (ra->L.total <= kMaxDynSmem) return ra->L.total < kRbMinSmem ? kRbMinSmem : ra->L.total;
     }
   return 0;
 }
 
-template <int WORDS, int GT, bool PROT, bool HALF>
-int launch_replay_block_half(const ReplayArgs& a, long long units, cudaStream_t stream) {
-  auto kernel = prefill_replay_block_kernel<WORDS, GT, PROT, HALF>;
+template <int WORDS, int GT, bool PROT, int FORM>
+int launch_replay_block_form(const ReplayArgs& a, long long units, cudaStream_t stream) {
+  auto kernel = prefill_replay_block_kernel<WORDS, GT, PROT, FORM>;
   RbArgs ra{};
   ra.r = a;
   ra.r.smem_slots = (a.cfg.max_budget + kRbTile - 1) / kRbTile * kRbTile;
@@ -534,7 +534,7 @@ int launch_replay_block_half(const ReplayArgs& a, long long units, cudaStream_t 
   int best_lg = -1, best_fit = 0;
   for (int lg = 0; (1 << lg) <= kRbMaxCluster && (lg == 0 || (1 << lg) <= tiles); ++lg) {
     const int n = 1 << lg;
-    if (rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, HALF ? kRbRows / 2 : kRbRows, &ra) == 0) continue;
+    if (rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, FORM, &ra) == 0) continue;
     int fit = sms;
     if (n > 1) {
       auto clusters_of = [&](int* got) -> int {
@@ -564,7 +564,7 @@ int launch_replay_block_half(const ReplayArgs& a, long long units, cudaStream_t 
   }
   if (best_lg < 0) return fail(HE_ERR_UNSUPPORTED, "max_budget %d does not fit the block replay's shared memory", a.cfg.max_budget);
   const int n = 1 << best_lg;
-  const size_t smem = rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, HALF ? kRbRows / 2 : kRbRows, &ra);
+  const size_t smem = rb_fit(WORDS, ra.r.smem_slots, a.cfg.group_size, n, FORM, &ra);
   if (int rc = set_smem(kernel, smem)) return rc;
   const long long clusters = units < best_fit ? units : best_fit;
   ra.ncta = n;
@@ -590,14 +590,20 @@ int launch_replay_block_half(const ReplayArgs& a, long long units, cudaStream_t 
 }
 
 // Two-word tables above about 8200 slots only fit with blocks of 64 steps.
+// The owner table of words costs 3 more bytes per slot and saves a pass 250 of its 600 cycles of claims: up to 6144 slots, where it
+// costs no operand stage. us per call with bytes / words: 32 units of 2048 slots 147.8 / 142.1, 128 of 1024 1554 / 1503, 512 of 512 to
+// 4096 with two words 1369 / 1354; beyond, where passes are a small share, 8 of 9830 1232 / 1238, 256 of 9830 7239 / 7367.
+constexpr int kRbWideSlots = 6144;
 template <int WORDS, int GT, bool PROT>
 int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t stream) {
-  if constexpr (WORDS == 2) {
-    RbArgs fit{};
-    if (rb_fit(WORDS, (a.cfg.max_budget + kRbTile - 1) / kRbTile * kRbTile, a.cfg.group_size, 1, kRbRows, &fit) == 0)
-      return launch_replay_block_half<WORDS, GT, PROT, true>(a, units, stream);
-  }
-  return launch_replay_block_half<WORDS, GT, PROT, false>(a, units, stream);
+  const int slots = (a.cfg.max_budget + kRbTile - 1) / kRbTile * kRbTile, G = a.cfg.group_size;
+  RbArgs fit{}, wide{};
+  const bool full = rb_fit(WORDS, slots, G, 1, kRbFull, &fit) != 0;
+  if constexpr (WORDS == 2)
+    if (!full) return launch_replay_block_form<WORDS, GT, PROT, kRbHalf>(a, units, stream);
+  if (slots <= kRbWideSlots && rb_fit(WORDS, slots, G, 1, kRbWide, &wide) != 0 && wide.abuf == fit.abuf && wide.lg_stage == fit.lg_stage)
+    return launch_replay_block_form<WORDS, GT, PROT, kRbWide>(a, units, stream);
+  return launch_replay_block_form<WORDS, GT, PROT, kRbFull>(a, units, stream);
 }
 
 template <int WORDS>
@@ -636,7 +642,7 @@ int launch_replay(const ReplayArgs& a, long long units, cudaStream_t stream) {
   const bool has_reg = a.cfg.group_size == 1 || a.cfg.group_size == 4;
   const int min_budget = units <= sms ? (has_reg ? 1 : 128) : (WORDS == 2 && a.cfg.group_size == 4 ? 256 : 384);
   bool block_ok = mode != 0 && (mode == 2 || a.cfg.max_budget >= min_budget) && a.cfg.max_budget <= kRbMaxSlots &&
-                  rb_fit(WORDS, slots, a.cfg.group_size, 1, WORDS == 2 ? kRbRows / 2 : kRbRows, &fit) != 0;
+                  rb_fit(WORDS, slots, a.cfg.group_size, 1, WORDS == 2 ? kRbHalf : kRbFull, &fit) != 0;
   if (block_ok && (a.cfg.n_sink > 0 || a.cfg.n_recent > 0)) {
     // protected windows: every budget must leave an eligible slot at every step (n_sink + n_recent < C), which the host
     // can only check on the caller's mirror of the budgets

@@ -6,11 +6,14 @@
 // so the distances of a block of steps to every slot are one [steps x K] * [K x slots] product of small integers. The
 // operands are 8-bit (e5m2 holds 2^n u for |u| <= 8, e4m3 every whole number up to 16), accumulation is fp32 over whole
 // numbers below 2^24, so the result is exact in any order. For even G the parity of D is the same for every slot of a
-// step, so the RANK D >> 1 orders the slots (D itself for odd G). Operands A = -alpha u, B = +-2 with 2 alpha = 2^12 (even
-// G) or 2^13 (odd G) and two index columns make the accumulator 2^14 * rank + (127 - slot in tile) + a constant of the
-// step: with the tile's number added, the largest accumulator of a 128-slot tile is the arg-max key of Eq. 6 over the
-// tile (largest distance, lowest slot on ties). A third column pushes slots past the budget and protected first tokens
-// below everything else.
+// step, so the RANK D >> 1 orders the slots (D itself for odd G). Operands A = -alpha u, B = +-2 with 2 alpha = 32 (even G) or 64
+// (odd G) and five more columns (a constant and the parity of the step, two digits of the index, 2^23) make the accumulator
+// 2^23 + 128 * rank + 128 - slot in tile: the largest of a 128-slot tile is the arg-max key of Eq. 6 over the tile (largest
+// distance, lowest slot on ties). Slots past the budget and protected first tokens have zeros in B and come to 2^23 alone, below
+// everything else. At 2^23 the last mantissa bit is worth one, so an accumulator's low 16 bits ARE that key (rank <= 448: below
+// 2^16), and the readers take them from tensor memory two to a register (tcgen05.ld.pack::16b) and compare two at a time: 36
+// instructions a tile and thread for 68 on the fp32 values, and half the registers. 256 units of 9830 slots, with the waits polled in
+// straight code (mbar_wait_warp): a pair of tiles 795 -> 630 cycles, a call 8580 -> 7210 us.
 //
 // What is sequential, and how it is settled side by side. Step r's victim depends on the victims s[0..r-1] of the block:
 // a base slot (the table as the block found it) may be taken already, and the keys of earlier steps are candidates
@@ -86,12 +89,12 @@ constexpr int kRbDnPitchHalf = 68;       // ... when blocks have at most 64 step
 constexpr int kRbMaxStages = 4;          // pairs of operand tiles
 
 // Byte offsets of the kernel's dynamic shared memory (after rounding its base up to 1024 bytes). Tile maxima: per CTA of the
-// cluster one block of fp32 keys, a row for each step, an odd number of words apart (a warp stores a column, a lane per
+// cluster one block of keys, a row for each step, an odd number of words apart (a warp stores a column, a lane per
 // step), then the best key of each step over each reader group's tiles.
 struct RbLayout {
   uint32_t a, bidx, b, codes, own, mx, mx_pitch, mx_block, top_at, dn, dn_buf, rn, nr, sv, sn, list, par, qraw, kraw, rec, total;
 };
-__host__ __device__ inline RbLayout rb_layout(int words, int slots, int G, int ncta, int nstage, int abuf, int rows_max) {
+__host__ __device__ inline RbLayout rb_layout(int words, int slots, int G, int ncta, int nstage, int abuf, int rows_max, bool wide) {
   RbLayout L;
   const uint32_t nt = (uint32_t)slots / kRbTile, ntl = (nt + ncta - 1) / ncta;
   uint32_t o = 0;
@@ -105,7 +108,7 @@ __host__ __device__ inline RbLayout rb_layout(int words, int slots, int G, int n
   L.bidx = take(kRbAtom);  // index columns: four variants side by side
   L.b = take(words == 2 ? (uint32_t)nstage * kRbAtom : (uint32_t)(nstage + 1) / 2 * kRbAtom);
   L.codes = take((uint32_t)slots * words * 4u);
-  L.own = take((uint32_t)slots);
+  L.own = take((uint32_t)slots * (wide ? 4u : 1u));
   L.mx_pitch = ntl | 1u;  // words
   // (one more row takes the threads without a step; whole 16-byte units, as the copies between CTAs want)
   L.top_at = (L.mx_pitch * (rows_max < kRbRows ? rows_max + 1 : rows_max) + 3u) & ~3u;
@@ -132,7 +135,7 @@ struct RbArgs {
   int scheduled;  // units are claimed from r.sched; 0: unit = cluster index
   int lg_stage;   // log2 of the pairs of operand tiles in shared memory
   int abuf;       // operand A buffers (2: the next block's is built during the tile phase)
-  int rows_max;   // steps per block at most: 128, or 64 (the HALF kernel)
+  int rows_max;   // steps per block at most: 128, or 64 (kRbHalf)
   RbLayout L;     // computed by the host: kernel parameters cost no registers
 };
 
@@ -166,10 +169,18 @@ __device__ __forceinline__ uint32_t rb_swz(int row, int chunk) {
   return (uint32_t)((row >> 3) * 1024 + (row & 7) * 128 + ((chunk ^ (row & 7)) << 4));
 }
 
-__device__ __forceinline__ float rb_fmax3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
+// The low halves of 64 accumulator columns, two to a register.
+__device__ __forceinline__ void rb_ld64_low(uint32_t taddr, uint32_t (&v)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.pack::16b.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+        "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+        "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr)
+      : "memory");
 }
 
 // Columns of a code word in operand order: output word m (four bytes) holds bits m, m + 8, m + 16, m + 24, in both
@@ -293,18 +304,22 @@ struct RbRank {
 
 // The walk through the steps fin .. rows - 1 of a block by the settling warps (file comment), every step on the table that the one
 // before it left. Every thread scans its slots (tid, tid + 384, ...), and a slot is rewritten by the thread that scans it, so that a
-// step needs one barrier: 400 cycles, and 35 (G = 1) or 55 (G = 4) more for each slot of a thread and word. `own` (all 0xFF before
-// and after) marks the slots of recent tokens meanwhile. Steps from writes_end on leave the table as it is; pos is null where
+// step needs one barrier: 400 cycles, and 35 (G = 1) or 55 (G = 4) more for each slot of a thread and word. The owner table (no claims
+// before and after) marks the slots of recent tokens meanwhile. Steps from writes_end on leave the table as it is; pos is null where
 // another CTA of the cluster writes the positions. Not inlined: inside the block loop it cost independent queries 2 % (64 ragged
 // prompts), and itself gains 6 %.
 extern __shared__ unsigned char rb_smem_raw[];
 template <int WORDS, int GT, bool PROT>
-__device__ __noinline__ void rb_walk(const RbLayout& L, int base, int cur, int32_t* pos, int t0, int fin, int rows, int writes_end, int C, int G,
+__device__ __noinline__ void rb_walk(const RbLayout& L, bool wide, int base, int cur, int32_t* pos, int t0, int fin, int rows, int writes_end, int C, int G,
                                      int S, int Rn) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, GW = G * WORDS;
   unsigned char* smem = rb_smem_raw + base;  // (not passed as pointers, so that the accesses stay shared-memory accesses)
   uint32_t* codes = reinterpret_cast<uint32_t*>(smem + L.codes);
-  uint8_t* own = smem + L.own;
+  auto recent = [&](int slot) { return wide ? reinterpret_cast<const uint32_t*>(smem + L.own)[slot] == 0u : smem[L.own + slot] == 0; };
+  auto mark = [&](int slot, uint32_t v) {
+    if (wide) reinterpret_cast<uint32_t*>(smem + L.own)[slot] = v;
+    else smem[L.own + slot] = (uint8_t)v;
+  };
   uint16_t* SV = reinterpret_cast<uint16_t*>(smem + L.sv);
   int32_t* SN = reinterpret_cast<int32_t*>(smem + L.sn);
   const int32_t* REC = reinterpret_cast<const int32_t*>(smem + L.rec);
@@ -314,7 +329,7 @@ __device__ __noinline__ void rb_walk(const RbLayout& L, int base, int cur, int32
   auto newest = [&](int r, int m) { return r >= m ? (int)SV[r - m] : REC[m - r - 1]; };  // slot of the m-th newest token at step r
   rb_bar<2, kRbResThreads>();
   if (PROT && Rn > 0) {
-    if (tid < Rn) own[newest(fin, tid + 1)] = 0;
+    if (tid < Rn) mark(newest(fin, tid + 1), 0u);
     rb_bar<2, kRbResThreads>();
   }
   const int mine = tid < C ? (C - tid + kRbResThreads - 1) / kRbResThreads : 0;  // slots of this thread
@@ -332,7 +347,7 @@ __device__ __noinline__ void rb_walk(const RbLayout& L, int base, int cur, int32
     const int out = PROT && Rn > 1 ? newest(r, Rn) : last;  // its token is recent no longer
     int best = -1, kx = kRbIdxMask - tid;
     const uint32_t* cp = codes + tid * WORDS;
-    const uint8_t* op = own + tid;
+    int slot = tid;
 #pragma unroll 4
     for (int i = 0; i < mine; ++i) {
       uint32_t h[WORDS];
@@ -343,10 +358,10 @@ __device__ __noinline__ void rb_walk(const RbLayout& L, int base, int cur, int32
         h[0] = *cp;
       }
       int key = (rk.rank(h) << kRbKeyShift) + kx;
-      if (PROT) key = kx <= kRbIdxMask - S && *op != 0 ? key : -1;
+      if (PROT) key = kx <= kRbIdxMask - S && !recent(slot) ? key : -1;
       best = max(best, key);
       cp += kRbResThreads * WORDS;
-      op += kRbResThreads;
+      slot += kRbResThreads;
       kx -= kRbResThreads;
     }
     int32_t* wbest = SN + (r & 1) * 16;
@@ -365,23 +380,26 @@ __device__ __noinline__ void rb_walk(const RbLayout& L, int base, int cur, int32
         for (int w = 0; w < WORDS; ++w) codes[last * WORDS + w] = kc[w];
         if (pos != nullptr) pos[last] = t0 + r;
       }
-      if (PROT && Rn > 0) own[last] = 0;
+      if (PROT && Rn > 0) mark(last, 0u);
     }
-    if (PROT && Rn > 0 && out % kRbResThreads == tid) own[out] = 0xFFu;
+    if (PROT && Rn > 0 && out % kRbResThreads == tid) mark(out, ~0u);
   }
   rb_bar<2, kRbResThreads>();
-  if (PROT && tid < Rn) own[newest(rows, tid + 1)] = 0xFFu;
+  if (PROT && tid < Rn) mark(newest(rows, tid + 1), ~0u);
 }
 
 // PROT: protected windows (Section 4 setup). The first n_sink tokens never leave slots 0 .. n_sink-1, so those slots are
 // masked like slots past the budget. A recent token that is already in the table is recognised by the list of the newest
 // slots, one of this block's own keys by its step. Needs every budget > n_sink + n_recent (so that some slot is always
 // eligible), n_sink <= 128 (one tile) and n_recent < 128.
-// HALF: blocks of at most 64 steps, where the largest two-word tables leave no room for the tables of more.
-template <int WORDS, int GT, bool PROT, bool HALF>
+// FORM: kRbHalf has blocks of at most 64 steps, where the largest two-word tables leave no room for the tables of more; kRbWide an
+// owner table of a word per slot instead of a byte (claims below).
+enum : int { kRbFull = 0, kRbHalf = 1, kRbWide = 2 };
+template <int WORDS, int GT, bool PROT, int FORM>
 __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(const __grid_constant__ RbArgs ar) {
   constexpr int NT = kRbThreads;
   constexpr int MS = kRbMaxStages;
+  constexpr bool HALF = FORM == kRbHalf, wide = FORM == kRbWide;
   constexpr int RM = HALF ? kRbRows / 2 : kRbRows;
   __shared__ __align__(8) unsigned long long bars[2 * MS + 4 + 5];
   __shared__ uint32_t tmem_base_s;
@@ -408,7 +426,8 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   unsigned char* Bs = smem + L.b;
   uint32_t* codes = reinterpret_cast<uint32_t*>(smem + L.codes);
   uint8_t* own = smem + L.own;
-  float* Mx = reinterpret_cast<float*>(smem + L.mx);
+  uint32_t* own32 = reinterpret_cast<uint32_t*>(own);  // wide
+  int32_t* Mx = reinterpret_cast<int32_t*>(smem + L.mx);
   const int top_at = HALF ? L.top_at : RM * L.mx_pitch;  // where a CTA's block of Mx holds its groups' best keys
   uint16_t* Dn = reinterpret_cast<uint16_t*>(smem + L.dn);
   int32_t* RN = reinterpret_cast<int32_t*>(smem + L.rn);    // per step: best base key
@@ -457,15 +476,16 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   // Scaling of the operands (file comment) and the e5m2 codes of -alpha (2 c - G) for c = 0..7 set bits among the group's
   // queries, as two words of a byte table; c = 8 (G = 8 only) is patched where it occurs.
   const bool even = (G & 1) == 0;
-  const int alpha = even ? 2048 : 4096;
-  const float off = (float)((even ? 4096 : 8192) * G * 32 * WORDS);  // accumulator + off - 2^13 parity (even G) = 2^14 * rank + index
+  const int alpha = even ? 16 : 32;
+  const int off = 2 * alpha * G * 32 * WORDS;  // data columns' sum + off - 64 parity (even G) = 128 * rank
   uint32_t lut_lo = 0u, lut_hi = 0u;
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     lut_lo |= rb_e5m2(-alpha * (2 * c - G)) << (8 * c);
     lut_hi |= (c + 4 <= G ? rb_e5m2(-alpha * (2 * (c + 4) - G)) : 0u) << (8 * c);
   }
-  for (int i = tid; i < a.smem_slots / 4; i += NT) reinterpret_cast<uint32_t*>(own)[i] = 0xFFFFFFFFu;
+  if (!wide)
+    for (int i = tid; i < a.smem_slots / 4; i += NT) own32[i] = 0xFFFFFFFFu;
   griddep_wait();  // everything above overlaps the hashing kernel's tail
   tc_fence_before();
   __syncthreads();
@@ -518,14 +538,18 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
       for (int w = 0; w < WORDS; ++w) codes[j * WORDS + w] = j < fill0 ? __ldg(kc_u + (long long)j * WORDS + w) : 0u;
     }
     for (int j = rank * NT + tid; j < (int)Cmax; j += ncta * NT) pos_g[j] = j < fill0 ? j : -1;
+    if (wide)
+      for (int j = tid; j < nbase * kRbTile; j += NT) own32[j] = 0xFFFFFFFFu;
+    uint32_t era = 0xFFFFFE00u;  // wide: claims of the current pass are era | step, of earlier ones larger
     if (PROT && tid < Rn) REC[tid] = C - 1 - tid;  // (the first C tokens sit in slot = position)
-    // Index columns of operand B (columns of A: 16, 1, 2^15): digits of 127 - x, and -256 for rows that may not win. Variant
-    // bit 0: the tile holds the protected first tokens, bit 1: the budget ends inside the tile.
+    // Further columns of operand B (columns of A: 16, 1, 2^15, off, -64 parity): digits of 128 - x, 256, 1, 1; rows that may not win
+    // have 256 alone. Variant bit 0: the tile holds the protected first tokens, bit 1: the budget ends inside the tile.
     if (tid < 4 * kRbTile) {
       const int x = tid & 127, v = tid >> 7;
       const bool bad = ((v & 1) && x < S) || ((v & 2) && x >= C - (nbase - 1) * kRbTile);
+      const uint32_t one = rb_e4m3(1), top = rb_e4m3(256) << 16;
       *reinterpret_cast<uint4*>(Bx + rb_swz(x, 2 * v)) =
-          make_uint4(rb_e4m3((127 - x) >> 4) | (rb_e4m3((127 - x) & 15) << 8) | (bad ? 0xF8u << 16 : 0u), 0u, 0u, 0u);
+          bad ? make_uint4(top, 0u, 0u, 0u) : make_uint4(rb_e4m3((128 - x) >> 4) | (rb_e4m3((128 - x) & 15) << 8) | top | (one << 24), one, 0u, 0u);
       *reinterpret_cast<uint4*>(Bx + rb_swz(x, 2 * v + 1)) = make_uint4(0u, 0u, 0u, 0u);
     }
     // The block's query and key codes into buffer `buf` (rows past the prompt keep what was there: nothing reads them).
@@ -540,7 +564,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(kd + i)), "l"(ks + i) : "memory");
       cp_async_commit();
     };
-    // Operand A, row r = step r of the block: -alpha u_t, then the three index columns. One thread per (row, word).
+    // Operand A, row r = step r of the block: -alpha u_t, then the five further columns. One thread per (row, word).
     auto build_a = [&](int buf, int nrows, int first, int nthreads) {
       const uint32_t* qd = qraw + buf * kRbRows * GW;
       unsigned char* ad = As + (WORDS == 2 && abuf > 1 ? buf * kRbAtom : 0);
@@ -562,15 +586,13 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         for (int m = 0; m < 8; ++m) {
           const uint32_t t = cnt[m] | (cnt[m] >> 4);
           v[m] = __byte_perm(lut_lo, lut_hi, __byte_perm(t, 0u, 0x4420));
-          // eight of eight: -2^14 = 0xF4 (selector 8 made the lookup give 0 there)
-          if (GT == 0) v[m] |= ((cnt[m] & 0x08080808u) * 0x1Eu) | ((cnt[m] & 0x08080808u) >> 1);
+          // eight of eight: -128 = 0xD8 (selector 8 made the lookup give 0 there)
+          if (GT == 0) v[m] |= (cnt[m] & 0x08080808u) * 0x1Bu;
           if (!valid) v[m] = 0u;
         }
         *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * w)) = make_uint4(v[0], v[1], v[2], v[3]);
         *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * w + 1)) = make_uint4(v[4], v[5], v[6], v[7]);
         if (w == 0) {
-          *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * WORDS)) = make_uint4(valid ? 0x4Cu | (0x3Cu << 8) | (0x78u << 16) : 0u, 0u, 0u, 0u);
-          *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * WORDS + 1)) = make_uint4(0u, 0u, 0u, 0u);
           int pc = 0;
           if (even && valid) {
 #pragma unroll
@@ -581,11 +603,14 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             }
           }
           PAR[buf * kRbRows + r] = pc;
+          *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * WORDS)) =
+              valid ? make_uint4(0x4Cu | (0x3Cu << 8) | (0x78u << 16) | (rb_e5m2(off) << 24), (pc & 1) ? 0xD4u : 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+          *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * WORDS + 1)) = make_uint4(0u, 0u, 0u, 0u);
         }
       }
     };
-    // One tile's row of operand B in operand stage sx (tile g of the pair): this thread's slot or key.
-    auto expand_row = [&](const uint32_t* h, int x, int sx, int g) {
+    // One tile's row of operand B in operand stage sx (tile g of the pair): this thread's slot or key; zeros for a slot that may not win.
+    auto expand_row = [&](const uint32_t* h, bool live, int x, int sx, int g) {
       unsigned char* bt = Bs + (WORDS == 2 ? sx : sx >> 1) * kRbAtom + (x >> 3) * 1024 + (x & 7) * 128;
       const int c0 = WORDS == 2 ? 4 * g : 2 * (2 * (sx & 1) + g);
 #pragma unroll
@@ -594,6 +619,10 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         const int m = (c & 1) * 4;
         *reinterpret_cast<uint4*>(bt + (((c0 + c) ^ (x & 7)) << 4)) =
             make_uint4(rb_expand4(hw, m), rb_expand4(hw, m + 1), rb_expand4(hw, m + 2), rb_expand4(hw, m + 3));
+      }
+      if (!live) {
+#pragma unroll
+        for (int c = 0; c < 2 * WORDS; ++c) *reinterpret_cast<uint4*>(bt + (((c0 + c) ^ (x & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
       }
     };
     auto a_desc_of = [&](int buf) { return umma_desc_k128(smem_u32(As)) + (uint64_t)((abuf > 1 ? buf * a_step : 0) >> 4); };
@@ -607,16 +636,16 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
     auto new_keys = [&](int buf, int n) {
       const int x = tid & 127, acc = n & 1, ph = (n >> 1) & 1, sx = stage_of(n);
       const uint32_t px = stage_phase(n);
-      if (!__all_sync(0xFFFFFFFFu, mbar_wait(sfree_bar(sx), px ^ 1, &abort_flag))) return;
+      if (!mbar_wait_warp(sfree_bar(sx), px ^ 1, &abort_flag)) return;
       uint32_t h[WORDS];
 #pragma unroll
       for (int w = 0; w < WORDS; ++w) h[w] = kraw[(buf * kRbRows + x) * WORDS + w];
-      expand_row(h, x, sx, 0);
+      expand_row(h, true, x, sx, 0);
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) mbar_arrive(full_bar(sx));
       if (warp == kRbMmaWarp) {
-        if (!__all_sync(0xFFFFFFFFu, mbar_wait2(afree_bar(acc), ph ^ 1, full_bar(sx), px, &abort_flag))) return;
+        if (!mbar_wait2_warp(afree_bar(acc), ph ^ 1, full_bar(sx), px, &abort_flag)) return;
         tc_fence_after();
         const uint64_t ad = a_desc_of(buf), bd = b_desc_of(sx, 0);
         if (rb_elect()) {
@@ -628,12 +657,12 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         }
         __syncwarp();
       }
-      if (!__all_sync(0xFFFFFFFFu, mbar_wait(afull_bar(acc), ph, &abort_flag))) return;
+      if (!mbar_wait_warp(afull_bar(acc), ph, &abort_flag)) return;
       tc_fence_after();
       // Conversions by an fp32 addition (the integer conversions run at a sixteenth of its rate): 2^22 + rank has 2 * rank
       // in its low bits, which is what is kept.
       const int r = x, last = PROT ? r - Rn : r;  // entries below `last` are candidates
-      const float magic = (off - (float)((PAR[buf * kRbRows + r] & 1) << 13)) * (1.f / 16384.f) + 4194304.f;
+      const float magic = (float)(off - ((PAR[buf * kRbRows + r] & 1) << 6)) * (1.f / 128.f) + 4194304.f;
       const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(2 * acc * kRbTile);
       uint16_t* dst = Dn + buf * L.dn_buf + rb_dn_at(r, RM);
       float dmax = -1e9f;
@@ -657,14 +686,14 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           uint32_t pk[2];
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
-            const float y0 = fmaf(__uint_as_float(v[4 * k + 2 * e]), 1.f / 16384.f, magic);
-            const float y1 = fmaf(__uint_as_float(v[4 * k + 2 * e + 1]), 1.f / 16384.f, magic);
+            const float y0 = fmaf(__uint_as_float(v[4 * k + 2 * e]), 1.f / 128.f, magic);
+            const float y1 = fmaf(__uint_as_float(v[4 * k + 2 * e + 1]), 1.f / 128.f, magic);
             pk[e] = __byte_perm(__float_as_uint(y0), __float_as_uint(y1), 0x5410);
           }
           if (c * 32 + 4 * k < r && r < RM) *reinterpret_cast<uint2*>(dst + c * 32 + 4 * k) = make_uint2(pk[0], pk[1]);
         }
       }
-      NR[buf * kRbRows + r] = last > 0 ? (int)(__float_as_uint(fmaf(dmax, 1.f / 16384.f, magic)) & 0xFFFFu) >> 1 : -1;
+      NR[buf * kRbRows + r] = last > 0 ? (int)(__float_as_uint(fmaf(dmax, 1.f / 128.f, magic)) & 0xFFFFu) >> 1 : -1;
     };
     int cur = 0;
     if (C < N) {
@@ -689,53 +718,46 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
       // ---------------------------------------------------------------- tile phase
       // this CTA's base tiles 0 .. ntl - 1 (tile i of the CTA is tile i * ncta + rank of the unit)
       const int npair = (ntl + 1) >> 1;
-      float topf = -1.f;  // readers: best base key of the thread's step so far
+      int top = -1;  // readers: best base key of the thread's step so far
       if (warp < kRbExpWarp) {
         const int r = tid & 127, grp = warp >> 2;  // this thread's step = its tensor-memory lane; tile grp of each pair
-        float* mrow = Mx + rank * L.mx_block + min(r, RM) * L.mx_pitch;
-        // 2^14 rank + index: the step's constant, and 127 - tile above the index within the tile (lower tiles first)
-        float ct = off - (float)((PAR[cur * kRbRows + r] & 1) << 13) + (float)((127 - ((grp << lg_ncta) + rank)) * 128);
-        const float cstep = (float)(256 << lg_ncta);
+        int32_t* mrow = Mx + rank * L.mx_block + min(r, RM) * L.mx_pitch;
+        int ct = (127 - ((grp << lg_ncta) + rank)) * 128;  // 127 - tile goes above the index within the tile (lower tiles first)
+        const int cstep = 256 << lg_ncta;
         const uint32_t taddr0 = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(grp * kRbTile);
         if (ncta > 1 && blk > 0) rb_wait_cluster(used_bar, (blk - 1) & 1, &abort_flag);  // peers still read the block before
         for (int p = 0; p < npair; ++p) {
           const int n = it + p, acc = n & 1, ph = (n >> 1) & 1, i = 2 * p + grp;
-          if (!__all_sync(0xFFFFFFFFu, mbar_wait(afull_bar(acc), ph, &abort_flag))) break;
+          if (!mbar_wait_warp(afull_bar(acc), ph, &abort_flag)) break;
           tc_fence_after();
           // (the second tile of an odd last pair holds an older product; nobody looks at its key)
           const uint32_t taddr = taddr0 + (uint32_t)(2 * acc * kRbTile);
-          uint32_t v0[32], v1[32];
-          float m[8];
-          tc_ld32(taddr, v0);
-          tc_ld32(taddr + 32, v1);
+          uint32_t v0[32], v1[32], m[8];
+          rb_ld64_low(taddr, v0);
+          rb_ld64_low(taddr + 64, v1);
           tc_wait_ld();
-#pragma unroll
-          for (int k = 0; k < 8; ++k) m[k] = rb_fmax3(__uint_as_float(v0[k]), __uint_as_float(v0[k + 8]), __uint_as_float(v0[k + 16]));
-#pragma unroll
-          for (int k = 0; k < 8; ++k) m[k] = rb_fmax3(m[k], __uint_as_float(v0[k + 24]), __uint_as_float(v1[k]));
-          tc_ld32(taddr + 64, v0);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) m[k] = rb_fmax3(m[k], __uint_as_float(v1[k + 8]), __uint_as_float(v1[k + 16]));
-#pragma unroll
-          for (int k = 0; k < 4; ++k) m[k] = rb_fmax3(m[k], __uint_as_float(v1[k + 24]), __uint_as_float(v1[k + 28]));
-          tc_ld32(taddr + 96, v1);
-          tc_wait_ld();
-          tc_fence_before();  // the last read: the accumulators go back
+          tc_fence_before();  // the accumulators go back
           __syncwarp();
           if (lane == 0) mbar_arrive(afree_bar(acc));
 #pragma unroll
-          for (int k0 = 0; k0 < 32; k0 += 8)
+          for (int k = 0; k < 8; ++k) m[k] = __vimax3_u16x2(v0[k], v0[k + 8], v0[k + 16]);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) m[k] = rb_fmax3(m[k], __uint_as_float(v0[k0 + k]), __uint_as_float(v1[k0 + k]));
-          // the tile's best key; negative: no slot of the tile may win
-          const float key = rb_fmax3(rb_fmax3(m[0], m[1], m[2]), rb_fmax3(m[3], m[4], m[5]), fmaxf(m[6], m[7])) + ct;
+          for (int k = 0; k < 8; ++k) m[k] = __vimax3_u16x2(m[k], v0[k + 24], v1[k]);
+#pragma unroll
+          for (int k = 0; k < 8; ++k) m[k] = __vimax3_u16x2(m[k], v1[k + 8], v1[k + 16]);
+          m[0] = __vimax3_u16x2(m[0], v1[24], v1[25]), m[1] = __vimax3_u16x2(m[1], v1[26], v1[27]);
+          m[2] = __vimax3_u16x2(m[2], v1[28], v1[29]), m[3] = __vimax3_u16x2(m[3], v1[30], v1[31]);
+          m[0] = __vimax3_u16x2(m[0], m[1], m[2]), m[3] = __vimax3_u16x2(m[3], m[4], m[5]);
+          m[0] = __vmaxu2(__vimax3_u16x2(m[0], m[3], m[6]), m[7]);
+          // the tile's best key, 2^14 rank + index; negative: no slot of the tile may win
+          const int k16 = (int)max(m[0] & 0xFFFFu, m[0] >> 16) - 1, key = ((k16 & ~127) << 7) + (k16 & 127) + ct;
           ct -= cstep;
           if (i < ntl) {
-            topf = fmaxf(topf, key);
+            top = max(top, key);
             mrow[i] = key;
           }
         }
-        if (r < RM) Mx[rank * L.mx_block + top_at + grp * RM + r] = topf;  // this group's best key of the step
+        if (r < RM) Mx[rank * L.mx_block + top_at + grp * RM + r] = top;  // this group's best key of the step
         if (ncta > 1) fence_proxy_async();
         rb_bar<4, 32 * kRbExpWarp>();  // the reader groups see each other's results
         if (tid < ncta - 1) {          // ... and every peer gets this CTA's block
@@ -754,6 +776,8 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         const int x = tid & 127;  // this thread's row of both tiles of a pair
         const uint32_t* base = codes + (rank * kRbTile + x) * WORDS;
         const int tstep = (kRbTile * WORDS) << lg_ncta;  // words between this CTA's tiles
+        const int jstep = kRbTile << lg_ncta;            // ... slots
+        int j0 = rank * kRbTile + x;                     // this thread's slot of the pair's first tile
         for (int p = 0; p < npair; ++p) {
           uint32_t h0[WORDS], h1[WORDS];
           const bool two = 2 * p + 1 < ntl;
@@ -763,9 +787,10 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             h1[w] = two ? base[(2 * p + 1) * tstep + w] : 0u;
           }
           const int sx = stage_of(it + p);
-          if (!__all_sync(0xFFFFFFFFu, mbar_wait(sfree_bar(sx), stage_phase(it + p) ^ 1, &abort_flag))) break;
-          expand_row(h0, x, sx, 0);
-          expand_row(h1, x, sx, 1);
+          if (!mbar_wait_warp(sfree_bar(sx), stage_phase(it + p) ^ 1, &abort_flag)) break;
+          expand_row(h0, j0 >= S && j0 < C, x, sx, 0);
+          expand_row(h1, j0 + jstep < C, x, sx, 1);
+          j0 += 2 * jstep;
           fence_proxy_async();
           __syncwarp();
           if (lane == 0) mbar_arrive(full_bar(sx));
@@ -780,7 +805,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             const uint64_t bd = b_desc_of(sx, 0), bd1 = bd + (uint64_t)((WORDS == 2 ? 64 : 32) >> 4);
             const uint64_t x0 = x_desc + (uint64_t)((i == first_i ? 2 : 0) + (i == last_i ? 4 : 0));
             const uint64_t x1 = x_desc + (uint64_t)(i + 1 == last_i ? 4 : 0);
-            if (!__all_sync(0xFFFFFFFFu, mbar_wait2(afree_bar(acc), ph ^ 1, full_bar(sx), stage_phase(n), &abort_flag))) break;
+            if (!mbar_wait2_warp(afree_bar(acc), ph ^ 1, full_bar(sx), stage_phase(n), &abort_flag)) break;
             tc_fence_after();
             if (rb_elect()) {
               const uint32_t d = tmem_base + (uint32_t)(2 * acc * kRbTile);
@@ -816,21 +841,29 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
       }
       it += npair + (tn < N ? 1 : 0);
       // ---------------------------------------------------------------- settle the block's steps
-      // Owner table: own[slot] = first step that claims the slot in this pass | pass parity << 7, so that claims of the
-      // pass before need not be cleared first; (own ^ tag) < r says that a step before r claims the slot (0xFF: nobody).
+      // Owner table: the first step that claims a slot in this pass. Wide: the smallest of era | step, by an atomic minimum; eras
+      // descend from pass to pass, so that older claims count as none and nothing is ever cleared: (own32 - era) < r says that a
+      // step before r claims the slot. Narrow: own[slot] = step | pass parity << 7, (own ^ tag) < r says so (0xFF: nobody), and
+      // claims of the pass before are taken back.
       if (warp < kRbResWarps) {
         tc_fence_before();
         const int r = tid;  // warps 0-3: this thread's step
+        era -= 256u;
+        if (wide && __builtin_expect(era < 0x20000u, 0)) {  // (16 million passes on)
+          for (int j = tid; j < nbase * kRbTile; j += kRbResThreads) own32[j] = 0xFFFFFFFFu;
+          era = 0xFFFFFE00u;
+          rb_bar<2, kRbResThreads>();
+        }
         const bool mine = tid < rows;
         int top_slot = 0, sv = 0, prev = 0;  // warps 0-3: best base slot, slot that the step writes (now, a pass ago)
-        bool forced = false, flagged = false;  // ... the best base slot may hold a recent token; or a new entry may win
+        bool forced = false, flagged = false;  // ... the best base slot holds a recent token; or a new entry may win
         if (warp < 4) {
           if (ncta > 1) rb_wait_cluster(tops_bar, blk & 1, &abort_flag);
-          for (int c = 0; c < kRbReadGroups * ncta; ++c) topf = fmaxf(topf, Mx[(c >> 1) * L.mx_block + top_at + (c & 1) * RM + (r < RM ? r : 0)]);
-          const int top = __float2int_rn(topf);
+          for (int c = 0; c < kRbReadGroups * ncta; ++c) top = max(top, Mx[(c >> 1) * L.mx_block + top_at + (c & 1) * RM + (r < RM ? r : 0)]);
           top_slot = max(0, min(kRbIdxMask - (top & kRbIdxMask), C - 1));
           sv = prev = top_slot;
-          forced = PROT && r < Rn;
+          if (PROT && 32 * warp < Rn)  // REC[m] entered m + 1 steps before the block: recent while r + m < Rn
+            for (int m = 0; m < Rn; ++m) forced |= m < Rn - r && REC[m] == top_slot;
           flagged = forced || NR[cur * kRbRows + r] >= (top >> kRbKeyShift);
           RN[r] = top;
           if (tid < 2) s_change[tid] = kRbRows;
@@ -842,26 +875,33 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           const int par = pass & 1;
           bool is_hard = false;
           if (warp < 4) {
-            // Claims: earlier warps store after later ones, so that a slot goes to its first warp; among that warp's lanes any
-            // may win, the earlier ones store again.
             SV[r] = mine ? (uint16_t)sv : (uint16_t)0xFFFFu;
-#pragma unroll
-            for (int k = 3; k >= 0; --k) {
-              if (warp == k && mine) own[sv] = (uint8_t)((uint32_t)r | tag);
+            bool stale;
+            if (wide) {
+              if (mine) atomicMin(&own32[sv], era | (uint32_t)r);
               rb_bar<1, kRbRows>();
+              stale = own32[top_slot] - era < (uint32_t)r;
+            } else {
+              // Earlier warps store after later ones, so that a slot goes to its first warp; among that warp's lanes any may win,
+              // the earlier ones store again.
+#pragma unroll
+              for (int k = 3; k >= 0; --k) {
+                if (warp == k && mine) own[sv] = (uint8_t)((uint32_t)r | tag);
+                rb_bar<1, kRbRows>();
+              }
+              for (;;) {
+                const uint32_t o = own[sv] ^ tag;
+                const bool again = mine && (int)(o >> 5) == warp && o > (uint32_t)r;
+                if (!__any_sync(0xFFFFFFFFu, again)) break;
+                if (again) own[sv] = (uint8_t)((uint32_t)r | tag);
+                __syncwarp();
+              }
+              rb_bar<1, kRbRows>();
+              const uint32_t o_top = own[top_slot];
+              if (prev != sv && (own[prev] ^ (tag ^ 0x80u)) < 128u) own[prev] = 0xFFu;  // claimed a pass ago, by nobody now
+              stale = (o_top ^ tag) < (uint32_t)r;
             }
-            for (;;) {
-              const uint32_t o = own[sv] ^ tag;
-              const bool again = mine && (int)(o >> 5) == warp && o > (uint32_t)r;
-              if (!__any_sync(0xFFFFFFFFu, again)) break;
-              if (again) own[sv] = (uint8_t)((uint32_t)r | tag);
-              __syncwarp();
-            }
-            rb_bar<1, kRbRows>();
-            const uint32_t o_top = own[top_slot];
-            if (prev != sv && (own[prev] ^ (tag ^ 0x80u)) < 128u) own[prev] = 0xFFu;  // claimed a pass ago, by nobody now
             // hard steps of the window
-            const bool stale = (o_top ^ tag) < (uint32_t)r;
             is_hard = r >= fb && r < wend && (flagged || stale);
             const uint32_t hm = __ballot_sync(0xFFFFFFFFu, is_hard);
             if (is_hard) LIST[warp * 32 + __popc(hm & ((1u << lane) - 1u))] = (uint8_t)((uint32_t)r | (stale || forced ? 0x80u : 0u));
@@ -900,7 +940,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             // entry may have been overwritten: it leaves the race. Each round takes a tile or an entry out.
             bool exact = (entry & 0x80) == 0;  // kb is a live slot's key
             bool loaded = false;
-            float mt[4];  // lane l: tiles l, l + 32, ...
+            int mt[4];  // lane l: tiles l, l + 32, ...
             RbRank<WORDS, GT> rk;
             int live = -1;  // best live slot of the tiles scanned so far, this lane's share
             for (int round = 0; round <= nbase + kRbRows; ++round) {
@@ -925,8 +965,8 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
               }
               if (exact || kb < 0) break;
               const int sb = min(kRbIdxMask - (kb & kRbIdxMask), C - 1);
-              if (loaded || PROT) {  // (the first time it is known to be taken)
-                bool bad = (own[sb] ^ tag) < (uint32_t)r2;
+              if (loaded) {  // (the first time it is known to be taken, or recent)
+                bool bad = wide ? own32[sb] - era < (uint32_t)r2 : (own[sb] ^ tag) < (uint32_t)r2;
                 if (PROT && r2 < Rn && !bad) {  // REC[m - 1] entered m steps before the block: recent while r2 + m <= Rn
                   bool hit = false;
                   for (int m0 = 0; m0 < Rn - r2; m0 += 32) hit |= m0 + lane < Rn - r2 && REC[m0 + lane] == sb;
@@ -939,17 +979,23 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                   const int T = lane + 32 * i;
-                  mt[i] = T < nbase ? Mx[(T & (ncta - 1)) * L.mx_block + r2 * L.mx_pitch + (T >> lg_ncta)] : -1.f;
+                  mt[i] = T < nbase ? Mx[(T & (ncta - 1)) * L.mx_block + r2 * L.mx_pitch + (T >> lg_ncta)] : -1;
                 }
                 rk.load(qb + r2 * GW, G, PAR[cur * kRbRows + r2]);
               }
               const int cb = sb >> 7, j0 = cb * kRbTile + 4 * lane;
-              const uint32_t o4 = *reinterpret_cast<const uint32_t*>(own + j0) ^ (tag * 0x01010101u);
               uint32_t hw[4 * WORDS];
 #pragma unroll
               for (int i = 0; i < WORDS; ++i) *reinterpret_cast<uint4*>(hw + 4 * i) = *reinterpret_cast<const uint4*>(codes + j0 * WORDS + 4 * i);
-              // bit 7 of a byte: nobody claims the slot before r2 (unclaimed bytes have bit 7 set, claims are below 128)
-              uint32_t ok4 = (((o4 | 0x80808080u) - (uint32_t)r2 * 0x01010101u) | o4);
+              uint32_t ok4;  // bit 7 of a byte: nobody claims the slot before r2
+              if (wide) {
+                const uint4 o = *reinterpret_cast<const uint4*>(own32 + j0);
+                ok4 = (o.x - era < (uint32_t)r2 ? 0u : 0x80u) | (o.y - era < (uint32_t)r2 ? 0u : 0x8000u) |
+                      (o.z - era < (uint32_t)r2 ? 0u : 0x800000u) | (o.w - era < (uint32_t)r2 ? 0u : 0x80000000u);
+              } else {  // (unclaimed bytes have bit 7 set, claims are below 128)
+                const uint32_t o4 = *reinterpret_cast<const uint32_t*>(own + j0) ^ (tag * 0x01010101u);
+                ok4 = (((o4 | 0x80808080u) - (uint32_t)r2 * 0x01010101u) | o4);
+              }
               if (PROT && r2 < Rn)
                 for (int m0 = 0; m0 < Rn - r2; ++m0) {
                   const int q = REC[m0] - j0;
@@ -965,14 +1011,12 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
                 const bool ok = (ok4 & (0x80u << (8 * e))) != 0u && e < hi && (!PROT || e >= lo);
                 live = max(live, ok ? key : -1);
               }
-              float mm = -1.f;
+              int km = -1;
 #pragma unroll
               for (int i = 0; i < 4; ++i) {
-                if (cb == lane + 32 * i) mt[i] = -1.f;
-                mm = fmaxf(mm, mt[i]);
+                if (cb == lane + 32 * i) mt[i] = -1;
+                km = max(km, mt[i]);
               }
-              // (keys are whole numbers below 2^23: the sum has them in its mantissa)
-              const int km = mm < 0.f ? -1 : (int)(__float_as_uint(mm + 8388608.f) & 0x7FFFFFu);
               kb = __reduce_max_sync(0xFFFFFFFFu, max(live, km));
             }
             const int slot = min(kRbIdxMask - (max(max(kb, kn), 0) & kRbIdxMask), C - 1);
@@ -983,6 +1027,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           }
           rb_bar<2, kRbResThreads>();
           const int ch = s_change[par];
+          era -= 256u;
           prev = sv;
           if (ch < kRbRows) {
             fb = ch + 1;
@@ -1004,27 +1049,35 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         };
         // last writers: the steps claim again, later ones over earlier ones (the prompt's last step waits until its scores
         // are taken)
+        era -= 256u;
         if (warp < 4) {
           const bool in = tid < fin && !(scoring && r == rows - 1);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            if (warp == k && in) own[sv] = (uint8_t)r;
+          if (wide) {
+            const uint32_t claim = era | (uint32_t)(kRbRows - 1 - r);
+            if (in) atomicMin(&own32[sv], claim);
             rb_bar<1, kRbRows>();
+            if (in && own32[sv] == claim) apply(sv);
+          } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              if (warp == k && in) own[sv] = (uint8_t)r;
+              rb_bar<1, kRbRows>();
+            }
+            for (;;) {
+              const int o = own[sv];
+              const bool again = in && (o >> 5) == warp && o < r;
+              if (!__any_sync(0xFFFFFFFFu, again)) break;
+              if (again) own[sv] = (uint8_t)r;
+              __syncwarp();
+            }
+            rb_bar<1, kRbRows>();
+            if (in && own[sv] == (uint8_t)r) apply(sv);
+            rb_bar<1, kRbRows>();
+            if (mine) own[sv] = 0xFFu;
           }
-          for (;;) {
-            const int o = own[sv];
-            const bool again = in && (o >> 5) == warp && o < r;
-            if (!__any_sync(0xFFFFFFFFu, again)) break;
-            if (again) own[sv] = (uint8_t)r;
-            __syncwarp();
-          }
-          rb_bar<1, kRbRows>();
-          if (in && own[sv] == (uint8_t)r) apply(sv);
-          rb_bar<1, kRbRows>();
-          if (mine) own[sv] = 0xFFu;
         }
         if (__builtin_expect(fin < rows, 0)) {
-          rb_walk<WORDS, GT, PROT>(L, (int)(smem - rb_smem_raw), cur, rank == 0 ? pos_g : nullptr, t0, fin, rows, scoring ? rows - 1 : rows, C, G, S, Rn);
+          rb_walk<WORDS, GT, PROT>(L, wide, (int)(smem - rb_smem_raw), cur, rank == 0 ? pos_g : nullptr, t0, fin, rows, scoring ? rows - 1 : rows, C, G, S, Rn);
           if (mine) sv = SV[r];
         }
         int keep = 0;

@@ -1,0 +1,29 @@
+"""The block replay at both ends of what its 16-bit tile keys hold and on both sides of where its owner table changes from words to
+bytes: the largest ranks (odd groups of two-word codes, groups of eight), codes of a few bits (most keys tie, and recent tokens hold
+best slots), and tables just within and just beyond the word table's limit, against the oracle, bit for bit."""
+import pytest
+
+from cases import C
+from parity import Case
+
+pytestmark = pytest.mark.gpu
+
+base = C["throughput_batch"].scaled(batch=1, n_kv_heads=2, ragged=False)
+SHAPES = {
+    "group_7_b64": base.scaled(group_size=7, budget=257, prompt_len=700),
+    "group_3_b32": base.scaled(group_size=3, hash_bits=32, budget=384, prompt_len=800),
+    "group_8_b64_protected": base.scaled(group_size=8, budget=300, prompt_len=700, n_sink=4, n_recent=10),
+    "group_4_b1": base.scaled(hash_bits=1, budget=200, prompt_len=500),
+    "group_1_b2_protected": base.scaled(group_size=1, hash_bits=2, budget=150, prompt_len=600, n_sink=3, n_recent=40),
+    "words_6144": base.scaled(n_kv_heads=1, hash_bits=32, budget=6144, prompt_len=6500),
+    "bytes_6148": base.scaled(n_kv_heads=1, hash_bits=32, budget=6148, prompt_len=6500, n_sink=4, n_recent=10),
+    "two_words_4096": base.scaled(n_kv_heads=1, budget=4096, prompt_len=4500),
+    "two_words_4100": base.scaled(n_kv_heads=1, budget=4100, prompt_len=4500),
+}
+
+
+@pytest.mark.parametrize("name", list(SHAPES))
+def test_replay_forms(name):
+    case = Case(SHAPES[name])
+    case.prefill()
+    case.compare_state()
