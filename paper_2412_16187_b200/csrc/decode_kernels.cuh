@@ -34,6 +34,7 @@ struct DecodeArgs {
   int32_t* evicted_pos_out;
   uint32_t* qcodes_out;
   const uint32_t* new_codes;               // PRE kernels: [B*Hkv*G + B*Hkv, Wd] codes of this step's q rows, then k rows
+  int pos_at;  // one-word tables: words into the dynamic shared memory where the unit's positions are copied to; 0: read where they are
   // What is in the union, copied from he_cache.budget_host (one of them > 0, or none):
   int n_budget16, n_budget32;  // the sequences' budgets
   int n_sched;                 // the sequences by budget, largest first (sequence << 21 | budget)
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
   static_assert(!PACKED || WORDS == 1, "packed tables hold codes of at most 24 bits");
   constexpr int SPV = 4 / WORDS;  // slots per 16-byte vector
   constexpr int BP = 32 * WORDS;
-  constexpr bool kGroupedCopy = WORDS == 2;
+  constexpr bool kGroupedCopy = WORDS == 2, kPosCopied = WORDS == 1 && !PACKED;
   using Ctx = QueryCtx<WORDS, GT>;
   extern __shared__ __align__(16) uint32_t dsm[];  // the unit's code words
   // staging of the rows to hash and of the partial sums: not needed when the codes come pre-hashed
@@ -92,8 +93,12 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
   const int cpr = d * es / 16;  // 16-byte chunks per row
   const bool dense = !PRE && nitems <= NT && R <= kRowBatch && cpr <= 32;  // one item per thread, one pass, one chunk per lane
   float wreg[kChunk];
-  if (dense && tid < nitems) {
-    const int c0 = (tid / BP) * kChunk, bi = tid % BP;
+  // Where there are twice as many threads as work items, the upper half takes rows 3 and 4 (a row's sum is in the same order).
+  const bool halves = WORDS == 1 && 2 * nitems <= NT && (nitems & (nitems - 1)) == 0;
+  const int item = halves ? tid & (nitems - 1) : tid, row0 = halves && tid >= nitems ? 3 : 0;
+  const bool hashes = dense && tid < (halves ? 2 * nitems : nitems) && row0 < R;
+  if (hashes) {
+    const int c0 = (item / BP) * kChunk, bi = item % BP;
     if (b == BP && d % kChunk == 0) {  // b = 32 or 64 and whole chunks: constant strides, no edge tests
       const float* wp = a.ca.W + c0 * BP + bi;
 #pragma unroll
@@ -106,7 +111,26 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
     }
   }
 
-  if (!PRE) griddep_wait();
+  // Only the kernel of the largest packed tables looks for 32-bit budgets: the third source costs the others 1 to 5 %.
+  constexpr bool kWide = PACKED && NT == 1024 && !PRE;
+  auto budget_of = [&]() {
+    return clamp_budget(a.n_budget16 > 0 ? (int)a.budget16[s] : (kWide && a.n_budget32 > 0 ? a.budget32[s] : a.ca.budget[s]), Cmax);
+  };
+  const int cb = PACKED ? (b + 7) >> 3 : 0;
+  auto vecs_of = [&](int c) { return PACKED ? (c * cb + 15) / 16 : (c * WORDS + 3) / 4; };
+  auto table_of = [&]() {
+    return PACKED ? reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(a.ca.codes) + (size_t)unit * Cmax * cb)
+                  : reinterpret_cast<const uint4*>(a.ca.codes + (size_t)unit * Cmax * WORDS);
+  };
+  if (!PRE) {
+    // The table comes to L2 under the previous kernel's tail (budgets do not change while a cache is in use, and a prefetch returns no
+    // data, so it cannot see a stale code).
+    if (tid == 0) {
+      const int n = vecs_of(budget_of());
+      if (n > 0) l2_prefetch_bulk(table_of(), (uint32_t)n * 16u);
+    }
+    griddep_wait();
+  }
   // The rows to hash are requested before the code table: they head the dependency chain, the table only has to
   // be there when hashing is done.
   uint4 xraw = make_uint4(0u, 0u, 0u, 0u);
@@ -123,19 +147,20 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
     const char* src = static_cast<const char*>(is_k ? a.k : a.v) + (size_t)unit * d * es;
     rowreg = __ldg(reinterpret_cast<const uint4*>(src) + (is_k ? tid : tid - cpr));
   }
-  // Only the kernel of the largest packed tables looks for 32-bit budgets: the third source costs the others 1 to 5 %.
-  constexpr bool kWide = PACKED && NT == 1024 && !PRE;
-  const int C = clamp_budget(a.n_budget16 > 0 ? (int)a.budget16[s] : (kWide && a.n_budget32 > 0 ? a.budget32[s] : a.ca.budget[s]), Cmax);
+  const int C = budget_of();
   const int fill = a.ca.fill[unit];
   const int t = a.ca.next_pos[unit];
 
   // (1) code words -> shared memory, asynchronously. The copy is sized by the budget alone: if the unit turns out
   // to be still filling (fill < C) the copied words are simply not used.
-  const int cb = PACKED ? (b + 7) >> 3 : 0;
-  const int nvec = PACKED ? (C * cb + 15) / 16 : (C * WORDS + 3) / 4;
+  const int nvec = vecs_of(C);
   {
-    const uint4* cvec = PACKED ? reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(a.ca.codes) + (size_t)unit * Cmax * cb)
-                               : reinterpret_cast<const uint4*>(a.ca.codes + (size_t)unit * Cmax * WORDS);
+    const uint4* cvec = table_of();
+    if (kPosCopied && a.pos_at > 0) {  // (protected windows: every slot's position, so that the scan does not wait for them)
+      const int32_t* pu = a.ca.pos + (size_t)unit * Cmax;
+      for (int vi = tid; 4 * vi < C; vi += NT) cp_async16(dsm + a.pos_at + 4 * vi, pu + 4 * vi);
+      cp_async_commit();
+    }
     // Two-word codes (b > 32): one commit group per vector of this thread; the scan waits for them one by one and
     // reads only what this thread copied itself, so it overlaps the rest of the transfer. Measured on B200 this is
     // 6 % faster per call at b = 64 but slower at b <= 32 (larger unrolled scan body), where a single group is used.
@@ -184,22 +209,22 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
   if (PRE) {
     // nothing to hash in this kernel
   } else if (dense) {
-    const bool active = tid < nitems;
-    const int qd = tid / BP, bi = tid % BP;
+    const int qd = item / BP, bi = item % BP;
     if (stages) store_chunk(xs[warp], xraw, lane, cfg.dtype);
     if (warp < kRowBatch)  // zeros for absent rows and for the channels that pad the last chunk
       for (int c = (warp < R ? d : 0) + lane; c < nch * kChunk; c += 32) xs[warp][c] = 0.f;
     __syncthreads();
-    if (active) {
-      float acc[kRowBatch];
+    auto project = [&](auto rows_c) {
+      constexpr int kRows = decltype(rows_c)::value;
+      float acc[kRows];
 #pragma unroll
-      for (int r = 0; r < kRowBatch; ++r) acc[r] = 0.f;
-      const float* xb = &xs[0][qd * kChunk];
+      for (int r = 0; r < kRows; ++r) acc[r] = 0.f;
+      const float* xb = &xs[row0][qd * kChunk];
 #pragma unroll
       for (int cc = 0; cc < kChunk; cc += 4) {
 #pragma unroll
-        for (int r = 0; r < kRowBatch; ++r) {
-          const float4 xv = *reinterpret_cast<const float4*>(xb + r * kMaxDim + cc);
+        for (int r = 0; r < kRows; ++r) {
+          const float4 xv = *reinterpret_cast<const float4*>(xb + (kRows < kRowBatch ? min(r, kRowBatch - 1 - row0) : r) * kMaxDim + cc);
           acc[r] = fmaf(xv.x, wreg[cc], acc[r]);
           acc[r] = fmaf(xv.y, wreg[cc + 1], acc[r]);
           acc[r] = fmaf(xv.z, wreg[cc + 2], acc[r]);
@@ -207,7 +232,12 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
         }
       }
 #pragma unroll
-      for (int r = 0; r < kRowBatch; ++r) part[qd][r][bi] = acc[r];
+      for (int r = 0; r < kRows; ++r)
+        if (row0 + r < kRowBatch) part[qd][row0 + r][bi] = acc[r];
+    };
+    if (hashes) {
+      if (halves) project(std::integral_constant<int, 3>{});
+      else project(std::integral_constant<int, kRowBatch>{});
     }
     __syncthreads();
     combine(0);
@@ -244,13 +274,14 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
       combine(r0);
     }
   }
-  if (!kGroupedCopy) cp_async_wait_all();  // this thread's code copies have landed
+  if (!kGroupedCopy) cp_async_wait_all();  // this thread's code (and position) copies have landed
   __syncthreads();                         // the codes of the new rows (and, ungrouped, the table) are in shared memory
   if (a.qcodes_out != nullptr && tid < G * WORDS) a.qcodes_out[(size_t)unit * G * WORDS + tid] = codes_s[tid];
 
   // (3) Eq. 5 / Eq. 6
   const bool evict = C >= 1 && fill >= C;
-  int slot = fill;
+  int slot = fill, ev = -1;
+  bool tail = tid == NT - 1;  // this thread writes the unit's positions, code and counters
   if (evict) {
     Ctx ctx;
     if (GT == 4) {  // build the bit-plane record in registers
@@ -287,14 +318,22 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
           rk[e] = ctx.rank(h);
         }
         if (j0 + SPV <= C) {  // every vector but possibly a unit's last one
+          int pv[4] = {0, 0, 0, 0};
+          if (PROT) {
+            const int32_t* src = kPosCopied && a.pos_at > 0 ? reinterpret_cast<const int32_t*>(dsm) + a.pos_at + j0 : pp + j0;
+            if (SPV == 4) {
+              const int4 p4 = *reinterpret_cast<const int4*>(src);
+              pv[0] = p4.x, pv[1] = p4.y, pv[2] = p4.z, pv[3] = p4.w;
+            } else {
+              const int2 p2 = *reinterpret_cast<const int2*>(src);
+              pv[0] = p2.x, pv[1] = p2.y;
+            }
+          }
 #pragma unroll
           for (int e = 0; e < SPV; ++e) {
             const uint32_t key = ((uint32_t)rk[e] << kKeyIdxBits) + (kKeyBase - (uint32_t)(j0 + e));
             best_all = max(best_all, key);
-            if (PROT) {
-              const int p = __ldg(pp + j0 + e);
-              if (p >= cfg.n_sink && p < t - cfg.n_recent) best_el = max(best_el, key);
-            }
+            if (PROT && pv[e] >= cfg.n_sink && pv[e] < t - cfg.n_recent) best_el = max(best_el, key);
           }
           if (SCORES) {
             if (SPV == 4)
@@ -382,12 +421,23 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
     } else {
       if (write_scores) scan(F{}, T{}); else scan(F{}, F{});
     }
-    uint32_t fin = block_max_key(best_all, wbest[0], lane, warp, NT / 32);
+    // Each warp reads the position of its own best slot while the block agrees on one of them: read once the victim was known, the
+    // evicted position ended every call with another trip to memory (64 ragged sequences 1.3 us).
+    const uint32_t best_w = __reduce_max_sync(0xFFFFFFFFu, best_all), best_we = prot ? __reduce_max_sync(0xFFFFFFFFu, best_el) : 0u;
+    const uint32_t cand = best_we != 0u ? best_we : best_w;  // (an eligible slot of this warp means that an eligible slot wins)
+    if (lane == 0) {
+      wbest[0][warp] = best_w;
+      if (prot) wbest[1][warp] = best_we;
+      if (a.evicted_pos_out != nullptr && cand != 0u) ev = __ldcg(pp + min((int)(kKeyIdxMask - (cand & kKeyIdxMask)), C - 1));
+    }
+    __syncthreads();
+    uint32_t fin = __reduce_max_sync(0xFFFFFFFFu, lane < NT / 32 ? wbest[0][lane] : 0u);
     if (prot) {
-      const uint32_t fin_el = block_max_key(best_el, wbest[1], lane, warp, NT / 32);
+      const uint32_t fin_el = __reduce_max_sync(0xFFFFFFFFu, lane < NT / 32 ? wbest[1][lane] : 0u);
       if (fin_el != 0u) fin = fin_el;
     }
     slot = (int)(kKeyIdxMask - (fin & kKeyIdxMask));
+    tail = lane == 0 && cand == fin;  // (keys differ between slots: one warp)
   }
 
   if (!evict) cp_async_wait_all();  // a unit that is still filling never looked at the copied table
@@ -405,9 +455,7 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
     char* dst = static_cast<char*>(is_k ? a.ca.k_cache : a.ca.v_cache) + slot_idx * d * es;
     reinterpret_cast<uint4*>(dst)[is_k ? tid : tid - cpr] = rowreg;
   }
-  if (tid == NT - 1) {
-    int ev = -1;
-    if (evict && a.evicted_pos_out != nullptr) ev = a.ca.pos[slot_idx];
+  if (tail) {
     a.ca.pos[slot_idx] = t;
     if (PACKED) {
       for (int i = 0; i < cb; ++i) reinterpret_cast<uint8_t*>(a.ca.codes)[slot_idx * cb + i] = (uint8_t)(codes_s[G] >> (8 * i));

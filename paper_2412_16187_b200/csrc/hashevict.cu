@@ -796,7 +796,7 @@ int he_decode_step(const he_config* cfg, const he_cache* cache, const void* q, c
   const int Wd = words_of(cfg->hash_bits);
   const int cb = packed_code_bytes(*cfg);  // 1..3 bytes per slot, or 0: word layout
   const long long nvec = cb ? ((long long)cfg->max_budget * cb + 15) / 16 : ((long long)cfg->max_budget * Wd + 3) / 4;
-  const size_t smem = (size_t)nvec * 16;
+  size_t smem = (size_t)nvec * 16;
   if (smem > 200 * 1024) return fail(HE_ERR_UNSUPPORTED, "max_budget %d with %d code words does not fit the decode kernel's shared memory", cfg->max_budget, Wd);
   int nt = 256;
   if (nvec > 2048) nt = 512;
@@ -818,6 +818,7 @@ int he_decode_step(const he_config* cfg, const he_cache* cache, const void* q, c
   a.evicted_pos_out = evicted_pos_out;
   a.qcodes_out = qcodes_out;
   a.n_budget16 = a.n_budget32 = a.n_sched = a.n_order = 0;
+  a.pos_at = 0;
   const bool mirror = cache->budget_host != nullptr && cfg->batch <= kBudgetVals;
   a.new_codes = nullptr;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -875,6 +876,16 @@ int he_decode_step(const he_config* cfg, const he_cache* cache, const void* q, c
     memcpy(a.budget32, cache->budget_host, sizeof(int32_t) * (size_t)cfg->batch);
   }
   const dim3 grid((unsigned)cfg->n_kv_heads, (unsigned)cfg->batch);
+  // With protected windows the scan wants every slot's position: they are copied beside a one-word code table where that leaves room
+  // for as many CTAs per SM as before (four of 256 threads beside 11 KB of static arrays each, one or two larger ones). 128 units of
+  // 1024 slots: 3.71 us a call in a graph without, 3.59 with (and two threads in place of one for each item of the projection).
+  if (!cb && Wd == 1 && (cfg->n_sink > 0 || cfg->n_recent > 0)) {
+    const size_t with_pos = smem + (size_t)cfg->max_budget * 4;
+    if (with_pos <= (nt == 256 ? 40 : 96) * 1024) {
+      a.pos_at = (int)(smem / 4);
+      smem = with_pos;
+    }
+  }
   if (cb) return launch_decode_g<1, true>(a, nt, smem, grid, st);
   return Wd == 1 ? launch_decode_g<1>(a, nt, smem, grid, st) : launch_decode_g<2>(a, nt, smem, grid, st);
 }
