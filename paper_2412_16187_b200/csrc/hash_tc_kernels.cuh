@@ -68,13 +68,6 @@ __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
     if (mbar_try_wait(bar, parity)) return;
 }
 
-// The same on two barriers, whose first polls overlap.
-__device__ __forceinline__ bool mbar_wait2(uint32_t bar_a, uint32_t parity_a, uint32_t bar_b, uint32_t parity_b, volatile int* abort_flag) {
-  const bool a = mbar_try_wait(bar_a, parity_a), b = mbar_try_wait(bar_b, parity_b);
-  if (a && b) return true;
-  return (a || mbar_wait(bar_a, parity_a, abort_flag)) && (b || mbar_wait(bar_b, parity_b, abort_flag));
-}
-
 // Bounded waits of a whole warp, with one answer for all of it. The first poll stands outside the loop, in straight code that votes
 // once: a completed phase costs 24 cycles that way, where the loop with its vote behind it costs 102 (164 on two barriers).
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
@@ -115,6 +108,17 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t tmem_d, uint64_t adesc, uin
       : "memory");
 }
 // 32 consecutive fp32 columns of this thread's tensor-memory lane
+// One lane of a converged warp.
+__device__ __forceinline__ bool tc_elect() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xFFFFFFFF;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -464,8 +468,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const __gri
     cp_async_wait_all();
     while (published < it) publish();
   } else if (warp == 5) {
-    // ------------------------------------------------------------------ MMA issue (one thread)
-    if (lane == 0) {
+    // ------------------------------------------------------------------ MMA issue (one elected lane of a warp-uniform loop)
+    // (from a divergent thread an instruction takes 90 cycles to issue, eight of them as long as they run at 64 bits: 2 M rows of 128
+    // channels 109.4 us a call that way, 102.8 this way; 90.6 at 32 bits either way)
+    {
       const uint32_t idesc = (1u << 4) /* fp32 accumulate */ | (1u << 7) /* A bf16 */ | (1u << 10) /* B bf16 */ |
                              ((uint32_t)(kAccCols >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
       const uint64_t b_desc0 = umma_desc_k128(smem_u32(Bs));
@@ -479,28 +485,31 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const __gri
         }
         const int s = it % kTcStages, acc = it & 1;
         // the epilogue has drained this accumulator and the stage's rows have landed
-        if (!mbar_wait2(tempty_bar(acc), ((it >> 1) & 1) ^ 1, full_bar(s), (it / kTcStages) & 1, &abort_flag)) break;
+        if (!mbar_wait2_warp(tempty_bar(acc), ((it >> 1) & 1) ^ 1, full_bar(s), (it / kTcStages) & 1, &abort_flag)) break;
         tc_fence_after();
         // Descriptors differ only in their 14-bit start-address field, so each MMA's pair is the tile's base
-        // descriptor plus a small constant: the issuing thread spends a few instructions per MMA, not dozens.
+        // descriptor plus a small constant.
         const uint64_t a_desc0 = umma_desc_k128(smem_u32(As + s * a_stage_bytes));
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kAccCols);
+        if (tc_elect()) {
 #pragma unroll
-        for (int kh = 0; kh < 2; ++kh) {
-          if (kh < KH) {
+          for (int kh = 0; kh < 2; ++kh) {
+            if (kh < KH) {
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks)  // K = 16 bf16 = 32 bytes per instruction inside the 128-byte swizzle span
-              tc_mma_bf16(d_tmem, a_desc0 + (uint64_t)((kh * (kTcRows * 128) + ks * 32) >> 4),
-                          b_desc0 + (uint64_t)((kh * 3 * (N * 128) + ks * 32) >> 4), idesc, !(kh == 0 && ks == 0));
+              for (int ks = 0; ks < 4; ++ks)  // K = 16 bf16 = 32 bytes per instruction inside the 128-byte swizzle span
+                tc_mma_bf16(d_tmem, a_desc0 + (uint64_t)((kh * (kTcRows * 128) + ks * 32) >> 4),
+                            b_desc0 + (uint64_t)((kh * 3 * (N * 128) + ks * 32) >> 4), idesc, !(kh == 0 && ks == 0));
+            }
           }
+          tc_commit(empty_bar(s));    // the stage may be refilled once these MMAs have read it
+          tc_commit(tfull_bar(acc));  // and the accumulator is complete
         }
-        tc_commit(empty_bar(s));    // the stage may be refilled once these MMAs have read it
-        tc_commit(tfull_bar(acc));  // and the accumulator is complete
+        __syncwarp();
         ++it;
       }
-      // ... nor free tensor memory under an MMA that is still writing it: one more commit tracks everything this thread
-      // has issued, and its completion is awaited (bounded) before the CTA goes on to the deallocation.
-      if (abort_flag) {
+      // ... nor free tensor memory under an MMA that is still writing it: one more commit tracks everything that was
+      // issued, and its completion is awaited (bounded) before the CTA goes on to the deallocation.
+      if (abort_flag && tc_elect()) {
         tc_commit(drain_bar);
         mbar_drain(drain_bar, 0);
       }

@@ -450,6 +450,8 @@ const SchedCache& sched_of(const int32_t* budget_host, int n, int cmax) {
   return c;
 }
 
+// The CUDA-core replay kernels have several CTAs on an SM. Launched programmatically behind the hashing kernel, which leaves room for
+// them on the SMs where it ends first, they crowd there: only a grid of at most one CTA per SM is.
 template <int WORDS, int GT>
 int launch_replay_smem(const ReplayArgs& a, long long units, cudaStream_t stream) {
   const size_t smem = (size_t)a.cfg.max_budget * (WORDS + 1) * 4;
@@ -458,7 +460,9 @@ int launch_replay_smem(const ReplayArgs& a, long long units, cudaStream_t stream
   if (a.cfg.max_budget > 4096) nt = 512;
   if (a.cfg.max_budget > 16384) nt = 1024;
   if (int rc = set_smem(prefill_replay_smem_kernel<WORDS, GT>, smem)) return rc;
-  return launch_pdl(prefill_replay_smem_kernel<WORDS, GT>, dim3((unsigned)units), nt, smem, true, stream, a);
+  int sms = 0;
+  if (int rc = sm_count(&sms)) return rc;
+  return launch_pdl(prefill_replay_smem_kernel<WORDS, GT>, dim3((unsigned)units), nt, smem, units <= sms, stream, a);
 }
 
 // The register kernel is persistent: as many CTAs as fit the GPU at once, each claiming units from the schedule.
@@ -480,7 +484,7 @@ int launch_replay_reg_one(const ReplayArgs& a, long long units, cudaStream_t str
   if (int rc = launch_pdl(prefill_schedule_kernel, dim3(1), kSchedThreads, 0, a.Nmax > 0, stream, a.cfg, a.ca.budget, a.prompt_len, nbins, a.sched, 0)) return rc;
   long long grid = (long long)sms * per_sm;
   if (grid > units) grid = units;
-  return launch_pdl(prefill_replay_reg_kernel<WORDS, GT, SPT, NT>, dim3((unsigned)grid), NT, smem, true, stream, a);
+  return launch_pdl(prefill_replay_reg_kernel<WORDS, GT, SPT, NT>, dim3((unsigned)grid), NT, smem, grid <= sms, stream, a);
 }
 
 // Smallest (threads x slots-per-thread) tile of the register kernel that holds max_budget slots.

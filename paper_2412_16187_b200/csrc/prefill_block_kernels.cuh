@@ -187,16 +187,6 @@ __device__ __forceinline__ void rb_ld64_low(uint32_t taddr, uint32_t (&v)[32]) {
 // operands, so that one shift and one logic operation expand four bits. Set: +2 (e4m3 0x40), clear: -2 (0xC0).
 __device__ __forceinline__ uint32_t rb_expand4(uint32_t h, int m) { return lop3<0x6A>(h << (7 - m), 0x80808080u, 0xC0C0C0C0u); }
 
-__device__ __forceinline__ bool rb_elect() {
-  uint32_t p;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "elect.sync _|p, 0xFFFFFFFF;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(p));
-  return p != 0;
-}
-
 // The ranks of a block's own keys at its steps: step r only needs those of the r steps before it, so steps 64 + k and 63 - k
 // share a row (64 + k entries from its start, 63 - k from the next multiple of four). Blocks of 64 have a row each.
 __device__ __forceinline__ int rb_dn_at(int r, int rows_max) {
@@ -648,7 +638,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         if (!mbar_wait2_warp(afree_bar(acc), ph ^ 1, full_bar(sx), px, &abort_flag)) return;
         tc_fence_after();
         const uint64_t ad = a_desc_of(buf), bd = b_desc_of(sx, 0);
-        if (rb_elect()) {
+        if (tc_elect()) {
 #pragma unroll
           for (int w = 0; w < WORDS; ++w)
             rb_mma_f8(tmem_base + (uint32_t)(2 * acc * kRbTile), ad + (uint64_t)(2 * w), bd + (uint64_t)(2 * w), idesc, w > 0);
@@ -807,7 +797,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             const uint64_t x1 = x_desc + (uint64_t)(i + 1 == last_i ? 4 : 0);
             if (!mbar_wait2_warp(afree_bar(acc), ph ^ 1, full_bar(sx), stage_phase(n), &abort_flag)) break;
             tc_fence_after();
-            if (rb_elect()) {
+            if (tc_elect()) {
               const uint32_t d = tmem_base + (uint32_t)(2 * acc * kRbTile);
 #pragma unroll
               for (int w = 0; w < WORDS; ++w) rb_mma_f8(d, a_desc + (uint64_t)(2 * w), bd + (uint64_t)(2 * w), idesc, w > 0);
@@ -822,7 +812,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             }
             __syncwarp();
           }
-          if (abuf == 1 && rb_elect()) tc_commit(adone_bar);
+          if (abuf == 1 && tc_elect()) tc_commit(adone_bar);
           __syncwarp();
         }
         if (tn < N) {  // the next block: its codes and operand A (warps 14-15, meanwhile), its own keys' ranks (all four)
@@ -1125,7 +1115,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   // A CTA that gave up must not free tensor memory under an MMA that is still writing it (the operands are written by
   // this CTA's own threads, so no copy from outside is ever in flight): one more commit of each MMA warp tracks everything
   // it has issued, and their completion is awaited (bounded) first.
-  if (abort_flag && (warp == kRbMmaWarp || warp == kRbMmaWarp + 1) && rb_elect()) {
+  if (abort_flag && (warp == kRbMmaWarp || warp == kRbMmaWarp + 1) && tc_elect()) {
     tc_commit(drain_bar);
     mbar_drain(drain_bar, 0);
   }
