@@ -1,6 +1,7 @@
 """The block replay at both ends of what its 16-bit tile keys hold and on both sides of where its owner table changes from words to
 bytes: the largest ranks (odd groups of two-word codes, groups of eight), codes of a few bits (most keys tie, and recent tokens hold
-best slots), and tables just within and just beyond the word table's limit, against the oracle, bit for bit."""
+best slots), tables just within and just beyond the word table's limit, and few-bit codes of more units than SMs, against the
+oracle, bit for bit."""
 import pytest
 
 from cases import C
@@ -19,6 +20,9 @@ SHAPES = {
     "bytes_6148": base.scaled(n_kv_heads=1, hash_bits=32, budget=6148, prompt_len=6500, n_sink=4, n_recent=10),
     "two_words_4096": base.scaled(n_kv_heads=1, budget=4096, prompt_len=4500),
     "two_words_4100": base.scaled(n_kv_heads=1, budget=4100, prompt_len=4500),
+    # more units than SMs: few-bit codes stay on the CUDA-core kernels, launched plainly behind the hashing
+    "few_bits_over_sms": base.scaled(batch=10, n_kv_heads=16, hash_bits=8, group_size=2, budget=400, prompt_len=520, head_dim=64),
+    "one_head_groups_over_sms": base.scaled(batch=10, n_kv_heads=16, hash_bits=16, group_size=1, budget=390, prompt_len=520, head_dim=64),
 }
 
 
