@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
       if (write_scores) scan(F{}, T{}); else scan(F{}, F{});
     }
     // Each warp reads the position of its own best slot while the block agrees on one of them: read once the victim was known, the
-    // evicted position ended every call with another trip to memory (64 ragged sequences 1.3 us).
+    // evicted position ended every call with another trip to memory.
     const uint32_t best_w = __reduce_max_sync(0xFFFFFFFFu, best_all), best_we = prot ? __reduce_max_sync(0xFFFFFFFFu, best_el) : 0u;
     const uint32_t cand = best_we != 0u ? best_we : best_w;  // (an eligible slot of this warp means that an eligible slot wins)
     if (lane == 0) {

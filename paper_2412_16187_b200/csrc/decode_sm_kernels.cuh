@@ -441,7 +441,6 @@ __global__ void __launch_bounds__(kSmThreads, 2) decode_step_sm_kernel(const Dec
   const bool write_scores = (flags & HE_FLAG_WRITE_SCORES) != 0;
   constexpr uint32_t kKeyBase = (1u << kKeyIdxBits) + kKeyIdxMask;  // key = (rank << 20) + kKeyBase - slot
   uint32_t rpos = 0;  // ring position of the next vector to consume
-  int wpos[kSmUnits] = {-1, -1, -1, -1};  // lane 0: position of the warp's best slot of each unit
   auto scan = [&](auto prot_c, auto scores_c) {
     constexpr bool PROT = decltype(prot_c)::value, SCORES = decltype(scores_c)::value;
 #pragma unroll
@@ -536,10 +535,6 @@ __global__ void __launch_bounds__(kSmThreads, 2) decode_step_sm_kernel(const Dec
       if (lane == 0) {
         wbest[0][i][warp] = best_all;
         if (PROT) wbest[1][i][warp] = best_el;
-        // the position of this warp's best slot, in case it is the unit's: read once the victim is known, the evicted position ended
-        // every call with another trip to memory
-        const uint32_t cand = PROT && best_el != 0u ? best_el : best_all;
-        if (su[i].evpos_p != nullptr && cand != 0u) wpos[i] = __ldcg(su[i].pp + min((int)(kKeyIdxMask - (cand & kKeyIdxMask)), C - 1));
       }
     }
   };
@@ -554,15 +549,7 @@ __global__ void __launch_bounds__(kSmThreads, 2) decode_step_sm_kernel(const Dec
   __syncthreads();
 
   // ---- Algorithm 1 lines 2-5: warp i finishes unit i; the slot takes the new token's K, V, code and position
-  auto best_of = [&](int i) {  // the unit's best key
-    uint32_t fin = __reduce_max_sync(0xFFFFFFFFu, lane < NW ? wbest[0][i][lane] : 0u);
-    if (prot) {
-      const uint32_t fin_el = __reduce_max_sync(0xFFFFFFFFu, lane < NW ? wbest[1][i][lane] : 0u);
-      if (fin_el != 0u) fin = fin_el;
-    }
-    return fin;
-  };
-  auto finish = [&]() {
+  if (warp < n_mine) {
     const int i = warp;
     int fill = 0, t = 0;
 #pragma unroll
@@ -579,7 +566,14 @@ __global__ void __launch_bounds__(kSmThreads, 2) decode_step_sm_kernel(const Dec
     }
     const bool evict = fill >= C;
     int slot = min(fill, Cmax - 1);
-    if (evict) slot = min((int)(kKeyIdxMask - (best_of(i) & kKeyIdxMask)), C - 1);  // (the clamp never acts on a scored table)
+    if (evict) {
+      uint32_t fin = __reduce_max_sync(0xFFFFFFFFu, lane < NW ? wbest[0][i][lane] : 0u);
+      if (prot) {
+        const uint32_t fin_el = __reduce_max_sync(0xFFFFFFFFu, lane < NW ? wbest[1][i][lane] : 0u);
+        if (fin_el != 0u) fin = fin_el;
+      }
+      slot = min((int)(kKeyIdxMask - (fin & kKeyIdxMask)), C - 1);  // (the clamp never acts on a scored table)
+    }
     if (!HE_IN_RANGE(slot, C)) return;
     const size_t row_bytes = (size_t)cpr * 16;
     for (int c = lane; c < 2 * cpr; c += 32) {
@@ -588,6 +582,8 @@ __global__ void __launch_bounds__(kSmThreads, 2) decode_step_sm_kernel(const Dec
       reinterpret_cast<uint4*>(dst)[is_k ? c : c - cpr] = kvs[i * 2 * cpr + c];
     }
     if (lane == 0) {
+      int ev = -1;
+      if (evict && u.evpos_p != nullptr) ev = __ldcg(u.pp + slot);
       u.pp[slot] = t;
 #pragma unroll
       for (int w = 0; w < WORDS; ++w) u.codes_p[(size_t)slot * WORDS + w] = codes_s[i][G * WORDS + w];
@@ -597,16 +593,7 @@ __global__ void __launch_bounds__(kSmThreads, 2) decode_step_sm_kernel(const Dec
       }
       *u.npos_p = t + 1;
       *u.victim_p = slot;
-      if (!evict && u.evpos_p != nullptr) *u.evpos_p = -1;
-    }
-  };
-  if (warp < n_mine) finish();
-  if (su[0].evpos_p != nullptr) {  // (all units or none) the warp that found a unit's victim has its position
-#pragma unroll
-    for (int i = 0; i < kSmUnits; ++i) {
-      if (i >= n_mine) break;
-      const uint32_t fin = best_of(i);
-      if (lane == 0 && fin != 0u && (wbest[0][i][warp] == fin || (prot && wbest[1][i][warp] == fin))) *su[i].evpos_p = wpos[i];
+      if (u.evpos_p != nullptr) *u.evpos_p = ev;
     }
   }
 }
