@@ -509,7 +509,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) hash_rows_tc_kernel(const __gri
       }
       // ... nor free tensor memory under an MMA that is still writing it: one more commit tracks everything that was
       // issued, and its completion is awaited (bounded) before the CTA goes on to the deallocation.
-      if (abort_flag && tc_elect()) {
+      const bool gave_up = __any_sync(0xFFFFFFFFu, abort_flag != 0);  // one answer for the warp: the election wants all its lanes
+      if (gave_up && tc_elect()) {
         tc_commit(drain_bar);
         mbar_drain(drain_bar, 0);
       }

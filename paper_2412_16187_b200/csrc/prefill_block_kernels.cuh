@@ -1115,9 +1115,12 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   // A CTA that gave up must not free tensor memory under an MMA that is still writing it (the operands are written by
   // this CTA's own threads, so no copy from outside is ever in flight): one more commit of each MMA warp tracks everything
   // it has issued, and their completion is awaited (bounded) first.
-  if (abort_flag && (warp == kRbMmaWarp || warp == kRbMmaWarp + 1) && tc_elect()) {
-    tc_commit(drain_bar);
-    mbar_drain(drain_bar, 0);
+  if (warp == kRbMmaWarp || warp == kRbMmaWarp + 1) {
+    const bool gave_up = __any_sync(0xFFFFFFFFu, abort_flag != 0);  // one answer for the warp: the election wants all its lanes
+    if (gave_up && tc_elect()) {
+      tc_commit(drain_bar);
+      mbar_drain(drain_bar, 0);
+    }
   }
   tc_fence_before();
   __syncthreads();
