@@ -124,12 +124,14 @@ int he_hash_keys(const he_config* cfg, const void* x, int64_t rows, int64_t row_
  * are left untouched and report victim -1.
  *
  * Ordering against earlier work of the stream. The kernel is launched with the programmatic-serialization attribute,
- * so it may start while the stream's previous kernel is still running. By default it reads only W (which must not
- * change while the cache is in use) before it waits for that kernel to finish; q, k, v may therefore be produced by
- * the kernel enqueued just before this call. With HE_FLAG_EARLY_INPUTS the call also reads q, k, v and hashes them
- * (Eq. 2) BEFORE that wait, so that this work overlaps the previous call's scan: consecutive decode calls (say, the
+ * so it may start while the stream's previous kernel is still running. By default only W (which must not change while
+ * the cache is in use) is read for good before it waits for that kernel to finish; without budget_host it also looks at
+ * `budget` then, as a hint of how much of the code table to ask into L2, and reads it again afterwards. q, k, v - and
+ * the budgets of a call without budget_host - may therefore be written by the kernel enqueued just before this call.
+ * With HE_FLAG_EARLY_INPUTS the call also reads q, k, v (and those budgets) and hashes the rows (Eq. 2) BEFORE that
+ * wait, so that this work overlaps the previous call's scan: consecutive decode calls (say, the
  * caches of a model's layers one after another, or one cache step after step) then run about twice as fast. The
- * caller promises in exchange that q, k, v were completely written before this call was ENQUEUED on the stream's
+ * caller promises in exchange that they were completely written before this call was ENQUEUED on the stream's
  * device timeline - by work the host has synchronised with, or by work ordered before everything still pending in
  * the stream (inputs staged ahead of a run of calls, or a captured graph whose inputs are final before it is
  * launched). If the rows are produced by a kernel enqueued shortly before the call, leave the flag off. Results are
@@ -171,7 +173,8 @@ size_t he_workspace_bytes(const he_config* cfg, int32_t max_prompt_len);
  * over the valid slots j < fill of unit (s, h). q: [B, Hkv*G, d] in the dtype of cfg (contiguous); out: [B, Hkv*G, d]
  * fp32. Products of bf16 inputs are exact; sums and the softmax are carried in fp32 (exp2 of scaled scores, running
  * maximum), so results agree with exact arithmetic to about 1e-5 of the largest |V| entry. A unit without valid
- * slots gives zeros. The cache is only read.
+ * slots gives zeros. The cache is only read. The kernel may start while the stream's previous kernel is still running; all it
+ * does with the cache before that one has finished is to ask first rows into L2, sized by a look at `fill` that it repeats.
  */
 int he_attend(const he_config* cfg, const he_cache* cache, const void* q, float* out, void* stream);
 

@@ -278,8 +278,9 @@ __device__ __forceinline__ void l2_prefetch_bulk(const void* gmem, uint32_t byte
 }
 
 // Programmatic dependent launch: a kernel launched with the programmatic-serialization attribute may start while
-// the previous kernel of the stream is still draining. Everything that touches memory another kernel may have
-// written comes after griddep_wait(); only W (read-only while a cache is in use) is read before it.
+// the previous kernel of the stream is still draining. Everything whose value counts and that another kernel may have
+// written is read after griddep_wait(); before it come W (read-only while a cache is in use), prefetches into L2, and reads past L1
+// that only size those (budget, fill) and are made again after it.
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

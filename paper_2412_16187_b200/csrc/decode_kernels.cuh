@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
   // Only the kernel of the largest packed tables looks for 32-bit budgets: the third source costs the others 1 to 5 %.
   constexpr bool kWide = PACKED && NT == 1024 && !PRE;
   auto budget_of = [&]() {
-    return clamp_budget(a.n_budget16 > 0 ? (int)a.budget16[s] : (kWide && a.n_budget32 > 0 ? a.budget32[s] : a.ca.budget[s]), Cmax);
+    return clamp_budget(a.n_budget16 > 0 ? (int)a.budget16[s] : (kWide && a.n_budget32 > 0 ? a.budget32[s] : __ldcg(a.ca.budget + s)), Cmax);
   };
   const int cb = PACKED ? (b + 7) >> 3 : 0;
   auto vecs_of = [&](int c) { return PACKED ? (c * cb + 15) / 16 : (c * WORDS + 3) / 4; };
@@ -123,8 +123,8 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
                   : reinterpret_cast<const uint4*>(a.ca.codes + (size_t)unit * Cmax * WORDS);
   };
   if (!PRE) {
-    // The table comes to L2 under the previous kernel's tail (budgets do not change while a cache is in use, and a prefetch returns no
-    // data, so it cannot see a stale code).
+    // The table comes to L2 under the previous kernel's tail (a prefetch returns no data, so it cannot see a stale code). The budget is
+    // a hint here: one from device memory is read again below, past L1, since that kernel may be writing it.
     if (tid == 0) {
       const int n = vecs_of(budget_of());
       if (n > 0) l2_prefetch_bulk(table_of(), (uint32_t)n * 16u);

@@ -122,6 +122,36 @@ def test_bf16_decode_from_an_empty_cache_matches_prefill_up_to_fragile_bits():
             assert torch.equal(getattr(a.gpu, n), getattr(b.gpu, n)), n
 
 
+@pytest.mark.parametrize("bits", [32, 64])
+def test_budgets_written_by_the_kernel_before_a_step_count_in_that_step(bits):
+    """Without a host mirror `budget` is read on the device, first as the hint that sizes a prefetch while the stream's earlier
+    kernels still run. Budgets that a kernel changes between steps of one queue give what the same steps give one by one."""
+    w = PARITY_CASES["llama3_8b_gqa"].scaled(batch=2, prompt_len=1200, budget=600, hash_bits=bits, decode_steps=12)
+    case = Case(w)
+    W, plans = torch.from_numpy(case.W), [600, 64, 301, 5] * 3
+    dq, dk, dv = (to_dev(wl.gen_decode_inputs(w, x, 0, 12), w) for x in "qkv")
+    scale = torch.tensor([[n, n] for n in plans], dtype=torch.int32, device="cuda")
+
+    def steps(one_by_one):
+        c = HashEvictCache(2, w.n_kv_heads, w.group_size, w.head_dim, bits, w.budgets(), W, dtype=torch.bfloat16, host_budget_mirror=False)
+        c.prefill_compress(case.dQ, case.dK, case.dV, case.dplen)
+        torch.cuda.synchronize()
+        out = []
+        if not one_by_one:
+            torch.cuda._sleep(3_000_000)  # the host gets ahead: the steps follow one another without a gap
+        for i in range(12):
+            torch.mul(scale[i], 1, out=c.budget)
+            if one_by_one:
+                torch.cuda.synchronize()
+            out.append(c.decode_step(dq[i], dk[i], dv[i]))
+        torch.cuda.synchronize()
+        return [torch.stack(out)] + [getattr(c, n) for n in STATE]
+
+    for name, x, y in zip(("victims",) + STATE, steps(True), steps(False)):
+        assert torch.equal(x, y), name
+    assert all((v < n).all() for v, n in zip(steps(False)[0], plans))
+
+
 DEBUG_SCRIPT = r"""
 import sys
 sys.path.insert(0, %r); sys.path.insert(0, %r)
