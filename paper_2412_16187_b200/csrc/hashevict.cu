@@ -35,6 +35,7 @@
 #include "oneshot_kernels.cuh"
 #include "prefill_block_kernels.cuh"
 #include "prefill_kernels.cuh"
+#include "replay_rule.h"
 
 using namespace he;
 
@@ -637,21 +638,7 @@ int launch_replay(const ReplayArgs& a, long long units, cudaStream_t stream) {
   int sms = 0;
   if (int rc = sm_count(&sms)) return rc;
   const int mode = block_replay_mode();
-  // The block kernel has one CTA per SM and pays a block's settling (8000 cycles) whatever the budget; the CUDA-core kernels
-  // scan every slot at every step, several units per SM. Measured on B200 (us with CUDA cores / block kernel): up to one unit per SM
-  // the block kernel is ahead from the smallest budgets where the register kernel exists (64 slots, G = 4, b = 32, N = 2 C: 38 / 31)
-  // and from 128 slots where it does not (G = 8, b = 64: 66 / 53). With more units they cross between 256 and 512 slots, sooner or
-  // later with the keys (320 units, b = 32, G = 4, N = 2.5 C: 411 / 418 at 512 slots on clustered keys, 410 / 316 on drifting ones),
-  // sooner with two code words and G = 4 (N = 3 C: 250 / 253 at 160, 336 / 302 at 224). Codes of few bits have few distinct distances,
-  // so that steps keep meeting in the same slots and a block needs more passes: clustered / drifting / independent keys of 320 units at
-  // N = 2.5 C, b = 8, G = 4 take 2094 us at 2048 slots and 5781 / 4482 / 4410; G = 2 5970 and 8623 / 7101 / 7435; b = 16, G = 1 584 at
-  // 1024 slots and 1019 / 561 / 480, 1510 at 2048 and 2612 / 966 / 717.
-  const bool has_reg = a.cfg.group_size == 1 || a.cfg.group_size == 4;
-  const int distances = a.cfg.group_size * a.cfg.hash_bits;
-  int min_budget = WORDS == 2 && a.cfg.group_size == 4 ? 256 : 384;
-  if (units <= sms) min_budget = has_reg ? 1 : 128;
-  else if (a.cfg.hash_bits <= 8 && distances <= 32) min_budget = has_reg ? 4096 : 2560;
-  else if (distances <= 16) min_budget = 2048;
+  const int min_budget = block_replay_min_budget(WORDS, a.cfg.group_size, a.cfg.hash_bits, units, sms);
   bool block_ok = mode != 0 && (mode == 2 || a.cfg.max_budget >= min_budget) && a.cfg.max_budget <= kRbMaxSlots &&
                   rb_fit(WORDS, slots, a.cfg.group_size, 1, WORDS == 2 ? kRbHalf : kRbFull, &fit) != 0;
   if (block_ok && (a.cfg.n_sink > 0 || a.cfg.n_recent > 0)) {

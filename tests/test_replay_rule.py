@@ -1,0 +1,41 @@
+"""The line between the CUDA-core replays and the block replay for codes of few bits (csrc/replay_rule.h) against measured calls: 320 units
+on 148 SMs, prompts 2.5 times the budget, us on CUDA cores and of the block kernel on clustered, drifting and independent keys. A
+shape goes to the kernel that is ahead over the three kinds of keys together."""
+import math
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2412_16187_b200", "csrc")
+# (bits, group, slots): CUDA cores, (block kernel on clustered, drifting, independent keys)
+MEASURED = {
+    (16, 1, 512): (362, (518, 333, 305)), (16, 1, 1024): (632, (976, 571, 524)), (16, 1, 1536): (1281, (1849, 731, 614)),
+    (16, 1, 2044): (1595, (2379, 940, 791)), (12, 1, 1024): (632, (1279, 656, 544)), (12, 1, 1536): (1280, (2545, 957, 677)),
+    (8, 1, 1024): (632, (1769, 1023, 676)), (8, 1, 3072): (2953, (7115, 3966, 2067)), (8, 4, 3072): (4530, (8945, 6513, 6823)),
+    (8, 2, 2048): (6060, (8539, 6927, 7522)), (8, 2, 3072): (12632, (12810, 10539, 11364)), (5, 3, 2048): (6130, (10146, 8149, 6094)),
+    (5, 3, 3072): (12764, (16320, 12292, 9276)), (4, 4, 1024): (792, (2731, 2826, 2606)),
+}
+PROGRAM = """
+#include <cstdio>
+#include <cstdlib>
+#include "replay_rule.h"
+int main(int argc, char** argv) {
+  for (int i = 1; i + 1 < argc; i += 2) std::printf("%d ", he::block_replay_min_budget(1, std::atoi(argv[i + 1]), std::atoi(argv[i]), 320, 148));
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lines(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rule")
+    (d / "t.cpp").write_text(PROGRAM)
+    subprocess.run(["g++", "-std=c++17", "-I", CSRC, "-o", d / "t", d / "t.cpp"], check=True)
+    out = subprocess.run([d / "t"] + [str(x) for k in MEASURED for x in k[:2]], capture_output=True, text=True, check=True).stdout.split()
+    return dict(zip(MEASURED, map(int, out)))
+
+
+@pytest.mark.parametrize("shape", list(MEASURED))
+def test_few_bit_shapes_go_to_the_kernel_that_is_ahead(shape, lines):
+    cores, block = MEASURED[shape]
+    assert (shape[2] >= lines[shape]) == (math.prod(block) < cores ** 3)
