@@ -20,12 +20,16 @@ namespace he {
 //   b = 12, G = 1   1024 slots 632 / 1279, 656, 544       1536 slots 1280 / 2545, 957, 677
 //   b = 16, G = 1   768 slots 523 / 742, 448, 407         1024 slots 632 / 976, 571, 524       1536 slots 1281 / 1849, 731, 614
 // (a thread of the register kernel holds four slots up to 1024 and eight beyond, which doubles its time there).
+// The block kernel's time goes with the rounds of units on the SMs, the others' less so: up to two units per SM codes of 13 to 16
+// distances are ahead from the smaller tables on (1024 slots, b = 16, G = 1: 160 units 503 / 682, 368, 339, 296 units 550 / 830, 436, 395,
+// 448 units 771 / 1208, 738, 682, 592 units 823 / 1530, 831, 763; 512 slots: 160 units 284 / 357, 215, 195, 592 units 486 / 826, 492, 443),
+// those of 12 are level (160 units 503 / 863, 432, 351, 296 units 551 / 1045, 497, 413) and stay with the line.
 inline int block_replay_min_budget(int words, int group_size, int hash_bits, long long units, int sms) {
   const bool has_reg = group_size == 1 || group_size == 4;  // group sizes with a register kernel
   const int distances = group_size * hash_bits;
   if (units <= sms) return has_reg ? 1 : 128;
   if (hash_bits <= 8 && distances <= 32) return has_reg ? 4096 : 2560;
-  if (distances <= 16) return 1025;
+  if (distances <= 16 && (distances <= 12 || units > 2LL * sms)) return 1025;
   return words == 2 && group_size == 4 ? 256 : 384;
 }
 
