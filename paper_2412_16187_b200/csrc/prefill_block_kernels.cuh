@@ -87,6 +87,16 @@ constexpr int kRbAtom = 128 * 128;       // 128 operand rows x one 128-byte swiz
 constexpr int kRbDnPitch = 136;          // 16-bit entries between rows of the new-entry table
 constexpr int kRbDnPitchHalf = 68;       // ... when blocks have at most 64 steps
 constexpr int kRbMaxStages = 4;          // pairs of operand tiles
+constexpr int kRbStaticSmem = 512;       // bytes kept back for the kernel's static arrays
+// Eras of the owner table of words: the passes of a unit go from the first one down, 256 apart, and start again at a block that finds
+// the last one behind it (a block uses a hundred or two, so none reaches the walk's mark of zero). The bounds-checking build starts over
+// every few blocks, so that its tests pass there.
+#ifdef HE_BOUNDS_CHECK
+constexpr uint32_t kRbFirstEra = 0x22800u;
+#else
+constexpr uint32_t kRbFirstEra = 0xFFFFFE00u;
+#endif
+constexpr uint32_t kRbLastEra = 0x20000u;
 
 // Byte offsets of the kernel's dynamic shared memory (after rounding its base up to 1024 bytes). Tile maxima: per CTA of the
 // cluster one block of keys, a row for each step, an odd number of words apart (a warp stores a column, a lane per
@@ -397,6 +407,8 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   __shared__ int s_unit[2];
   __shared__ int s_change[2];                    // by pass parity: first step that changed
   __shared__ __align__(4) uint8_t s_hard[2][4];  // by pass parity: lengths of warps 0-3's lists of hard steps
+  static_assert(sizeof(bars) + sizeof(tmem_base_s) + sizeof(abort_flag) + sizeof(s_unit) + sizeof(s_change) + sizeof(s_hard) <= kRbStaticSmem,
+                "the host sizes the dynamic shared memory beside these");
 
   griddep_launch_dependents();
   const ReplayArgs& a = ar.r;
@@ -530,7 +542,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
     for (int j = rank * NT + tid; j < (int)Cmax; j += ncta * NT) pos_g[j] = j < fill0 ? j : -1;
     if (wide)
       for (int j = tid; j < nbase * kRbTile; j += NT) own32[j] = 0xFFFFFFFFu;
-    uint32_t era = 0xFFFFFE00u;  // wide: claims of the current pass are era | step, of earlier ones larger
+    uint32_t era = kRbFirstEra;  // wide: claims of the current pass are era | step, of earlier ones larger
     if (PROT && tid < Rn) REC[tid] = C - 1 - tid;  // (the first C tokens sit in slot = position)
     // Further columns of operand B (columns of A: 16, 1, 2^15, off, -64 parity): digits of 128 - x, 256, 1, 1; rows that may not win
     // have 256 alone. Variant bit 0: the tile holds the protected first tokens, bit 1: the budget ends inside the tile.
@@ -839,9 +851,9 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         tc_fence_before();
         const int r = tid;  // warps 0-3: this thread's step
         era -= 256u;
-        if (wide && __builtin_expect(era < 0x20000u, 0)) {  // (16 million passes on)
+        if (wide && __builtin_expect(era < kRbLastEra, 0)) {  // (16 million passes on)
           for (int j = tid; j < nbase * kRbTile; j += kRbResThreads) own32[j] = 0xFFFFFFFFu;
-          era = 0xFFFFFE00u;
+          era = kRbFirstEra;
           rb_bar<2, kRbResThreads>();
         }
         const bool mine = tid < rows;
