@@ -62,7 +62,9 @@ __device__ __forceinline__ float neg_small_int(int D) { return 8388608.0f - __ui
 // PACKED = true (HE_FLAG_PACKED_CODES with fewer bytes per slot than the word layout; WORDS = 1): the table holds
 // cb = ceil(b/8) bytes per slot, 1 to 3. A thread takes four consecutive slots (cb words) at a time, widens each code
 // to a word in registers and scores it like a word-layout slot.
-template <int WORDS, int GT, int NT, bool PRE, bool PACKED = false>
+//
+// SPLIT = false: the rows of a one-word step are projected by as many threads as there are work items (launch_decode_nt has the rule).
+template <int WORDS, int GT, int NT, bool PRE, bool PACKED = false, bool SPLIT = true>
 __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_step_kernel(const DecodeArgs a) {
   static_assert(!PACKED || WORDS == 1, "packed tables hold codes of at most 24 bits");
   constexpr int SPV = 4 / WORDS;  // slots per 16-byte vector
@@ -94,7 +96,7 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? (PRE ? 6 : 4) : 1)) decode_st
   const bool dense = !PRE && nitems <= NT && R <= kRowBatch && cpr <= 32;  // one item per thread, one pass, one chunk per lane
   float wreg[kChunk];
   // Where there are twice as many threads as work items, the upper half takes rows 3 and 4 (a row's sum is in the same order).
-  const bool halves = WORDS == 1 && 2 * nitems <= NT && (nitems & (nitems - 1)) == 0;
+  const bool halves = SPLIT && WORDS == 1 && 2 * nitems <= NT && (nitems & (nitems - 1)) == 0;
   const int item = halves ? tid & (nitems - 1) : tid, row0 = halves && tid >= nitems ? 3 : 0;
   const bool hashes = dense && tid < (halves ? 2 * nitems : nitems) && row0 < R;
   if (hashes) {

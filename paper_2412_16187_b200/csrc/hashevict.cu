@@ -352,9 +352,10 @@ int launch_hash(const HashJob& job, long long max_rows_per_segment, int segments
   return HE_OK;
 }
 
-template <int WORDS, int GT, int NT, bool PRE, bool PACKED = false>
+template <int WORDS, int GT, int NT, bool PRE, bool PACKED = false, bool SPLIT = true>
 int launch_decode_one(const DecodeArgs& a, size_t smem, dim3 grid, cudaStream_t stream) {
-  if (int rc = set_smem(decode_step_kernel<WORDS, GT, NT, PRE, PACKED>, smem)) return rc;
+  auto kernel = decode_step_kernel<WORDS, GT, NT, PRE, PACKED, SPLIT>;
+  if (int rc = set_smem(kernel, smem)) return rc;
   cudaLaunchConfig_t lc{};
   lc.gridDim = grid;
   lc.blockDim = dim3(NT);
@@ -365,7 +366,7 @@ int launch_decode_one(const DecodeArgs& a, size_t smem, dim3 grid, cudaStream_t 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
   lc.numAttrs = pdl_enabled() ? 1 : 0;
-  HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, decode_step_kernel<WORDS, GT, NT, PRE, PACKED>, a));
+  HE_CUDA_CHECK(cudaLaunchKernelEx(&lc, kernel, a));
   return HE_OK;
 }
 
@@ -376,6 +377,18 @@ int launch_decode_nt(const DecodeArgs& a, int nt, size_t smem, dim3 grid, cudaSt
     if (nt == 512) return launch_decode_one<WORDS, GT, 512, true, PACKED>(a, smem, grid, stream);
     return launch_decode_one<WORDS, GT, 1024, true, PACKED>(a, smem, grid, stream);
   }
+  // A thread of either half reads W for itself. While at most two units share an SM, and for one or two query rows (where splitting only
+  // means fewer rows a thread), the shorter chain is worth it; four query rows of narrow codes, whose W has no constant strides, pay for
+  // the second read where more CTAs share an SM. us per 32 calls in a graph, split / not, b = 16, G = 4, d = 128: windows (4, 10), 128
+  // units of 1024 slots 107 / 125, 296 of 256 103 / 104, 512 of 256 146 / 134, 1024 of 48 279 / 257; none, 512 of 256 139 / 131, 1024 of
+  // 1024 323 / 301. Whole words (b = 32) are level or better split: 512 of 256 126 / 131 without windows, 135 / 130 with, 1024 of 256 238 /
+  // 244 and 246 / 248.
+  if constexpr (WORDS == 1 && GT == 4)
+    if (nt == 256 && a.cfg.hash_bits < 32) {
+      int sms = 0;
+      if (int rc = sm_count(&sms)) return rc;
+      if ((long long)grid.x * grid.y > 2LL * sms) return launch_decode_one<WORDS, GT, 256, false, PACKED, false>(a, smem, grid, stream);
+    }
   if (nt == 256) return launch_decode_one<WORDS, GT, 256, false, PACKED>(a, smem, grid, stream);
   if (nt == 512) return launch_decode_one<WORDS, GT, 512, false, PACKED>(a, smem, grid, stream);
   return launch_decode_one<WORDS, GT, 1024, false, PACKED>(a, smem, grid, stream);
