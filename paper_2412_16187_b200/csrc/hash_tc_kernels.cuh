@@ -107,7 +107,6 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t tmem_d, uint64_t adesc, uin
       ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
       : "memory");
 }
-// 32 consecutive fp32 columns of this thread's tensor-memory lane
 // One lane of a converged warp.
 __device__ __forceinline__ bool tc_elect() {
   uint32_t p;
@@ -119,6 +118,7 @@ __device__ __forceinline__ bool tc_elect() {
   return p != 0;
 }
 
+// 32 consecutive fp32 columns of this thread's tensor-memory lane
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "

@@ -37,12 +37,12 @@
 // whole packed code table (at most 48 KB at 32 bits), copies its tiles' maxima to the others through distributed shared
 // memory, and all of them settle the block redundantly: one exchange per block.
 //
-// One CTA per SM, 512 threads (16 warps, so that each may have 128 registers: with 96 the accumulator loads spill and a
-// tile takes the readers 540 cycles instead of 160):
+// One CTA per SM, 512 threads (16 warps, so that each may have 128 registers; 107 to 128 are used. With 20 warps and 96 registers the
+// loads of fp32 accumulators spilled, a tile took the readers 540 cycles instead of 160; not tried since they come as 16-bit pairs):
 //   warps 0-7    tile phase: read accumulators from tensor memory, one step per thread, four warps a tile
 //   warps 8-11   tile phase: expand packed codes into +-2 operand tiles (K-major, 128-byte swizzle), one slot per thread
 //   warps 12-13  issue tcgen05.mma (M = 128 steps, N = 128 slots, K = 32) for every other pair of tiles: one warp's chain of
-//                waits, instructions and commits is 800 cycles a pair, twice what the tensor pipe needs. The loop is
+//                waits, instructions and commits is 600 to 770 cycles a pair, two to three times what the tensor pipe needs. The loop is
 //                warp-uniform and one elected lane issues, which keeps the descriptors in uniform registers
 //   warps 12-15  prepare the next block beside everything else: its codes, its operand A (14-15) and the distances between
 //                its own keys and queries, none of which depend on this block's outcome
