@@ -524,11 +524,10 @@ constexpr size_t kMaxDynSmem = 227 * 1024 - kRbStaticSmem;  // dynamic shared me
 // Shared memory of the block replay with as many operand stages as fit (fewer for large two-word tables); 0: does not fit.
 size_t rb_fit(int words, int slots, int G, int ncta, int form, RbArgs* ra) {
   ra->rows_max = form == kRbHalf ? kRbRows / 2 : kRbRows;
-  for (ra->abuf = 2; ra->abuf >= 1; --ra->abuf)
-    for (ra->lg_stage = 2; ra->lg_stage >= 1; --ra->lg_stage) {
-      ra->L = rb_layout(words, slots, G, ncta, 1 << ra->lg_stage, ra->abuf, ra->rows_max, form == kRbWide);
-      if (ra->L.total <= kMaxDynSmem) return ra->L.total < kRbMinSmem ? kRbMinSmem : ra->L.total;
-    }
+  for (ra->abuf = 2; ra->abuf >= 1; --ra->abuf) {
+    ra->L = rb_layout(words, slots, G, ncta, ra->abuf, ra->rows_max, form == kRbWide);
+    if (ra->L.total <= kMaxDynSmem) return ra->L.total < kRbMinSmem ? kRbMinSmem : ra->L.total;
+  }
   return 0;
 }
 
@@ -626,7 +625,7 @@ int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t s
   const bool full = rb_fit(WORDS, slots, G, 1, kRbFull, &fit) != 0;
   if constexpr (WORDS == 2)
     if (!full) return launch_replay_block_form<WORDS, GT, PROT, kRbHalf>(a, units, stream);
-  if (slots <= kRbWideSlots && rb_fit(WORDS, slots, G, 1, kRbWide, &wide) != 0 && wide.abuf == fit.abuf && wide.lg_stage == fit.lg_stage)
+  if (slots <= kRbWideSlots && rb_fit(WORDS, slots, G, 1, kRbWide, &wide) != 0 && wide.abuf == fit.abuf)
     return launch_replay_block_form<WORDS, GT, PROT, kRbWide>(a, units, stream);
   return launch_replay_block_form<WORDS, GT, PROT, kRbFull>(a, units, stream);
 }

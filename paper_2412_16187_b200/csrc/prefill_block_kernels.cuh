@@ -12,8 +12,7 @@
 // distance, lowest slot on ties). Slots past the budget and protected first tokens have zeros in B and come to 2^23 alone, below
 // everything else. At 2^23 the last mantissa bit is worth one, so an accumulator's low 16 bits ARE that key (rank <= 448: below
 // 2^16), and the readers take them from tensor memory two to a register (tcgen05.ld.pack::16b) and compare two at a time: 36
-// instructions a tile and thread for 68 on the fp32 values, and half the registers. 256 units of 9830 slots, with the waits polled in
-// straight code (mbar_wait_warp): a pair of tiles 795 -> 630 cycles, a call 8580 -> 7210 us.
+// instructions a tile and thread for 68 on the fp32 values, and half the registers.
 //
 // What is sequential, and how it is settled side by side. Step r's victim depends on the victims s[0..r-1] of the block:
 // a base slot (the table as the block found it) may be taken already, and the keys of earlier steps are candidates
@@ -37,16 +36,23 @@
 // whole packed code table (at most 48 KB at 32 bits), copies its tiles' maxima to the others through distributed shared
 // memory, and all of them settle the block redundantly: one exchange per block.
 //
-// One CTA per SM, 512 threads (16 warps, so that each may have 128 registers; 107 to 128 are used. With 20 warps and 96 registers the
-// loads of fp32 accumulators spilled, a tile took the readers 540 cycles instead of 160; not tried since they come as 16-bit pairs):
-//   warps 0-7    tile phase: read accumulators from tensor memory, one step per thread, four warps a tile
-//   warps 8-11   tile phase: expand packed codes into +-2 operand tiles (K-major, 128-byte swizzle), one slot per thread
-//   warps 12-13  issue tcgen05.mma (M = 128 steps, N = 128 slots, K = 32) for every other pair of tiles: one warp's chain of
-//                waits, instructions and commits is 600 to 770 cycles a pair, two to three times what the tensor pipe needs. The loop is
-//                warp-uniform and one elected lane issues, which keeps the descriptors in uniform registers
-//   warps 12-15  prepare the next block beside everything else: its codes, its operand A (14-15) and the distances between
-//                its own keys and queries, none of which depend on this block's outcome
+// One CTA per SM, 18 warps of at most 96 registers:
+//   warps 0-11   tile phase: groups of four read accumulators from tensor memory, one step per thread, a group a tile: three groups, or two
+//                for two-word codes, whose warps 8-11 expand with the next four
+//   warps 12-15  tile phase: expand packed codes into +-2 operand tiles (K-major, 128-byte swizzle), teams of two warps a tile, two slots
+//                per thread; then they prepare the next block beside everything else: its operand A and the distances between its own
+//                keys and queries, none of which depend on this block's outcome
+//   warps 16-17  issue tcgen05.mma (M = 128 steps, N = 128 slots, K = 32) for the even and the odd tiles. The loop is warp-uniform, its counters
+//                come out of a reduction so that they sit in uniform registers, and one elected lane issues
 //   afterwards   warps 0-11 settle the block's steps
+// A tile's tensor time is 64 cycles a K step (128 with one word, 192 with two), its read 64 and its maxima 72; what a tile costs instead is the
+// latency of the hand-overs around them: 100 cycles for a wait on a completed mbarrier and 170 from an arrival to the waiter, 260 from
+// the last MMA to its commit. So every tile has an accumulator of its own (pairs of tiles, with two groups and two accumulator pairs, took
+// 630 cycles a pair), a freed accumulator and a written operand tile meet the issuing warp in ONE named barrier (45 cycles; two mbarriers
+// 120), and no warp handles more than every second tile. A tile now takes 245 cycles with one word at 9830 slots. In a program of the tile
+// phase alone: three groups 201, two 246, one 393 (in this kernel a single issuing warp is the bound, at 290 to 430 cycles a tile); two words
+// 271 with three groups and 285 with two; with mbarriers instead 235 to 290. Replay of 256 units of 9830 slots: 5630 -> 4800 us; of 512 units of
+// 512 to 4096 slots, two words, 835 -> 810 (840 with three groups and four expanding warps).
 // Every wait on an mbarrier is bounded; a CTA that gives up raises a flag that turns its later waits into no-ops, but it
 // still walks the same blocks and cluster barriers as its peers (their copies into its shared memory must find it), then
 // releases tensor memory and raises the device error counter.
@@ -58,13 +64,17 @@
 
 namespace he {
 
-constexpr int kRbThreads = 512;
-constexpr int kRbReadGroups = 2;         // groups of four warps that read accumulators
-constexpr int kRbExpWarp = 4 * kRbReadGroups, kRbMmaWarp = kRbExpWarp + 4;
 constexpr int kRbResWarps = 12;          // warps that settle a block
 constexpr int kRbResThreads = 32 * kRbResWarps;
-constexpr int kRbAuxThreads = 128;       // warps kRbMmaWarp .. kRbMmaWarp + 3
-constexpr int kRbBuildThreads = 64;      // ... of which the last two build operand A
+constexpr int kRbAuxWarp = kRbResWarps;  // the four warps that prepare the next block
+constexpr int kRbAuxThreads = 128;
+constexpr int kRbMmaWarp = 16;           // the two warps that issue products
+constexpr int kRbThreads = 32 * (kRbMmaWarp + 2);
+// Groups of four warps that read accumulators; the warps from there to kRbMmaWarp expand.
+__host__ __device__ constexpr int rb_read_groups(int words) { return words == 2 ? 2 : 3; }
+constexpr int kRbAccs = 4;               // accumulators, and tiles of operand B in shared memory
+constexpr int kRbDoneBars = 2 * kRbAccs; // mbarriers that say a product is complete
+constexpr int kRbTileBar = 8;            // named barriers kRbTileBar .. + 3: one for each accumulator
 constexpr int kRbRows = 128;             // steps per block at most = MMA M
 constexpr int kRbTile = 128;             // slots per tile = MMA N
 constexpr int kRbKeyShift = 14;
@@ -86,7 +96,6 @@ __host__ __device__ constexpr int rb_walk_cost(int words, int gt, bool prot, int
 constexpr int kRbAtom = 128 * 128;       // 128 operand rows x one 128-byte swizzle atom
 constexpr int kRbDnPitch = 136;          // 16-bit entries between rows of the new-entry table
 constexpr int kRbDnPitchHalf = 68;       // ... when blocks have at most 64 steps
-constexpr int kRbMaxStages = 4;          // pairs of operand tiles
 constexpr int kRbStaticSmem = 512;       // bytes kept back for the kernel's static arrays
 // Eras of the owner table of words: the passes of a unit go from the first one down, 256 apart, and start again at a block that finds
 // the last one behind it (a block uses a hundred or two, so none reaches the walk's mark of zero). The bounds-checking build starts over
@@ -104,7 +113,7 @@ constexpr uint32_t kRbLastEra = 0x20000u;
 struct RbLayout {
   uint32_t a, bidx, b, codes, own, mx, mx_pitch, mx_block, top_at, dn, dn_buf, rn, nr, sv, sn, list, par, qraw, kraw, rec, total;
 };
-__host__ __device__ inline RbLayout rb_layout(int words, int slots, int G, int ncta, int nstage, int abuf, int rows_max, bool wide) {
+__host__ __device__ inline RbLayout rb_layout(int words, int slots, int G, int ncta, int abuf, int rows_max, bool wide) {
   RbLayout L;
   const uint32_t nt = (uint32_t)slots / kRbTile, ntl = (nt + ncta - 1) / ncta;
   uint32_t o = 0;
@@ -116,13 +125,13 @@ __host__ __device__ inline RbLayout rb_layout(int words, int slots, int G, int n
   // a 128-byte atom row holds two tiles' 64-bit rows or four tiles' 32-bit rows, and both buffers of a 32-bit operand A
   L.a = take(words == 2 ? (uint32_t)abuf * kRbAtom : kRbAtom);
   L.bidx = take(kRbAtom);  // index columns: four variants side by side
-  L.b = take(words == 2 ? (uint32_t)nstage * kRbAtom : (uint32_t)(nstage + 1) / 2 * kRbAtom);
+  L.b = take((uint32_t)kRbAccs / (words == 2 ? 2 : 4) * kRbAtom);
   L.codes = take((uint32_t)slots * words * 4u);
   L.own = take((uint32_t)slots * (wide ? 4u : 1u));
   L.mx_pitch = ntl | 1u;  // words
   // (one more row takes the threads without a step; whole 16-byte units, as the copies between CTAs want)
   L.top_at = (L.mx_pitch * (rows_max < kRbRows ? rows_max + 1 : rows_max) + 3u) & ~3u;
-  L.mx_block = L.top_at + kRbReadGroups * rows_max;
+  L.mx_block = L.top_at + (uint32_t)rb_read_groups(words) * rows_max;
   L.mx = take(L.mx_block * ncta * 4u);
   L.dn_buf = rows_max == kRbRows ? kRbRows / 2 * kRbDnPitch : rows_max * kRbDnPitchHalf;  // entries
   L.dn = take(2u * L.dn_buf * 2u);
@@ -143,7 +152,6 @@ struct RbArgs {
   ReplayArgs r;
   int ncta;       // CTAs per unit (cluster size, a power of two)
   int scheduled;  // units are claimed from r.sched; 0: unit = cluster index
-  int lg_stage;   // log2 of the pairs of operand tiles in shared memory
   int abuf;       // operand A buffers (2: the next block's is built during the tile phase)
   int rows_max;   // steps per block at most: 128, or 64 (kRbHalf)
   RbLayout L;     // computed by the host: kernel parameters cost no registers
@@ -193,6 +201,31 @@ __device__ __forceinline__ void rb_ld64_low(uint32_t taddr, uint32_t (&v)[32]) {
       : "memory");
 }
 
+// tcgen05.wait::ld that the loaded registers pass through, so that nothing uses them ahead of it.
+__device__ __forceinline__ void rb_wait_ld(uint32_t (&v)[32]) {
+  asm volatile(
+      "tcgen05.wait::ld.sync.aligned;"
+      : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]),
+        "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]), "+r"(v[16]),
+        "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]), "+r"(v[24]),
+        "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+      :
+      : "memory");
+}
+// Pairwise maximum of 64 registers: a tree of three-input maxima, four levels deep.
+__device__ __forceinline__ uint32_t rb_max64(const uint32_t (&a)[32], const uint32_t (&b)[32]) {
+  uint32_t t[21], u[7];
+#pragma unroll
+  for (int k = 0; k < 10; ++k) {
+    t[k] = __vimax3_u16x2(a[3 * k], a[3 * k + 1], a[3 * k + 2]);
+    t[10 + k] = __vimax3_u16x2(b[3 * k], b[3 * k + 1], b[3 * k + 2]);
+  }
+  t[20] = __vimax3_u16x2(a[30], a[31], b[30]);
+#pragma unroll
+  for (int k = 0; k < 7; ++k) u[k] = __vimax3_u16x2(t[3 * k], t[3 * k + 1], t[3 * k + 2]);
+  return __vimax3_u16x2(__vimax3_u16x2(u[0], u[1], u[2]), __vimax3_u16x2(u[3], u[4], u[5]), __vmaxu2(u[6], b[31]));
+}
+
 // Columns of a code word in operand order: output word m (four bytes) holds bits m, m + 8, m + 16, m + 24, in both
 // operands, so that one shift and one logic operation expand four bits. Set: +2 (e4m3 0x40), clear: -2 (0xC0).
 __device__ __forceinline__ uint32_t rb_expand4(uint32_t h, int m) { return lop3<0x6A>(h << (7 - m), 0x80808080u, 0xC0C0C0C0u); }
@@ -227,8 +260,22 @@ __device__ __forceinline__ void rb_copy_to_peer(uint32_t dst, uint32_t src, uint
 __device__ __forceinline__ void rb_arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// mbar_wait_warp with its loop left rolled: unrolled by the compiler, each of this kernel's waits was 5 KB of code, half of the kernel's 143 KB
+// (128 units of 1024 slots, b = 16, windows, the kernel otherwise as it was: 1290 -> 1230 us).
+__device__ __forceinline__ bool rb_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  if (__builtin_expect(__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)), 1)) return true;
+  bool ok = false, on = true;
+#pragma unroll 1
+  for (uint32_t i = 0; i < kTcSpinLimit && on; ++i) {
+    ok = mbar_try_wait(bar, parity);
+    on = !ok && *abort_flag == 0;
+  }
+  if (!ok) *abort_flag = 1;
+  return __all_sync(0xFFFFFFFFu, ok);
+}
 // Bounded wait for copies and arrivals of other CTAs of the cluster.
 __device__ __forceinline__ bool rb_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+#pragma unroll 1
   for (uint32_t i = 0; i < kTcSpinLimit; ++i) {
     uint32_t ok;
     asm volatile(
@@ -251,6 +298,11 @@ template <int ID, int THREADS>
 __device__ __forceinline__ void rb_bar() {
   asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
 }
+// An accumulator's named barrier (`acc` 0 .. 3): four warps that have read it, two that have written the operand tile of the same number,
+// and the issuing warp, which waits.
+constexpr int kRbTileBarThreads = 128 + 64 + 32;
+__device__ __forceinline__ void rb_tile_arrive(int acc) { asm volatile("bar.arrive %0, %1;" ::"r"(kRbTileBar + acc), "n"(kRbTileBarThreads) : "memory"); }
+__device__ __forceinline__ void rb_tile_sync(int acc) { asm volatile("bar.sync %0, %1;" ::"r"(kRbTileBar + acc), "n"(kRbTileBarThreads) : "memory"); }
 
 // Rank of one slot's code at a step from the packed words. GT = 4 uses the bit-plane form, which yields (D - pc) / 2 with pc
 // the bits set in the exclusive or of the step's query codes (`parity_bits`, worked out with operand A).
@@ -336,6 +388,7 @@ __device__ __noinline__ void rb_walk(const RbLayout& L, bool wide, int base, int
   RbRank<WORDS, GT> rk;
   rk.load(qb + fin * GW, G, par[fin]);
   int last = PROT && Rn == 1 ? newest(fin, 1) : 0;  // slot of the step before
+#pragma unroll 1
   for (int r = fin; r < rows; ++r) {
     // what the rewrite and the next step want and this step's outcome does not decide
     RbRank<WORDS, GT> next;
@@ -398,10 +451,10 @@ enum : int { kRbFull = 0, kRbHalf = 1, kRbWide = 2 };
 template <int WORDS, int GT, bool PROT, int FORM>
 __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(const __grid_constant__ RbArgs ar) {
   constexpr int NT = kRbThreads;
-  constexpr int MS = kRbMaxStages;
+  constexpr int kGroups = rb_read_groups(WORDS), kExpWarp = 4 * kGroups, kTeams = (kRbMmaWarp - kExpWarp) / 2;
   constexpr bool HALF = FORM == kRbHalf, wide = FORM == kRbWide;
   constexpr int RM = HALF ? kRbRows / 2 : kRbRows;
-  __shared__ __align__(8) unsigned long long bars[2 * MS + 4 + 5];
+  __shared__ __align__(8) unsigned long long bars[kRbDoneBars + 5];
   __shared__ uint32_t tmem_base_s;
   __shared__ volatile int abort_flag;
   __shared__ int s_unit[2];
@@ -418,7 +471,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   const int GW = G * WORDS;
   const long long Cmax = cfg.max_budget;
   const bool write_scores = (cfg.flags & HE_FLAG_WRITE_SCORES) != 0;
-  const int ncta = ar.ncta, lg_ncta = 31 - __clz(ncta), lg_stage = ar.lg_stage, abuf = ar.abuf;
+  const int ncta = ar.ncta, lg_ncta = 31 - __clz(ncta), abuf = ar.abuf;
   const int rank = ncta > 1 ? (int)rb_cluster_rank() : 0;
   // rounded up to 1024 bytes by an offset from the array itself: the accesses stay shared-memory accesses
   unsigned char* smem = rb_smem_raw + ((1024u - (smem_u32(rb_smem_raw) & 1023u)) & 1023u);
@@ -444,34 +497,25 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   const int a_step = WORDS == 2 ? kRbAtom : 64;             // bytes between the two buffers of operand A
 
   const uint32_t bar0 = smem_u32(bars);
-  auto full_bar = [&](int s) { return bar0 + 8u * s; };                  // expanders -> MMA: the pair's operand tiles are written
-  auto sfree_bar = [&](int s) { return bar0 + 8u * (MS + s); };          // MMA -> expanders: they may be rewritten
-  auto afull_bar = [&](int x) { return bar0 + 8u * (2 * MS + x); };      // MMA -> readers: the pair's accumulators are complete
-  auto afree_bar = [&](int x) { return bar0 + 8u * (2 * MS + 2 + x); };  // readers -> MMA: they have been read
-  const uint32_t peer_bar = bar0 + 8u * (2 * MS + 4);                    // peers' copies of their tiles' maxima have arrived
-  const uint32_t used_bar = bar0 + 8u * (2 * MS + 5);                    // peers: they are done with this CTA's maxima
-  const uint32_t adone_bar = bar0 + 8u * (2 * MS + 6);                   // one operand A buffer: the block's tiles are multiplied
-  const uint32_t drain_bar = bar0 + 8u * (2 * MS + 7);                   // abort path
-  const uint32_t tops_bar = bar0 + 8u * (2 * MS + 8);                    // peers' copies of their best keys have arrived
+  auto done_bar = [&](int n) { return bar0 + 8u * (n & (kRbDoneBars - 1)); };  // product n is complete: its accumulator may be read, its operand tile rewritten
+  auto done_phase = [&](int n) { return (uint32_t)(n >> 3) & 1u; };
+  const uint32_t peer_bar = bar0 + 8u * kRbDoneBars;           // peers' copies of their tiles' maxima have arrived
+  const uint32_t used_bar = bar0 + 8u * (kRbDoneBars + 1);     // peers: they are done with this CTA's maxima
+  const uint32_t adone_bar = bar0 + 8u * (kRbDoneBars + 2);    // one operand A buffer: the block's tiles are multiplied
+  const uint32_t drain_bar = bar0 + 8u * (kRbDoneBars + 3);    // abort path
+  const uint32_t tops_bar = bar0 + 8u * (kRbDoneBars + 4);     // peers' copies of their best keys have arrived
   if (tid == 0) {
     abort_flag = 0;
     mbar_init(drain_bar, 2);
     mbar_init(adone_bar, 2);
-    for (int i = 0; i < MS; ++i) {
-      mbar_init(full_bar(i), 4);
-      mbar_init(sfree_bar(i), 1);
-    }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(afull_bar(i), 1);
-      mbar_init(afree_bar(i), 8);
-    }
+    for (int i = 0; i < kRbDoneBars; ++i) mbar_init(done_bar(i), 1);
     mbar_init(peer_bar, 1);
     mbar_init(tops_bar, 1);
     mbar_init(used_bar, ncta > 1 ? ncta - 1 : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == kRbMmaWarp) {  // four accumulators of 128 columns
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(4 * kRbTile)
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(kRbAccs * kRbTile)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -487,6 +531,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
     lut_hi |= (c + 4 <= G ? rb_e5m2(-alpha * (2 * (c + 4) - G)) : 0u) << (8 * c);
   }
   if (!wide)
+#pragma unroll 1
     for (int i = tid; i < a.smem_slots / 4; i += NT) own32[i] = 0xFFFFFFFFu;
   griddep_wait();  // everything above overlaps the hashing kernel's tail
   tc_fence_before();
@@ -496,14 +541,17 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   const uint32_t tmem_base = tmem_base_s;
   // instruction descriptor: fp32 accumulate, e5m2 x e4m3, both operands K-major, N = 128, M = 128
   const uint32_t idesc = (1u << 4) | (1u << 7) | ((uint32_t)(kRbTile >> 3) << 17) | ((uint32_t)(kRbRows >> 4) << 24);
-  // Pairs of tiles so far; every role counts the same sequence. Pair n lives in operand stage n mod (1 << lg_stage) and
-  // accumulator pair n mod 2.
+  // Tiles so far; every role counts the same sequence. Tile n lives in operand tile and accumulator n mod 4; warp 16 + (n mod 2) issues its
+  // product, so that the even and the odd products each complete in order. A wait for product n may only be begun once product n - 8
+  // is known to be complete (the barrier's phases alternate): readers have read product n - 6 before it or come from a block's start, where
+  // everything is complete, and expanding warps have waited for products of the same parity.
   int it = 0;
-  int blk = 0;  // blocks so far
-  auto stage_of = [&](int n) { return n & ((1 << lg_stage) - 1); };
-  auto stage_phase = [&](int n) { return (uint32_t)(n >> lg_stage) & 1u; };
+  int blk = 0, turn = 0;  // blocks settled and turns of the block loop so far
+  if (warp < 4)
+    for (int x = 0; x < kRbAccs; ++x) rb_tile_arrive(x);  // nothing is in the accumulators
 
   // (the unit number is double-buffered: a peer may still be reading the one before)
+#pragma unroll 1
   for (int nunit = 0;; ++nunit) {
     if (ar.scheduled) {
       if (rank == 0 && warp == 0) {
@@ -532,7 +580,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
     int32_t* pos_g = a.ca.pos + unit * Cmax;
     const int S = PROT ? cfg.n_sink : 0, Rn = PROT ? cfg.n_recent : 0;
     const int nbase = (C + kRbTile - 1) / kRbTile;
-    const int ntl = nbase > rank ? (nbase - rank + ncta - 1) >> lg_ncta : 0;  // this CTA's tiles: rank, rank + ncta, ...
+    const int ntl_unit = nbase > rank ? (nbase - rank + ncta - 1) >> lg_ncta : 0;  // this CTA's tiles: rank, rank + ncta, ...
     const int R = min(rb_block_rows(C, G * cfg.hash_bits), RM);
     // the first C tokens fill the cache in order; everything beyond `fill` is reset
     for (int j = tid; j < nbase * kRbTile; j += NT) {
@@ -560,8 +608,10 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
       uint32_t* kd = kraw + buf * kRbRows * WORDS;
       const uint32_t* qs = qc_u + (long long)tb * GW;
       const uint32_t* ks = kc_u + (long long)tb * WORDS;
+#pragma unroll 1
       for (int i = first; i < nrows * GW; i += nthreads)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(qd + i)), "l"(qs + i) : "memory");
+#pragma unroll 1
       for (int i = first; i < nrows * WORDS; i += nthreads)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(kd + i)), "l"(ks + i) : "memory");
       cp_async_commit();
@@ -571,6 +621,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
       const uint32_t* qd = qraw + buf * kRbRows * GW;
       unsigned char* ad = As + (WORDS == 2 && abuf > 1 ? buf * kRbAtom : 0);
       const int c0 = WORDS == 1 && abuf > 1 ? 4 * buf : 0;
+#pragma unroll 1
       for (int item = first; item < kRbRows * WORDS; item += nthreads) {
         const int r = item & (kRbRows - 1), w = item >> 7;
         const bool valid = r < nrows;
@@ -611,61 +662,66 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         }
       }
     };
-    // One tile's row of operand B in operand stage sx (tile g of the pair): this thread's slot or key; zeros for a slot that may not win.
-    auto expand_row = [&](const uint32_t* h, bool live, int x, int sx, int g) {
-      unsigned char* bt = Bs + (WORDS == 2 ? sx : sx >> 1) * kRbAtom + (x >> 3) * 1024 + (x & 7) * 128;
-      const int c0 = WORDS == 2 ? 4 * g : 2 * (2 * (sx & 1) + g);
+    // Shared-memory address of the first chunk of row x of operand tile sx.
+    auto row_at = [&](int x, int sx) {
+      const int c0 = WORDS == 2 ? 4 * (sx & 1) : 2 * sx;
+      return smem_u32(Bs) + (uint32_t)((WORDS == 2 ? sx >> 1 : 0) * kRbAtom + (x >> 3) * 1024 + (x & 7) * 128 + ((c0 ^ (x & 7)) << 4));
+    };
+    auto st_chunk = [](uint32_t at, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3) {
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v0), "r"(v1), "r"(v2), "r"(v3) : "memory");
+    };
+    // A slot's or a key's code as a row (c0 is a multiple of the row's chunks, so chunk c is where c0 is, xor c).
+    auto expand_row = [&](const uint32_t* h, uint32_t at) {
 #pragma unroll
       for (int c = 0; c < 2 * WORDS; ++c) {
         const uint32_t hw = h[c >> 1];
         const int m = (c & 1) * 4;
-        *reinterpret_cast<uint4*>(bt + (((c0 + c) ^ (x & 7)) << 4)) =
-            make_uint4(rb_expand4(hw, m), rb_expand4(hw, m + 1), rb_expand4(hw, m + 2), rb_expand4(hw, m + 3));
+        st_chunk(at ^ (uint32_t)(c << 4), rb_expand4(hw, m), rb_expand4(hw, m + 1), rb_expand4(hw, m + 2), rb_expand4(hw, m + 3));
       }
-      if (!live) {
+    };
+    auto clear_row = [&](uint32_t at) {
 #pragma unroll
-        for (int c = 0; c < 2 * WORDS; ++c) *reinterpret_cast<uint4*>(bt + (((c0 + c) ^ (x & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
-      }
+      for (int c = 0; c < 2 * WORDS; ++c) st_chunk(at ^ (uint32_t)(c << 4), 0u, 0u, 0u, 0u);
     };
     auto a_desc_of = [&](int buf) { return umma_desc_k128(smem_u32(As)) + (uint64_t)((abuf > 1 ? buf * a_step : 0) >> 4); };
-    auto b_desc_of = [&](int sx, int g) {
-      return umma_desc_k128(smem_u32(Bs)) +
-             (uint64_t)((WORDS == 2 ? sx * kRbAtom + g * 64 : (sx >> 1) * kRbAtom + (2 * (sx & 1) + g) * 32) >> 4);
+    auto b_desc_of = [&](int sx) {
+      return umma_desc_k128(smem_u32(Bs)) + (uint64_t)((WORDS == 2 ? (sx >> 1) * kRbAtom + (sx & 1) * 64 : sx * 32) >> 4);
     };
-    // Ranks of a block's own keys (buffer `buf`) at its steps, by warps 12-15: one more tile, as pair n, without index
+    // Product n of operand A `buf` with operand tile n mod 4, by the issuing warp; xd: index columns, none for a block's own keys.
+    auto issue = [&](int n, uint32_t tmem, uint64_t ad, bool index, uint64_t xd) {
+      const int acc = n & 3;
+      const uint64_t bd = b_desc_of(acc);
+      rb_tile_sync(acc);
+      tc_fence_after();
+      if (tc_elect()) {
+        const uint32_t d = tmem + (uint32_t)(acc * kRbTile);
+#pragma unroll
+        for (int w = 0; w < WORDS; ++w) rb_mma_f8(d, ad + (uint64_t)(2 * w), bd + (uint64_t)(2 * w), idesc, w > 0);
+        if (index) rb_mma_f8(d, ad + (uint64_t)(2 * WORDS), xd, idesc, true);
+        tc_commit(done_bar(n));
+      }
+      __syncwarp();
+    };
+    // Ranks of a block's own keys (buffer `buf`) at its steps, by warps 12-15: one more tile, as product n, without index
     // columns. Also each step's largest rank of any key that enters before it (and is no longer recent): no new entry can
-    // beat that. (Both MMA warps have issued every earlier pair when this runs, so no wait here can meet an older phase.)
+    // beat that.
     auto new_keys = [&](int buf, int n) {
-      const int x = tid & 127, acc = n & 1, ph = (n >> 1) & 1, sx = stage_of(n);
-      const uint32_t px = stage_phase(n);
-      if (!mbar_wait_warp(sfree_bar(sx), px ^ 1, &abort_flag)) return;
+      const int x = tid & 127, acc = n & 3;
+      rb_wait(done_bar(n - 4), done_phase(n - 4), &abort_flag);
       uint32_t h[WORDS];
 #pragma unroll
       for (int w = 0; w < WORDS; ++w) h[w] = kraw[(buf * kRbRows + x) * WORDS + w];
-      expand_row(h, true, x, sx, 0);
+      expand_row(h, row_at(x, acc));
       fence_proxy_async();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(full_bar(sx));
-      if (warp == kRbMmaWarp) {
-        if (!mbar_wait2_warp(afree_bar(acc), ph ^ 1, full_bar(sx), px, &abort_flag)) return;
-        tc_fence_after();
-        const uint64_t ad = a_desc_of(buf), bd = b_desc_of(sx, 0);
-        if (tc_elect()) {
-#pragma unroll
-          for (int w = 0; w < WORDS; ++w)
-            rb_mma_f8(tmem_base + (uint32_t)(2 * acc * kRbTile), ad + (uint64_t)(2 * w), bd + (uint64_t)(2 * w), idesc, w > 0);
-          tc_commit(afull_bar(acc));
-          tc_commit(sfree_bar(sx));
-        }
-        __syncwarp();
-      }
-      if (!mbar_wait_warp(afull_bar(acc), ph, &abort_flag)) return;
+      rb_bar<3, kRbAuxThreads>();
+      if (warp < kRbAuxWarp + 2) rb_tile_arrive(acc);
+      rb_wait(done_bar(n), done_phase(n), &abort_flag);
       tc_fence_after();
       // Conversions by an fp32 addition (the integer conversions run at a sixteenth of its rate): 2^22 + rank has 2 * rank
       // in its low bits, which is what is kept.
       const int r = x, last = PROT ? r - Rn : r;  // entries below `last` are candidates
       const float magic = (float)(off - ((PAR[buf * kRbRows + r] & 1) << 6)) * (1.f / 128.f) + 4194304.f;
-      const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(2 * acc * kRbTile);
+      const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(acc * kRbTile);
       uint16_t* dst = Dn + buf * L.dn_buf + rb_dn_at(r, RM);
       float dmax = -1e9f;
 #pragma unroll 1
@@ -675,8 +731,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         tc_wait_ld();
         if (c == 3) {
           tc_fence_before();
-          __syncwarp();
-          if (lane < 2) mbar_arrive(afree_bar(acc));  // (four warps, eight arrivals)
+          rb_tile_arrive(acc);
         }
         if (c > (warp & 3)) continue;  // no step of this warp comes after those keys
         const int lc = last - c * 32;
@@ -697,161 +752,132 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
       }
       NR[buf * kRbRows + r] = last > 0 ? (int)(__float_as_uint(fmaf(dmax, 1.f / 128.f, magic)) & 0xFFFFu) >> 1 : -1;
     };
-    int cur = 0;
-    if (C < N) {
-      const int rows = min(N - C, R);
-      stage_codes(0, C, rows, tid, NT);
-      cp_async_wait_all();
-      __syncthreads();
-      build_a(0, rows, tid, NT);
-      fence_proxy_async();
-      __syncthreads();
-      if (warp >= kRbMmaWarp) new_keys(0, it);
-      ++it;
-    }
     fence_proxy_async();
     __syncthreads();
-
-    for (int t0 = C; t0 < N; t0 += R) {
-      const int rows = min(N - t0, R);
-      const int tn = t0 + rows;
+    // A turn works on the block of steps t0 .. tn - 1 and prepares the next one; a unit's first turn has no steps yet.
+    int cur = 0, rows = 0;
+#pragma unroll 1
+    for (int t0 = C; t0 < N;) {
+      const int tn = t0 + rows, ntl = rows > 0 ? ntl_unit : 0;
       const uint32_t* qb = qraw + cur * kRbRows * GW;
       const uint32_t* kb_codes = kraw + cur * kRbRows * WORDS;
       // ---------------------------------------------------------------- tile phase
       // this CTA's base tiles 0 .. ntl - 1 (tile i of the CTA is tile i * ncta + rank of the unit)
-      const int npair = (ntl + 1) >> 1;
       int top = -1;  // readers: best base key of the thread's step so far
-      if (warp < kRbExpWarp) {
-        const int r = tid & 127, grp = warp >> 2;  // this thread's step = its tensor-memory lane; tile grp of each pair
+      if (warp < kExpWarp) {
+        const int r = tid & 127, grp = warp >> 2;  // this thread's step = its tensor-memory lane; tiles grp, grp + kGroups, ...
         int32_t* mrow = Mx + rank * L.mx_block + min(r, RM) * L.mx_pitch;
         int ct = (127 - ((grp << lg_ncta) + rank)) * 128;  // 127 - tile goes above the index within the tile (lower tiles first)
-        const int cstep = 256 << lg_ncta;
-        const uint32_t taddr0 = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(grp * kRbTile);
-        if (ncta > 1 && blk > 0) rb_wait_cluster(used_bar, (blk - 1) & 1, &abort_flag);  // peers still read the block before
-        for (int p = 0; p < npair; ++p) {
-          const int n = it + p, acc = n & 1, ph = (n >> 1) & 1, i = 2 * p + grp;
-          if (!mbar_wait_warp(afull_bar(acc), ph, &abort_flag)) break;
+        const int cstep = (128 * kGroups) << lg_ncta;
+        const uint32_t taddr0 = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+        if (ncta > 1 && blk > 0 && rows > 0) rb_wait_cluster(used_bar, (blk - 1) & 1, &abort_flag);  // peers still read the block before
+#pragma unroll 1
+        for (int i = grp; i < ntl; i += kGroups) {
+          const int n = it + i, acc = n & 3;
+          rb_wait(done_bar(n), done_phase(n), &abort_flag);
           tc_fence_after();
-          // (the second tile of an odd last pair holds an older product; nobody looks at its key)
-          const uint32_t taddr = taddr0 + (uint32_t)(2 * acc * kRbTile);
-          uint32_t v0[32], v1[32], m[8];
+          const uint32_t taddr = taddr0 + (uint32_t)(acc * kRbTile);
+          uint32_t v0[32], v1[32];
           rb_ld64_low(taddr, v0);
           rb_ld64_low(taddr + 64, v1);
-          tc_wait_ld();
-          tc_fence_before();  // the accumulators go back
-          __syncwarp();
-          if (lane == 0) mbar_arrive(afree_bar(acc));
-#pragma unroll
-          for (int k = 0; k < 8; ++k) m[k] = __vimax3_u16x2(v0[k], v0[k + 8], v0[k + 16]);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) m[k] = __vimax3_u16x2(m[k], v0[k + 24], v1[k]);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) m[k] = __vimax3_u16x2(m[k], v1[k + 8], v1[k + 16]);
-          m[0] = __vimax3_u16x2(m[0], v1[24], v1[25]), m[1] = __vimax3_u16x2(m[1], v1[26], v1[27]);
-          m[2] = __vimax3_u16x2(m[2], v1[28], v1[29]), m[3] = __vimax3_u16x2(m[3], v1[30], v1[31]);
-          m[0] = __vimax3_u16x2(m[0], m[1], m[2]), m[3] = __vimax3_u16x2(m[3], m[4], m[5]);
-          m[0] = __vmaxu2(__vimax3_u16x2(m[0], m[3], m[6]), m[7]);
+          rb_wait_ld(v0);
+          rb_wait_ld(v1);
+          tc_fence_before();  // the accumulator goes back
+          rb_tile_arrive(acc);
+          const uint32_t m = rb_max64(v0, v1);
           // the tile's best key, 2^14 rank + index; negative: no slot of the tile may win
-          const int k16 = (int)max(m[0] & 0xFFFFu, m[0] >> 16) - 1, key = ((k16 & ~127) << 7) + (k16 & 127) + ct;
+          const int k16 = (int)max(m & 0xFFFFu, m >> 16) - 1, key = ((k16 & ~127) << 7) + (k16 & 127) + ct;
           ct -= cstep;
-          if (i < ntl) {
-            top = max(top, key);
-            mrow[i] = key;
-          }
+          top = max(top, key);
+          mrow[i] = key;
         }
-        if (r < RM) Mx[rank * L.mx_block + top_at + grp * RM + r] = top;  // this group's best key of the step
+        if (rows > 0 && r < RM) Mx[rank * L.mx_block + top_at + grp * RM + r] = top;  // this group's best key of the step
         if (ncta > 1) fence_proxy_async();
-        rb_bar<4, 32 * kRbExpWarp>();  // the reader groups see each other's results
-        if (tid < ncta - 1) {          // ... and every peer gets this CTA's block
+      } else if (warp < kRbMmaWarp) {
+        if (ncta > 1 && rows > 0 && tid == 32 * kRbAuxWarp) {
+          mbar_arrive_expect_tx(tops_bar, (uint32_t)(kGroups * RM * (ncta - 1)) * 4u);
+          mbar_arrive_expect_tx(peer_bar, 4u * (uint32_t)(top_at * (ncta - 1)));
+        }
+        const int aux = tid - 32 * kRbAuxWarp, nrows = min(N - tn, R);
+        if (tn < N && warp >= kRbAuxWarp) stage_codes(cur ^ 1, tn, nrows, aux, kRbAuxThreads);  // the next block's codes arrive meanwhile
+        // teams of two warps write the operand tiles in turn, rows x and x + 64 by a thread
+        const int x = tid & 63;
+        uint32_t h0[WORDS], h1[WORDS];
+        auto fetch = [&](int i) {
+          const uint32_t* src = codes + (((i << lg_ncta) + rank) * kRbTile + x) * WORDS;
+          if (WORDS == 2) {
+            const uint2 a2 = *reinterpret_cast<const uint2*>(src), b2 = *reinterpret_cast<const uint2*>(src + 64 * WORDS);
+            h0[0] = a2.x, h0[WORDS - 1] = a2.y, h1[0] = b2.x, h1[WORDS - 1] = b2.y;
+          } else {
+            h0[0] = src[0], h1[0] = src[64];
+          }
+        };
+        int i = (((warp - kExpWarp) >> 1) - it) & (kTeams - 1);
+        uint32_t at = row_at(x, (it + i) & 3), at_next = row_at(x, (it + i + kTeams) & 3);  // row x + 64 is 8 KB further on
+        const int whole = S > 0 ? 1 : 0, part = C / kRbTile;  // tiles of the unit from `whole` to `part` - 1 hold candidates only
+        if (i < ntl) fetch(i);
+#pragma unroll 1
+        for (; i < ntl; i += kTeams) {
+          const int n = it + i, tile = (i << lg_ncta) + rank;
+          rb_wait(done_bar(n - 4), done_phase(n - 4), &abort_flag);  // product n - 4 is done with the operand tile
+          expand_row(h0, at);
+          expand_row(h1, at + 8192u);
+          if (__builtin_expect(tile < whole || tile >= part, 0)) {
+            const int j = tile * kRbTile + x;
+            if (j < S || j >= C) clear_row(at);
+            if (j + 64 < S || j + 64 >= C) clear_row(at + 8192u);
+          }
+          fence_proxy_async();
+          rb_tile_arrive(n & 3);
+          if (i + kTeams < ntl) fetch(i + kTeams);
+          const uint32_t t = at;
+          at = at_next, at_next = t;
+        }
+        if (tn < N && warp >= kRbAuxWarp) {  // the next block: operand A, its own keys' ranks
+          cp_async_wait_all();
+          if (abuf == 1) rb_wait(adone_bar, turn & 1, &abort_flag);  // a single operand A is free after the block's last tile
+          rb_bar<3, kRbAuxThreads>();
+          build_a(cur ^ 1, nrows, aux, kRbAuxThreads);
+          new_keys(cur ^ 1, it + ntl);
+        }
+      } else {
+        // (a reduction's result sits in a uniform register: the loop's counters and the descriptors then stay in those)
+        auto uniform = [](uint32_t v) { return (int)__reduce_max_sync(0xFFFFFFFFu, v); };
+        const int it_u = uniform(it), ntl_u = uniform(ntl), cur_u = uniform(cur);
+        const uint32_t tmem_u = uniform(tmem_base);
+        const uint64_t ad = a_desc_of(cur_u), xd = umma_desc_k128(smem_u32(Bx));
+        // index-column variants: the unit's first tile (protected first tokens) and its last (the budget ends in it)
+        const int first_i = S > 0 && rank == 0 ? 0 : -1, last_i = uniform(((nbase - 1 - rank) & (ncta - 1)) == 0 ? ntl : 0) - 1;
+        const int odd = warp - kRbMmaWarp;  // this warp's products: the even or the odd ones
+#pragma unroll 1
+        for (int i = (it_u ^ odd) & 1; i < ntl_u; i += 2) issue(it_u + i, tmem_u, ad, true, xd + (uint64_t)((i == first_i ? 2 : 0) + (i == last_i ? 4 : 0)));
+        if (abuf == 1 && tc_elect()) tc_commit(adone_bar);
+        __syncwarp();
+        if (tn < N && ((it_u + ntl_u) & 1) == odd) issue(it_u + ntl_u, tmem_u, a_desc_of(cur_u ^ 1), false, 0);
+      }
+      it += ntl + (tn < N ? 1 : 0);
+      if (warp < kRbResWarps && rows > 0) {
+        rb_bar<2, kRbResThreads>();  // the reader groups see each other's results
+        if (tid < ncta - 1) {        // ... and every peer gets this CTA's block
           const uint32_t peer = (uint32_t)((rank + 1 + tid) & (ncta - 1)), la = smem_u32(Mx + rank * L.mx_block);
           // the best keys, which the settling starts from, then the tiles' (1 KB each against 6 KB at 9830 slots and 8 CTAs)
           const uint32_t tops = la + 4u * (uint32_t)top_at;
-          rb_copy_to_peer(rb_mapa(tops, peer), tops, (uint32_t)(kRbReadGroups * RM) * 4u, rb_mapa(tops_bar, peer));
+          rb_copy_to_peer(rb_mapa(tops, peer), tops, (uint32_t)(kGroups * RM) * 4u, rb_mapa(tops_bar, peer));
           rb_copy_to_peer(rb_mapa(la, peer), la, 4u * (uint32_t)top_at, rb_mapa(peer_bar, peer));
         }
         __syncwarp();
-      } else if (warp < kRbMmaWarp) {
-        if (ncta > 1 && tid == 32 * kRbExpWarp) {
-          mbar_arrive_expect_tx(tops_bar, (uint32_t)(kRbReadGroups * RM * (ncta - 1)) * 4u);
-          mbar_arrive_expect_tx(peer_bar, 4u * (uint32_t)(top_at * (ncta - 1)));
-        }
-        const int x = tid & 127;  // this thread's row of both tiles of a pair
-        const uint32_t* base = codes + (rank * kRbTile + x) * WORDS;
-        const int tstep = (kRbTile * WORDS) << lg_ncta;  // words between this CTA's tiles
-        const int jstep = kRbTile << lg_ncta;            // ... slots
-        int j0 = rank * kRbTile + x;                     // this thread's slot of the pair's first tile
-        for (int p = 0; p < npair; ++p) {
-          uint32_t h0[WORDS], h1[WORDS];
-          const bool two = 2 * p + 1 < ntl;
-#pragma unroll
-          for (int w = 0; w < WORDS; ++w) {
-            h0[w] = base[2 * p * tstep + w];
-            h1[w] = two ? base[(2 * p + 1) * tstep + w] : 0u;
-          }
-          const int sx = stage_of(it + p);
-          if (!mbar_wait_warp(sfree_bar(sx), stage_phase(it + p) ^ 1, &abort_flag)) break;
-          expand_row(h0, j0 >= S && j0 < C, x, sx, 0);
-          expand_row(h1, j0 + jstep < C, x, sx, 1);
-          j0 += 2 * jstep;
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(full_bar(sx));
-        }
-      } else {
-        if (warp < kRbMmaWarp + 2) {
-          const uint64_t a_desc = a_desc_of(cur), x_desc = umma_desc_k128(smem_u32(Bx));
-          // index-column variants: the unit's first tile (protected first tokens) and its last (the budget ends in it)
-          const int first_i = S > 0 && rank == 0 ? 0 : -1, last_i = ((nbase - 1 - rank) & (ncta - 1)) == 0 ? ntl - 1 : -1;
-          for (int p = (it ^ warp) & 1; p < npair; p += 2) {  // pairs of this warp's parity
-            const int n = it + p, acc = n & 1, ph = (n >> 1) & 1, i = 2 * p, sx = stage_of(n);
-            const uint64_t bd = b_desc_of(sx, 0), bd1 = bd + (uint64_t)((WORDS == 2 ? 64 : 32) >> 4);
-            const uint64_t x0 = x_desc + (uint64_t)((i == first_i ? 2 : 0) + (i == last_i ? 4 : 0));
-            const uint64_t x1 = x_desc + (uint64_t)(i + 1 == last_i ? 4 : 0);
-            if (!mbar_wait2_warp(afree_bar(acc), ph ^ 1, full_bar(sx), stage_phase(n), &abort_flag)) break;
-            tc_fence_after();
-            if (tc_elect()) {
-              const uint32_t d = tmem_base + (uint32_t)(2 * acc * kRbTile);
-#pragma unroll
-              for (int w = 0; w < WORDS; ++w) rb_mma_f8(d, a_desc + (uint64_t)(2 * w), bd + (uint64_t)(2 * w), idesc, w > 0);
-              rb_mma_f8(d, a_desc + (uint64_t)(2 * WORDS), x0, idesc, true);
-              if (i + 1 < ntl) {
-#pragma unroll
-                for (int w = 0; w < WORDS; ++w) rb_mma_f8(d + kRbTile, a_desc + (uint64_t)(2 * w), bd1 + (uint64_t)(2 * w), idesc, w > 0);
-                rb_mma_f8(d + kRbTile, a_desc + (uint64_t)(2 * WORDS), x1, idesc, true);
-              }
-              tc_commit(afull_bar(acc));
-              tc_commit(sfree_bar(sx));
-            }
-            __syncwarp();
-          }
-          if (abuf == 1 && tc_elect()) tc_commit(adone_bar);
-          __syncwarp();
-        }
-        if (tn < N) {  // the next block: its codes and operand A (warps 14-15, meanwhile), its own keys' ranks (all four)
-          const int nrows = min(N - tn, R), first = tid - 32 * (kRbMmaWarp + 2);
-          if (first >= 0) {
-            stage_codes(cur ^ 1, tn, nrows, first, kRbBuildThreads);
-            cp_async_wait_all();
-            if (abuf == 1) mbar_wait(adone_bar, blk & 1, &abort_flag);  // a single operand A is free after the block's last tile
-            rb_bar<5, kRbBuildThreads>();
-            build_a(cur ^ 1, nrows, first, kRbBuildThreads);
-            fence_proxy_async();
-          }
-          rb_bar<3, kRbAuxThreads>();
-          new_keys(cur ^ 1, it + npair);
-        }
       }
-      it += npair + (tn < N ? 1 : 0);
       // ---------------------------------------------------------------- settle the block's steps
       // Owner table: the first step that claims a slot in this pass. Wide: the smallest of era | step, by an atomic minimum; eras
       // descend from pass to pass, so that older claims count as none and nothing is ever cleared: (own32 - era) < r says that a
       // step before r claims the slot. Narrow: own[slot] = step | pass parity << 7, (own ^ tag) < r says so (0xFF: nobody), and
       // claims of the pass before are taken back.
-      if (warp < kRbResWarps) {
+      if (warp < kRbResWarps && rows > 0) {
         tc_fence_before();
         const int r = tid;  // warps 0-3: this thread's step
         era -= 256u;
         if (wide && __builtin_expect(era < kRbLastEra, 0)) {  // (16 million passes on)
+#pragma unroll 1
           for (int j = tid; j < nbase * kRbTile; j += kRbResThreads) own32[j] = 0xFFFFFFFFu;
           era = kRbFirstEra;
           rb_bar<2, kRbResThreads>();
@@ -861,7 +887,10 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         bool forced = false, flagged = false;  // ... the best base slot holds a recent token; or a new entry may win
         if (warp < 4) {
           if (ncta > 1) rb_wait_cluster(tops_bar, blk & 1, &abort_flag);
-          for (int c = 0; c < kRbReadGroups * ncta; ++c) top = max(top, Mx[(c >> 1) * L.mx_block + top_at + (c & 1) * RM + (r < RM ? r : 0)]);
+#pragma unroll 1
+          for (int c = 0; c < ncta; ++c)
+#pragma unroll
+            for (int g = 0; g < kGroups; ++g) top = max(top, Mx[c * L.mx_block + top_at + g * RM + (r < RM ? r : 0)]);
           top_slot = max(0, min(kRbIdxMask - (top & kRbIdxMask), C - 1));
           sv = prev = top_slot;
           if (PROT && 32 * warp < Rn)  // REC[m] entered m + 1 steps before the block: recent while r + m < Rn
@@ -871,6 +900,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           if (tid < 2) s_change[tid] = kRbRows;
         }
         int fb = 0;                    // steps below are final
+#pragma unroll 1
         for (int pass = 0;; ++pass) {  // every pass but the last of a window makes at least one more step final
           const int wend = min(fb + (pass < kRbWidePasses ? kRbRows : kRbResWarps), rows);
           const uint32_t tag = (uint32_t)(pass & 1) << 7;
@@ -891,6 +921,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
                 if (warp == k && mine) own[sv] = (uint8_t)((uint32_t)r | tag);
                 rb_bar<1, kRbRows>();
               }
+#pragma unroll 1
               for (;;) {
                 const uint32_t o = own[sv] ^ tag;
                 const bool again = mine && (int)(o >> 5) == warp && o > (uint32_t)r;
@@ -921,6 +952,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             const int walk = rb_walk_cost(WORDS, GT, PROT, (C + kRbResThreads - 1) / kRbResThreads);
             if (pass * rb_pass_cost(n3) > 2 * fb * walk && 2 * pass * (rows - fb) > rows) break;  // the rest is walked
           }
+#pragma unroll 1
           for (int e0 = warp; e0 < n3; e0 += kRbResWarps) {
             const int entry = LIST[e0 < n1 ? (e0 < n0 ? e0 : 32 + e0 - n0) : (e0 < n2 ? 64 + e0 - n1 : 96 + e0 - n2)];
             const int r2 = entry & 127;
@@ -945,6 +977,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             int mt[4];  // lane l: tiles l, l + 32, ...
             RbRank<WORDS, GT> rk;
             int live = -1;  // best live slot of the tiles scanned so far, this lane's share
+#pragma unroll 1
             for (int round = 0; round <= nbase + kRbRows; ++round) {
               if (kn > kb) {
                 const uint32_t slot = (uint32_t)(kRbIdxMask - (kn & kRbIdxMask));
@@ -971,6 +1004,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
                 bool bad = wide ? own32[sb] - era < (uint32_t)r2 : (own[sb] ^ tag) < (uint32_t)r2;
                 if (PROT && r2 < Rn && !bad) {  // REC[m - 1] entered m steps before the block: recent while r2 + m <= Rn
                   bool hit = false;
+#pragma unroll 1
                   for (int m0 = 0; m0 < Rn - r2; m0 += 32) hit |= m0 + lane < Rn - r2 && REC[m0 + lane] == sb;
                   bad = __any_sync(0xFFFFFFFFu, hit);
                 }
@@ -999,6 +1033,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
                 ok4 = (((o4 | 0x80808080u) - (uint32_t)r2 * 0x01010101u) | o4);
               }
               if (PROT && r2 < Rn)
+#pragma unroll 1
                 for (int m0 = 0; m0 < Rn - r2; ++m0) {
                   const int q = REC[m0] - j0;
                   if (q >= 0 && q < 4) ok4 &= ~(0x80u << (8 * q));
@@ -1065,6 +1100,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
               if (warp == k && in) own[sv] = (uint8_t)r;
               rb_bar<1, kRbRows>();
             }
+#pragma unroll 1
             for (;;) {
               const int o = own[sv];
               const bool again = in && (o >> 5) == warp && o < r;
@@ -1088,6 +1124,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           rb_bar<2, kRbResThreads>();
           RbRank<WORDS, GT> rk;
           rk.load(qb + (rows - 1) * GW, G, PAR[cur * kRbRows + rows - 1]);
+#pragma unroll 1
           for (int j = rank * kRbResThreads + tid; j < C; j += ncta * kRbResThreads) {
             uint32_t h[WORDS];
 #pragma unroll
@@ -1102,8 +1139,11 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           if (tid < Rn) REC[tid] = tid < rows ? (int)SV[rows - 1 - tid] : keep;
         }
       }
-      ++blk;
+      blk += rows > 0 ? 1 : 0;
+      ++turn;
       cur ^= 1;
+      t0 = tn;
+      rows = min(N - tn, R);
       __syncthreads();
       tc_fence_after();
     }
@@ -1124,10 +1164,14 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
     __syncthreads();  // the tables and s_unit are reused by the next unit
   }
 
+  // The readers' last arrivals still stand in the tile barriers: their phases are completed.
+  if (warp == kRbAuxWarp || warp == kRbAuxWarp + 1)
+    for (int x = 0; x < kRbAccs; ++x) rb_tile_arrive(x);
   // A CTA that gave up must not free tensor memory under an MMA that is still writing it (the operands are written by
-  // this CTA's own threads, so no copy from outside is ever in flight): one more commit of each MMA warp tracks everything
-  // it has issued, and their completion is awaited (bounded) first.
+  // this CTA's own threads, so no copy from outside is ever in flight): one more commit tracks everything that the issuing
+  // warp has issued, and its completion is awaited (bounded) first.
   if (warp == kRbMmaWarp || warp == kRbMmaWarp + 1) {
+    for (int x = warp - kRbMmaWarp; x < kRbAccs; x += 2) rb_tile_sync(x);
     const bool gave_up = __any_sync(0xFFFFFFFFu, abort_flag != 0);  // one answer for the warp: the election wants all its lanes
     if (gave_up && tc_elect()) {
       tc_commit(drain_bar);
@@ -1138,7 +1182,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   __syncthreads();
   if (warp == kRbMmaWarp) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(4 * kRbTile) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kRbAccs * kRbTile) : "memory");
   }
   if (tid == 0 && abort_flag) atomicAdd(&g_tc_error, 1);
   if (ncta > 1) rb_cluster_sync();  // no CTA leaves while a peer may still copy into its shared memory
