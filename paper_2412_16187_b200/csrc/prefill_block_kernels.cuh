@@ -49,10 +49,11 @@
 // latency of the hand-overs around them: 100 cycles for a wait on a completed mbarrier and 170 from an arrival to the waiter, 260 from
 // the last MMA to its commit. So every tile has an accumulator of its own (pairs of tiles, with two groups and two accumulator pairs, took
 // 630 cycles a pair), a freed accumulator and a written operand tile meet the issuing warp in ONE named barrier (45 cycles; two mbarriers
-// 120), and no warp handles more than every second tile. A tile now takes 245 cycles with one word at 9830 slots. In a program of the tile
+// 120), and no warp handles more than every second tile. A tile now takes 235 cycles with one word at 9830 slots. In a program of the tile
 // phase alone: three groups 201, two 246, one 393 (in this kernel a single issuing warp is the bound, at 290 to 430 cycles a tile); two words
-// 271 with three groups and 285 with two; with mbarriers instead 235 to 290. Replay of 256 units of 9830 slots: 5630 -> 4800 us; of 512 units of
-// 512 to 4096 slots, two words, 835 -> 810 (840 with three groups and four expanding warps).
+// 271 with three groups and 285 with two; with mbarriers instead 235 to 290. Here two words take two groups, so that eight warps expand:
+// replay of 512 units of 512 to 4096 slots 835 -> 810 us (840 with three groups and four expanding warps); of 256 units of 9830 slots, one word, 5630 ->
+// 4800 us (5400 with two groups).
 // Every wait on an mbarrier is bounded; a CTA that gives up raises a flag that turns its later waits into no-ops, but it
 // still walks the same blocks and cluster barriers as its peers (their copies into its shared memory must find it), then
 // releases tensor memory and raises the device error counter.
@@ -262,8 +263,8 @@ __device__ __forceinline__ void rb_arrive_remote(uint32_t bar) {
 }
 // mbar_wait_warp with its loop left rolled: unrolled by the compiler, each of this kernel's waits was 5 KB of code, half of the kernel's 143 KB
 // (128 units of 1024 slots, b = 16, windows, the kernel otherwise as it was: 1290 -> 1230 us).
-__device__ __forceinline__ bool rb_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  if (__builtin_expect(__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)), 1)) return true;
+__device__ __forceinline__ bool rb_wait_polled(bool done, uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  if (__builtin_expect(__all_sync(0xFFFFFFFFu, done), 1)) return true;
   bool ok = false, on = true;
 #pragma unroll 1
   for (uint32_t i = 0; i < kTcSpinLimit && on; ++i) {
@@ -272,6 +273,9 @@ __device__ __forceinline__ bool rb_wait(uint32_t bar, uint32_t parity, volatile 
   }
   if (!ok) *abort_flag = 1;
   return __all_sync(0xFFFFFFFFu, ok);
+}
+__device__ __forceinline__ bool rb_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return rb_wait_polled(mbar_try_wait(bar, parity), bar, parity, abort_flag);
 }
 // Bounded wait for copies and arrivals of other CTAs of the cluster.
 __device__ __forceinline__ bool rb_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
@@ -303,6 +307,98 @@ __device__ __forceinline__ void rb_bar() {
 constexpr int kRbTileBarThreads = 128 + 64 + 32;
 __device__ __forceinline__ void rb_tile_arrive(int acc) { asm volatile("bar.arrive %0, %1;" ::"r"(kRbTileBar + acc), "n"(kRbTileBarThreads) : "memory"); }
 __device__ __forceinline__ void rb_tile_sync(int acc) { asm volatile("bar.sync %0, %1;" ::"r"(kRbTileBar + acc), "n"(kRbTileBarThreads) : "memory"); }
+
+// The loops of the tile phase, and the preparation of the next block. Functions of their own, so that their registers and their code
+// don't change with what the settling around them needs: inlined, a change of the settling moved a tile by 4 % either way. Replay, us
+// inlined / as functions: 256 units of 9830 slots 4970 / 4600, 512 of 512 to 4096, two words, 810 / 763, 128 of 1024 with windows 1228 / 1182,
+// 8 of 9830 1155 / 1140. (The evaluation of a hard step as a function: 1182 -> 1328, its caller's registers go to the stack.)
+// `bars`: the products' mbarriers (product n's is n mod 8, its phase n / 8).
+__device__ __forceinline__ uint32_t rb_done_bar(uint32_t bars, int n) { return bars + 8u * (uint32_t)(n & (kRbDoneBars - 1)); }
+__device__ __forceinline__ uint32_t rb_done_phase(int n) { return (uint32_t)(n >> 3) & 1u; }
+
+// One group's tiles i = grp, grp + GROUPS, ...: the best key of each into mrow[i]. taddr: this warp's lanes of the first accumulator; ct: 127 - tile of
+// the unit goes above the index within the tile (lower tiles first), cstep less from tile to tile. Returns the best of all.
+template <int GROUPS>
+__device__ __noinline__ int rb_read_tiles(uint32_t bars, volatile int* abort_flag, int it, int grp, int ntl, uint32_t taddr, uint32_t mrow, int ct, int cstep) {
+  int top = -1;
+#pragma unroll 1
+  for (int i = grp; i < ntl; i += GROUPS) {
+    const int n = it + i, acc = n & 3;
+    rb_wait(rb_done_bar(bars, n), rb_done_phase(n), abort_flag);
+    tc_fence_after();
+    uint32_t v0[32], v1[32];
+    rb_ld64_low(taddr + (uint32_t)(acc * kRbTile), v0);
+    rb_ld64_low(taddr + (uint32_t)(acc * kRbTile) + 64, v1);
+    rb_wait_ld(v0);
+    rb_wait_ld(v1);
+    tc_fence_before();  // the accumulator goes back
+    rb_tile_arrive(acc);
+    const uint32_t m = rb_max64(v0, v1);
+    // the tile's best key, 2^14 rank + index; negative: no slot of the tile may win
+    const int k16 = (int)max(m & 0xFFFFu, m >> 16) - 1, key = ((k16 & ~127) << 7) + (k16 & 127) + ct;
+    ct -= cstep;
+    top = max(top, key);
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(mrow + 4u * (uint32_t)i), "r"(key) : "memory");
+  }
+  return top;
+}
+
+__device__ __forceinline__ void rb_st_chunk(uint32_t at, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v0), "r"(v1), "r"(v2), "r"(v3) : "memory");
+}
+// A slot's or a key's code as a row of an operand tile whose first chunk is at `at` (a multiple of the row's chunks, so chunk c is at `at` xor c).
+template <int WORDS>
+__device__ __forceinline__ void rb_expand_row(const uint32_t (&h)[WORDS], uint32_t at) {
+#pragma unroll
+  for (int c = 0; c < 2 * WORDS; ++c) {
+    const uint32_t hw = h[c >> 1];
+    const int m = (c & 1) * 4;
+    rb_st_chunk(at ^ (uint32_t)(c << 4), rb_expand4(hw, m), rb_expand4(hw, m + 1), rb_expand4(hw, m + 2), rb_expand4(hw, m + 3));
+  }
+}
+template <int WORDS>
+__device__ __forceinline__ void rb_clear_row(uint32_t at) {
+#pragma unroll
+  for (int c = 0; c < 2 * WORDS; ++c) rb_st_chunk(at ^ (uint32_t)(c << 4), 0u, 0u, 0u, 0u);
+}
+
+// One team's tiles i, i + TEAMS, ...: rows x and x + 64 (8 KB further on) of the tile by a thread. src: the thread's first code of the CTA's tile 0, step:
+// bytes from tile to tile; at, at_next: where its row is in this tile and the next. The CTA's tiles below `whole` and from `part` on hold slots that
+// may not win: those below S and from C on, with j the thread's first slot of tile 0 and jstep slots from tile to tile.
+template <int WORDS, int TEAMS>
+__device__ __noinline__ void rb_expand_tiles(uint32_t bars, volatile int* abort_flag, int it, int i, int ntl, uint32_t src, uint32_t step, uint32_t at, uint32_t at_next, int j,
+                                             int jstep, int S, int C) {
+  uint32_t h0[WORDS], h1[WORDS];
+  auto fetch = [&](int t) {
+    const uint32_t from = src + step * (uint32_t)t;
+    if (WORDS == 2) {
+      asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(h0[0]), "=r"(h0[WORDS - 1]) : "r"(from));
+      asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(h1[0]), "=r"(h1[WORDS - 1]) : "r"(from + 64u * 4u * WORDS));
+    } else {
+      asm volatile("ld.shared.b32 %0, [%1];" : "=r"(h0[0]) : "r"(from));
+      asm volatile("ld.shared.b32 %0, [%1];" : "=r"(h1[0]) : "r"(from + 64u * 4u));
+    }
+  };
+  if (i < ntl) fetch(i);
+#pragma unroll 1
+  for (; i < ntl; i += TEAMS) {
+    const int n = it + i;
+    rb_wait(rb_done_bar(bars, n - 4), rb_done_phase(n - 4), abort_flag);  // product n - 4 is done with the operand tile
+    rb_expand_row<WORDS>(h0, at);
+    rb_expand_row<WORDS>(h1, at + 8192u);
+    const int j0 = j + jstep * i;
+    if (__any_sync(0xFFFFFFFFu, j0 < S || j0 + 64 >= C)) {  // some slots of the tile may not win
+      if (j0 < S || j0 >= C) rb_clear_row<WORDS>(at);
+      if (j0 + 64 < S || j0 + 64 >= C) rb_clear_row<WORDS>(at + 8192u);
+      __syncwarp();
+    }
+    fence_proxy_async();
+    rb_tile_arrive(n & 3);
+    if (i + TEAMS < ntl) fetch(i + TEAMS);
+    const uint32_t t = at;
+    at = at_next, at_next = t;
+  }
+}
 
 // Rank of one slot's code at a step from the packed words. GT = 4 uses the bit-plane form, which yields (D - pc) / 2 with pc
 // the bits set in the exclusive or of the step's query codes (`parity_bits`, worked out with operand A).
@@ -441,6 +537,168 @@ __device__ __noinline__ void rb_walk(const RbLayout& L, bool wide, int base, int
   if (PROT && tid < Rn) mark(newest(rows, tid + 1), ~0u);
 }
 
+// First chunk of row x of operand tile sx, as an offset into operand B.
+template <int WORDS>
+__device__ __forceinline__ uint32_t rb_row_at(int x, int sx) {
+  const int c0 = WORDS == 2 ? 4 * (sx & 1) : 2 * sx;
+  return (uint32_t)((WORDS == 2 ? sx >> 1 : 0) * kRbAtom + (x >> 3) * 1024 + (x & 7) * 128 + ((c0 ^ (x & 7)) << 4));
+}
+
+// Scaling of the operands (file comment): data columns' sum + off - 64 parity (even G) = 128 * rank.
+__device__ __forceinline__ int rb_alpha(int G) { return (G & 1) == 0 ? 16 : 32; }
+template <int WORDS>
+__device__ __forceinline__ int rb_off(int G) {
+  return 2 * rb_alpha(G) * G * 32 * WORDS;
+}
+
+// An issuing warp's products of a turn, the even (odd = 0) or the odd ones: the block's tiles with operand A at `a`, then, if there is a next block,
+// its own keys (product it + ntl, no index columns) with operand A at `a_next`. bidx, b: index columns and operand tiles. first, last: the
+// tiles that take the index-column variants (-1: none). adone: mbarrier to tell when the tiles are multiplied (0: nobody asks).
+template <int WORDS>
+__device__ __noinline__ void rb_issue_tiles(uint32_t bars, int it_, int ntl_, int odd, uint32_t tmem_, uint32_t a_, uint32_t a_next_, uint32_t bidx_, uint32_t b_, int first,
+                                            int last, uint32_t adone, bool next) {
+  // (a reduction's result sits in a uniform register: the loop's counters and the descriptors then stay in those)
+  auto uniform = [](uint32_t v) { return __reduce_max_sync(0xFFFFFFFFu, v); };
+  const int it = (int)uniform((uint32_t)it_), ntl = (int)uniform((uint32_t)ntl_), first_i = (int)uniform((uint32_t)(first + 1)) - 1, last_i = (int)uniform((uint32_t)(last + 1)) - 1;
+  const uint32_t tmem = uniform(tmem_);
+  const uint64_t ad = umma_desc_k128(uniform(a_)), ad_next = umma_desc_k128(uniform(a_next_)), xd = umma_desc_k128(uniform(bidx_)), bd0 = umma_desc_k128(uniform(b_));
+  // instruction descriptor: fp32 accumulate, e5m2 x e4m3, both operands K-major, N = 128, M = 128
+  const uint32_t idesc = (1u << 4) | (1u << 7) | ((uint32_t)(kRbTile >> 3) << 17) | ((uint32_t)(kRbRows >> 4) << 24);
+  auto issue = [&](int n, uint64_t a, bool index, uint64_t x) {
+    const int acc = n & 3;
+    const uint64_t bd = bd0 + (uint64_t)((WORDS == 2 ? (acc >> 1) * kRbAtom + (acc & 1) * 64 : acc * 32) >> 4);
+    rb_tile_sync(acc);
+    tc_fence_after();
+    if (tc_elect()) {
+      const uint32_t d = tmem + (uint32_t)(acc * kRbTile);
+#pragma unroll
+      for (int w = 0; w < WORDS; ++w) rb_mma_f8(d, a + (uint64_t)(2 * w), bd + (uint64_t)(2 * w), idesc, w > 0);
+      if (index) rb_mma_f8(d, a + (uint64_t)(2 * WORDS), x, idesc, true);
+      tc_commit(rb_done_bar(bars, n));
+    }
+    __syncwarp();
+  };
+#pragma unroll 1
+  for (int i = (it ^ odd) & 1; i < ntl; i += 2) issue(it + i, ad, true, xd + (uint64_t)((i == first_i ? 2 : 0) + (i == last_i ? 4 : 0)));
+  if (adone != 0u && tc_elect()) tc_commit(adone);
+  __syncwarp();
+  if (next && ((it + ntl) & 1) == odd) issue(it + ntl, ad_next, false, 0);
+}
+
+// Warps 12-15 prepare a block in buffer `buf`: operand A from the queries' codes, then the ranks of its own keys at its steps (product n).
+template <int WORDS, int GT, bool PROT, int RM>
+__device__ __noinline__ void rb_prepare(const RbLayout& L, int base, int buf, int nrows, int n, int G_, int Rn, int abuf, uint32_t bars, volatile int* abort_flag,
+                                        uint32_t tmem_base) {
+  const int tid = threadIdx.x, warp = tid >> 5, first = tid & (kRbAuxThreads - 1);
+  const int G = GT > 0 ? GT : G_, GW = G * WORDS;
+  unsigned char* smem = rb_smem_raw + base;
+  const uint32_t* kraw = reinterpret_cast<const uint32_t*>(smem + L.kraw);
+  int32_t* PAR = reinterpret_cast<int32_t*>(smem + L.par);
+  int32_t* NR = reinterpret_cast<int32_t*>(smem + L.nr);
+  uint16_t* Dn = reinterpret_cast<uint16_t*>(smem + L.dn);
+  const bool even = (G & 1) == 0;
+  const int alpha = rb_alpha(G), off = rb_off<WORDS>(G);
+  // the e5m2 codes of -alpha (2 c - G) for c = 0..7 set bits among the group's queries, as two words of a byte table; c = 8 (G = 8 only) is
+  // patched where it occurs
+  uint32_t lut_lo = 0u, lut_hi = 0u;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    lut_lo |= rb_e5m2(-alpha * (2 * c - G)) << (8 * c);
+    lut_hi |= (c + 4 <= G ? rb_e5m2(-alpha * (2 * (c + 4) - G)) : 0u) << (8 * c);
+  }
+  // operand A, row r = step r of the block: -alpha u_t, then the five further columns; one thread per (row, word)
+  const uint32_t* qd = reinterpret_cast<const uint32_t*>(smem + L.qraw) + buf * kRbRows * GW;
+  unsigned char* ad = smem + L.a + (WORDS == 2 && abuf > 1 ? buf * kRbAtom : 0);
+  const int c0 = WORDS == 1 && abuf > 1 ? 4 * buf : 0;
+#pragma unroll 1
+  for (int item = first; item < kRbRows * WORDS; item += kRbAuxThreads) {
+    const int r = item & (kRbRows - 1), w = item >> 7;
+    const bool valid = r < nrows;
+    uint32_t cnt[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) cnt[m] = 0u;
+    if (valid)
+      for (int g = 0; g < G; ++g) {
+        const uint32_t x = qd[r * GW + g * WORDS + w];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) cnt[m] += (x >> m) & 0x01010101u;  // set bits among the queries, one counter per byte
+      }
+    uint32_t v[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const uint32_t t = cnt[m] | (cnt[m] >> 4);
+      v[m] = __byte_perm(lut_lo, lut_hi, __byte_perm(t, 0u, 0x4420));
+      // eight of eight: -128 = 0xD8 (selector 8 made the lookup give 0 there)
+      if (GT == 0) v[m] |= (cnt[m] & 0x08080808u) * 0x1Bu;
+      if (!valid) v[m] = 0u;
+    }
+    *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * w)) = make_uint4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * w + 1)) = make_uint4(v[4], v[5], v[6], v[7]);
+    if (w == 0) {
+      int pc = 0;
+      if (even && valid) {
+#pragma unroll
+        for (int v2 = 0; v2 < WORDS; ++v2) {
+          uint32_t x = 0u;
+          for (int g = 0; g < G; ++g) x ^= qd[r * GW + g * WORDS + v2];
+          pc += __popc(x);
+        }
+      }
+      PAR[buf * kRbRows + r] = pc;
+      *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * WORDS)) =
+          valid ? make_uint4(0x4Cu | (0x3Cu << 8) | (0x78u << 16) | (rb_e5m2(off) << 24), (pc & 1) ? 0xD4u : 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * WORDS + 1)) = make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+  // The ranks: one more tile, without index columns. Also each step's largest rank of any key that enters before it (and is no longer recent):
+  // no new entry can beat that.
+  const int x = tid & 127, acc = n & 3;
+  rb_wait(rb_done_bar(bars, n - 4), rb_done_phase(n - 4), abort_flag);
+  uint32_t h[WORDS];
+#pragma unroll
+  for (int w = 0; w < WORDS; ++w) h[w] = kraw[(buf * kRbRows + x) * WORDS + w];
+  rb_expand_row<WORDS>(h, smem_u32(smem + L.b) + rb_row_at<WORDS>(x, acc));
+  fence_proxy_async();
+  rb_bar<3, kRbAuxThreads>();
+  if (warp < kRbAuxWarp + 2) rb_tile_arrive(acc);
+  rb_wait(rb_done_bar(bars, n), rb_done_phase(n), abort_flag);
+  tc_fence_after();
+  // Conversions by an fp32 addition (the integer conversions run at a sixteenth of its rate): 2^22 + rank has 2 * rank
+  // in its low bits, which is what is kept.
+  const int r = x, last = PROT ? r - Rn : r;  // entries below `last` are candidates
+  const float magic = (float)(off - ((PAR[buf * kRbRows + r] & 1) << 6)) * (1.f / 128.f) + 4194304.f;
+  const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(acc * kRbTile);
+  uint16_t* dst = Dn + buf * L.dn_buf + rb_dn_at(r, RM);
+  float dmax = -1e9f;
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {
+    uint32_t v[32];
+    tc_ld32(taddr + c * 32, v);
+    tc_wait_ld();
+    if (c == 3) {
+      tc_fence_before();
+      rb_tile_arrive(acc);
+    }
+    if (c > (warp & 3)) continue;  // no step of this warp comes after those keys
+    const int lc = last - c * 32;
+#pragma unroll
+    for (int k = 0; k < 32; ++k)
+      if (k < lc) dmax = fmaxf(dmax, __uint_as_float(v[k]));
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      uint32_t pk[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float y0 = fmaf(__uint_as_float(v[4 * k + 2 * e]), 1.f / 128.f, magic);
+        const float y1 = fmaf(__uint_as_float(v[4 * k + 2 * e + 1]), 1.f / 128.f, magic);
+        pk[e] = __byte_perm(__float_as_uint(y0), __float_as_uint(y1), 0x5410);
+      }
+      if (c * 32 + 4 * k < r && r < RM) *reinterpret_cast<uint2*>(dst + c * 32 + 4 * k) = make_uint2(pk[0], pk[1]);
+    }
+  }
+  NR[buf * kRbRows + r] = last > 0 ? (int)(__float_as_uint(fmaf(dmax, 1.f / 128.f, magic)) & 0xFFFFu) >> 1 : -1;
+}
+
 // PROT: protected windows (Section 4 setup). The first n_sink tokens never leave slots 0 .. n_sink-1, so those slots are
 // masked like slots past the budget. A recent token that is already in the table is recognised by the list of the newest
 // slots, one of this block's own keys by its step. Needs every budget > n_sink + n_recent (so that some slot is always
@@ -459,8 +717,9 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   __shared__ volatile int abort_flag;
   __shared__ int s_unit[2];
   __shared__ int s_change[2];                    // by pass parity: first step that changed
-  __shared__ __align__(4) uint8_t s_hard[2][4];  // by pass parity: lengths of warps 0-3's lists of hard steps
-  static_assert(sizeof(bars) + sizeof(tmem_base_s) + sizeof(abort_flag) + sizeof(s_unit) + sizeof(s_change) + sizeof(s_hard) <= kRbStaticSmem,
+  __shared__ __align__(4) uint8_t s_hard[2][4];   // by pass parity: lengths of warps 0-3's lists of hard steps
+  __shared__ __align__(4) uint8_t s_stale[2][4];  // ... and of the stale ones at their heads
+  static_assert(sizeof(bars) + sizeof(tmem_base_s) + sizeof(abort_flag) + sizeof(s_unit) + sizeof(s_change) + sizeof(s_hard) + sizeof(s_stale) <= kRbStaticSmem,
                 "the host sizes the dynamic shared memory beside these");
 
   griddep_launch_dependents();
@@ -497,8 +756,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   const int a_step = WORDS == 2 ? kRbAtom : 64;             // bytes between the two buffers of operand A
 
   const uint32_t bar0 = smem_u32(bars);
-  auto done_bar = [&](int n) { return bar0 + 8u * (n & (kRbDoneBars - 1)); };  // product n is complete: its accumulator may be read, its operand tile rewritten
-  auto done_phase = [&](int n) { return (uint32_t)(n >> 3) & 1u; };
+  // bar0 ..: product n mod 8 is complete, its accumulator may be read and its operand tile rewritten
   const uint32_t peer_bar = bar0 + 8u * kRbDoneBars;           // peers' copies of their tiles' maxima have arrived
   const uint32_t used_bar = bar0 + 8u * (kRbDoneBars + 1);     // peers: they are done with this CTA's maxima
   const uint32_t adone_bar = bar0 + 8u * (kRbDoneBars + 2);    // one operand A buffer: the block's tiles are multiplied
@@ -508,7 +766,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
     abort_flag = 0;
     mbar_init(drain_bar, 2);
     mbar_init(adone_bar, 2);
-    for (int i = 0; i < kRbDoneBars; ++i) mbar_init(done_bar(i), 1);
+    for (int i = 0; i < kRbDoneBars; ++i) mbar_init(rb_done_bar(bar0, i), 1);
     mbar_init(peer_bar, 1);
     mbar_init(tops_bar, 1);
     mbar_init(used_bar, ncta > 1 ? ncta - 1 : 1);
@@ -519,17 +777,6 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // Scaling of the operands (file comment) and the e5m2 codes of -alpha (2 c - G) for c = 0..7 set bits among the group's
-  // queries, as two words of a byte table; c = 8 (G = 8 only) is patched where it occurs.
-  const bool even = (G & 1) == 0;
-  const int alpha = even ? 16 : 32;
-  const int off = 2 * alpha * G * 32 * WORDS;  // data columns' sum + off - 64 parity (even G) = 128 * rank
-  uint32_t lut_lo = 0u, lut_hi = 0u;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    lut_lo |= rb_e5m2(-alpha * (2 * c - G)) << (8 * c);
-    lut_hi |= (c + 4 <= G ? rb_e5m2(-alpha * (2 * (c + 4) - G)) : 0u) << (8 * c);
-  }
   if (!wide)
 #pragma unroll 1
     for (int i = tid; i < a.smem_slots / 4; i += NT) own32[i] = 0xFFFFFFFFu;
@@ -539,8 +786,6 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   if (ncta > 1) rb_cluster_sync();  // every CTA of the cluster runs before anyone copies into it
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
-  // instruction descriptor: fp32 accumulate, e5m2 x e4m3, both operands K-major, N = 128, M = 128
-  const uint32_t idesc = (1u << 4) | (1u << 7) | ((uint32_t)(kRbTile >> 3) << 17) | ((uint32_t)(kRbRows >> 4) << 24);
   // Tiles so far; every role counts the same sequence. Tile n lives in operand tile and accumulator n mod 4; warp 16 + (n mod 2) issues its
   // product, so that the even and the odd products each complete in order. A wait for product n may only be begun once product n - 8
   // is known to be complete (the barrier's phases alternate): readers have read product n - 6 before it or come from a block's start, where
@@ -616,142 +861,6 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(kd + i)), "l"(ks + i) : "memory");
       cp_async_commit();
     };
-    // Operand A, row r = step r of the block: -alpha u_t, then the five further columns. One thread per (row, word).
-    auto build_a = [&](int buf, int nrows, int first, int nthreads) {
-      const uint32_t* qd = qraw + buf * kRbRows * GW;
-      unsigned char* ad = As + (WORDS == 2 && abuf > 1 ? buf * kRbAtom : 0);
-      const int c0 = WORDS == 1 && abuf > 1 ? 4 * buf : 0;
-#pragma unroll 1
-      for (int item = first; item < kRbRows * WORDS; item += nthreads) {
-        const int r = item & (kRbRows - 1), w = item >> 7;
-        const bool valid = r < nrows;
-        uint32_t cnt[8];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) cnt[m] = 0u;
-        if (valid)
-          for (int g = 0; g < G; ++g) {
-            const uint32_t x = qd[r * GW + g * WORDS + w];
-#pragma unroll
-            for (int m = 0; m < 8; ++m) cnt[m] += (x >> m) & 0x01010101u;  // set bits among the queries, one counter per byte
-          }
-        uint32_t v[8];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          const uint32_t t = cnt[m] | (cnt[m] >> 4);
-          v[m] = __byte_perm(lut_lo, lut_hi, __byte_perm(t, 0u, 0x4420));
-          // eight of eight: -128 = 0xD8 (selector 8 made the lookup give 0 there)
-          if (GT == 0) v[m] |= (cnt[m] & 0x08080808u) * 0x1Bu;
-          if (!valid) v[m] = 0u;
-        }
-        *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * w)) = make_uint4(v[0], v[1], v[2], v[3]);
-        *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * w + 1)) = make_uint4(v[4], v[5], v[6], v[7]);
-        if (w == 0) {
-          int pc = 0;
-          if (even && valid) {
-#pragma unroll
-            for (int v2 = 0; v2 < WORDS; ++v2) {
-              uint32_t x = 0u;
-              for (int g = 0; g < G; ++g) x ^= qd[r * GW + g * WORDS + v2];
-              pc += __popc(x);
-            }
-          }
-          PAR[buf * kRbRows + r] = pc;
-          *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * WORDS)) =
-              valid ? make_uint4(0x4Cu | (0x3Cu << 8) | (0x78u << 16) | (rb_e5m2(off) << 24), (pc & 1) ? 0xD4u : 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
-          *reinterpret_cast<uint4*>(ad + rb_swz(r, c0 + 2 * WORDS + 1)) = make_uint4(0u, 0u, 0u, 0u);
-        }
-      }
-    };
-    // Shared-memory address of the first chunk of row x of operand tile sx.
-    auto row_at = [&](int x, int sx) {
-      const int c0 = WORDS == 2 ? 4 * (sx & 1) : 2 * sx;
-      return smem_u32(Bs) + (uint32_t)((WORDS == 2 ? sx >> 1 : 0) * kRbAtom + (x >> 3) * 1024 + (x & 7) * 128 + ((c0 ^ (x & 7)) << 4));
-    };
-    auto st_chunk = [](uint32_t at, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3) {
-      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v0), "r"(v1), "r"(v2), "r"(v3) : "memory");
-    };
-    // A slot's or a key's code as a row (c0 is a multiple of the row's chunks, so chunk c is where c0 is, xor c).
-    auto expand_row = [&](const uint32_t* h, uint32_t at) {
-#pragma unroll
-      for (int c = 0; c < 2 * WORDS; ++c) {
-        const uint32_t hw = h[c >> 1];
-        const int m = (c & 1) * 4;
-        st_chunk(at ^ (uint32_t)(c << 4), rb_expand4(hw, m), rb_expand4(hw, m + 1), rb_expand4(hw, m + 2), rb_expand4(hw, m + 3));
-      }
-    };
-    auto clear_row = [&](uint32_t at) {
-#pragma unroll
-      for (int c = 0; c < 2 * WORDS; ++c) st_chunk(at ^ (uint32_t)(c << 4), 0u, 0u, 0u, 0u);
-    };
-    auto a_desc_of = [&](int buf) { return umma_desc_k128(smem_u32(As)) + (uint64_t)((abuf > 1 ? buf * a_step : 0) >> 4); };
-    auto b_desc_of = [&](int sx) {
-      return umma_desc_k128(smem_u32(Bs)) + (uint64_t)((WORDS == 2 ? (sx >> 1) * kRbAtom + (sx & 1) * 64 : sx * 32) >> 4);
-    };
-    // Product n of operand A `buf` with operand tile n mod 4, by the issuing warp; xd: index columns, none for a block's own keys.
-    auto issue = [&](int n, uint32_t tmem, uint64_t ad, bool index, uint64_t xd) {
-      const int acc = n & 3;
-      const uint64_t bd = b_desc_of(acc);
-      rb_tile_sync(acc);
-      tc_fence_after();
-      if (tc_elect()) {
-        const uint32_t d = tmem + (uint32_t)(acc * kRbTile);
-#pragma unroll
-        for (int w = 0; w < WORDS; ++w) rb_mma_f8(d, ad + (uint64_t)(2 * w), bd + (uint64_t)(2 * w), idesc, w > 0);
-        if (index) rb_mma_f8(d, ad + (uint64_t)(2 * WORDS), xd, idesc, true);
-        tc_commit(done_bar(n));
-      }
-      __syncwarp();
-    };
-    // Ranks of a block's own keys (buffer `buf`) at its steps, by warps 12-15: one more tile, as product n, without index
-    // columns. Also each step's largest rank of any key that enters before it (and is no longer recent): no new entry can
-    // beat that.
-    auto new_keys = [&](int buf, int n) {
-      const int x = tid & 127, acc = n & 3;
-      rb_wait(done_bar(n - 4), done_phase(n - 4), &abort_flag);
-      uint32_t h[WORDS];
-#pragma unroll
-      for (int w = 0; w < WORDS; ++w) h[w] = kraw[(buf * kRbRows + x) * WORDS + w];
-      expand_row(h, row_at(x, acc));
-      fence_proxy_async();
-      rb_bar<3, kRbAuxThreads>();
-      if (warp < kRbAuxWarp + 2) rb_tile_arrive(acc);
-      rb_wait(done_bar(n), done_phase(n), &abort_flag);
-      tc_fence_after();
-      // Conversions by an fp32 addition (the integer conversions run at a sixteenth of its rate): 2^22 + rank has 2 * rank
-      // in its low bits, which is what is kept.
-      const int r = x, last = PROT ? r - Rn : r;  // entries below `last` are candidates
-      const float magic = (float)(off - ((PAR[buf * kRbRows + r] & 1) << 6)) * (1.f / 128.f) + 4194304.f;
-      const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(acc * kRbTile);
-      uint16_t* dst = Dn + buf * L.dn_buf + rb_dn_at(r, RM);
-      float dmax = -1e9f;
-#pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        uint32_t v[32];
-        tc_ld32(taddr + c * 32, v);
-        tc_wait_ld();
-        if (c == 3) {
-          tc_fence_before();
-          rb_tile_arrive(acc);
-        }
-        if (c > (warp & 3)) continue;  // no step of this warp comes after those keys
-        const int lc = last - c * 32;
-#pragma unroll
-        for (int k = 0; k < 32; ++k)
-          if (k < lc) dmax = fmaxf(dmax, __uint_as_float(v[k]));
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          uint32_t pk[2];
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float y0 = fmaf(__uint_as_float(v[4 * k + 2 * e]), 1.f / 128.f, magic);
-            const float y1 = fmaf(__uint_as_float(v[4 * k + 2 * e + 1]), 1.f / 128.f, magic);
-            pk[e] = __byte_perm(__float_as_uint(y0), __float_as_uint(y1), 0x5410);
-          }
-          if (c * 32 + 4 * k < r && r < RM) *reinterpret_cast<uint2*>(dst + c * 32 + 4 * k) = make_uint2(pk[0], pk[1]);
-        }
-      }
-      NR[buf * kRbRows + r] = last > 0 ? (int)(__float_as_uint(fmaf(dmax, 1.f / 128.f, magic)) & 0xFFFFu) >> 1 : -1;
-    };
     fence_proxy_async();
     __syncthreads();
     // A turn works on the block of steps t0 .. tn - 1 and prepares the next one; a unit's first turn has no steps yet.
@@ -763,34 +872,14 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
       const uint32_t* kb_codes = kraw + cur * kRbRows * WORDS;
       // ---------------------------------------------------------------- tile phase
       // this CTA's base tiles 0 .. ntl - 1 (tile i of the CTA is tile i * ncta + rank of the unit)
-      int top = -1;  // readers: best base key of the thread's step so far
       if (warp < kExpWarp) {
         const int r = tid & 127, grp = warp >> 2;  // this thread's step = its tensor-memory lane; tiles grp, grp + kGroups, ...
         int32_t* mrow = Mx + rank * L.mx_block + min(r, RM) * L.mx_pitch;
-        int ct = (127 - ((grp << lg_ncta) + rank)) * 128;  // 127 - tile goes above the index within the tile (lower tiles first)
+        const int ct = (127 - ((grp << lg_ncta) + rank)) * 128;  // 127 - tile goes above the index within the tile (lower tiles first)
         const int cstep = (128 * kGroups) << lg_ncta;
         const uint32_t taddr0 = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
         if (ncta > 1 && blk > 0 && rows > 0) rb_wait_cluster(used_bar, (blk - 1) & 1, &abort_flag);  // peers still read the block before
-#pragma unroll 1
-        for (int i = grp; i < ntl; i += kGroups) {
-          const int n = it + i, acc = n & 3;
-          rb_wait(done_bar(n), done_phase(n), &abort_flag);
-          tc_fence_after();
-          const uint32_t taddr = taddr0 + (uint32_t)(acc * kRbTile);
-          uint32_t v0[32], v1[32];
-          rb_ld64_low(taddr, v0);
-          rb_ld64_low(taddr + 64, v1);
-          rb_wait_ld(v0);
-          rb_wait_ld(v1);
-          tc_fence_before();  // the accumulator goes back
-          rb_tile_arrive(acc);
-          const uint32_t m = rb_max64(v0, v1);
-          // the tile's best key, 2^14 rank + index; negative: no slot of the tile may win
-          const int k16 = (int)max(m & 0xFFFFu, m >> 16) - 1, key = ((k16 & ~127) << 7) + (k16 & 127) + ct;
-          ct -= cstep;
-          top = max(top, key);
-          mrow[i] = key;
-        }
+        const int top = rb_read_tiles<kGroups>(bar0, &abort_flag, it, grp, ntl, taddr0, smem_u32(mrow), ct, cstep);
         if (rows > 0 && r < RM) Mx[rank * L.mx_block + top_at + grp * RM + r] = top;  // this group's best key of the step
         if (ncta > 1) fence_proxy_async();
       } else if (warp < kRbMmaWarp) {
@@ -800,60 +889,22 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         }
         const int aux = tid - 32 * kRbAuxWarp, nrows = min(N - tn, R);
         if (tn < N && warp >= kRbAuxWarp) stage_codes(cur ^ 1, tn, nrows, aux, kRbAuxThreads);  // the next block's codes arrive meanwhile
-        // teams of two warps write the operand tiles in turn, rows x and x + 64 by a thread
-        const int x = tid & 63;
-        uint32_t h0[WORDS], h1[WORDS];
-        auto fetch = [&](int i) {
-          const uint32_t* src = codes + (((i << lg_ncta) + rank) * kRbTile + x) * WORDS;
-          if (WORDS == 2) {
-            const uint2 a2 = *reinterpret_cast<const uint2*>(src), b2 = *reinterpret_cast<const uint2*>(src + 64 * WORDS);
-            h0[0] = a2.x, h0[WORDS - 1] = a2.y, h1[0] = b2.x, h1[WORDS - 1] = b2.y;
-          } else {
-            h0[0] = src[0], h1[0] = src[64];
-          }
-        };
-        int i = (((warp - kExpWarp) >> 1) - it) & (kTeams - 1);
-        uint32_t at = row_at(x, (it + i) & 3), at_next = row_at(x, (it + i + kTeams) & 3);  // row x + 64 is 8 KB further on
-        const int whole = S > 0 ? 1 : 0, part = C / kRbTile;  // tiles of the unit from `whole` to `part` - 1 hold candidates only
-        if (i < ntl) fetch(i);
-#pragma unroll 1
-        for (; i < ntl; i += kTeams) {
-          const int n = it + i, tile = (i << lg_ncta) + rank;
-          rb_wait(done_bar(n - 4), done_phase(n - 4), &abort_flag);  // product n - 4 is done with the operand tile
-          expand_row(h0, at);
-          expand_row(h1, at + 8192u);
-          if (__builtin_expect(tile < whole || tile >= part, 0)) {
-            const int j = tile * kRbTile + x;
-            if (j < S || j >= C) clear_row(at);
-            if (j + 64 < S || j + 64 >= C) clear_row(at + 8192u);
-          }
-          fence_proxy_async();
-          rb_tile_arrive(n & 3);
-          if (i + kTeams < ntl) fetch(i + kTeams);
-          const uint32_t t = at;
-          at = at_next, at_next = t;
-        }
+        // teams of two warps write the operand tiles in turn
+        const int x = tid & 63, i = (((warp - kExpWarp) >> 1) - it) & (kTeams - 1), j = rank * kRbTile + x;
+        rb_expand_tiles<WORDS, kTeams>(bar0, &abort_flag, it, i, ntl, smem_u32(codes + j * WORDS), (uint32_t)(kRbTile * WORDS * 4) << lg_ncta, smem_u32(Bs) + rb_row_at<WORDS>(x, (it + i) & 3),
+                                       smem_u32(Bs) + rb_row_at<WORDS>(x, (it + i + kTeams) & 3), j, kRbTile << lg_ncta, S, C);
         if (tn < N && warp >= kRbAuxWarp) {  // the next block: operand A, its own keys' ranks
           cp_async_wait_all();
           if (abuf == 1) rb_wait(adone_bar, turn & 1, &abort_flag);  // a single operand A is free after the block's last tile
           rb_bar<3, kRbAuxThreads>();
-          build_a(cur ^ 1, nrows, aux, kRbAuxThreads);
-          new_keys(cur ^ 1, it + ntl);
+          rb_prepare<WORDS, GT, PROT, RM>(L, (int)(smem - rb_smem_raw), cur ^ 1, nrows, it + ntl, G, Rn, abuf, bar0, &abort_flag, tmem_base);
         }
       } else {
-        // (a reduction's result sits in a uniform register: the loop's counters and the descriptors then stay in those)
-        auto uniform = [](uint32_t v) { return (int)__reduce_max_sync(0xFFFFFFFFu, v); };
-        const int it_u = uniform(it), ntl_u = uniform(ntl), cur_u = uniform(cur);
-        const uint32_t tmem_u = uniform(tmem_base);
-        const uint64_t ad = a_desc_of(cur_u), xd = umma_desc_k128(smem_u32(Bx));
         // index-column variants: the unit's first tile (protected first tokens) and its last (the budget ends in it)
-        const int first_i = S > 0 && rank == 0 ? 0 : -1, last_i = uniform(((nbase - 1 - rank) & (ncta - 1)) == 0 ? ntl : 0) - 1;
-        const int odd = warp - kRbMmaWarp;  // this warp's products: the even or the odd ones
-#pragma unroll 1
-        for (int i = (it_u ^ odd) & 1; i < ntl_u; i += 2) issue(it_u + i, tmem_u, ad, true, xd + (uint64_t)((i == first_i ? 2 : 0) + (i == last_i ? 4 : 0)));
-        if (abuf == 1 && tc_elect()) tc_commit(adone_bar);
-        __syncwarp();
-        if (tn < N && ((it_u + ntl_u) & 1) == odd) issue(it_u + ntl_u, tmem_u, a_desc_of(cur_u ^ 1), false, 0);
+        const int first_i = S > 0 && rank == 0 ? 0 : -1, last_i = ((nbase - 1 - rank) & (ncta - 1)) == 0 ? ntl - 1 : -1;
+        const uint32_t a_at = smem_u32(As);
+        rb_issue_tiles<WORDS>(bar0, it, ntl, warp - kRbMmaWarp, tmem_base, a_at + (abuf > 1 ? cur * a_step : 0), a_at + (abuf > 1 ? (cur ^ 1) * a_step : 0), smem_u32(Bx),
+                              smem_u32(Bs), first_i, last_i, abuf == 1 ? adone_bar : 0u, tn < N);
       }
       it += ntl + (tn < N ? 1 : 0);
       if (warp < kRbResWarps && rows > 0) {
@@ -887,6 +938,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
         bool forced = false, flagged = false;  // ... the best base slot holds a recent token; or a new entry may win
         if (warp < 4) {
           if (ncta > 1) rb_wait_cluster(tops_bar, blk & 1, &abort_flag);
+          int top = -1;
 #pragma unroll 1
           for (int c = 0; c < ncta; ++c)
 #pragma unroll
@@ -894,7 +946,11 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           top_slot = max(0, min(kRbIdxMask - (top & kRbIdxMask), C - 1));
           sv = prev = top_slot;
           if (PROT && 32 * warp < Rn)  // REC[m] entered m + 1 steps before the block: recent while r + m < Rn
-            for (int m = 0; m < Rn; ++m) forced |= m < Rn - r && REC[m] == top_slot;
+            for (int m = 0; m < Rn; m += 4) {
+              const int4 q = *reinterpret_cast<const int4*>(REC + m);
+              const int left = Rn - r - m;
+              forced |= (left > 0 && q.x == top_slot) | (left > 1 && q.y == top_slot) | (left > 2 && q.z == top_slot) | (left > 3 && q.w == top_slot);
+            }
           flagged = forced || NR[cur * kRbRows + r] >= (top >> kRbKeyShift);
           RN[r] = top;
           if (tid < 2) s_change[tid] = kRbRows;
@@ -937,24 +993,32 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             // hard steps of the window
             is_hard = r >= fb && r < wend && (flagged || stale);
             const uint32_t hm = __ballot_sync(0xFFFFFFFFu, is_hard);
-            if (is_hard) LIST[warp * 32 + __popc(hm & ((1u << lane) - 1u))] = (uint8_t)((uint32_t)r | (stale || forced ? 0x80u : 0u));
-            if (lane == 0) s_hard[par][warp] = (uint8_t)__popc(hm);
+            const bool scan = is_hard && (stale || forced);
+            const uint32_t sm = __ballot_sync(0xFFFFFFFFu, scan), lt = (1u << lane) - 1u;
+            if (is_hard) LIST[warp * 32 + (scan ? __popc(sm & lt) : __popc(sm) + __popc(hm & ~sm & lt))] = (uint8_t)((uint32_t)r | (scan ? 0x80u : 0u));
+            if (lane == 0) s_hard[par][warp] = (uint8_t)__popc(hm), s_stale[par][warp] = (uint8_t)__popc(sm);
             if (!is_hard && r >= fb && r < wend && sv != top_slot) atomicMin(&s_change[par], r);
             if (ncta > 1 && pass == 0) rb_wait_cluster(peer_bar, blk & 1, &abort_flag);  // the peers' tile maxima
           }
           rb_bar<2, kRbResThreads>();
           if (tid == 0) s_change[par ^ 1] = kRbRows;
-          // The hard steps are dealt round-robin over all warps (later steps are hard more often than earlier ones): entry e
-          // of the four lists one after another.
-          const uint32_t nhard = *reinterpret_cast<const uint32_t*>(s_hard[par]);
-          const int n0 = nhard & 0xFFu, n1 = n0 + ((nhard >> 8) & 0xFFu), n2 = n1 + ((nhard >> 16) & 0xFFu), n3 = n2 + (nhard >> 24);
+          // The stale steps of the four lists first, then the others, dealt to and fro over the warps: an evaluation with a scan takes twice as
+          // long as one without (900 to 1400 cycles, 450 to 680), so that a warp with a second one has two short ones. 128 units of 1024 slots,
+          // windows: 1243 -> 1225 us; dealing to 18 warps instead gained nothing, as the longest evaluation counts. (Bytes w: steps in the lists
+          // up to warp w's.)
+          const uint32_t nhard = *reinterpret_cast<const uint32_t*>(s_hard[par]), nstale = *reinterpret_cast<const uint32_t*>(s_stale[par]);
+          const uint32_t upto_s = nstale * 0x01010101u, upto_f = (nhard - nstale) * 0x01010101u;
+          const int ns = (int)(upto_s >> 24), n3 = ns + (int)(upto_f >> 24);
           if (__builtin_expect(32 * n3 > 31 * (wend - fb), 0)) {
             const int walk = rb_walk_cost(WORDS, GT, PROT, (C + kRbResThreads - 1) / kRbResThreads);
             if (pass * rb_pass_cost(n3) > 2 * fb * walk && 2 * pass * (rows - fb) > rows) break;  // the rest is walked
           }
 #pragma unroll 1
-          for (int e0 = warp; e0 < n3; e0 += kRbResWarps) {
-            const int entry = LIST[e0 < n1 ? (e0 < n0 ? e0 : 32 + e0 - n0) : (e0 < n2 ? 64 + e0 - n1 : 96 + e0 - n2)];
+          for (int e0 = warp, fro = kRbResWarps - 1 - 2 * warp; e0 < n3; e0 += kRbResWarps + fro, fro = -fro) {
+            const uint32_t upto = e0 < ns ? upto_s : upto_f;
+            const int e1 = e0 < ns ? e0 : e0 - ns;
+            const int of = (e1 >= (int)(upto & 0xFFu)) + (e1 >= (int)((upto >> 8) & 0xFFu)) + (e1 >= (int)((upto >> 16) & 0xFFu));  // whose list
+            const int entry = LIST[32 * of + e1 - (int)(((upto << 8) >> (8 * of)) & 0xFFu) + (e0 < ns ? 0 : (int)((nstale >> (8 * of)) & 0xFFu))];
             const int r2 = entry & 127;
             const uint2 dd = *reinterpret_cast<const uint2*>(Dn + cur * L.dn_buf + rb_dn_at(r2, RM) + (4 * lane < r2 ? 4 * lane : 0));
             const uint2 s4 = *reinterpret_cast<const uint2*>(SV + 4 * lane);
@@ -1032,11 +1096,15 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
                 const uint32_t o4 = *reinterpret_cast<const uint32_t*>(own + j0) ^ (tag * 0x01010101u);
                 ok4 = (((o4 | 0x80808080u) - (uint32_t)r2 * 0x01010101u) | o4);
               }
-              if (PROT && r2 < Rn)
+              if (PROT && r2 < Rn)  // recent tokens in this tile
 #pragma unroll 1
-                for (int m0 = 0; m0 < Rn - r2; ++m0) {
-                  const int q = REC[m0] - j0;
-                  if (q >= 0 && q < 4) ok4 &= ~(0x80u << (8 * q));
+                for (int m0 = 0; m0 < Rn - r2; m0 += 32) {
+                  const int q = m0 + lane < Rn - r2 ? REC[m0 + lane] : -1;
+#pragma unroll 1
+                  for (uint32_t in = __ballot_sync(0xFFFFFFFFu, q >> 7 == cb); in != 0u; in &= in - 1u) {
+                    const int at = __shfl_sync(0xFFFFFFFFu, q, __ffs(in) - 1) - j0;
+                    if (at >= 0 && at < 4) ok4 &= ~(0x80u << (8 * at));
+                  }
                 }
               const int hi = C - j0, lo = PROT ? S - j0 : 0;
 #pragma unroll
