@@ -521,7 +521,7 @@ int launch_replay_reg(const ReplayArgs& a, long long units, cudaStream_t stream)
 constexpr size_t kRbMinSmem = 120 * 1024;
 constexpr size_t kMaxDynSmem = 227 * 1024 - kRbStaticSmem;  // dynamic shared memory of a CTA beside the kernel's static arrays
 
-// Shared memory of the block replay with as many operand stages as fit (fewer for large two-word tables); 0: does not fit.
+// Shared memory of the block replay, with one operand A buffer instead of two where a large two-word table leaves no room; 0: does not fit.
 size_t rb_fit(int words, int slots, int G, int ncta, int form, RbArgs* ra) {
   ra->rows_max = form == kRbHalf ? kRbRows / 2 : kRbRows;
   for (ra->abuf = 2; ra->abuf >= 1; --ra->abuf) {
@@ -544,10 +544,9 @@ int launch_replay_block_form(const ReplayArgs& a, long long units, cudaStream_t 
   // protected windows), 380 per tile of its own and 3000 for the exchange with its peers; the number of rounds is what the
   // clusters that fit the GPU need for the units. A wider cluster never pays with more rounds unless there are about 90 tiles (200
   // units: two rounds of single CTAs against three of pairs cross at 89 tiles with 8000, at 74 with 5000, where they are level
-  // within 1 %), so one figure does for every block length. The figures are those of fp32 tile keys; a tile takes 315 since, settling 5000 to
-  // 8000. Every width measured at 4 to 200 units of 256 to 9830 slots (170 points, N = 2 C): the choice is within 2 % of the best but for
-  // 1024 slots with up to 64 units, where four CTAs (two from 48 units on) would take 2 to 8 % less than the one chosen (8 units, b = 64:
-  // 114 / 107 us; b = 32: 104 / 99).
+  // within 1 %), so one figure does for every block length. A tile takes 235 to 300 since, settling 5000 to 8000. Every width measured at 4 to
+  // 200 units of 256 to 9830 slots, four code shapes (160 points, N = 2 C, drifting keys): the choice is within 2 % of the best but for two-word
+  // tables of 1024 slots with up to 32 units, where four CTAs would take 2 to 3 % less (8 units 111.4 / 108.4 us, 32 units 122.8 / 119.2).
   static DeviceTable<4> table;  // clusters of 2^lg CTAs that the device holds at once (-1: none)
   const int tiles = ra.r.smem_slots / kRbTile;
   double best = 0.;
@@ -611,12 +610,12 @@ int launch_replay_block_form(const ReplayArgs& a, long long units, cudaStream_t 
 
 // Two-word tables above about 8200 slots only fit with blocks of 64 steps.
 // The owner table of words costs 3 more bytes per slot and saves a pass 250 of its 600 cycles of claims: up to 6144 slots, where it
-// costs a CTA on its own no operand stage. us per call with bytes / words: 32 units of 2048 slots 147.8 / 142.1, 128 of 1024 1554 / 1503,
-// 512 of 512 to 4096 with two words 1369 / 1354; beyond, where passes are a small share, 8 of 9830 1232 / 1238, 256 of 9830 7239 /
+// costs no operand A buffer. us per call with bytes / words, both measured with pairs of tiles: 32 units of 2048 slots 147.8 / 142.1, 128 of 1024
+// 1554 / 1503, 512 of 512 to 4096 with two words 1369 / 1354; beyond, where passes are a small share, 8 of 9830 1232 / 1238, 256 of 9830 7239 /
 // 7367. One word, G = 4, words over bytes: 128 and 320 units 1.00 at 6144 slots and 1.01 at 8192, 8 and 32 units 0.98 to 0.99 up to there
-// (G = 1 stays at 0.97 to 0.99 up to 9830). In a cluster the tiles' maxima of every CTA can cost the words a stage that the bytes keep (two
-// words from 3968 slots); the shorter passes outweigh it: 4096 slots, G = 4, 8 units in clusters of 8 296 / 284, 32 units in fours 368 / 355,
-// 64 in pairs 462 / 459 on clustered keys and 389 / 392 on drifting ones.
+// (G = 1 stays at 0.97 to 0.99 up to 9830). Two words, drifting keys, measured
+// tile by tile, bytes / words: 3072 slots, G = 4, 8 units 191 / 184, 200 units 717 / 693; 4096 slots, 64 units 389 / 379; 6144 slots, 8 units 350 / 338,
+// 200 units 1669 / 1631 (G = 1 alike).
 constexpr int kRbWideSlots = 6144;
 template <int WORDS, int GT, bool PROT>
 int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t stream) {
