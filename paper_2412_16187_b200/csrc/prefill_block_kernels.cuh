@@ -717,9 +717,8 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   __shared__ volatile int abort_flag;
   __shared__ int s_unit[2];
   __shared__ int s_change[2];                    // by pass parity: first step that changed
-  __shared__ __align__(4) uint8_t s_hard[2][4];   // by pass parity: lengths of warps 0-3's lists of hard steps
-  __shared__ __align__(4) uint8_t s_stale[2][4];  // ... and of the stale ones at their heads
-  static_assert(sizeof(bars) + sizeof(tmem_base_s) + sizeof(abort_flag) + sizeof(s_unit) + sizeof(s_change) + sizeof(s_hard) + sizeof(s_stale) <= kRbStaticSmem,
+  __shared__ uint32_t s_hard[2];                 // by pass parity: stale steps to evaluate, others << 16
+  static_assert(sizeof(bars) + sizeof(tmem_base_s) + sizeof(abort_flag) + sizeof(s_unit) + sizeof(s_change) + sizeof(s_hard) <= kRbStaticSmem,
                 "the host sizes the dynamic shared memory beside these");
 
   griddep_launch_dependents();
@@ -748,7 +747,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   int32_t* NR = reinterpret_cast<int32_t*>(smem + L.nr);    // per step: largest rank of any earlier key of the block, two buffers
   uint16_t* SV = reinterpret_cast<uint16_t*>(smem + L.sv);  // per step: the slot it writes, as far as known
   int32_t* SN = reinterpret_cast<int32_t*>(smem + L.sn);    // what the evaluation of a hard step gave
-  uint8_t* LIST = smem + L.list;                            // hard steps that warps 0-3 found in the pass: step | stale << 7
+  uint8_t* LIST = smem + L.list;                            // the pass's hard steps: step | stale << 7
   int32_t* PAR = reinterpret_cast<int32_t*>(smem + L.par);  // per step: bits set in the xor of its query codes, two buffers
   uint32_t* qraw = reinterpret_cast<uint32_t*>(smem + L.qraw);
   uint32_t* kraw = reinterpret_cast<uint32_t*>(smem + L.kraw);
@@ -953,7 +952,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             }
           flagged = forced || NR[cur * kRbRows + r] >= (top >> kRbKeyShift);
           RN[r] = top;
-          if (tid < 2) s_change[tid] = kRbRows;
+          if (tid < 2) s_change[tid] = kRbRows, s_hard[tid] = 0u;
         }
         int fb = 0;                    // steps below are final
 #pragma unroll 1
@@ -994,31 +993,30 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
             is_hard = r >= fb && r < wend && (flagged || stale);
             const uint32_t hm = __ballot_sync(0xFFFFFFFFu, is_hard);
             const bool scan = is_hard && (stale || forced);
-            const uint32_t sm = __ballot_sync(0xFFFFFFFFu, scan), lt = (1u << lane) - 1u;
-            if (is_hard) LIST[warp * 32 + (scan ? __popc(sm & lt) : __popc(sm) + __popc(hm & ~sm & lt))] = (uint8_t)((uint32_t)r | (scan ? 0x80u : 0u));
-            if (lane == 0) s_hard[par][warp] = (uint8_t)__popc(hm), s_stale[par][warp] = (uint8_t)__popc(sm);
+            const uint32_t sm = __ballot_sync(0xFFFFFFFFu, scan), fm = hm & ~sm, lt = (1u << lane) - 1u;
+            uint32_t at = 0u;
+            if (lane == 0 && hm != 0u) at = atomicAdd(&s_hard[par], (uint32_t)(__popc(sm) | __popc(fm) << 16));
+            at = __shfl_sync(0xFFFFFFFFu, at, 0);
+            // the stale steps from the list's start on, the others from its end
+            if (is_hard) LIST[scan ? (at & 0xFFFFu) + __popc(sm & lt) : kRbRows - 1 - (at >> 16) - __popc(fm & lt)] = (uint8_t)((uint32_t)r | (scan ? 0x80u : 0u));
             if (!is_hard && r >= fb && r < wend && sv != top_slot) atomicMin(&s_change[par], r);
             if (ncta > 1 && pass == 0) rb_wait_cluster(peer_bar, blk & 1, &abort_flag);  // the peers' tile maxima
           }
           rb_bar<2, kRbResThreads>();
-          if (tid == 0) s_change[par ^ 1] = kRbRows;
-          // The stale steps of the four lists first, then the others, dealt to and fro over the warps: an evaluation with a scan takes twice as
-          // long as one without (900 to 1400 cycles, 450 to 680), so that a warp with a second one has two short ones. 128 units of 1024 slots,
-          // windows: 1243 -> 1225 us; dealing to 18 warps instead gained nothing, as the longest evaluation counts. (Bytes w: steps in the lists
-          // up to warp w's.)
-          const uint32_t nhard = *reinterpret_cast<const uint32_t*>(s_hard[par]), nstale = *reinterpret_cast<const uint32_t*>(s_stale[par]);
-          const uint32_t upto_s = nstale * 0x01010101u, upto_f = (nhard - nstale) * 0x01010101u;
-          const int ns = (int)(upto_s >> 24), n3 = ns + (int)(upto_f >> 24);
+          if (tid == 0) s_change[par ^ 1] = kRbRows, s_hard[par ^ 1] = 0u;
+          // The stale steps first, then the others, dealt to and fro over the warps: an evaluation with a scan takes twice as long as one without
+          // (900 to 1400 cycles, 450 to 680), so that a warp with a second one has two short ones. 128 units of 1024 slots, windows: 1243 -> 1225 us
+          // of replay; dealing to 18 warps instead gained nothing, as the longest evaluation counts. One list, filled from both ends by an atomic
+          // addition a warp: with a list for each of the four warps, looked through at every evaluation, the same call took 1404 us for 1359, and
+          // 128 units of 2048 slots with b = 8 lost 5 % to what the order gained.
+          const int ns = (int)(s_hard[par] & 0xFFFFu), n3 = ns + (int)(s_hard[par] >> 16);
           if (__builtin_expect(32 * n3 > 31 * (wend - fb), 0)) {
             const int walk = rb_walk_cost(WORDS, GT, PROT, (C + kRbResThreads - 1) / kRbResThreads);
             if (pass * rb_pass_cost(n3) > 2 * fb * walk && 2 * pass * (rows - fb) > rows) break;  // the rest is walked
           }
 #pragma unroll 1
           for (int e0 = warp, fro = kRbResWarps - 1 - 2 * warp; e0 < n3; e0 += kRbResWarps + fro, fro = -fro) {
-            const uint32_t upto = e0 < ns ? upto_s : upto_f;
-            const int e1 = e0 < ns ? e0 : e0 - ns;
-            const int of = (e1 >= (int)(upto & 0xFFu)) + (e1 >= (int)((upto >> 8) & 0xFFu)) + (e1 >= (int)((upto >> 16) & 0xFFu));  // whose list
-            const int entry = LIST[32 * of + e1 - (int)(((upto << 8) >> (8 * of)) & 0xFFu) + (e0 < ns ? 0 : (int)((nstale >> (8 * of)) & 0xFFu))];
+            const int entry = LIST[e0 < ns ? e0 : kRbRows - 1 - (e0 - ns)];
             const int r2 = entry & 127;
             const uint2 dd = *reinterpret_cast<const uint2*>(Dn + cur * L.dn_buf + rb_dn_at(r2, RM) + (4 * lane < r2 ? 4 * lane : 0));
             const uint2 s4 = *reinterpret_cast<const uint2*>(SV + 4 * lane);
