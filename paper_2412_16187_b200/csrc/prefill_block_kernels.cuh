@@ -56,7 +56,10 @@
 // 4800 us (5400 with two groups).
 // Every wait on an mbarrier is bounded; a CTA that gives up raises a flag that turns its later waits into no-ops, but it
 // still walks the same blocks and cluster barriers as its peers (their copies into its shared memory must find it), then
-// releases tensor memory and raises the device error counter.
+// releases tensor memory and raises the device error counter. The tiles' named barriers count arrivals and have no limit of their
+// own, and what keeps the arrivals of one tile apart from those of four tiles on are the mbarriers: once roles run on without them a
+// barrier's phases may pass without its issuing warp, which would then wait for arrivals that nobody owes. So a warp that is not needed
+// elsewhere sees the issuing warps out of every turn, and arrives for them where the flag is up (rb_see_out).
 #pragma once
 #include <cuda_fp16.h>
 
@@ -307,6 +310,23 @@ __device__ __forceinline__ void rb_bar() {
 constexpr int kRbTileBarThreads = 128 + 64 + 32;
 __device__ __forceinline__ void rb_tile_arrive(int acc) { asm volatile("bar.arrive %0, %1;" ::"r"(kRbTileBar + acc), "n"(kRbTileBarThreads) : "memory"); }
 __device__ __forceinline__ void rb_tile_sync(int acc) { asm volatile("bar.sync %0, %1;" ::"r"(kRbTileBar + acc), "n"(kRbTileBarThreads) : "memory"); }
+
+// Until both issuing warps have come through the turn (`turns`: the last one of each): once the abort flag is up nobody else waits at the tiles'
+// barriers, and an arrival at each lets an issuing warp on after seven rounds at the latest. The limit is several times that of the
+// waits after which other roles raise the flag (seconds); what is still out there then is given up on as a wait is.
+__device__ __noinline__ void rb_see_out(volatile int* turns, int turn, volatile int* abort_flag) {
+#pragma unroll 1
+  for (uint32_t i = 0; i < 8u * kTcSpinLimit && __any_sync(0xFFFFFFFFu, turns[0] < turn || turns[1] < turn); ++i) {
+    if (i == 7u * kTcSpinLimit) *abort_flag = 1;
+    if (__any_sync(0xFFFFFFFFu, *abort_flag != 0)) {
+#pragma unroll 1
+      for (int x = 0; x < kRbAccs; ++x) rb_tile_arrive(x);
+    } else {
+      __nanosleep(100);
+    }
+    __syncwarp();
+  }
+}
 
 // The loops of the tile phase, and the preparation of the next block. Functions of their own, so that their registers and their code
 // don't change with what the settling around them needs: inlined, a change of the settling moved a tile by 4 % either way. Replay, us
@@ -715,10 +735,11 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   __shared__ __align__(8) unsigned long long bars[kRbDoneBars + 5];
   __shared__ uint32_t tmem_base_s;
   __shared__ volatile int abort_flag;
+  __shared__ volatile int s_turns[2];            // the issuing warps' last turns
   __shared__ int s_unit[2];
   __shared__ int s_change[2];                    // by pass parity: first step that changed
   __shared__ uint32_t s_hard[2];                 // by pass parity: stale steps to evaluate, others << 16
-  static_assert(sizeof(bars) + sizeof(tmem_base_s) + sizeof(abort_flag) + sizeof(s_unit) + sizeof(s_change) + sizeof(s_hard) <= kRbStaticSmem,
+  static_assert(sizeof(bars) + sizeof(tmem_base_s) + sizeof(abort_flag) + sizeof(s_turns) + sizeof(s_unit) + sizeof(s_change) + sizeof(s_hard) <= kRbStaticSmem,
                 "the host sizes the dynamic shared memory beside these");
 
   griddep_launch_dependents();
@@ -763,6 +784,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
   const uint32_t tops_bar = bar0 + 8u * (kRbDoneBars + 4);     // peers' copies of their best keys have arrived
   if (tid == 0) {
     abort_flag = 0;
+    s_turns[0] = s_turns[1] = -1;
     mbar_init(drain_bar, 2);
     mbar_init(adone_bar, 2);
     for (int i = 0; i < kRbDoneBars; ++i) mbar_init(rb_done_bar(bar0, i), 1);
@@ -898,12 +920,15 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           rb_bar<3, kRbAuxThreads>();
           rb_prepare<WORDS, GT, PROT, RM>(L, (int)(smem - rb_smem_raw), cur ^ 1, nrows, it + ntl, G, Rn, abuf, bar0, &abort_flag, tmem_base);
         }
+        if (warp == kRbAuxWarp) rb_see_out(s_turns, turn, &abort_flag);
       } else {
         // index-column variants: the unit's first tile (protected first tokens) and its last (the budget ends in it)
         const int first_i = S > 0 && rank == 0 ? 0 : -1, last_i = ((nbase - 1 - rank) & (ncta - 1)) == 0 ? ntl - 1 : -1;
         const uint32_t a_at = smem_u32(As);
-        rb_issue_tiles<WORDS>(bar0, it, ntl, warp - kRbMmaWarp, tmem_base, a_at + (abuf > 1 ? cur * a_step : 0), a_at + (abuf > 1 ? (cur ^ 1) * a_step : 0), smem_u32(Bx),
-                              smem_u32(Bs), first_i, last_i, abuf == 1 ? adone_bar : 0u, tn < N);
+        if (__builtin_expect(!__any_sync(0xFFFFFFFFu, abort_flag != 0), 1))
+          rb_issue_tiles<WORDS>(bar0, it, ntl, warp - kRbMmaWarp, tmem_base, a_at + (abuf > 1 ? cur * a_step : 0), a_at + (abuf > 1 ? (cur ^ 1) * a_step : 0), smem_u32(Bx),
+                                smem_u32(Bs), first_i, last_i, abuf == 1 ? adone_bar : 0u, tn < N);
+        s_turns[warp - kRbMmaWarp] = turn;
       }
       it += ntl + (tn < N ? 1 : 0);
       if (warp < kRbResWarps && rows > 0) {
@@ -1230,15 +1255,16 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
     __syncthreads();  // the tables and s_unit are reused by the next unit
   }
 
-  // The readers' last arrivals still stand in the tile barriers: their phases are completed.
-  if (warp == kRbAuxWarp || warp == kRbAuxWarp + 1)
+  // The readers' last arrivals still stand in the tile barriers: their phases are completed, unless the CTA gave up (every wait that
+  // could raise the flag lies before the last barrier of the block loop).
+  const bool gave_up = __any_sync(0xFFFFFFFFu, abort_flag != 0);  // one answer for the warp: the election below wants all its lanes
+  if (!gave_up && (warp == kRbAuxWarp || warp == kRbAuxWarp + 1))
     for (int x = 0; x < kRbAccs; ++x) rb_tile_arrive(x);
   // A CTA that gave up must not free tensor memory under an MMA that is still writing it (the operands are written by
   // this CTA's own threads, so no copy from outside is ever in flight): one more commit tracks everything that the issuing
   // warp has issued, and its completion is awaited (bounded) first.
   if (warp == kRbMmaWarp || warp == kRbMmaWarp + 1) {
-    for (int x = warp - kRbMmaWarp; x < kRbAccs; x += 2) rb_tile_sync(x);
-    const bool gave_up = __any_sync(0xFFFFFFFFu, abort_flag != 0);  // one answer for the warp: the election wants all its lanes
+    for (int x = warp - kRbMmaWarp; x < kRbAccs && !gave_up; x += 2) rb_tile_sync(x);
     if (gave_up && tc_elect()) {
       tc_commit(drain_bar);
       mbar_drain(drain_bar, 0);
