@@ -609,23 +609,24 @@ int launch_replay_block_form(const ReplayArgs& a, long long units, cudaStream_t 
 }
 
 // Two-word tables above about 8200 slots only fit with blocks of 64 steps.
-// The owner table of words costs 3 more bytes per slot and saves a pass 250 of its 600 cycles of claims: up to 6144 slots, where it
-// costs no operand A buffer. us per call with bytes / words, both measured with pairs of tiles: 32 units of 2048 slots 147.8 / 142.1, 128 of 1024
-// 1554 / 1503, 512 of 512 to 4096 with two words 1369 / 1354; beyond, where passes are a small share, 8 of 9830 1232 / 1238, 256 of 9830 7239 /
-// 7367. One word, G = 4, words over bytes: 128 and 320 units 1.00 at 6144 slots and 1.01 at 8192, 8 and 32 units 0.98 to 0.99 up to there
-// (G = 1 stays at 0.97 to 0.99 up to 9830). Two words, drifting keys, measured
-// tile by tile, bytes / words: 3072 slots, G = 4, 8 units 191 / 184, 200 units 717 / 693; 4096 slots, 64 units 389 / 379; 6144 slots, 8 units 350 / 338,
-// 200 units 1669 / 1631 (G = 1 alike).
-constexpr int kRbWideSlots = 6144;
+// The owner table of words costs 3 more bytes per slot and saves a pass its four barriers in turn and the claims' clearing. One word: wherever it fits
+// clusters of every width (up to 10368 slots with G = 1, 9984 with G = 4, 9472 with G = 8; further on few units would lose the widest cluster, a third
+// of their time). us per call with bytes / words, 80 points of 8 to 320 units and 4096 to 9830 slots, drifting and clustered keys,
+// words ahead at each by 1 to 4 %: 9830 slots, G = 4, 8 units 537 / 527, 32 units 662 / 650, 128 units 1345 / 1324 and 2098 / 2063; G = 1, 128 units
+// 1195 / 1175; 6144 slots, 320 units 1970 / 1928. Two words: up to 6144 slots, where it costs no operand A buffer; drifting keys, bytes / words: 3072 slots, G = 4, 8 units
+// 191 / 184, 200 units 717 / 693; 4096 slots, 64 units 389 / 379; 6144 slots, 8 units 350 / 338, 200 units 1669 / 1631 (G = 1 alike).
+constexpr int kRbWideSlots2 = 6144;
 template <int WORDS, int GT, bool PROT>
 int launch_replay_block_one(const ReplayArgs& a, long long units, cudaStream_t stream) {
   const int slots = (a.cfg.max_budget + kRbTile - 1) / kRbTile * kRbTile, G = a.cfg.group_size;
   RbArgs fit{}, wide{};
-  const bool full = rb_fit(WORDS, slots, G, 1, kRbFull, &fit) != 0;
-  if constexpr (WORDS == 2)
-    if (!full) return launch_replay_block_form<WORDS, GT, PROT, kRbHalf>(a, units, stream);
-  if (slots <= kRbWideSlots && rb_fit(WORDS, slots, G, 1, kRbWide, &wide) != 0 && wide.abuf == fit.abuf)
-    return launch_replay_block_form<WORDS, GT, PROT, kRbWide>(a, units, stream);
+  if constexpr (WORDS == 2) {
+    if (rb_fit(2, slots, G, 1, kRbFull, &fit) == 0) return launch_replay_block_form<WORDS, GT, PROT, kRbHalf>(a, units, stream);
+    if (slots <= kRbWideSlots2 && rb_fit(2, slots, G, 1, kRbWide, &wide) != 0 && wide.abuf == fit.abuf)
+      return launch_replay_block_form<WORDS, GT, PROT, kRbWide>(a, units, stream);
+  } else {
+    if (rb_fit(1, slots, G, kRbMaxCluster, kRbWide, &wide) != 0) return launch_replay_block_form<WORDS, GT, PROT, kRbWide>(a, units, stream);
+  }
   return launch_replay_block_form<WORDS, GT, PROT, kRbFull>(a, units, stream);
 }
 

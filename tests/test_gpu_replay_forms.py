@@ -18,6 +18,13 @@ SHAPES = {
     "group_1_b2_protected": base.scaled(group_size=1, hash_bits=2, budget=150, prompt_len=600, n_sink=3, n_recent=40),
     "words_6144": base.scaled(n_kv_heads=1, hash_bits=32, budget=6144, prompt_len=6500),
     "bytes_6148": base.scaled(n_kv_heads=1, hash_bits=32, budget=6148, prompt_len=6500, n_sink=4, n_recent=10),
+    # one word: the owner table of words wherever it fits a cluster of eight, with and without several units to a CTA
+    "words_9984": base.scaled(n_kv_heads=1, hash_bits=32, budget=9984, prompt_len=10300),
+    "bytes_9985": base.scaled(n_kv_heads=1, hash_bits=32, budget=9985, prompt_len=10300),
+    "words_9472_group_8": base.scaled(n_kv_heads=1, group_size=8, hash_bits=32, budget=9472, prompt_len=9700),
+    "bytes_9473_group_8_protected": base.scaled(n_kv_heads=1, group_size=8, hash_bits=32, budget=9473, prompt_len=9700, n_sink=4, n_recent=10),
+    "words_10368_group_1": base.scaled(n_kv_heads=1, group_size=1, hash_bits=16, budget=10368, prompt_len=10700),
+    "words_9000_over_sms": base.scaled(batch=75, group_size=1, hash_bits=32, head_dim=64, budget=9000, prompt_len=9150),
     "two_words_4096": base.scaled(n_kv_heads=1, budget=4096, prompt_len=4500),
     "two_words_4100": base.scaled(n_kv_heads=1, budget=4100, prompt_len=4500),
     # more units than SMs: few-bit codes stay on the CUDA-core kernels, launched plainly behind the hashing
