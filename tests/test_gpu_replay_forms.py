@@ -27,6 +27,10 @@ SHAPES = {
     "words_9000_over_sms": base.scaled(batch=75, group_size=1, hash_bits=32, head_dim=64, budget=9000, prompt_len=9150),
     "two_words_4096": base.scaled(n_kv_heads=1, budget=4096, prompt_len=4500),
     "two_words_4100": base.scaled(n_kv_heads=1, budget=4100, prompt_len=4500),
+    "two_words_6144": base.scaled(n_kv_heads=1, budget=6144, prompt_len=6500),
+    "two_words_bytes_6145": base.scaled(n_kv_heads=1, budget=6145, prompt_len=6500),
+    "two_words_5632_group_8": base.scaled(n_kv_heads=1, group_size=8, budget=5632, prompt_len=5900),
+    "two_words_bytes_5633_group_8_protected": base.scaled(n_kv_heads=1, group_size=8, budget=5633, prompt_len=5900, n_sink=4, n_recent=10),
     # more units than SMs: few-bit codes stay on the CUDA-core kernels, launched plainly behind the hashing
     "few_bits_over_sms": base.scaled(batch=10, n_kv_heads=16, hash_bits=8, group_size=2, budget=400, prompt_len=520, head_dim=64),
     "one_head_groups_over_sms": base.scaled(batch=10, n_kv_heads=16, hash_bits=16, group_size=1, budget=390, prompt_len=520, head_dim=64),
