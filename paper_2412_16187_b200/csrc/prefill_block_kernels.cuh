@@ -266,8 +266,8 @@ __device__ __forceinline__ void rb_arrive_remote(uint32_t bar) {
 }
 // mbar_wait_warp with its loop left rolled: unrolled by the compiler, each of this kernel's waits was 5 KB of code, half of the kernel's 143 KB
 // (128 units of 1024 slots, b = 16, windows, the kernel otherwise as it was: 1290 -> 1230 us).
-__device__ __forceinline__ bool rb_wait_polled(bool done, uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  if (__builtin_expect(__all_sync(0xFFFFFFFFu, done), 1)) return true;
+__device__ __forceinline__ bool rb_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  if (__builtin_expect(__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)), 1)) return true;
   bool ok = false, on = true;
 #pragma unroll 1
   for (uint32_t i = 0; i < kTcSpinLimit && on; ++i) {
@@ -276,9 +276,6 @@ __device__ __forceinline__ bool rb_wait_polled(bool done, uint32_t bar, uint32_t
   }
   if (!ok) *abort_flag = 1;
   return __all_sync(0xFFFFFFFFu, ok);
-}
-__device__ __forceinline__ bool rb_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  return rb_wait_polled(mbar_try_wait(bar, parity), bar, parity, abort_flag);
 }
 // Bounded wait for copies and arrivals of other CTAs of the cluster.
 __device__ __forceinline__ bool rb_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
@@ -329,9 +326,9 @@ __device__ __noinline__ void rb_see_out(volatile int* turns, int turn, volatile 
 }
 
 // The loops of the tile phase, and the preparation of the next block. Functions of their own, so that their registers and their code
-// don't change with what the settling around them needs: inlined, a change of the settling moved a tile by 4 % either way. Replay, us
-// inlined / as functions: 256 units of 9830 slots 4970 / 4600, 512 of 512 to 4096, two words, 810 / 763, 128 of 1024 with windows 1228 / 1182,
-// 8 of 9830 1155 / 1140. (The evaluation of a hard step as a function: 1182 -> 1328, its caller's registers go to the stack.)
+// don't change with what the settling around them needs: inlined, a change of the settling moved a tile by 4 % either way. Replay when they became
+// functions, us inlined / as functions: 256 units of 9830 slots 4970 / 4600, 512 of 512 to 4096, two words, 810 / 763, 128 of 1024 with windows
+// 1228 / 1182, 8 of 9830 1155 / 1140. (Today 4600, 761, 1138 and 1115: the first with an owner table of words; where code falls still moves it by 1 to 2 %.) (The evaluation of a hard step as a function: 1182 -> 1328, its caller's registers go to the stack.)
 // `bars`: the products' mbarriers (product n's is n mod 8, its phase n / 8).
 __device__ __forceinline__ uint32_t rb_done_bar(uint32_t bars, int n) { return bars + 8u * (uint32_t)(n & (kRbDoneBars - 1)); }
 __device__ __forceinline__ uint32_t rb_done_phase(int n) { return (uint32_t)(n >> 3) & 1u; }
@@ -383,8 +380,8 @@ __device__ __forceinline__ void rb_clear_row(uint32_t at) {
 }
 
 // One team's tiles i, i + TEAMS, ...: rows x and x + 64 (8 KB further on) of the tile by a thread. src: the thread's first code of the CTA's tile 0, step:
-// bytes from tile to tile; at, at_next: where its row is in this tile and the next. The CTA's tiles below `whole` and from `part` on hold slots that
-// may not win: those below S and from C on, with j the thread's first slot of tile 0 and jstep slots from tile to tile.
+// bytes from tile to tile; at, at_next: where its row is in this tile and the next. Slots below S and from C on may not win and get zeros: j is the
+// thread's first slot of tile 0, jstep slots from tile to tile.
 template <int WORDS, int TEAMS>
 __device__ __noinline__ void rb_expand_tiles(uint32_t bars, volatile int* abort_flag, int it, int i, int ntl, uint32_t src, uint32_t step, uint32_t at, uint32_t at_next, int j,
                                              int jstep, int S, int C) {
@@ -1032,8 +1029,11 @@ __global__ void __launch_bounds__(kRbThreads, 1) prefill_replay_block_kernel(con
           // The stale steps first, then the others, dealt to and fro over the warps: an evaluation with a scan takes twice as long as one without
           // (900 to 1400 cycles, 450 to 680), so that a warp with a second one has two short ones. 128 units of 1024 slots, windows: 1243 -> 1225 us
           // of replay; dealing to 18 warps instead gained nothing, as the longest evaluation counts. One list, filled from both ends by an atomic
-          // addition a warp: with a list for each of the four warps, looked through at every evaluation, the same call took 1404 us for 1359, and
-          // 128 units of 2048 slots with b = 8 lost 5 % to what the order gained.
+          // addition a warp. The addition costs a pass 110 cycles (one layer of 32 units: 560 a pass for 450), 0.9 % of a block of the longest tables, which
+          // have five hard steps a pass and gain nothing; what else there is costs more. Four lists looked through at every evaluation: the same call
+          // 1404 us for 1359, b = 8 2 to 4 %; the ballots as words, an entry found in them by lane: 250 cycles a pass, but 490 more in its
+          // evaluations, 1424 us; places from the warps' counts behind one more barrier: 1377; four lists without an order: 1427, while 256 units of 9830
+          // slots take 6181 for 6208 and b = 8 stays where it is.
           const int ns = (int)(s_hard[par] & 0xFFFFu), n3 = ns + (int)(s_hard[par] >> 16);
           if (__builtin_expect(32 * n3 > 31 * (wend - fb), 0)) {
             const int walk = rb_walk_cost(WORDS, GT, PROT, (C + kRbResThreads - 1) / kRbResThreads);

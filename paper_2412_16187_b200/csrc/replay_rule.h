@@ -3,10 +3,13 @@
 
 namespace he {
 
-// Smallest max_budget of the block kernel. It has one CTA per SM and pays a block's settling (5000 to 12 000 cycles) whatever the budget; the
-// CUDA-core kernels scan every slot at every step, several units per SM. us with CUDA cores / block kernel:
+// Smallest max_budget of the block kernel. It has one CTA per SM and pays a block's settling (5500 to 11 500 cycles, with 8-bit codes
+// up to 130 000) whatever the budget; the CUDA-core kernels scan every slot at every step, several units per SM. us with CUDA cores / block kernel:
 //   up to one unit per SM the block kernel is ahead from the smallest budgets where the register kernel exists (64 slots, G = 4,
-//   b = 32, N = 2 C: 38 / 31) and from 128 slots where it does not (G = 8, b = 64: 66 / 53);
+//   b = 32, N = 2 C: 38 / 31) and from 128 slots where it does not (G = 8, b = 64: 66 / 53); codes of 8 bits are not split off there, though on
+//   some keys the register kernel is ahead (N = 2 C, block kernel on independent, drifting, clustered keys): G = 1, 4 units 64 slots 35 / 32, 37,
+//   47, 128 slots 50 / 41, 45, 70, 384 slots 115 / 68, 89, 181, 128 units 128 slots clustered 78 / 75, 384 slots 169 / 222; G = 4, 4 units 64 slots
+//   38 / 41, 44, 45, 200 slots 76 / 86, 96, 120, 384 slots 129 / 128, 145, 213, 32 and 128 units behind on clustered keys alone;
 //   with more units they cross between 256 and 512 slots, sooner or later with the keys (320 units, b = 32, G = 4, N = 2.5 C: 411 / 418
 //   at 512 slots on clustered keys, 410 / 316 on drifting ones), sooner with two words and G = 4 (N = 3 C: 250 / 253 at 160 slots,
 //   336 / 302 at 224).
