@@ -543,8 +543,8 @@ int launch_replay_block_form(const ReplayArgs& a, long long units, cudaStream_t 
   // Cluster size: a block costs a CTA about 8000 cycles of settling, 380 per tile of its own and 3000 for the exchange with its peers; the
   // number of rounds is what the clusters that fit the GPU need for the units. A wider cluster never pays with more rounds unless there are about
   // 90 tiles (200 units: two rounds of single CTAs against three of pairs cross at 89 tiles with 8000, at 74 with 5000, where they are level
-  // within 1 %), so one figure does for every block length. They are those of an older kernel (a tile takes 235 to 300 today, settling 5500 for
-  // the largest tables to 11 500 for 64 steps with protected windows), and the choice still holds: of every width measured at 4 to 200 units of
+  // within 1 %), so one figure does for every block length. They are those of an older kernel (a tile takes 235 to 300 today, settling 5200 for
+  // the largest tables to 11 000 for 64 steps with protected windows), and the choice still holds: of every width measured at 4 to 200 units of
   // 256 to 9830 slots (158 points: b = 32 and 64 with G = 4, b = 16 with G = 1, N = 2 or 3 C, drifting and clustered keys) the one chosen is
   // within 0.8 % of the best, but for 1024 slots with G = 4 and up to 32 units, where four CTAs would take 2 % less (4 units, b = 32, 100.7 / 98.6
   // us; 32 units, b = 64, 137.5 / 134.9).

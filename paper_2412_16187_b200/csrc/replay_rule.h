@@ -3,7 +3,7 @@
 
 namespace he {
 
-// Smallest max_budget of the block kernel. It has one CTA per SM and pays a block's settling (5500 to 11 500 cycles, with 8-bit codes
+// Smallest max_budget of the block kernel. It has one CTA per SM and pays a block's settling (5200 to 11 000 cycles, with 8-bit codes
 // up to 130 000) whatever the budget; the CUDA-core kernels scan every slot at every step, several units per SM. us with CUDA cores / block kernel:
 //   up to one unit per SM the block kernel is ahead from the smallest budgets where the register kernel exists (64 slots, G = 4,
 //   b = 32, N = 2 C: 38 / 31) and from 128 slots where it does not (G = 8, b = 64: 66 / 53); codes of 8 bits are not split off there, though on
